@@ -41,11 +41,20 @@ __device__ __forceinline__ int64_t graph_of(const int64_t *graph_ptr, int G, int
 }
 
 // ---------------------------------------------------------------------------------------------
-// Aggregation, one warp per destination vertex, lanes over channels (d <= 64):
+// Aggregation, one warp per destination vertex:
 //   mode 0: Y_i = (1/deg_i) sum_{j in N(i)} X_j               (A_mean X)
 //   mode 1: Y_j = sum_{i in N(j)} X_i / deg_i                 (A_mean^T X, graph symmetric)
 //   mode 2: Y_i = 0.5 X_i + 0.5 sum_{j in N(i)} X_j / sqrt(deg_i deg_j)   (lazy normalised walk)
 // accumulate: Y += result instead of Y = result.
+__device__ __forceinline__ float edge_weight(int mode, const int64_t *row_ptr, int64_t j, float degi)
+{
+    if (mode == 0) return 1.f;
+    const float dj = (float)(row_ptr[j + 1] - row_ptr[j]);
+    return mode == 1 ? 1.f / dj : rsqrtf(degi * dj);
+}
+
+// Any width d <= 64, lanes over channels, neighbours one after the other: the widths and alignments
+// that the vector kernel below does not take.
 __global__ void aggregate_kernel(int64_t N, const int64_t *row_ptr, const int32_t *col, const float *X,
                                  int d, float *Y, int mode, int accumulate)
 {
@@ -76,6 +85,68 @@ __global__ void aggregate_kernel(int64_t N, const int64_t *row_ptr, const int32_
         }
         if (lane < d) Y[i * d + lane] = accumulate ? Y[i * d + lane] + a0 : a0;
         if (lane + 32 < d) Y[i * d + lane + 32] = accumulate ? Y[i * d + lane + 32] + a1 : a1;
+    }
+}
+
+// Rows of D = 8, 16 or 64 floats on a 16-byte boundary: a row is D / 4 lanes of 16 bytes, so a warp
+// reads 128 / D neighbours at once (2 of the 64-wide rows, 8 of the 16-wide).  The warp takes its
+// columns 32 at a time, one coalesced load, and every lane forms the weight of one edge; a lane
+// group then gets its neighbour and weight by shuffle, with four gathers in flight.  Bound by the
+// L2 gathers (N = 46 thousand, 1.0 M edges, D = 64: 256 MB a launch; one neighbour at a time over 32
+// lanes took 36 us, and 80 us with the transpose's weights formed once per channel group).
+template <int D>
+__global__ void __launch_bounds__(256) aggregate_vec_kernel(int64_t N, const int64_t *row_ptr, const int32_t *col,
+                                                            const float *X, float *Y, int mode, int accumulate)
+{
+    constexpr int LPR = D / 4;              // lanes of a row
+    constexpr int NB = 32 / LPR;            // neighbours at once
+    const int lane = threadIdx.x & 31, sub = lane / LPR, c4 = lane % LPR;
+    const int64_t wglob = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const float4 *X4 = reinterpret_cast<const float4 *>(X);
+    for (int64_t i = wglob; i < N; i += nw) {
+        const int64_t e0 = row_ptr[i], e1 = row_ptr[i + 1];
+        const float degi = (float)(e1 - e0);
+        float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int64_t eb = e0; eb < e1; eb += 32) {
+            const int cnt = (int)min((int64_t)32, e1 - eb);
+            int j = 0;
+            float w = 0.f;
+            if (lane < cnt) {
+                j = col[eb + lane];
+                w = edge_weight(mode, row_ptr, j, degi);
+            }
+#pragma unroll 4
+            for (int k = 0; k < cnt; k += NB) {
+                const int jj = __shfl_sync(0xFFFFFFFFu, j, (k + sub) & 31);
+                const float ww = __shfl_sync(0xFFFFFFFFu, w, (k + sub) & 31);
+                if (k + sub < cnt) {
+                    const float4 v = X4[(int64_t)jj * LPR + c4];
+                    a.x += ww * v.x; a.y += ww * v.y; a.z += ww * v.z; a.w += ww * v.w;
+                }
+            }
+        }
+#pragma unroll
+        for (int o = LPR; o < 32; o <<= 1) {
+            a.x += __shfl_xor_sync(0xFFFFFFFFu, a.x, o);
+            a.y += __shfl_xor_sync(0xFFFFFFFFu, a.y, o);
+            a.z += __shfl_xor_sync(0xFFFFFFFFu, a.z, o);
+            a.w += __shfl_xor_sync(0xFFFFFFFFu, a.w, o);
+        }
+        if (sub == 0) {
+            if (mode == 0 && e1 > e0) { a.x /= degi; a.y /= degi; a.z /= degi; a.w /= degi; }
+            if (mode == 2) {
+                const float4 x = X4[i * LPR + c4];
+                a.x = 0.5f * x.x + 0.5f * a.x; a.y = 0.5f * x.y + 0.5f * a.y;
+                a.z = 0.5f * x.z + 0.5f * a.z; a.w = 0.5f * x.w + 0.5f * a.w;
+            }
+            float4 *y = reinterpret_cast<float4 *>(Y) + i * LPR + c4;
+            if (accumulate) {
+                const float4 o = *y;
+                a.x += o.x; a.y += o.y; a.z += o.z; a.w += o.w;
+            }
+            *y = a;
+        }
     }
 }
 
@@ -169,57 +240,65 @@ __device__ __forceinline__ void split_bf16x2(float x0, float x1, uint32_t &hi, u
     lo = (uint32_t)__bfloat16_as_ushort(l0) | ((uint32_t)__bfloat16_as_ushort(l1) << 16);
 }
 
-// H = ReLU([X | AGG] [Ws; Wn] + b): K = 2 DIN, 64 outputs = 8 column tiles.
+// H = ReLU([X | AGG] [Ws; Wn] + b): K = 2 DIN, 64 outputs = 8 column tiles.  Bound by reading X and
+// AGG and writing H once.  The rows of X and of AGG that a warp's tile needs are all in flight before
+// the first is multiplied (64 registers for DIN = 64: 8 KB a warp, 128 KB an SM with two blocks), and
+// a block stays for several tiles (at most two blocks per SM), since laying the weights out as pairs
+// costs as much as a tile (2,432 blocks that each laid them out for about one tile per warp: 161 us at
+// N = 390 thousand, DIN = 64).
 template <int DIN>
-__global__ void __launch_bounds__(256) dense_fwd_mma_kernel(int64_t N, const float *X, const float *AGG,
-                                                            const uint16_t *Ws, const uint16_t *Wn,
-                                                            const float *b, float *H)
+__global__ void __launch_bounds__(256, 2) dense_fwd_mma_kernel(int64_t N, const float *X, const float *AGG,
+                                                               const uint16_t *Ws, const uint16_t *Wn,
+                                                               const float *b, float *H)
 {
     constexpr int K = 2 * DIN, KP = K / 2 + 4;           // pairs per output column (+4: banks)
+    constexpr int KS = DIN / 16;                          // k-steps of X, and of AGG
     __shared__ uint32_t wt[HID * KP];                     // [n][k pair]: (k, k+1) of output n
     for (int t = threadIdx.x; t < HID * (K / 2); t += blockDim.x) {
-        const int n = t / (K / 2), kp = t % (K / 2), k = 2 * kp;
-        const uint16_t w0 = k < DIN ? Ws[k * HID + n] : Wn[(k - DIN) * HID + n];
-        const uint16_t w1 = k + 1 < DIN ? Ws[(k + 1) * HID + n] : Wn[(k + 1 - DIN) * HID + n];
-        wt[n * KP + kp] = (uint32_t)w0 | ((uint32_t)w1 << 16);
+        const int n = t % HID, kp = t / HID, k = 2 * kp;  // a warp reads 32 consecutive columns
+        const uint16_t *W = k < DIN ? Ws + k * HID : Wn + (k - DIN) * HID;
+        wt[n * KP + kp] = (uint32_t)W[n] | ((uint32_t)W[HID + n] << 16);
     }
     __syncthreads();
     const int lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
     const int64_t wglob = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    float bias[8][2];
-#pragma unroll
-    for (int nt = 0; nt < 8; ++nt) { bias[nt][0] = b[nt * 8 + 2 * q]; bias[nt][1] = b[nt * 8 + 2 * q + 1]; }
     for (int64_t tile = wglob; tile * 16 < N; tile += nw) {
         const int64_t r0 = tile * 16 + g, r1 = r0 + 8;
+        float2 v[2][KS][4];
+#pragma unroll
+        for (int m = 0; m < 2; ++m) {
+            const float *src = m == 0 ? X : AGG;
+#pragma unroll
+            for (int ks = 0; ks < KS; ++ks)
+#pragma unroll
+                for (int h = 0; h < 4; ++h) {
+                    const int64_t r = (h & 1) ? r1 : r0;
+                    const int kk = ks * 16 + 2 * q + ((h & 2) ? 8 : 0);
+                    v[m][ks][h] = r < N ? *reinterpret_cast<const float2 *>(src + r * DIN + kk) : make_float2(0.f, 0.f);
+                }
+        }
         float acc[8][4];
 #pragma unroll
         for (int nt = 0; nt < 8; ++nt) {
-            acc[nt][0] = acc[nt][2] = bias[nt][0];
-            acc[nt][1] = acc[nt][3] = bias[nt][1];
+            acc[nt][0] = acc[nt][2] = __ldg(b + nt * 8 + 2 * q);
+            acc[nt][1] = acc[nt][3] = __ldg(b + nt * 8 + 2 * q + 1);
         }
 #pragma unroll
-        for (int ks = 0; ks < K / 16; ++ks) {
-            const float *src = ks * 16 < DIN ? X : AGG;     // a k-step never straddles the two
-            const int kk = (ks * 16) % DIN + 2 * q;
-            const float2 z = make_float2(0.f, 0.f);
-            const float2 v00 = r0 < N ? *reinterpret_cast<const float2 *>(src + r0 * DIN + kk) : z;
-            const float2 v10 = r1 < N ? *reinterpret_cast<const float2 *>(src + r1 * DIN + kk) : z;
-            const float2 v01 = r0 < N ? *reinterpret_cast<const float2 *>(src + r0 * DIN + kk + 8) : z;
-            const float2 v11 = r1 < N ? *reinterpret_cast<const float2 *>(src + r1 * DIN + kk + 8) : z;
-            uint32_t ah[4], al[4];
-            split_bf16x2(v00.x, v00.y, ah[0], al[0]);
-            split_bf16x2(v10.x, v10.y, ah[1], al[1]);
-            split_bf16x2(v01.x, v01.y, ah[2], al[2]);
-            split_bf16x2(v11.x, v11.y, ah[3], al[3]);
+        for (int m = 0; m < 2; ++m)
 #pragma unroll
-            for (int nt = 0; nt < 8; ++nt) {
-                const uint32_t *wr = wt + (nt * 8 + g) * KP + ks * 8 + q;
-                const uint32_t b0 = wr[0], b1 = wr[4];
-                mma_bf16_16816(acc[nt], ah, b0, b1);
-                mma_bf16_16816(acc[nt], al, b0, b1);
+            for (int ks = 0; ks < KS; ++ks) {
+                uint32_t ah[4], al[4];
+#pragma unroll
+                for (int h = 0; h < 4; ++h) split_bf16x2(v[m][ks][h].x, v[m][ks][h].y, ah[h], al[h]);
+#pragma unroll
+                for (int nt = 0; nt < 8; ++nt) {
+                    const uint32_t *wr = wt + (nt * 8 + g) * KP + (m * KS + ks) * 8 + q;
+                    const uint32_t b0 = wr[0], b1 = wr[4];
+                    mma_bf16_16816(acc[nt], ah, b0, b1);
+                    mma_bf16_16816(acc[nt], al, b0, b1);
+                }
             }
-        }
 #pragma unroll
         for (int nt = 0; nt < 8; ++nt) {
             const int c = nt * 8 + 2 * q;
@@ -289,51 +368,158 @@ __global__ void __launch_bounds__(256) dense_bwd_mma_kernel(int64_t N, const uin
     }
 }
 
-// out[din x dout] += A^T B over the rows of a chunk; A: N x din, B: N x dout (dout <= 64).
-// Also colsum[dout] += sum of the rows of B when colsum != null.
-__global__ void wgrad_kernel(int64_t N, const float *A, int din, const float *B, int dout, float *out,
-                             float *colsum, int64_t chunk)
+// out[din x dout] += A^T B over the rows of a chunk; A: N x din, B: N x dout (both at most 64 wide).
+// Also colsum[dout] += sum of the rows of B when colsum != null.  One block of 512 threads per SM:
+// tiles of 32 rows go through shared memory (the next tile's loads are in flight while this one is
+// multiplied), a thread keeps a 4 x 4 block of the product in registers (two 16-byte shared loads
+// for 16 multiply-adds), and the 512 / (4 DK) thread groups take different rows of a tile.  Each
+// tile is summed on its own before it joins the running sum, so a sum is a tree of 16 (or 4), then
+// tiles, then blocks.  Bound by the FP32 multiply-adds.  (One block per 1,024 rows with two shared
+// loads per multiply-add took 480 us at N = 46 thousand, DK = 64, 45 blocks; with it a training batch
+// of 16 graphs took 2.57 ms, with this kernel and the two above and below 0.38 ms.)  DK = 16 or 64
+// is din rounded up; columns and rows beyond the matrices are zeros.
+constexpr int WG_T = 512, WG_R = 32;
+
+// tile rows [t0, t0 + 32) of M (N x d, d <= DP): this thread's share, as DP * 32 / 512 floats
+template <int DP>
+__device__ __forceinline__ void wg_load(const float *M, int d, int64_t t0, int64_t r1, bool vec, float (&v)[DP * WG_R / WG_T])
 {
-    extern __shared__ float sm[];
-    float *sa = sm;                      // [32][din]
-    float *sb = sm + 32 * din;           // [32][dout]
+    constexpr int PER = DP * WG_R / WG_T;          // 1 (DP = 16) or 4 (DP = 64)
+    if (PER == 4 && vec) {                         // d == DP, rows contiguous, 16-byte aligned
+        const int o = threadIdx.x * 4;
+        const float4 x = t0 + o / DP < r1 ? *reinterpret_cast<const float4 *>(M + t0 * DP + o) : make_float4(0.f, 0.f, 0.f, 0.f);
+        v[0] = x.x; v[1 % PER] = x.y; v[2 % PER] = x.z; v[3 % PER] = x.w;
+    } else {
+#pragma unroll
+        for (int u = 0; u < PER; ++u) {
+            const int o = threadIdx.x * PER + u, rr = o / DP, k = o % DP;
+            v[u] = k < d && t0 + rr < r1 ? M[(t0 + rr) * d + k] : 0.f;
+        }
+    }
+}
+
+template <int DP>
+__device__ __forceinline__ void wg_store(float *s, const float (&v)[DP * WG_R / WG_T])
+{
+    constexpr int PER = DP * WG_R / WG_T;
+    if (PER == 4) *reinterpret_cast<float4 *>(s + threadIdx.x * 4) = make_float4(v[0], v[1 % PER], v[2 % PER], v[3 % PER]);
+    else s[threadIdx.x] = v[0];
+}
+
+template <int DK>
+__global__ void __launch_bounds__(WG_T, 1) wgrad_kernel(int64_t N, const float *A, int din, const float *B, int dout,
+                                                        float *out, float *colsum, int64_t chunk, int vec)
+{
+    constexpr int TG = DK * HID / 16;              // threads of a group: one 4 x 4 block of out each
+    constexpr int NG = WG_T / TG, RG = WG_R / NG;  // groups, rows of a tile per group
+    __shared__ __align__(16) float sa[2][WG_R * DK];
+    __shared__ __align__(16) float sb[2][WG_R * HID];
+    __shared__ __align__(16) float red[DK * HID];
     const int64_t r0 = (int64_t)blockIdx.x * chunk, r1 = min(N, r0 + chunk);
-    const int outs = din * dout;
-    float acc[16];
+    const int grp = threadIdx.x / TG, ty = (threadIdx.x % TG) / 16, tx = threadIdx.x % 16;
+    float acc[4][4];
 #pragma unroll
-    for (int q = 0; q < 16; ++q) acc[q] = 0.f;
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
     float cs = 0.f;
-    for (int64_t t0 = r0; t0 < r1; t0 += 32) {
-        const int rows = (int)min((int64_t)32, r1 - t0);
+    float va[DK * WG_R / WG_T], vb[HID * WG_R / WG_T];
+    wg_load<DK>(A, din, r0, r1, vec & 1, va);
+    wg_load<HID>(B, dout, r0, r1, (vec >> 1) & 1, vb);
+    int buf = 0;
+    for (int64_t t0 = r0; t0 < r1; t0 += WG_R, buf ^= 1) {
+        // two buffers: the barrier below also says that everyone is done with the tile before last
+        wg_store<DK>(sa[buf], va);
+        wg_store<HID>(sb[buf], vb);
         __syncthreads();
-        for (int t = threadIdx.x; t < 32 * din; t += blockDim.x) {
-            const int rr = t / din, k = t % din;
-            sa[t] = rr < rows ? A[(t0 + rr) * din + k] : 0.f;
+        if (t0 + WG_R < r1) {
+            wg_load<DK>(A, din, t0 + WG_R, r1, vec & 1, va);
+            wg_load<HID>(B, dout, t0 + WG_R, r1, (vec >> 1) & 1, vb);
         }
-        for (int t = threadIdx.x; t < 32 * dout; t += blockDim.x) {
-            const int rr = t / dout, c = t % dout;
-            sb[t] = rr < rows ? B[(t0 + rr) * dout + c] : 0.f;
-        }
-        __syncthreads();
+        float s[4][4];
 #pragma unroll
-        for (int q = 0; q < 16; ++q) {
-            const int o = threadIdx.x + q * blockDim.x;
-            if (o < outs) {
-                const int k = o / dout, c = o % dout;
-                float s = 0.f;
-                for (int rr = 0; rr < 32; ++rr) s += sa[rr * din + k] * sb[rr * dout + c];
-                acc[q] += s;
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) s[i][j] = 0.f;
+#pragma unroll
+        for (int rr = 0; rr < RG; ++rr) {
+            const float4 x = *reinterpret_cast<const float4 *>(&sa[buf][(grp * RG + rr) * DK + 4 * ty]);
+            const float4 y = *reinterpret_cast<const float4 *>(&sb[buf][(grp * RG + rr) * HID + 4 * tx]);
+            const float xs[4] = {x.x, x.y, x.z, x.w}, ys[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) s[i][j] += xs[i] * ys[j];
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) acc[i][j] += s[i][j];
+        if (colsum) {                              // thread: column t % 64, 4 rows of the tile
+            float c = 0.f;
+#pragma unroll
+            for (int rr = 0; rr < WG_R * HID / WG_T; ++rr)
+                c += sb[buf][(threadIdx.x / HID + rr * (WG_T / HID)) * HID + threadIdx.x % HID];
+            cs += c;
+        }
+    }
+    // the groups' products meet in shared memory, then one 16-byte atomic per four outputs
+    for (int g = 0; g < NG; ++g) {
+        __syncthreads();
+        if (grp == g) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                float4 *q = reinterpret_cast<float4 *>(&red[(4 * ty + i) * HID + 4 * tx]);
+                float4 o = g ? *q : make_float4(0.f, 0.f, 0.f, 0.f);
+                o.x += acc[i][0]; o.y += acc[i][1]; o.z += acc[i][2]; o.w += acc[i][3];
+                *q = o;
             }
         }
-        if (colsum && threadIdx.x < dout)
-            for (int rr = 0; rr < 32; ++rr) cs += sb[rr * dout + threadIdx.x];
     }
+    __syncthreads();
+    if (vec & 4) {                                 // dout == 64 and out 16-byte aligned
+        for (int t = threadIdx.x; t < din * (HID / 4); t += WG_T)
+            atomicAdd(reinterpret_cast<float4 *>(out) + t, *reinterpret_cast<const float4 *>(&red[4 * t]));
+    } else {
+        for (int t = threadIdx.x; t < din * dout; t += WG_T)
+            atomicAdd(&out[t], red[(t / dout) * HID + t % dout]);
+    }
+    if (colsum) {
+        __syncthreads();
+        if (threadIdx.x < HID) red[threadIdx.x] = 0.f;
+        __syncthreads();
+        atomicAdd(&red[threadIdx.x % HID], cs);
+        __syncthreads();
+        if (threadIdx.x < dout) atomicAdd(&colsum[threadIdx.x], red[threadIdx.x]);
+    }
+}
+
+// the same for one column B (dout == 1): out[k] += sum_i A[i][k] B[i].  Bound by reading A once:
+// lanes over columns, the four thread groups take every fourth row.
+__global__ void __launch_bounds__(256) wgrad1_kernel(int64_t N, const float *A, int din, const float *B, float *out,
+                                                     float *colsum, int64_t chunk)
+{
+    __shared__ float red[4][HID + 1];
+    const int64_t r0 = (int64_t)blockIdx.x * chunk, r1 = min(N, r0 + chunk);
+    const int k = threadIdx.x % HID, grp = threadIdx.x / HID;
+    float acc = 0.f, cs = 0.f;
+    for (int64_t t0 = r0 + grp; t0 < r1; t0 += 4 * 8) {
+        float s = 0.f, c = 0.f;
 #pragma unroll
-    for (int q = 0; q < 16; ++q) {
-        const int o = threadIdx.x + q * blockDim.x;
-        if (o < outs && acc[q] != 0.f) atomicAdd(&out[o], acc[q]);
+        for (int u = 0; u < 8; ++u) {
+            const int64_t r = t0 + 4 * u;
+            const float bv = r < r1 ? B[r] : 0.f;
+            if (k < din && r < r1) s += A[r * din + k] * bv;
+            c += bv;
+        }
+        acc += s;
+        cs += c;
     }
-    if (colsum && threadIdx.x < dout && cs != 0.f) atomicAdd(&colsum[threadIdx.x], cs);
+    red[grp][k] = acc;
+    if (k == 0) red[grp][HID] = cs;
+    __syncthreads();
+    if (threadIdx.x < din) atomicAdd(&out[threadIdx.x], (red[0][k] + red[1][k]) + (red[2][k] + red[3][k]));
+    if (colsum && threadIdx.x == 0) atomicAdd(colsum, (red[0][HID] + red[1][HID]) + (red[2][HID] + red[3][HID]));
 }
 
 // z = H wo + bo
@@ -575,6 +761,19 @@ int grid_for(int64_t work, int per_block)
     return (int)g;
 }
 
+// 8-, 16- and 64-wide rows (the network's) on a 16-byte boundary take the vector kernel, other widths
+// and alignments the general one.
+void launch_aggregate(int64_t N, const int64_t *row_ptr, const int32_t *col, const float *X, int d, float *Y,
+                      int mode, int accumulate, cudaStream_t st)
+{
+    const int grid = grid_for(N * 32, 256);
+    const bool vec = aligned(X, 16) && aligned(Y, 16);
+    if (vec && d == 64) aggregate_vec_kernel<64><<<grid, 256, 0, st>>>(N, row_ptr, col, X, Y, mode, accumulate);
+    else if (vec && d == 16) aggregate_vec_kernel<16><<<grid, 256, 0, st>>>(N, row_ptr, col, X, Y, mode, accumulate);
+    else if (vec && d == 8) aggregate_vec_kernel<8><<<grid, 256, 0, st>>>(N, row_ptr, col, X, Y, mode, accumulate);
+    else aggregate_kernel<<<grid, 256, 0, st>>>(N, row_ptr, col, X, d, Y, mode, accumulate);
+}
+
 }  // namespace
 
 extern "C" {
@@ -602,8 +801,7 @@ int gdi_mpnn_aggregate(int64_t N, const int64_t *row_ptr, const int32_t *col, co
                        float *Y, int32_t mode, int32_t accumulate, void *stream)
 {
     if (N < 1 || d < 1 || d > 64 || mode < 0 || mode > 2) return GDI_ERR_INVALID_ARG;
-    aggregate_kernel<<<grid_for(N * 32, 256), 256, 0, (cudaStream_t)stream>>>(N, row_ptr, col, X, d, Y, mode,
-                                                                              accumulate);
+    launch_aggregate(N, row_ptr, col, X, d, Y, mode, accumulate, (cudaStream_t)stream);
     return cudaGetLastError() == cudaSuccess ? GDI_OK : GDI_ERR_CUDA;
 }
 
@@ -612,7 +810,7 @@ int gdi_mpnn_dense_fwd(int64_t N, const float *X, const float *AGG, int32_t din,
 {
     if (N < 1 || din < 1 || din > 64) return GDI_ERR_INVALID_ARG;
     cudaStream_t st = (cudaStream_t)stream;
-    const int tb = (int)min((N + 15) / 16 * 32 / 256 + 1, (int64_t)152 * 16);   // tiles of 16 rows, 8 warps a block
+    const int tb = (int)min(((N + 15) / 16 + 7) / 8, (int64_t)152 * 2);         // tiles of 16 rows, 8 warps a block
     // the tensor-core kernels move activations in pairs (8-byte accesses)
     const bool pairs = aligned(X, 8) && aligned(AGG, 8) && aligned(H, 8);
     if (din == 64 && pairs) {
@@ -650,10 +848,21 @@ int gdi_mpnn_wgrad(int64_t N, const float *A, int32_t din, const float *B, int32
                    float *colsum, void *stream)
 {
     if (N < 1 || din < 1 || din > 64 || dout < 1 || dout > 64) return GDI_ERR_INVALID_ARG;
-    const int64_t chunk = 1024;
+    cudaStream_t st = (cudaStream_t)stream;
+    if (dout == 1) {
+        // two blocks per SM, at least 64 rows each
+        const int64_t chunk = max((int64_t)64, (N + 303) / 304);
+        wgrad1_kernel<<<(int)((N + chunk - 1) / chunk), 256, 0, st>>>(N, A, din, B, out, colsum, chunk);
+        return cudaGetLastError() == cudaSuccess ? GDI_OK : GDI_ERR_CUDA;
+    }
+    // one block per SM, whole tiles of 32 rows
+    const int64_t chunk = ((N + 151) / 152 + WG_R - 1) / WG_R * WG_R;
     const int grid = (int)((N + chunk - 1) / chunk);
-    const size_t smem = 32 * (size_t)(din + dout) * sizeof(float);
-    wgrad_kernel<<<grid, 256, smem, (cudaStream_t)stream>>>(N, A, din, B, dout, out, colsum, chunk);
+    const int dk = din <= 16 ? 16 : 64;
+    const int vec = (din == dk && aligned(A, 16) ? 1 : 0) | (dout == HID && aligned(B, 16) ? 2 : 0) |
+                    (dout == HID && aligned(out, 16) ? 4 : 0);
+    if (dk == 16) wgrad_kernel<16><<<grid, WG_T, 0, st>>>(N, A, din, B, dout, out, colsum, chunk, vec);
+    else wgrad_kernel<64><<<grid, WG_T, 0, st>>>(N, A, din, B, dout, out, colsum, chunk, vec);
     return cudaGetLastError() == cudaSuccess ? GDI_OK : GDI_ERR_CUDA;
 }
 
@@ -675,7 +884,7 @@ int gdi_mpnn_loss(int32_t G, const int64_t *graph_ptr, const float *z, const int
                   float *stats, float *dz, float *loss, void *stream)
 {
     if (G < 1) return GDI_ERR_INVALID_ARG;
-    loss_kernel<<<G, 256, 0, (cudaStream_t)stream>>>(G, graph_ptr, z, y, lambda, stats, dz, loss);
+    loss_kernel<<<G, 1024, 0, (cudaStream_t)stream>>>(G, graph_ptr, z, y, lambda, stats, dz, loss);
     return cudaGetLastError() == cudaSuccess ? GDI_OK : GDI_ERR_CUDA;
 }
 

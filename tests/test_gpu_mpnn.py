@@ -172,3 +172,73 @@ def test_trained_start_against_untrained_and_plain_annealer(gdi):
     assert reached["trained"] > reached["untrained"]
     assert reached["trained"] >= 8 and reached["random_T3.0"] == 0
     assert reached["noise_channel0"] >= 8
+
+
+def _ring_graph(n, extra, seed):
+    """A ring with `extra` random chords and, past vertex n - 3, two isolated vertices and a leaf."""
+    from gdi_synth.graphs import from_edges
+    rng = np.random.default_rng(seed)
+    m = n - 3
+    u, v = np.arange(m), (np.arange(m) + 1) % m
+    u = np.concatenate([u, rng.integers(0, m, extra), [0]])
+    v = np.concatenate([v, rng.integers(0, m, extra), [n - 1]])
+    return from_edges(n, u, v)
+
+
+@pytest.mark.parametrize("d,shift", [(8, 0), (16, 0), (64, 0), (64, 1), (5, 0), (33, 0)])
+@pytest.mark.parametrize("mode", [0, 1, 2])
+def test_aggregate_widths_and_alignments(gdi, d, shift, mode):
+    """Every width the vector kernel takes, the same width off a 16-byte boundary, and other widths;
+    rows of 0, 1 and more than 32 neighbours.  Sums of at most 70 float32 products: 1e-5 of the
+    largest value."""
+    import torch
+    from paper_1908_00210_gb300 import learn
+    g = _ring_graph(203, 900, d)
+    hub = np.arange(1, 70)
+    from gdi_synth.graphs import from_edges
+    u, v, _ = g.edges()
+    g = from_edges(g.n, np.concatenate([u, np.zeros(69, np.int64)]), np.concatenate([v, hub]))
+    rng = np.random.default_rng(d + mode)
+    x = rng.standard_normal((g.n, d)).astype(np.float32)
+    y0 = rng.standard_normal((g.n, d)).astype(np.float32)
+    buf = torch.empty(2 * (g.n * d + 4), device="cuda")
+    X = buf[shift:shift + g.n * d]
+    Y = buf[g.n * d + 4 - (g.n * d) % 4 + shift:][:g.n * d]
+    rp, col = torch.from_numpy(g.row_ptr).cuda(), torch.from_numpy(g.col).cuda()
+    f = [ref.mean_aggregate, ref.mean_aggregate_T, ref.lazy_walk][mode](g.row_ptr, g.col, x.astype(np.float64))
+    f = np.where(np.isfinite(f), f, 0.0)
+    for acc in (0, 1):
+        X.copy_(torch.from_numpy(x.ravel()))
+        Y.copy_(torch.from_numpy(y0.ravel()))
+        rc = learn.lib().gdi_mpnn_aggregate(g.n, rp.data_ptr(), col.data_ptr(), X.data_ptr(), d, Y.data_ptr(), mode,
+                                            acc, None)
+        assert rc == 0
+        want = f + acc * y0
+        got = Y.cpu().numpy().reshape(g.n, d)
+        assert np.max(np.abs(got - want)) < 1e-5 * np.max(np.abs(want)), (acc, np.max(np.abs(got - want)))
+
+
+@pytest.mark.parametrize("n", [1, 31, 33, 4865, 9801])
+@pytest.mark.parametrize("din,dout,shift", [(64, 64, 0), (16, 64, 0), (64, 64, 1), (7, 64, 0), (64, 1, 0), (16, 5, 0),
+                                            (33, 33, 0), (1, 1, 0)])
+def test_wgrad_shapes(gdi, n, din, dout, shift):
+    """Row counts around the tiles and the blocks' chunks, widths that fill the tile and not, operands
+    off a 16-byte boundary; the result is added to what is there.  A float32 sum of n products of
+    standard normals, summed in trees of depth about 40, is expected 6e-8 sqrt(40 n) off, 4.5 times that at
+    the worst of 4,096: 1e-5 (1 + sqrt(n)) is some five times as much."""
+    import torch
+    from paper_1908_00210_gb300 import learn
+    rng = np.random.default_rng(n + din + dout)
+    a, b = rng.standard_normal((n, din)).astype(np.float32), rng.standard_normal((n, dout)).astype(np.float32)
+    o0, c0 = rng.standard_normal((din, dout)).astype(np.float32), rng.standard_normal(dout).astype(np.float32)
+
+    def dev(x):
+        t = torch.empty(x.size + 4, device="cuda")[shift:shift + x.size]
+        t.copy_(torch.from_numpy(x.ravel()))
+        return t
+    A, Bm, out, cs = dev(a), dev(b), dev(o0), dev(c0)
+    assert learn.lib().gdi_mpnn_wgrad(n, A.data_ptr(), din, Bm.data_ptr(), dout, out.data_ptr(), cs.data_ptr(), None) == 0
+    want = o0 + a.astype(np.float64).T @ b.astype(np.float64)
+    tol = 1e-5 * (1 + np.sqrt(n))
+    assert np.max(np.abs(out.cpu().numpy().reshape(din, dout) - want)) < tol
+    assert np.max(np.abs(cs.cpu().numpy() - (c0 + b.astype(np.float64).sum(0)))) < tol
