@@ -242,3 +242,31 @@ def test_wgrad_shapes(gdi, n, din, dout, shift):
     tol = 1e-5 * (1 + np.sqrt(n))
     assert np.max(np.abs(out.cpu().numpy().reshape(din, dout) - want)) < tol
     assert np.max(np.abs(cs.cpu().numpy() - (c0 + b.astype(np.float64).sum(0)))) < tol
+
+
+@pytest.mark.parametrize("steps", [1, 5, 6])
+def test_features_one_launch_and_the_rest(gdi, steps):
+    """Graphs at the edges of the one-launch walk: one vertex, isolated vertices, sizes around the 32-row
+    slices, a hub whose degree exceeds the counting sort's bins, a graph too dense for the laid-out
+    columns and one too large for a block (both walked by the grid-wide kernel), and a batch whose mean is too
+    large for a block.  Features are float32 sums of at most 9,100 terms, scaled to unit RMS: 1e-4."""
+    from gdi_synth.graphs import from_edges, star_graph
+    from paper_1908_00210_gb300 import learn
+    rng = np.random.default_rng(steps)
+    dense = np.triu_indices(400, 1)
+    keep = rng.random(dense[0].size) < 0.5
+    small = [from_edges(1, np.zeros(0), np.zeros(0)), _ring_graph(31, 5, 1), _ring_graph(32, 9, 2), _ring_graph(33, 0, 3),
+             star_graph(700), from_edges(400, dense[0][keep], dense[1][keep]), _ring_graph(2047, 9000, 4)]
+    big = _ring_graph(9101, 3000, 5)
+    for gs in (small, small + [big] + small[1:], [big, big]):
+        gp, u = batch_union(gs)
+        ids = np.arange(3, 3 + len(gs), dtype=np.uint32)
+        b = learn.GraphBatch.from_graphs(gs, graph_ids=ids)
+        m = learn.MPNN(seed=1, feat_seed=77, steps=steps)
+        X = m.features(b).cpu().numpy()
+        Xr = ref.features(gp, ids, u.row_ptr, u.col, 77, steps)
+        for q in range(len(gs)):
+            if gs[q].n == 1:
+                continue                       # one vertex: centred to 0, scaled by 1e-12
+            s = slice(gp[q], gp[q + 1])
+            assert np.max(np.abs(X[s] - Xr[s])) < 1e-4, (q, np.max(np.abs(X[s] - Xr[s])))
