@@ -73,7 +73,7 @@ struct gdi_ctx {
     int device = 0;
     int32_t Q = 0, R = 1, A = 0, B = 1, W = 0;
     int64_t N = 0, nnz = 0;
-    int32_t max_n = 0, max_window = 0, max_degree = 0, max_class = 0;
+    int32_t max_n = 0, max_window = 0, max_degree = 0, max_class = 0, max_class_nnz = 0;
     int32_t path = 0;                        // GDI_PATH_*
     DevBuf<uint8_t> g_packed, g_rflags;
     DevBuf<int16_t> g_tables;
@@ -141,6 +141,7 @@ struct gdi_ctx {
         P.max_window = max_window;
         P.max_degree = max_degree;
         P.max_class = max_class;
+        P.max_class_nnz = max_class_nnz;
         return P;
     }
     void release()
@@ -311,6 +312,7 @@ struct HostRankSpace {
     std::vector<int64_t> rp;
     std::vector<uint32_t> cr;
     int32_t max_n = 0, max_window = 0, max_class = 0, max_degree = 0;
+    int64_t max_class_nnz = 0;
 };
 
 int build_rank_space(const gdi_graph *g, const std::vector<int64_t> &inst, int32_t W, HostRankSpace &H)
@@ -429,6 +431,10 @@ int build_rank_space(const gdi_graph *g, const std::vector<int64_t> &inst, int32
         }
         rp[(size_t)N] = e_out;
     }
+    for (int32_t k = 0; k < Q; ++k)
+        for (int32_t c = class_off[(size_t)k]; c + 1 < class_off[(size_t)k + 1]; ++c)
+            H.max_class_nnz = std::max(H.max_class_nnz, rp[(size_t)(inst[(size_t)k] + class_ptr[(size_t)c + 1])] -
+                                                            rp[(size_t)(inst[(size_t)k] + class_ptr[(size_t)c])]);
     return GDI_OK;
 }
 
@@ -484,6 +490,7 @@ int gdi_create(gdi_ctx **out, const gdi_graph *g, const gdi_model *m)
     c->max_window = H.max_window;
     c->max_class = H.max_class;
     c->max_degree = H.max_degree;
+    c->max_class_nnz = H.max_class_nnz <= (1 << 20) ? (int32_t)H.max_class_nnz : 0;
     // window costs for the grid path's weighted split: a rank costs its degree plus a constant for
     // its threshold and its share of the window sort (both measured as about 12 neighbour reads)
     if (Q == 1 && c->W >= 1) {
@@ -516,8 +523,9 @@ int gdi_create(gdi_ctx **out, const gdi_graph *g, const gdi_model *m)
     GDI_UP(c->row_ptr, rp);
     GDI_UP(c->col, cr);
     if (H.max_n <= 32767) {
-        // 16-bit columns for the CTA-resident kernels' neighbour sums (half the CSR bytes)
-        std::vector<uint16_t> c16(cr.size());
+        // 16-bit columns for the CTA-resident kernels' neighbour sums (half the CSR bytes), padded so
+        // that whole 16-byte pieces can be read up to the last column
+        std::vector<uint16_t> c16(cr.size() + 8, 0);
         for (size_t e = 0; e < cr.size(); ++e)
             c16[e] = (uint16_t)((cr[e] & 0x7FFFu) | ((cr[e] >> 31) << 15));
         GDI_UP(c->col16, c16);
@@ -728,8 +736,7 @@ int gdi_anneal(gdi_ctx *c, const gdi_schedule *S, const gdi_run *run)
     R.item_counter = c->item_counter.p;
 
     size_t need = 0;
-    int H = 0;
-    gdi_cta_smem_bytes(P, R, c->block, &need, &H);
+    gdi_cta_smem_bytes(P, R, c->block, &need);
     int max_optin = 0, sms = 0;
     cudaDeviceGetAttribute(&max_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
@@ -796,8 +803,9 @@ int gdi_anneal(gdi_ctx *c, const gdi_schedule *S, const gdi_run *run)
         if (c->max_degree > 32767) return fail(GDI_ERR_TOO_LARGE, "degree above 32767 on the grid-scale path");
         int spc = 0, wpc = 0;
         size_t smem = 0;
+        bool counted = false;
         const int nblk = c->grid_limit > 0 ? std::min(c->grid_limit, sms) : sms;
-        if (gdi_grid_plan(P, max_row, nblk, (size_t)max_optin, &spc, &wpc, &smem) != 0)
+        if (gdi_grid_plan(P, max_row, nblk, (size_t)max_optin, &spc, &wpc, &smem, &counted) != 0)
             return fail(GDI_ERR_TOO_LARGE, "grid-scale plan needs " + std::to_string(smem) +
                                                " bytes of shared memory per block; use a smaller W");
         const int D = c->max_degree;
@@ -812,7 +820,7 @@ int gdi_anneal(gdi_ctx *c, const gdi_schedule *S, const gdi_run *run)
         if (e == cudaSuccess) e = c->g_rties.alloc((size_t)8 * 152 * 4);
         if (e == cudaSuccess) e = c->g_rparams.alloc(32);
         if (e == cudaSuccess) e = c->g_bar.alloc(4);
-        if (e == cudaSuccess && c->W <= 256) e = c->g_hfield.alloc((size_t)2 * c->N);
+        if (e == cudaSuccess && counted) e = c->g_hfield.alloc((size_t)2 * c->N);
         if (e != cudaSuccess) return fail(GDI_ERR_OOM, "device allocation failed (grid scratch)");
         cudaMemsetAsync(c->g_err.p, 0, sizeof(int32_t), st);
         cudaMemsetAsync(c->g_status.p, 0, 16 * sizeof(int32_t), st);
@@ -823,7 +831,7 @@ int gdi_anneal(gdi_ctx *c, const gdi_schedule *S, const gdi_run *run)
             c->inject_limit = 0;
         }
         const int32_t *wbnd = nullptr;
-        if (c->W <= 256 && !c->wcost_off.empty()) {
+        if (counted && !c->wcost_off.empty()) {
             if (c->wbnd_blocks != nblk || c->wbnd_wpc != wpc) {
                 const int ncls = (int)c->wcost_off.size() - 1;
                 std::vector<int32_t> bnd((size_t)ncls * (nblk + 1));
@@ -837,7 +845,7 @@ int gdi_anneal(gdi_ctx *c, const gdi_schedule *S, const gdi_run *run)
             }
             wbnd = c->g_wbnd.p;
         }
-        int ke = gdi_launch_grid_anneal(P, R, X, c->spins.p, nblk, spc, wpc, smem, wbnd, &timer, st);
+        int ke = gdi_launch_grid_anneal(P, R, X, c->spins.p, nblk, spc, wpc, smem, counted, wbnd, &timer, st);
         if (ke) return cuda_fail((cudaError_t)ke, "grid anneal launch");
         ke = gdi_launch_grid_finish(P, R, X, c->spins.p, (run->flags & GDI_FLAG_NO_REPAIR) ? 0 : 1, st);
         if (ke) return cuda_fail((cudaError_t)ke, "grid finish kernels");

@@ -273,7 +273,7 @@ struct GSmem {
     int32_t *longq;    // [spc]
     int16_t *wtab;     // [wpc][8][TW]
     int32_t *win;      // [wpc][8]
-    int32_t *hist;     // [NWARP][2][HB] (tabulated path) or [NWARP][HA] (sorted path)
+    int32_t *hist;     // [NWARP][2][HB] (tabulated path)
     int32_t *nchunk;   // [spc] chunk counts of the long rows
     int16_t *ctab;     // [P][TW]
     uint32_t *row;     // [max_row]
@@ -905,7 +905,8 @@ __global__ void __launch_bounds__(GB, 1) gdi_grid_anneal_kernel(GridArgs A)
 // entering G up from c: at most 160 / 16 + 15 byte lookups, without a grid barrier.  Where the walk leaves the lattice, the block whose table failed publishes its exact
 // outgoing G (it knows its own entering G and replays exactly), and the walk continues from it.
 // One grid barrier per class remains: the next class reads this class's spins.
-constexpr int SMAXW = 256;
+constexpr int SMAXW = 256;              // windows a warp holds in registers
+constexpr int CMAXW = 32767;            // windows whose counts fit 16 bits
 constexpr int RUN = 16;                 // blocks per run table
 __host__ __device__ inline int nruns(int P) { return (P + RUN - 1) / RUN; }
 // per replica warp: run tables [nruns] + own-run block tables [RUN] + descent tables [RUN]
@@ -913,8 +914,7 @@ __host__ __device__ inline int walk_slots(int P) { return nruns(P) + 2 * RUN; }
 
 
 struct SortedLayout {
-    size_t off_h, off_gam, off_es, off_s0, off_fm, off_fbits, off_longq, off_smap, off_hist, off_walk, off_row,
-        off_misc, total;
+    size_t off_h, off_gam, off_es, off_s0, off_fm, off_fbits, off_longq, off_smap, off_walk, off_row, off_misc, total;
     int fw;                             // words of one replica's flip bitmap
     int gs;                             // threshold row stride (ints): >= spc + 7, 4 mod 32
     int es;                             // E* row stride (int16): >= spc + 7, 16 mod 32; 0 = no E* rows
@@ -924,7 +924,9 @@ __host__ __device__ inline SortedLayout sorted_layout(int spc, int wpc, int max_
 {
     SortedLayout L;
     size_t o = 0;
-    L.off_h = o; o = align16(o + (size_t)spc * 8 * sizeof(int16_t));      // fields, then rel
+    // the fields; once the thresholds are made, the counting warps' bins
+    const size_t fields = (size_t)spc * 8 * sizeof(int16_t), bins = (size_t)NWARP * WBINS * sizeof(uint32_t);
+    L.off_h = o; o = align16(o + (fields > bins ? fields : bins));
     // thresholds [r][gs]: a row starts 4 words (16 banks' worth of bytes) after the previous
     // one's bank, so the 8 replicas' 16-byte stores of one quad of ranks hit disjoint banks
     L.gs = ((spc + 3 + 31) & ~31) + 4;
@@ -933,12 +935,11 @@ __host__ __device__ inline SortedLayout sorted_layout(int spc, int wpc, int max_
     L.es = es_rows ? ((spc + 3 + 31) & ~31) + 16 : 0;
     L.off_es = o; o = align16(o + (size_t)L.es * 8 * sizeof(int16_t));
     L.off_s0 = o; o = align16(o + (size_t)spc);
-    L.off_fm = o; o = align16(o + (size_t)((spc + 3) / 4) * sizeof(uint32_t));
+    L.off_fm = o; o = align16(o + (size_t)((spc + 3) / 4) * sizeof(uint32_t));   // racy variant's flips
     L.fw = spc / 32 + 2;
     L.off_fbits = o; o = align16(o + (size_t)8 * L.fw * sizeof(uint32_t));
     L.off_longq = o; o = align16(o + (size_t)2 * spc * sizeof(int32_t));   // long rows, chunk counts
     L.off_smap = o; o = align16(o + (size_t)wpc * 8 * 2 * sizeof(StageMap));
-    L.off_hist = o; o = align16(o + (size_t)NWARP * HA * sizeof(int32_t));    // exact-replay bins
     L.off_walk = o; o = align16(o + (size_t)8 * walk_slots(P) * NT);
     L.off_row = o; o = align16(o + (size_t)(max_row + 4) * sizeof(uint32_t));
     L.off_misc = o; o = align16(o + 64 * sizeof(int64_t));
@@ -1061,7 +1062,8 @@ __device__ bool fetch_valid(const int8_t *a, int na, int8_t *da, const int8_t *b
     return ok;
 }
 
-// SL = members per lane of a window sort (1, 2, 4 or 8): one instantiation per window size class
+// SL = members per lane of a window (1, 2, 4 or 8; 0: windows above 256, members read from shared
+// memory): one instantiation per window size class
 template <int SL>
 __global__ void __launch_bounds__(GB, 1) gdi_grid_sorted_kernel(GridArgs A)
 {
@@ -1073,18 +1075,16 @@ __global__ void __launch_bounds__(GB, 1) gdi_grid_sorted_kernel(GridArgs A)
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int spc = A.spc;
     const SortedLayout L = sorted_layout(spc, A.wpc, R.max_row, Pb, A.es_pre);
-    int16_t *hb = reinterpret_cast<int16_t *>(smem_raw + L.off_h);   // fields [i*8 + r], then rel [r*spc + i]
+    int16_t *hb = reinterpret_cast<int16_t *>(smem_raw + L.off_h);   // fields [i*8 + r], then the counting warps' bins
     int32_t *gam = reinterpret_cast<int32_t *>(smem_raw + L.off_gam);
     int16_t *esb = reinterpret_cast<int16_t *>(smem_raw + L.off_es);   // E* drawn ahead [r][L.es]
     uint8_t *s0 = smem_raw + L.off_s0;
-    uint32_t *fm = reinterpret_cast<uint32_t *>(smem_raw + L.off_fm);
     StageMap *smap = reinterpret_cast<StageMap *>(smem_raw + L.off_smap);
-    int32_t *hist = reinterpret_cast<int32_t *>(smem_raw + L.off_hist);
+    uint32_t *hist = reinterpret_cast<uint32_t *>(smem_raw + L.off_h);
     int8_t *walk = reinterpret_cast<int8_t *>(smem_raw + L.off_walk);
     uint32_t *fbits = reinterpret_cast<uint32_t *>(smem_raw + L.off_fbits);   // [r][fw] fast-path flips
     GSmem S = {};
     S.longq = reinterpret_cast<int32_t *>(smem_raw + L.off_longq);
-    S.hist = hist;
     S.nchunk = S.longq + spc;
     S.row = reinterpret_cast<uint32_t *>(smem_raw + L.off_row);
     S.misc = reinterpret_cast<int64_t *>(smem_raw + L.off_misc);
@@ -1165,16 +1165,36 @@ __global__ void __launch_bounds__(GB, 1) gdi_grid_sorted_kernel(GridArgs A)
             int32_t *gamc = gam + (a0 & 3);
             range_thresholds(A, S, a0, a1, sw, true, 0, gamc, 1, L.gs, s0, hb, rlen, Tsw, true,
                              have_es ? esb : nullptr, L.es, threadIdx.x < nrep ? Gc : nullptr, gcl);
-            // ---- sorted groups: rel values and stage maps of every (window, replica)
-            for (int task = warp; task < nwin * nrep; task += NWARP) {
-                const int kk = task / nrep, r = task % nrep;
-                const int ws = kk * W, wlen = min(W, ns - ws);
-                const int32_t *gr = gamc + (size_t)r * L.gs;
-                int16_t *rr = hb + (size_t)r * spc;
-                StageMap *o = smap + ((size_t)kk * 8 + r) * 2;
-                window_maps<SL>(gr, s0, rr, ws, wlen, r, Gc[r], o);
+            // ---- counts and stage maps of every (window, replica)
+            if constexpr (SL > 0) {
+                for (int task = warp; task < nwin * nrep; task += NWARP) {
+                    const int kk = task / nrep, r = task % nrep;
+                    const int ws = kk * W, wlen = min(W, ns - ws);
+                    window_maps<SL>(gamc + (size_t)r * L.gs, s0, ws, wlen, r, Gc[r], hist + (size_t)warp * WBINS,
+                                    smap + ((size_t)kk * 8 + r) * 2);
+                }
+            } else {
+                // large windows are few: several warps count the parts of one (window, replica)
+                const int ntask = nwin * nrep;
+                const int parts = ntask > 0 && ntask < NWARP ? NWARP / ntask : 1;
+                const int per = NWARP / parts, grp = warp / parts, part = warp % parts;
+                for (int t0 = 0; t0 < ntask; t0 += per) {
+                    const int task = t0 + grp;
+                    const bool mine = grp < per && task < ntask;
+                    const int kk = task / nrep, r = task % nrep;
+                    uint32_t *bins = hist + (size_t)grp * WBINS;
+                    if (mine && part == 0)
+                        for (int b = lane; b < WBINS; b += 32) bins[b] = 0;
+                    __syncthreads();
+                    if (mine) {
+                        const int ws = kk * W, we = min(ws + W, ns), len = ((we - ws + parts - 1) / parts + 31) & ~31;
+                        count_members(gamc + (size_t)r * L.gs, s0, min(ws + part * len, we), min(ws + (part + 1) * len, we), r,
+                                      Gc[r], bins);
+                    }
+                    __syncthreads();
+                    if (mine && part == 0) bins_to_maps(bins, smap + ((size_t)kk * 8 + r) * 2);
+                }
             }
-            for (int i = threadIdx.x; i < (ns + 3) / 4; i += GB) fm[i] = 0;
             for (int i = threadIdx.x; i < 8 * L.fw; i += GB) fbits[i] = 0;
             if (threadIdx.x == 0) npush = 0;
             __syncthreads();
@@ -1267,19 +1287,28 @@ __global__ void __launch_bounds__(GB, 1) gdi_grid_sorted_kernel(GridArgs A)
                     const int own = __shfl_sync(0xFFFFFFFFu, (idx >= 0 && idx < 32) ? t0 : t1, idx & 31);
                     const bool need_exact = idx < 0 || own < 0;
                     uint32_t *fb = fbits + (size_t)r * L.fw;
-                    int32_t x = gin - c0;
+                    int32_t gout = gin;
                     const int32_t *gr = gamc + (size_t)r * L.gs;
-                    const int16_t *rr = hb + (size_t)r * spc;
-                    int32_t *bins = hist + (size_t)warp * HA;
                     for (int kk = 0; kk < nwin; ++kk) {
                         const int ws = kk * W, we = min(ws + W, ns);
-                        // a narrow window's rel values hold on the lattice only (see window_maps)
-                        const bool on = smap[((size_t)kk * 8 + r) * 2].narrow ? (x >= -NT && x <= NT - 2)
-                                                                            : (x >= -FAST_X && x <= FAST_X);
-                        x = on ? replay_window<SL>(rr, s0, r, ws, we, x, plus_first, fb, W)
-                               : window_replay_exact(gr, s0, r, ws, we, c0 + x, plus_first, bins, fm) - c0;
+                        const int32_t x = gout - c0;
+                        const int t = x >= -NT && x <= NT - 2 ? (x + NT) >> 1 : -1;
+                        const StageMap *maps = smap + ((size_t)kk * 8 + r) * 2;
+                        if constexpr (SL > 0) {
+                            gout = replay_mapped<SL>(gr, s0, r, ws, we, gout, plus_first, t, maps,
+                                                     [&](const uint32_t (&wb)[SL]) { flips_to_bitmap<SL>(wb, ws, we, fb, W); });
+                        } else {
+                            int K1, K2;
+                            mapped_flips(plus_first, t, maps, K1, K2);
+                            gout = replay_large(gr, s0, r, ws, we, gout, plus_first, K1, K2, [&](int i0, unsigned bits) {
+                                if (lane == 0) {
+                                    const int sh = i0 & 31;
+                                    fb[i0 >> 5] |= bits << sh;
+                                    if (sh && bits >> (32 - sh)) fb[(i0 >> 5) + 1] |= bits >> (32 - sh);
+                                }
+                            });
+                        }
                     }
-                    const int32_t gout = c0 + x;
                     if (lane == 0) {
                         if (need_exact) {
                             st_release_u64(exg + (size_t)p * 8 + r,
@@ -1323,7 +1352,6 @@ __global__ void __launch_bounds__(GB, 1) gdi_grid_sorted_kernel(GridArgs A)
                 }
                 uint32_t f = 0;
                 if (i < ns) {
-                    f = (fm[i >> 2] >> (8 * (i & 3))) & 0xFFu;
                     for (int r = 0; r < nrep; ++r) f |= ((fbits[(size_t)r * L.fw + (i >> 5)] >> (i & 31)) & 1u) << r;
                 }
                 if (f) X.packed[base + a0 + i] = (uint8_t)(s0[i] ^ f);
@@ -1434,7 +1462,6 @@ __global__ void __launch_bounds__(GB, 1) gdi_grid_racy_kernel(GridArgs A)
     uint32_t *fm = reinterpret_cast<uint32_t *>(smem_raw + L.off_fm);
     GSmem S = {};
     S.longq = reinterpret_cast<int32_t *>(smem_raw + L.off_longq);
-    S.hist = reinterpret_cast<int32_t *>(smem_raw + L.off_hist);
     S.nchunk = S.longq + spc;
     S.row = reinterpret_cast<uint32_t *>(smem_raw + L.off_row);
     S.misc = reinterpret_cast<int64_t *>(smem_raw + L.off_misc);
@@ -1697,7 +1724,7 @@ __global__ void repair_apply_kernel(int8_t *spins, int64_t N, int nrep, const ui
 
 // ---------------------------------------------------------------------------------------------
 int gdi_grid_plan(const GdiDevProblem &P, int max_row, int sms, size_t smem_limit, int *spc, int *wpc,
-                  size_t *smem)
+                  size_t *smem, bool *counted)
 {
     if (P.num_instances != 1 || P.W < 1) return -1;
     // the kernels' static shared memory (class bounds, a few words) counts against the same limit
@@ -1707,18 +1734,22 @@ int gdi_grid_plan(const GdiDevProblem &P, int max_row, int sms, size_t smem_limi
     const int w = (wp + sms - 1) / sms;
     *wpc = w < 1 ? 1 : w;
     *spc = *wpc * P.W;
-    if (P.W <= SMAXW) {
+    *counted = true;
+    if (P.W <= CMAXW) {
         // the cost-weighted split stays within the even share of windows per block: more shared
         // memory per block (less L1) costs more than the finer balance gains
         // with rows for the E* drawn ahead when they fit, else without
         *smem = sorted_layout(*spc, *wpc, max_row, sms, true).total;
         if (*smem <= smem_limit) return 0;
         *smem = sorted_layout(*spc, *wpc, max_row, sms, false).total;
-        return *smem <= smem_limit ? 0 : -1;
+        if (*smem <= smem_limit) return 0;
+        if (P.W <= SMAXW) return -1;
     }
-    // the tabulated path keeps the long rows' chunk counts in the histogram area, and its exact
+    // larger windows whose buffers do not fit the counted path (its E* and push queue take about 10 bytes
+    // a rank more): tabulated.  It keeps the long rows' chunk counts in the histogram area, and its exact
     // chain fallback the thresholds, fields, start signs and bins of one block's windows (one
     // replica)
+    *counted = false;
     if ((size_t)*spc > (size_t)NWARP * 2 * HB) return -1;
     if ((size_t)*spc * 7 + 64 + HA * sizeof(int32_t) > (size_t)NWARP * 2 * HB * sizeof(int32_t)) return -1;
     *smem = grid_layout(*spc, *wpc, sms, max_row).total;
@@ -1766,19 +1797,20 @@ void gdi_grid_window_bounds(const int64_t *cost, const int64_t *cost_off, int nu
 }
 
 int gdi_launch_grid_anneal(const GdiDevProblem &P, const GdiDevRun &R, const GdiGridScratch &X,
-                           int8_t *spins, int sms, int spc, int wpc, size_t smem, const int32_t *wbnd,
-                           GdiKernelTimer *timer, void *stream)
+                           int8_t *spins, int sms, int spc, int wpc, size_t smem, bool counted,
+                           const int32_t *wbnd, GdiKernelTimer *timer, void *stream)
 {
     cudaStream_t st = (cudaStream_t)stream;
     const bool racy = (R.flags & GDI_DEV_RACY) != 0;
-    const bool sorted = P.W <= SMAXW && !racy;
+    const bool sorted = counted && !racy;
     if (racy) smem = sorted_layout(spc, wpc, R.max_row, sms, false).total;
     const void *kern = racy ? (const void *)gdi_grid_racy_kernel
                      : !sorted ? (const void *)gdi_grid_anneal_kernel
                      : P.W <= 32 ? (const void *)gdi_grid_sorted_kernel<1>
                      : P.W <= 64 ? (const void *)gdi_grid_sorted_kernel<2>
                      : P.W <= 128 ? (const void *)gdi_grid_sorted_kernel<4>
-                                  : (const void *)gdi_grid_sorted_kernel<8>;
+                     : P.W <= SMAXW ? (const void *)gdi_grid_sorted_kernel<8>
+                                    : (const void *)gdi_grid_sorted_kernel<0>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return (int)e;
     int per_sm = 0;

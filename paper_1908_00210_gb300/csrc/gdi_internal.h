@@ -19,13 +19,15 @@ struct GdiDevProblem {
     const int64_t *row_ptr;          // [N+1] rank-space CSR offsets
     const uint32_t *col;             // [nnz] local neighbour rank | (weight < 0) << 31
     const uint16_t *col16;           // [nnz] the same in 16 bits (rank | (weight < 0) << 15) when
-                                     // every instance has at most 32,767 vertices, else null
+                                     // every instance has at most 32,767 vertices, else null; 16-byte
+                                     // aligned and readable 8 entries past its end
     const int32_t *rank_of;          // [N] original vertex -> global rank
     int32_t A, B, W;
     int32_t max_n;                   // largest instance
     int32_t max_window;              // largest window (W or class size) over instances
     int32_t max_degree;
     int32_t max_class;               // largest colour class
+    int32_t max_class_nnz;           // most row entries of one colour class (0: not known, or above 2^20)
 };
 
 // Global scratch of the grid-scale path (single large instance).
@@ -69,6 +71,7 @@ struct GdiDevRun {
     int32_t *err;                    // device error word (0 = ok)
     const int32_t *item_order;       // [Q*R] items, largest instance first (CTA path)
     int32_t *item_counter;           // [1] next item to take (zeroed before the launch)
+    int32_t cta_opts, cta_stage;     // CTA path's shared-memory options (gdi_kernels.cu), set by the launch
 };
 
 // record a failure for gdi_last_error() (gdi_api.cpp); returns code
@@ -82,13 +85,14 @@ int gdi_launch_init(const GdiDevProblem &P, int8_t *spins, const int8_t *init_or
                     uint32_t key0, uint32_t key1, void *stream);
 int gdi_launch_cta_anneal(const GdiDevProblem &P, const GdiDevRun &R, int block, int grid_limit,
                           void *stream, int *grid_used, size_t *smem_used);
-int gdi_cta_smem_bytes(const GdiDevProblem &P, const GdiDevRun &R, int block, size_t *bytes, int *hist);
+int gdi_cta_smem_bytes(const GdiDevProblem &P, const GdiDevRun &R, int block, size_t *bytes);
 // resident CTA-path blocks per SM for this problem and block size (0 when the block does not fit)
 int gdi_cta_blocks_per_sm(const GdiDevProblem &P, const GdiDevRun &R, int block, int *per_sm);
 // Grid plan for `sms` blocks: spans of ranks (spc) and windows (wpc) per block and per class, and
-// the dynamic shared memory; -1 if the instance does not fit smem_limit.
+// the dynamic shared memory; counted: the counted-window kernel runs it (else the tabulated one); -1 if
+// the instance does not fit smem_limit.
 int gdi_grid_plan(const GdiDevProblem &P, int max_row, int sms, size_t smem_limit, int *spc, int *wpc,
-                  size_t *smem);
+                  size_t *smem, bool *counted);
 // Host: first window of every block, per class, for the sorted-window grid path.  cost[k] is the
 // cost of window k of the class (windows of one class consecutive, class c starting at
 // cost_off[c]); every block gets at most wpc windows.  bnd has num_classes * (blocks + 1) entries.
@@ -101,8 +105,8 @@ struct GdiKernelTimer {
     int n;                           // pairs recorded
 };
 int gdi_launch_grid_anneal(const GdiDevProblem &P, const GdiDevRun &R, const GdiGridScratch &X,
-                           int8_t *spins, int sms, int spc, int wpc, size_t smem, const int32_t *wbnd,
-                           GdiKernelTimer *timer, void *stream);
+                           int8_t *spins, int sms, int spc, int wpc, size_t smem, bool counted,
+                           const int32_t *wbnd, GdiKernelTimer *timer, void *stream);
 int gdi_launch_grid_finish(const GdiDevProblem &P, const GdiDevRun &R, const GdiGridScratch &X,
                            int8_t *spins, int do_repair, void *stream);
 int gdi_launch_gather_spins(const GdiDevProblem &P, const int8_t *spins_rank, int8_t *out_orig,

@@ -17,15 +17,16 @@
 //        s_i = -1 flips iff G <= gamma_i = floor((E* + B h_i - 4A) / 4A)
 //      (dE = B s_i h_i + 4A (1 - s_i G), Eq. 4-6 with G counting the other spins).
 //   2. the +1 group and the -1 group of the window each see the exact running G in threshold
-//      order (Algorithm 3's atomically updated G, serialised): with d_i = G - gamma_i (+1 group) or
-//      gamma_i - G (-1 group), the k-th spin in d-descending order flips iff d_(k) >= 2k.  The
-//      number of flips K and the cut-off d* come from a shared-memory histogram of d with suffix
-//      sums; ties at d* are resolved by rank with a block prefix count.
+//      order (Algorithm 3's atomically updated G, serialised): with e_i = G - gamma_i (+1 group) or
+//      gamma_i - G (-1 group), the k-th spin in e-descending order flips iff e_(k) >= 2k, ties by rank.
+//      The number of flips K and the last margin come from counts of e, not from a sort.
 //   3. G changes by -2K (+1 group) or +2K (-1 group): one shared-memory update per group, the
 //      block-level analogue of the paper's atomicAdd on G.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
+
+#include <algorithm>
 
 #include "gdi_device.cuh"
 #include "gdi_internal.h"
@@ -39,11 +40,8 @@ using namespace gdi::win;
 // ---------------------------------------------------------------------------------------------
 struct Smem {
     int8_t *sig;        // [max_n] spins of the current item, rank order
-    int8_t *s0;         // [max_window] group (sign at window start) of each window position
-    int8_t *flag;       // [max_n] repair decisions
-    int32_t *gam;       // [max_window] flip thresholds
-    int32_t *hist;      // [H] histogram of d / suffix counts
-    uint32_t *row;      // [max_row] table row of the current sweep
+    int8_t *flag;       // [max_n] repair decisions (during the sweeps: bins)
+    uint32_t *row;      // [1 or 2][row_stride] table rows
     int32_t *red32;     // [BS/32 + 2]
     int64_t *red64;     // [BS/32 + 2]
     int32_t *G;         // running magnetisation of the item
@@ -63,167 +61,40 @@ __device__ __forceinline__ int32_t local_field(const GdiDevProblem &P, int64_t b
     return h;
 }
 
-// the same sum over the 16-bit column copy (instances of at most 32,767 vertices)
-__device__ __forceinline__ int32_t local_field16(const GdiDevProblem &P, int64_t base, int32_t r,
-                                                 const int8_t *sig)
-{
-    const int64_t e0 = P.row_ptr[base + r], e1 = P.row_ptr[base + r + 1];
-    int32_t h = 0;
-    for (int64_t e = e0; e < e1; ++e) {
-        const uint32_t c = __ldg(P.col16 + e);
-        const int32_t s = sig[c & 0x7FFFu];
-        h += (c >> 15) ? -s : s;
-    }
-    return h;
-}
-
-// count of members of group grp with d >= x (exact d), block-wide
-template <int BS>
-__device__ int32_t count_ge(const Smem &S, int32_t Wn, int grp, int32_t Gc, int64_t x)
-{
-    int32_t c = 0;
-    for (int32_t p = threadIdx.x; p < Wn; p += BS) {
-        if (S.s0[p] != grp) continue;
-        const int64_t d = grp > 0 ? (int64_t)Gc - S.gam[p] : (int64_t)S.gam[p] - Gc;
-        c += (d >= x);
-    }
-    return block_sum<BS, int32_t>(c, S.red32);
-}
-
-// Decide the flips of one group of a window and apply them (see file header, step 2).
-template <int BS>
-__device__ void select_and_flip(const Smem &S, int32_t wlo, int32_t Wn, int grp, int H)
-{
-    __syncthreads();
-    const int32_t Gc = *S.G;
-    for (int32_t b = threadIdx.x; b < H; b += BS) S.hist[b] = 0;
-    __syncthreads();
-    for (int32_t p = threadIdx.x; p < Wn; p += BS) {
-        if (S.s0[p] != grp) continue;
-        const int32_t d = grp > 0 ? Gc - S.gam[p] : S.gam[p] - Gc;
-        if (d >= 0) atomicAdd(&S.hist[d < H - 1 ? d : H - 1], 1);
-    }
-    __syncthreads();
-    // suffix sums in place: hist[x] := #{members with min(d, H-1) >= x}
-    {
-        const int32_t c = (H + BS - 1) / BS;
-        const int32_t b0 = threadIdx.x * c;
-        const int32_t b1 = min(b0 + c, H);
-        int32_t loc = 0;
-        for (int32_t b = b0; b < b1; ++b) loc += S.hist[b];
-        int32_t total;
-        const int32_t before = block_excl_scan<BS>(loc, S.red32, &total);
-        int32_t run = total - before;
-        for (int32_t b = b0; b < b1; ++b) {
-            const int32_t hb = S.hist[b];
-            S.hist[b] = run;
-            run -= hb;
-        }
-    }
-    __syncthreads();
-    const int32_t n_top = S.hist[H - 1];
-    const bool safe = n_top <= (H - 1) / 2 + 1;
-    int32_t K, t;
-    int64_t dstar;
-    if (safe) {
-        int32_t cnt = 0;
-        for (int32_t k = threadIdx.x; 2 * k <= H - 1; k += BS) cnt += (S.hist[2 * k] >= k + 1);
-        K = block_sum<BS, int32_t>(cnt, S.red32);
-        if (K == 0) return;
-        int32_t cx = 0;
-        for (int32_t x = threadIdx.x; x < H; x += BS) cx += (S.hist[x] >= K);
-        dstar = block_sum<BS, int32_t>(cx, S.red32) - 1;
-        const int32_t above = (dstar + 1 <= H - 1) ? S.hist[dstar + 1] : 0;
-        t = K - above;
-    } else {
-        // exact counting passes (rare: more than H/2 members far above the running G)
-        const int32_t n0 = count_ge<BS>(S, Wn, grp, Gc, 0);
-        int32_t lo = 0, hi = n0 - 1;
-        while (lo < hi) {
-            const int32_t mid = (lo + hi + 1) >> 1;
-            if (count_ge<BS>(S, Wn, grp, Gc, 2 * (int64_t)mid) >= mid + 1) lo = mid; else hi = mid - 1;
-        }
-        K = lo + 1;
-        int64_t dl = 2 * (int64_t)(K - 1), dh = (int64_t)1 << 32;
-        while (dl < dh) {
-            const int64_t mid = (dl + dh + 1) >> 1;
-            if (count_ge<BS>(S, Wn, grp, Gc, mid) >= K) dl = mid; else dh = mid - 1;
-        }
-        dstar = dl;
-        t = K - count_ge<BS>(S, Wn, grp, Gc, dstar + 1);
-    }
-    // apply: contiguous position chunks so that the tie prefix follows rank order
-    const int32_t chunk = (Wn + BS - 1) / BS;
-    const int32_t p0 = threadIdx.x * chunk;
-    const int32_t p1 = min(p0 + chunk, Wn);
-    int32_t ties = 0;
-    for (int32_t p = p0; p < p1; ++p) {
-        if (S.s0[p] != grp) continue;
-        int64_t d = grp > 0 ? (int64_t)Gc - S.gam[p] : (int64_t)S.gam[p] - Gc;
-        if (safe && d > H - 1) d = H - 1;
-        ties += (d == dstar);
-    }
-    int32_t total;
-    int32_t idx = block_excl_scan<BS>(ties, S.red32, &total);
-    for (int32_t p = p0; p < p1; ++p) {
-        if (S.s0[p] != grp) continue;
-        int64_t d = grp > 0 ? (int64_t)Gc - S.gam[p] : (int64_t)S.gam[p] - Gc;
-        if (safe && d > H - 1) d = H - 1;
-        bool flip = d > dstar;
-        if (d == dstar) flip = (idx++ < t);
-        if (flip) S.sig[wlo + p] = (int8_t)(-grp);
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) *S.G = Gc - 2 * grp * K;
-}
-
 // Algorithm 2 (the paper's standard annealer, GDI_FLAG_STANDARD): every spin of the window forms
 // the balance term from the complete graph of Eq. 5, i.e. sums all n spins itself (an O(n) read per
 // spin, which is what the decoupled G of Algorithm 3 removes), on the state at the window start,
 // and flips iff its draw accepts dE = B s h + 4A (1 - s G) -- the same test as "G >= gamma" with
 // the threshold gamma of step 1.  All decisions are taken before any spin of the window changes.
+// The sums are read 16 spins at a time (every lane of a warp reads the same 16 bytes) into four
+// independent dot-product chains.
 template <int BS>
-__device__ void standard_window(const Smem &S, int32_t wlo, int32_t Wn, int32_t n)
+__device__ void standard_window(const Smem &S, const int32_t *gam, const int8_t *s0, int32_t wlo, int32_t Wn, int32_t n)
 {
-    __syncthreads();
     int32_t dG = 0;
-    // the spin vector is read in 4-byte words from its first 4-byte boundary on (the shared
-    // layout aligns it to 8 bytes only); the bytes before and after are read one by one
-    const int32_t head = (int32_t)((4 - (reinterpret_cast<uintptr_t>(S.sig) & 3)) & 3) < n
-                             ? (int32_t)((4 - (reinterpret_cast<uintptr_t>(S.sig) & 3)) & 3) : n;
-    const int32_t nwords = (n - head) >> 2;
-    const int32_t *sw = reinterpret_cast<const int32_t *>(S.sig + head);
+    const uint4 *sv = reinterpret_cast<const uint4 *>(S.sig);    // 16-byte aligned by the layout
+    const int32_t nv = n >> 4;
     for (int32_t p = threadIdx.x; p < Wn; p += BS) {
-        int32_t G = 0;                              // sum of all spins, read by this spin
-        for (int32_t j = 0; j < head; ++j) G += S.sig[j];
-        for (int32_t k = 0; k < nwords; ++k) G += __dp4a(sw[k], 0x01010101, 0);
-        for (int32_t j = head + 4 * nwords; j < n; ++j) G += S.sig[j];
-        const int sg = S.s0[p];
-        const bool flip = sg > 0 ? G >= S.gam[p] : G <= S.gam[p];
+        int32_t a0 = 0, a1 = 0, a2 = 0, a3 = 0;     // sum of all spins, read by this spin
+#pragma unroll 4
+        for (int32_t k = 0; k < nv; ++k) {
+            const uint4 v = sv[k];
+            a0 = __dp4a((int)v.x, 0x01010101, a0);
+            a1 = __dp4a((int)v.y, 0x01010101, a1);
+            a2 = __dp4a((int)v.z, 0x01010101, a2);
+            a3 = __dp4a((int)v.w, 0x01010101, a3);
+        }
+        for (int32_t j = 16 * nv; j < n; ++j) a0 += S.sig[j];
+        const int32_t G = (a0 + a1) + (a2 + a3);
+        const int sg = s0[p];
+        const bool flip = sg > 0 ? G >= gam[p] : G <= gam[p];
         S.flag[wlo + p] = flip ? 1 : 0;
         dG += flip ? -2 * sg : 0;
     }
     dG = block_sum<BS, int32_t>(dG, S.red32);
     for (int32_t p = threadIdx.x; p < Wn; p += BS)
-        if (S.flag[wlo + p]) S.sig[wlo + p] = (int8_t)(-S.s0[p]);
-    __syncthreads();
+        if (S.flag[wlo + p]) S.sig[wlo + p] = (int8_t)(-s0[p]);
     if (threadIdx.x == 0) *S.G += dG;
-}
-
-// cut of the item: (1/2) sum_i sum_j w_ij [s_i != s_j]
-template <int BS>
-__device__ int64_t item_cut(const GdiDevProblem &P, int64_t base, int32_t n, const Smem &S)
-{
-    int64_t c = 0;
-    for (int32_t r = threadIdx.x; r < n; r += BS) {
-        const int8_t sr = S.sig[r];
-        const int64_t e0 = P.row_ptr[base + r], e1 = P.row_ptr[base + r + 1];
-        for (int64_t e = e0; e < e1; ++e) {
-            const uint32_t cc = __ldg(P.col + e);
-            if (S.sig[cc & 0x7FFFFFFFu] != sr) c += (cc >> 31) ? -1 : 1;
-        }
-    }
-    return block_sum<BS, int64_t>(c, S.red64) / 2;
 }
 
 // #majority spins with repair key (s_i h_i) <= x, and with key == x (when eq != null)
@@ -289,25 +160,389 @@ __device__ void repair(const GdiDevProblem &P, int64_t base, int32_t n, const Sm
     __syncthreads();
 }
 
+// One pass over the item's rows, a team of lanes per row: the item's cut (the sum of the weights whose
+// ends differ, / 2).  mode 1: also counts the repair keys s_i h_i of the majority spins in hist[key + D];
+// mode 2: instead marks each majority spin's flag, 1 for a key below kappa and 2 for one equal to it.
 template <int BS>
-__global__ void __launch_bounds__(BS) gdi_cta_anneal_kernel(GdiDevProblem P, GdiDevRun R, int H)
+__device__ int64_t item_fields(const GdiDevProblem &P, int64_t base, int32_t n, int32_t mean_deg, const Smem &S, int mode,
+                               int maj, int32_t *hist, int32_t kappa)
+{
+    const int tl = mean_deg >= 16 ? 3 : (mean_deg >= 8 ? 2 : (mean_deg >= 4 ? 1 : 0));
+    const int T = 1 << tl, sub = threadIdx.x & (T - 1);
+    int64_t c = 0;
+    for (int32_t k0 = 0; k0 < n; k0 += BS >> tl) {
+        const int32_t i = k0 + ((int32_t)threadIdx.x >> tl);
+        int32_t diff = 0, deg = 0;                      // weights of the differing neighbours, of all
+        int8_t si = 0;
+        if (i < n) {
+            si = S.sig[i];
+            const int64_t e0 = P.row_ptr[base + i], e1 = P.row_ptr[base + i + 1];
+            if (P.col16) {
+                for (int64_t e = e0 + sub; e < e1; e += T) {
+                    const uint32_t cc = __ldg(P.col16 + e);
+                    const int32_t w = (cc >> 15) ? -1 : 1;
+                    deg += w;
+                    diff += S.sig[cc & 0x7FFFu] != si ? w : 0;
+                }
+            } else {
+                for (int64_t e = e0 + sub; e < e1; e += T) {
+                    const uint32_t cc = __ldg(P.col + e);
+                    const int32_t w = (cc >> 31) ? -1 : 1;
+                    deg += w;
+                    diff += S.sig[cc & 0x7FFFFFFFu] != si ? w : 0;
+                }
+            }
+        }
+        c += diff;
+        if (mode) {
+            int32_t key = deg - 2 * diff;                // s_i h_i
+            for (int o = T >> 1; o >= 1; o >>= 1) key += __shfl_xor_sync(0xFFFFFFFFu, key, o);
+            if (i < n && sub == 0) {
+                if (mode == 1) {
+                    if (si == maj) atomicAdd(&hist[key + P.max_degree], 1);
+                } else {
+                    S.flag[i] = si != maj ? 0 : (key < kappa ? 1 : (key == kappa ? 2 : 0));
+                }
+            }
+        }
+    }
+    return block_sum<BS, int64_t>(c, S.red64) / 2;
+}
+
+// Results of an annealed item: cut and G before and after the exact-balance repair (the k majority spins
+// with the smallest (s_i h_i, rank) keys flip).  The keys are counted in scratch while the cut is taken,
+// so the repair costs two more passes over the rows; where 2 max_degree + 1 bins do not fit the scratch,
+// the key bound is searched instead, a pass per step.  Ends with a block barrier.
+template <int BS>
+__device__ void finish_item(const GdiDevProblem &P, const GdiDevRun &R, int64_t base, int32_t n, int32_t mean_deg,
+                            const Smem &S, int32_t *scratch, int scratch_words, int32_t item, bool write)
+{
+    __shared__ int32_t sel[2];
+    __syncthreads();
+    const int32_t raw_G = *S.G;
+    const int32_t target = n & 1, aG = raw_G < 0 ? -raw_G : raw_G;
+    const bool fix = !(R.flags & GDI_DEV_NO_REPAIR) && aG > target;
+    const int32_t nb = 2 * P.max_degree + 1;
+    const bool counted = fix && nb <= scratch_words;
+    const int maj = raw_G > 0 ? 1 : -1;
+    if (counted) {
+        for (int32_t b = threadIdx.x; b < nb; b += BS) scratch[b] = 0;
+        __syncthreads();
+    }
+    const int64_t raw_cut = item_fields<BS>(P, base, n, mean_deg, S, counted ? 1 : 0, maj, scratch, 0);
+    int64_t fin_cut = raw_cut;
+    if (counted) {
+        const int32_t k = (aG - target) / 2;
+        __syncthreads();
+        if (threadIdx.x < 32) {
+            // kappa = the smallest key with k keys at or below it; t = how many keys equal to it flip
+            const int lane = threadIdx.x;
+            int32_t before = 0;
+            for (int32_t b0 = 0; b0 < nb; b0 += 32) {
+                int32_t x = b0 + lane < nb ? scratch[b0 + lane] : 0;
+                const int32_t own = x;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int32_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
+                    if (lane >= o) x += y;
+                }
+                const unsigned m = __ballot_sync(0xFFFFFFFFu, before + x >= k);
+                if (m) {
+                    const int f = __ffs(m) - 1;
+                    if (lane == f) {
+                        sel[0] = b0 + f - P.max_degree;
+                        sel[1] = k - (before + x - own);
+                    }
+                    break;
+                }
+                before += __shfl_sync(0xFFFFFFFFu, x, 31);
+            }
+        }
+        __syncthreads();
+        const int32_t kappa = sel[0], t = sel[1];
+        item_fields<BS>(P, base, n, mean_deg, S, 2, maj, nullptr, kappa);
+        __syncthreads();
+        // equal keys flip in rank order: contiguous chunks keep it
+        const int32_t chunk = (n + BS - 1) / BS;
+        const int32_t p0 = min((int32_t)threadIdx.x * chunk, n), p1 = min(p0 + chunk, n);
+        int32_t ties = 0;
+        for (int32_t r = p0; r < p1; ++r) ties += S.flag[r] == 2;
+        int32_t total;
+        int32_t idx = block_excl_scan<BS>(ties, S.red32, &total);
+        for (int32_t r = p0; r < p1; ++r) {
+            const int f = S.flag[r];
+            if (f == 1 || (f == 2 && idx++ < t)) S.sig[r] = (int8_t)-maj;
+        }
+        if (threadIdx.x == 0) *S.G = raw_G - 2 * maj * k;
+        __syncthreads();
+        fin_cut = item_fields<BS>(P, base, n, mean_deg, S, 0, 0, nullptr, 0);
+    } else if (fix) {
+        repair<BS>(P, base, n, S);
+        fin_cut = item_fields<BS>(P, base, n, mean_deg, S, 0, 0, nullptr, 0);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0 && write) {
+        R.raw_G[item] = raw_G;
+        R.raw_cut[item] = raw_cut;
+        R.final_G[item] = *S.G;
+        R.final_cut[item] = fin_cut;
+    }
+    __syncthreads();
+}
+
+__host__ __device__ inline size_t align16c(size_t x) { return (x + 15) & ~(size_t)15; }
+
+// what a launch keeps in shared memory beyond the necessary (GdiDevRun::cta_opts)
+constexpr int CTA_OPT_ROWS2 = 1;    // the next sweep's table row beside the current one
+constexpr int CTA_OPT_ES = 2;       // whole-block windows: the next window's E* (else drawn in place)
+constexpr int CTA_OPT_BINS = 4;     // whole-block windows: 512 bins of margins (else 16)
+// GdiDevRun::cta_stage: columns the staging buffer of the next class (window) holds; a class with more
+// is read from global memory
+
+// lanes per rank of a field sum: the layout whose longest chain of dependent reads is shortest
+// (rounds x (row / T + about 4 reads' worth of reduction and threshold latency per round))
+template <int BS>
+__device__ __forceinline__ int team_log2(int32_t nown, int32_t mean_deg)
+{
+    int best = 0x7FFFFFFF, tl = 0;
+    for (int l = 0; l <= 5; ++l) {
+        const int32_t rounds = ((nown << l) + BS - 1) / BS;
+        const int32_t chain = rounds * (((mean_deg + (1 << l) - 1) >> l) + 4);
+        if (chain < best) { best = chain; tl = l; }
+    }
+    return tl;
+}
+
+__device__ __forceinline__ void cp_async16(void *dst, const void *src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// E* of ranks [r0, r1) of an item at sweep sw (table row `row` of length rlen) into es[r - org], by threads
+// t of nth: one Philox call per aligned quad of ranks
+__device__ __forceinline__ void draw_estar(const GdiDevRun &R, int32_t r0, int32_t r1, int32_t org, int32_t q, int32_t rep,
+                                           int32_t sw, const uint32_t *row, int32_t rlen, float Tsw, int32_t *es, int t,
+                                           int nth)
+{
+    if (r1 <= r0) return;
+    for (int32_t qd = (r0 >> 2) + t; qd <= ((r1 - 1) >> 2); qd += nth) {
+        const uint4 u4 = philox4x32_10(make_uint4((uint32_t)qd, (uint32_t)sw, (uint32_t)q, (uint32_t)rep), R.key0, R.key1);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int32_t r = 4 * qd + j;
+            if (r >= r0 && r < r1) es[r - org] = estar_of(row, rlen, R.mode, word_of(u4, j), Tsw);
+        }
+    }
+}
+
+// whether columns [eb, ee), staged in whole 16-byte pieces, fit a buffer of cap columns
+__device__ __forceinline__ bool stage_fits(int64_t eb, int64_t ee, int32_t cap)
+{
+    return ((ee - (eb & ~(int64_t)7) + 7) & ~(int64_t)7) <= cap;
+}
+
+// Columns [eb, ee) and the offsets of nrows rows (bounds rp) into shared memory, by threads t of nth:
+// whole 16-byte pieces from the boundary at or before the first column (the column array is padded).
+// The caller waits (cp_async_wait_all) before its block barrier.
+__device__ __forceinline__ void stage_rows(const GdiDevProblem &P, const int64_t *rp, int32_t nrows, int64_t eb, int64_t ee,
+                                           int32_t *rofs, uint16_t *cbuf, int t, int nth)
+{
+    const int64_t al = eb & ~(int64_t)7;
+    const int32_t pieces = (int32_t)((ee - al + 7) >> 3);
+    for (int32_t k = t; k < pieces; k += nth) cp_async16(cbuf + 8 * k, P.col16 + al + 8 * (int64_t)k);
+    for (int32_t i = t; i <= nrows; i += nth) rofs[i] = (int32_t)(rp[i] - al);
+}
+
+// Flip thresholds of ranks [lo + rb, lo + re) of an item from the shared spins and E* (es[i], i counted from
+// lo), a team of 2^tl lanes per rank; put(i, sign, threshold) by each team's first lane.  rofs != null:
+// rows staged in shared memory (row i at rofs[i - rb]).  Teams are aligned lane groups of one warp; every
+// lane takes part in every round's shuffles (the round count is the block's).
+template <int BS, class Put>
+__device__ __forceinline__ void team_thresholds(const GdiDevProblem &P, const int8_t *sig, int64_t base, int32_t lo, int32_t rb,
+                                                int32_t re, int tl, const int32_t *rofs, const uint16_t *cbuf,
+                                                const int32_t *es, int a_shift, const Put &put)
+{
+    const int T = 1 << tl, sub = threadIdx.x & (T - 1);
+    for (int32_t k0 = rb; k0 < re; k0 += BS >> tl) {
+        const int32_t i = k0 + ((int32_t)threadIdx.x >> tl);
+        int32_t h = 0;
+        if (i < re) {
+            if (rofs) {
+                const int32_t e1 = rofs[i - rb + 1];
+#pragma unroll 4
+                for (int32_t e = rofs[i - rb] + sub; e < e1; e += T) {
+                    const uint32_t cc = cbuf[e];
+                    const int32_t sv = sig[cc & 0x7FFFu];
+                    h += (cc >> 15) ? -sv : sv;
+                }
+            } else {
+                const int64_t e0 = P.row_ptr[base + lo + i], e1 = P.row_ptr[base + lo + i + 1];
+                if (P.col16) {
+                    for (int64_t e = e0 + sub; e < e1; e += T) {
+                        const uint32_t cc = __ldg(P.col16 + e);
+                        const int32_t sv = sig[cc & 0x7FFFu];
+                        h += (cc >> 15) ? -sv : sv;
+                    }
+                } else {
+                    for (int64_t e = e0 + sub; e < e1; e += T) {
+                        const uint32_t cc = __ldg(P.col + e);
+                        const int32_t sv = sig[cc & 0x7FFFFFFFu];
+                        h += (cc >> 31) ? -sv : sv;
+                    }
+                }
+            }
+        }
+        for (int o = T >> 1; o >= 1; o >>= 1) h += __shfl_xor_sync(0xFFFFFFFFu, h, o);
+        if (i < re && sub == 0) {
+            const int sg = sig[lo + i];
+            const int32_t e = es[i];
+            put(i, sg, a_shift >= 0 ? gamma_of_shift(sg, h, e, P.A, P.B, a_shift) : gamma_of(sg, h, e, P.A, P.B));
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------------------------
+// CTA-resident kernel for windows that one warp does not hold: whole colour classes (W = 0), W > 256,
+// instances whose class buffers do not fit the counting kernel, and Algorithm 2.  Windows are taken one
+// after another from the exact running G.  Per window: every thread counts its thresholds' margins e
+// (the distance on the flipping side of the window-start G) into shared bins as it makes them; one warp
+// reads both groups' flips off the bins -- members flip in e order, the k-th iff e >= 2k, so the first
+// k with N(2k) <= k is the number of flips K, and the last one has e >= 2K, = 2K - 1 or = 2K - 2; the
+// second group sees the same margins shifted by the first group's 2K -- and then every thread decides its
+// ranks, equal margins by position.  Four block barriers per window (two less where no tie is cut); a
+// counting pass and a scan per group with its own barriers took about 26.  Draws and rows of the next
+// window are prepared by the other warps while one reads the bins, as in the counting kernel.
+struct CtaBlockLayout {
+    size_t red64, red32, G, row, sig, flag, gam, es, s0, rofs, cbuf, total;
+    int row_stride, nb;
+};
+
+__host__ __device__ inline CtaBlockLayout cta_block_layout(const GdiDevProblem &P, int32_t max_row, int BS, int opts,
+                                                           int32_t stage)
+{
+    CtaBlockLayout L;
+    const size_t mw = (size_t)P.max_window + 8;
+    size_t o = 0;
+    L.red64 = o; o = align16c(o + sizeof(int64_t) * (BS / 32 + 2));
+    L.red32 = o; o = align16c(o + sizeof(int32_t) * (BS / 32 + 2));
+    L.G = o; o = align16c(o + 16);
+    L.row_stride = (max_row + 3) & ~3;
+    L.row = o; o = align16c(o + sizeof(uint32_t) * (size_t)L.row_stride * ((opts & CTA_OPT_ROWS2) ? 2 : 1));
+    L.sig = o; o = align16c(o + (size_t)P.max_n);
+    // the repair flags and, during the sweeps, the bins (nb first group, 2 nb second) and the tie counts
+    // of 32 ranks each share their bytes
+    L.nb = (opts & CTA_OPT_BINS) ? 512 : 16;
+    const size_t bins = 4 * (3 * (size_t)L.nb + mw / 32 + 1), fl = (size_t)P.max_n;
+    L.flag = o; o = align16c(o + (fl > bins ? fl : bins));
+    L.gam = o; o = align16c(o + 4 * (size_t)P.max_window);
+    L.es = o; o = align16c(o + ((opts & CTA_OPT_ES) ? 4 * (size_t)P.max_window : 0));
+    L.s0 = o; o = align16c(o + (size_t)P.max_window);
+    L.rofs = o; o = align16c(o + (stage ? 4 * mw : 0));
+    L.cbuf = o; o = align16c(o + 2 * (size_t)stage);
+    L.total = o;
+    return L;
+}
+
+// one group's flips off its bins h[m] (members with margin m < lim), of which n0 members have margin >= 0,
+// by one warp: K, and (y, left) such that the members with e > y flip and of those with e == y the first
+// `left` in position order.  False when K lies beyond the bins.
+__device__ __forceinline__ bool group_flips(const int32_t *h, int lim, int32_t n0, int32_t &K, int32_t &y, int32_t &left)
+{
+    const int lane = threadIdx.x & 31;
+    int32_t above = n0;                                  // members with margin >= m0
+    for (int m0 = 0; m0 < lim; m0 += 32) {
+        const int m = m0 + lane;
+        const int32_t own = m < lim ? h[m] : 0;
+        int32_t x = own;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int32_t v = __shfl_up_sync(0xFFFFFFFFu, x, o);
+            if (lane >= o) x += v;
+        }
+        const int32_t N = above - (x - own);             // members with margin >= m
+        const unsigned hit = __ballot_sync(0xFFFFFFFFu, !(lane & 1) && m < lim && N <= (m >> 1));
+        if (hit) {
+            const int f = __ffs(hit) - 1;
+            K = (m0 + f) >> 1;
+            y = INT32_MAX;
+            left = 0;
+            if (K == 0) return true;
+            const int32_t n2 = __shfl_sync(0xFFFFFFFFu, N, f), h1 = h[2 * K - 1], h2 = h[2 * K - 2];
+            int32_t ties = 0;
+            if (n2 == K) {
+                y = 2 * K - 1;
+            } else if (n2 + h1 >= K) {
+                y = 2 * K - 1;
+                left = K - n2;
+                ties = h1;
+            } else {
+                y = 2 * K - 2;
+                left = K - n2 - h1;
+                ties = h2;
+            }
+            if (left && left == ties) { --y; left = 0; }
+            return true;
+        }
+        above -= __shfl_sync(0xFFFFFFFFu, x, 31);
+    }
+    return false;
+}
+
+// count of members of group grp (signs s0) with margin >= x relative to g, block-wide
+template <int BS>
+__device__ int32_t count_ge(const int32_t *gam, const int8_t *s0, int32_t Wn, int grp, int32_t g, int64_t x, int32_t *red)
+{
+    int32_t c = 0;
+    for (int32_t p = threadIdx.x; p < Wn; p += BS) {
+        if (s0[p] != grp) continue;
+        const int64_t d = grp > 0 ? (int64_t)g - gam[p] : (int64_t)gam[p] - g;
+        c += (d >= x);
+    }
+    return block_sum<BS, int32_t>(c, red);
+}
+
+template <int BS>
+__global__ void __launch_bounds__(BS, 1024 / BS) gdi_cta_block_kernel(GdiDevProblem P, GdiDevRun R)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    Smem S;
+    Smem S = {};
+    const bool rows2 = (R.cta_opts & CTA_OPT_ROWS2) != 0, staged = R.cta_stage > 0;
+    const bool pre = (R.cta_opts & CTA_OPT_ES) != 0;
+    const CtaBlockLayout L = cta_block_layout(P, R.max_row, BS, R.cta_opts, R.cta_stage);
+    S.red64 = reinterpret_cast<int64_t *>(smem_raw + L.red64);
+    S.red32 = reinterpret_cast<int32_t *>(smem_raw + L.red32);
+    S.G = reinterpret_cast<int32_t *>(smem_raw + L.G);
+    S.row = reinterpret_cast<uint32_t *>(smem_raw + L.row);
+    S.sig = reinterpret_cast<int8_t *>(smem_raw + L.sig);
+    S.flag = reinterpret_cast<int8_t *>(smem_raw + L.flag);
+    const int NB = L.nb;
+    int32_t *h1 = reinterpret_cast<int32_t *>(smem_raw + L.flag);      // [NB] first group, margin 0 ...
+    int32_t *h2 = h1 + NB;                                             // [2 NB] second group, margin -NB ...
+    int32_t *tcnt = h2 + 2 * NB;                                       // [windows' ranks / 32] ties
+    int32_t *gam = reinterpret_cast<int32_t *>(smem_raw + L.gam);
+    int32_t *es = pre ? reinterpret_cast<int32_t *>(smem_raw + L.es) : gam;   // in place: E*, then gamma
+    int8_t *s0 = reinterpret_cast<int8_t *>(smem_raw + L.s0);
+    int32_t *rofs = reinterpret_cast<int32_t *>(smem_raw + L.rofs);
+    uint16_t *cbuf = reinterpret_cast<uint16_t *>(smem_raw + L.cbuf);
     {
-        unsigned char *p = smem_raw;
-        S.red64 = reinterpret_cast<int64_t *>(p); p += sizeof(int64_t) * (BS / 32 + 2);
-        S.red32 = reinterpret_cast<int32_t *>(p); p += sizeof(int32_t) * (BS / 32 + 2);
-        S.G = reinterpret_cast<int32_t *>(p); p += 16;
-        S.hist = reinterpret_cast<int32_t *>(p); p += sizeof(int32_t) * H;
-        S.gam = reinterpret_cast<int32_t *>(p); p += sizeof(int32_t) * ((P.max_window + 3) & ~3);
-        S.row = reinterpret_cast<uint32_t *>(p); p += sizeof(uint32_t) * ((R.max_row + 3) & ~3);
-        S.s0 = reinterpret_cast<int8_t *>(p); p += (P.max_window + 15) & ~15;
-        S.sig = reinterpret_cast<int8_t *>(p); p += (P.max_n + 15) & ~15;
-        S.flag = reinterpret_cast<int8_t *>(p);
+        // the launch must have given the whole layout (the host sizes it with the same function)
+        uint32_t dyn;
+        asm volatile("mov.u32 %0, %%dynamic_smem_size;" : "=r"(dyn));
+        if ((size_t)dyn < L.total) {
+            if (threadIdx.x == 0 && blockIdx.x == 0) atomicCAS(R.err, 0, GDI_DEVERR_INPUT);
+            return;
+        }
     }
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const bool standard = (R.flags & GDI_DEV_STANDARD) != 0;
+    const int a_shift = (P.A > 0 && (P.A & (P.A - 1)) == 0) ? 2 + __ffs(P.A) - 1 : -1;   // log2(4A)
     const int32_t items = P.num_instances * P.replicas;
     __shared__ int32_t next_item;
+    __shared__ int32_t nge[2];                          // members with margin >= 0, by group
+    struct Decision { int32_t y[2], left[2], slow; };
+    __shared__ Decision dec;
     while (true) {
         // persistent blocks take (instance, replica) items from a queue sorted by size, largest
         // first; items are independent, so the assignment does not change any result
@@ -324,6 +559,16 @@ __global__ void __launch_bounds__(BS) gdi_cta_anneal_kernel(GdiDevProblem P, Gdi
         const int32_t *cls = P.class_ptr + P.class_off[q];
         const int32_t ncls = P.class_off[q + 1] - P.class_off[q] - 1;
         int8_t *gsig = R.spins + (int64_t)rep * P.N + base;
+        const int64_t nnz_item = P.row_ptr[base + n] - P.row_ptr[base];
+        const int32_t mean_deg = n > 0 ? (int32_t)min((nnz_item + n - 1) / n, (int64_t)64) : 1;
+
+        // the window at ranks [wlo, whi): its E* and rows, by threads t of nth
+        auto prepare = [&](int32_t wlo, int32_t whi, int32_t sw, const uint32_t *row, int32_t rlen, float Tsw, int t, int nth) {
+            const int64_t *rp = P.row_ptr + base + wlo;
+            if (staged && stage_fits(rp[0], rp[whi - wlo], R.cta_stage))
+                stage_rows(P, rp, whi - wlo, rp[0], rp[whi - wlo], rofs, cbuf, t, nth);
+            if (pre) draw_estar(R, wlo, whi, wlo, q, rep, sw, row, rlen, Tsw, es, t, nth);
+        };
 
         int32_t g = 0;
         for (int32_t r = threadIdx.x; r < n; r += BS) {
@@ -331,47 +576,204 @@ __global__ void __launch_bounds__(BS) gdi_cta_anneal_kernel(GdiDevProblem P, Gdi
             S.sig[r] = s;
             g += s;
         }
+        for (int b = threadIdx.x; b < 3 * NB; b += BS) h1[b] = 0;
+        if (threadIdx.x < 2) nge[threadIdx.x] = 0;
+        {
+            const int32_t roff = R.tab_off[R.s_begin], rlen = R.tab_off[R.s_begin + 1] - roff;
+            uint32_t *row = S.row + (rows2 && (R.s_begin & 1) ? L.row_stride : 0);
+            for (int32_t k = threadIdx.x; k < rlen; k += BS) row[k] = R.tab[roff + k];
+        }
         g = block_sum<BS, int32_t>(g, S.red32);
         if (threadIdx.x == 0) *S.G = g;
+        __syncthreads();
+        if (R.s_begin < R.s_end && ncls > 0) {
+            prepare(cls[0], P.W > 0 ? min(cls[0] + P.W, cls[1]) : cls[1], R.s_begin,
+                    S.row + (rows2 && (R.s_begin & 1) ? L.row_stride : 0),
+                    R.tab_off[R.s_begin + 1] - R.tab_off[R.s_begin], R.temp ? R.temp[R.s_begin] : 0.f, threadIdx.x, BS);
+            cp_async_wait_all();
+        }
         __syncthreads();
 
         for (int32_t sw = R.s_begin; sw < R.s_end; ++sw) {
             const int32_t roff = R.tab_off[sw];
             const int32_t rlen = R.tab_off[sw + 1] - roff;
-            for (int32_t k = threadIdx.x; k < rlen; k += BS) S.row[k] = R.tab[roff + k];
+            const uint32_t *row = S.row + (rows2 && (sw & 1) ? L.row_stride : 0);
+            // this sweep's row (its first window was drawn before), or the next sweep's beside it
+            if (!rows2 && sw > R.s_begin)
+                for (int32_t k = threadIdx.x; k < rlen; k += BS) S.row[k] = R.tab[roff + k];
+            const int32_t roff1 = sw + 1 < R.s_end ? roff + rlen : 0;
+            const int32_t rlen1 = sw + 1 < R.s_end ? R.tab_off[sw + 2] - roff1 : 0;
+            uint32_t *row1 = S.row + (sw & 1 ? 0 : L.row_stride);
+            if (rows2)
+                for (int32_t k = threadIdx.x; k < rlen1; k += BS) row1[k] = R.tab[roff1 + k];
             const float Tsw = R.temp ? R.temp[sw] : 0.f;
-            __syncthreads();
+            const int first = (sw & 1) ? -1 : 1;            // the group that goes first
+            if (!pre) __syncthreads();
             for (int32_t c = 0; c < ncls; ++c) {
                 const int32_t clo = cls[c], chi = cls[c + 1];
                 const int32_t Wn0 = P.W > 0 ? P.W : (chi - clo);
+                const int tl = team_log2<BS>(min(Wn0, chi - clo), mean_deg);
                 for (int32_t wlo = clo; wlo < chi; wlo += Wn0) {
-                    const int32_t whi = min(wlo + Wn0, chi);
-                    const int32_t Wn = whi - wlo;
-                    // step 1: thresholds, one Philox call per aligned quad of ranks
-                    const int32_t q0 = wlo >> 2, q1 = (whi - 1) >> 2;
-                    for (int32_t qd = q0 + threadIdx.x; qd <= q1; qd += BS) {
-                        const uint4 u4 = philox4x32_10(
-                            make_uint4((uint32_t)qd, (uint32_t)sw, (uint32_t)q, (uint32_t)rep),
-                            R.key0, R.key1);
-#pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            const int32_t r = 4 * qd + j;
-                            if (r < wlo || r >= whi) continue;
-                            const int sg = S.sig[r];
-                            const int32_t h = local_field(P, base, r, S.sig);
-                            const int32_t es = estar_of(S.row, rlen, R.mode, word_of(u4, j), Tsw);
-                            S.gam[r - wlo] = gamma_of(sg, h, es, P.A, P.B);
-                            S.s0[r - wlo] = (int8_t)sg;
-                        }
+                    const int32_t whi = min(wlo + Wn0, chi), Wn = whi - wlo;
+                    const int32_t c0 = *S.G;
+                    if (!pre) {
+                        draw_estar(R, wlo, whi, wlo, q, rep, sw, row, rlen, Tsw, es, threadIdx.x, BS);
+                        __syncthreads();
                     }
-                    if (R.flags & GDI_DEV_STANDARD) {
-                        standard_window<BS>(S, wlo, Wn, n);
+                    // ---- thresholds, counted by margin
+                    const int64_t *wrp = P.row_ptr + base + wlo;
+                    const bool st = staged && stage_fits(wrp[0], wrp[Wn], R.cta_stage);
+                    int32_t ge1 = 0, ge2 = 0;
+                    team_thresholds<BS>(P, S.sig, base, wlo, 0, Wn, tl, st ? rofs : nullptr, cbuf, es, a_shift,
+                                        [&](int32_t i, int sg, int32_t gm) {
+                                            gam[i] = gm;
+                                            s0[i] = (int8_t)sg;
+                                            if (standard) return;
+                                            const int32_t e = sg > 0 ? c0 - gm : gm - c0;
+                                            if (sg == first) {
+                                                ge1 += e >= 0;
+                                                if (e >= 0 && e < NB) atomicAdd(&h1[e], 1);
+                                            } else {
+                                                ge2 += e >= 0;
+                                                if (e >= -NB && e < NB) atomicAdd(&h2[e + NB], 1);
+                                            }
+                                        });
+                    if (!standard) {
+                        ge1 = __reduce_add_sync(0xFFFFFFFFu, ge1);
+                        ge2 = __reduce_add_sync(0xFFFFFFFFu, ge2);
+                        if (lane == 0 && ge1) atomicAdd(&nge[0], ge1);
+                        if (lane == 0 && ge2) atomicAdd(&nge[1], ge2);
+                    }
+                    __syncthreads();
+                    // the next window: its E* and rows do not depend on the spins
+                    auto ahead = [&](int t, int nth) {
+                        int32_t nlo = whi, nhi, nsw = sw;
+                        if (whi < chi) {
+                            nhi = min(whi + Wn0, chi);
+                        } else {
+                            if (c + 1 == ncls) {
+                                if (sw + 1 >= R.s_end) return;
+                                nsw = sw + 1;
+                            }
+                            const int nc = nsw == sw ? c + 1 : 0;
+                            nlo = cls[nc];
+                            nhi = P.W > 0 ? min(nlo + P.W, cls[nc + 1]) : cls[nc + 1];
+                        }
+                        const bool same = nsw == sw;
+                        prepare(nlo, nhi, nsw, same ? row : (rows2 ? row1 : R.tab + roff1), same ? rlen : rlen1,
+                                same ? Tsw : (R.temp ? R.temp[nsw] : 0.f), t, nth);
+                    };
+                    if (standard) {
+                        standard_window<BS>(S, gam, s0, wlo, Wn, n);
+                        ahead(threadIdx.x, BS);
+                        if (staged) cp_async_wait_all();
+                        __syncthreads();
                         continue;
                     }
-                    // step 2/3: the two groups in the canonical order (+1 first on even sweeps)
-                    const int first = (sw & 1) ? -1 : 1;
-                    select_and_flip<BS>(S, wlo, Wn, first, H);
-                    select_and_flip<BS>(S, wlo, Wn, -first, H);
+                    if (warp == 0) {
+                        int32_t K1 = 0, K2 = 0, y1, y2, l1, l2;
+                        bool ok = group_flips(h1, NB, nge[0], K1, y1, l1);
+                        if (ok) {
+                            // second group: margins grow by 2 K1
+                            int32_t n2 = 0;
+                            for (int m = NB - 2 * K1 + lane; m < NB; m += 32) n2 += h2[m];
+                            n2 = nge[1] + __reduce_add_sync(0xFFFFFFFFu, n2);
+                            ok = group_flips(h2 + NB - 2 * K1, NB + 2 * K1, n2, K2, y2, l2);
+                        }
+                        if (lane == 0) {
+                            dec.slow = ok ? 0 : 1;
+                            if (ok) {
+                                dec.y[0] = y1;
+                                dec.left[0] = l1;
+                                dec.y[1] = K2 ? y2 - 2 * K1 : INT32_MAX;
+                                dec.left[1] = l2;
+                                *S.G = c0 - 2 * first * K1 + 2 * first * K2;
+                            }
+                        }
+                    } else {
+                        ahead(threadIdx.x - 32, BS - 32);
+                    }
+                    __syncthreads();
+                    if (dec.slow) {
+                        // more flips than the bins cover: both groups by counting passes over the window
+                        int32_t gg = c0;
+                        for (int ph = 0; ph < 2; ++ph) {
+                            const int grp = ph == 0 ? first : -first;
+                            int32_t lo = 0, hi = count_ge<BS>(gam, s0, Wn, grp, gg, 0, S.red32);
+                            while (lo < hi) {
+                                const int32_t mid = (lo + hi + 1) >> 1;
+                                if (count_ge<BS>(gam, s0, Wn, grp, gg, 2 * (int64_t)mid - 2, S.red32) >= mid) lo = mid;
+                                else hi = mid - 1;
+                            }
+                            const int32_t K = lo;
+                            int32_t y = INT32_MAX, left = 0;
+                            if (K > 0) {
+                                const int32_t n2 = count_ge<BS>(gam, s0, Wn, grp, gg, 2 * (int64_t)K, S.red32);
+                                const int32_t n1 = count_ge<BS>(gam, s0, Wn, grp, gg, 2 * (int64_t)K - 1, S.red32);
+                                y = n2 == K || n1 >= K ? 2 * K - 1 : 2 * K - 2;
+                                left = n2 == K ? 0 : (n1 >= K ? K - n2 : K - n1);
+                                // margins are taken from the window-start G below
+                                y += grp > 0 ? c0 - gg : gg - c0;
+                            }
+                            if (threadIdx.x == 0) {
+                                dec.y[ph] = y;
+                                dec.left[ph] = left;
+                            }
+                            gg -= 2 * grp * K;
+                        }
+                        if (threadIdx.x == 0) *S.G = gg;
+                        __syncthreads();
+                    }
+                    const int32_t y1 = dec.y[0], y2 = dec.y[1], l1 = dec.left[0], l2 = dec.left[1];
+                    const bool cut = l1 | l2;               // some group's ties flip in part: by position
+                    // (also the bins' next use starts from zero)
+                    for (int b = threadIdx.x; b < 3 * NB; b += BS) h1[b] = 0;
+                    if (threadIdx.x < 2) nge[threadIdx.x] = 0;
+                    const int32_t rounds = (Wn + BS - 1) / BS;
+                    if (cut) {
+                        for (int32_t k = 0; k < rounds; ++k) {
+                            const int32_t i = k * BS + threadIdx.x;
+                            bool t1 = false, t2 = false;
+                            if (i < Wn) {
+                                const int sg = s0[i];
+                                const int32_t e = sg > 0 ? c0 - gam[i] : gam[i] - c0;
+                                t1 = sg == first && e == y1;
+                                t2 = sg != first && e == y2;
+                            }
+                            const unsigned b1 = __ballot_sync(0xFFFFFFFFu, t1), b2 = __ballot_sync(0xFFFFFFFFu, t2);
+                            if (lane == 0 && i < Wn) tcnt[i >> 5] = __popc(b1) | (__popc(b2) << 16);
+                        }
+                        __syncthreads();
+                    }
+                    for (int32_t k = 0; k < rounds; ++k) {
+                        const int32_t i = k * BS + threadIdx.x;
+                        int32_t e = 0;
+                        int sg = 0;
+                        if (i < Wn) {
+                            sg = s0[i];
+                            e = sg > 0 ? c0 - gam[i] : gam[i] - c0;
+                        }
+                        const bool g1 = sg == first, g2 = sg == -first;
+                        bool flip = (g1 && e > y1) || (g2 && e > y2);
+                        if (cut) {
+                            const bool t1 = g1 && e == y1, t2 = g2 && e == y2;
+                            const unsigned b1 = __ballot_sync(0xFFFFFFFFu, t1), b2 = __ballot_sync(0xFFFFFFFFu, t2);
+                            if (b1 | b2) {
+                                // ties of the ranks before this warp's 32
+                                const int32_t ch = (k * BS + (int32_t)(threadIdx.x & ~31u)) >> 5;
+                                int32_t p1 = 0, p2 = 0;
+                                for (int32_t j = lane; j < ch; j += 32) {
+                                    p1 += tcnt[j] & 0xFFFF;
+                                    p2 += tcnt[j] >> 16;
+                                }
+                                p1 = __reduce_add_sync(0xFFFFFFFFu, p1) + __popc(b1 & ((1u << lane) - 1u));
+                                p2 = __reduce_add_sync(0xFFFFFFFFu, p2) + __popc(b2 & ((1u << lane) - 1u));
+                                flip |= (t1 && p1 < l1) || (t2 && p2 < l2);
+                            }
+                        }
+                        if (flip) S.sig[wlo + i] = (int8_t)-sg;
+                    }
+                    if (staged) cp_async_wait_all();
                     __syncthreads();
                 }
             }
@@ -382,56 +784,49 @@ __global__ void __launch_bounds__(BS) gdi_cta_anneal_kernel(GdiDevProblem P, Gdi
                         dg += splitmix64_fin((uint64_t)(uint32_t)r | ((uint64_t)(sw & 0xFFFF) << 32) |
                                              ((uint64_t)(rep & 0xFFFF) << 48));
                 dg = block_sum<BS, uint64_t>(dg, reinterpret_cast<uint64_t *>(S.red64));
-                const int64_t ct = item_cut<BS>(P, base, n, S);
+                const int64_t ct = item_fields<BS>(P, base, n, mean_deg, S, 0, 0, nullptr, 0);
                 if (threadIdx.x == 0) {
                     const int64_t o = (int64_t)item * R.sweeps + sw;
                     R.tr_digest[o] = dg;
                     R.tr_G[o] = *S.G;
                     R.tr_cut[o] = ct;
                 }
+                __syncthreads();
             }
-            __syncthreads();
         }
-        // outputs before and after the exact-balance repair
-        const int64_t raw_cut = item_cut<BS>(P, base, n, S);
-        __syncthreads();
-        const int32_t raw_G = *S.G;
-        if (!(R.flags & GDI_DEV_NO_REPAIR)) repair<BS>(P, base, n, S);
-        const int64_t fin_cut = item_cut<BS>(P, base, n, S);
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            R.raw_G[item] = raw_G;
-            R.raw_cut[item] = raw_cut;
-            R.final_G[item] = *S.G;
-            R.final_cut[item] = fin_cut;
-        }
+        finish_item<BS>(P, R, base, n, mean_deg, S, gam, (int)((L.total - L.gam) / 4), item, true);
         for (int32_t r = threadIdx.x; r < n; r += BS) gsig[r] = S.sig[r];
         __syncthreads();
     }
 }
 
 // ---------------------------------------------------------------------------------------------
-// CTA-resident sorted-window kernel (1 <= W <= 256): the same results as gdi_cta_anneal_kernel with
-// far fewer block barriers per window.  Per colour class: the thresholds of the class's ranks
-// (fields gathered from the shared spins); every warp sorts whole windows of the class
-// (window_maps: one comparison value per member, valid for any G entering the window, and the
-// window's stage maps on the lattice, gdi_window.cuh); one thread walks the stage maps from the
-// class-start G, every window entered on the lattice is replayed at once by its own warp -- two
-// rounds of ballots -- and the rest in rank order; then the flips are applied.  The windows of a
-// class share no edge, so only the running G passes from one window to the next.  SL = members per
-// lane of a window.
+// CTA-resident counting kernel (1 <= W <= 256): the same results as gdi_cta_anneal_kernel with far
+// fewer block barriers per window.  Per colour class:
+//   1. thresholds of the class's ranks: a team of T lanes sums a rank's row over the shared spins;
+//   2. a class of three or more windows: every warp counts whole windows into their stage maps on the
+//      lattice (gdi_window.cuh), one thread walks the maps from the class-start G, and every window
+//      entered on the lattice is replayed at once by its own warp; the rest, and classes of one or two
+//      windows, are replayed in rank order from the exact G by one warp.  A replay writes its flips
+//      to the spins itself: nothing reads them again before the class ends.
+// The windows of a class share no edge, so only the running G passes from one window to the next.
+// SL = members per lane of a window.
+//
+// What bounds it is the chain of dependent steps of a class (a few hundred ranks), not bandwidth, so
+// everything that does not depend on spins leaves the chain: while one warp walks or replays, the
+// other warps draw the next class's E* (Philox and the table search) into shared memory and stage the
+// next class's columns and row offsets there (cp.async: contiguous in rank order), so that a threshold
+// is a few shared loads.
 struct SortedCta {
     int32_t *gam;       // [max_class] flip thresholds of the class
-    int16_t *rel;       // [max_class] comparison values
+    int32_t *es;        // [max_class] E* of the next class's ranks, drawn ahead
     uint8_t *s0;        // [max_class] 1 = the member was -1 at window start
-    uint8_t *narrow;    // [windows of the largest class] window sorted with 16-bit keys
-    uint32_t *fbits;    // [2][max_class / 32 + 2] flips of the fast replay (two class buffers)
-    uint32_t *fm;       // [2][max_class / 4 + 2] flips of the exact replay (byte per member)
-    int32_t *bins;      // [HA] exact-replay histogram
-    StageMap *maps;     // [warps][2] stage maps of the window a warp sorts (classes of many windows)
-    StageMap *wmaps;    // [nwm][2] stage maps of every window (classes of at most nwm windows)
+    uint32_t *bins;     // [warps that count][WBINS]
+    StageMap *wmaps;    // [nwm][2] stage maps of every window (classes of 3 to nwm windows)
     int32_t *tin;       // [nwm + 2] entering lattice index of every window; then the walk's
                         // first failing window and its last lattice index
+    int32_t *rofs;      // [max_class + 1] row offsets of the next class's ranks in cbuf
+    uint16_t *cbuf;     // [cta_stage] its columns
 };
 
 // windows per class whose stage maps are kept for the walk (more: one warp replays them in order)
@@ -444,61 +839,68 @@ __host__ __device__ inline int cta_walk_windows(int32_t max_class, int W)
     return nw < CTA_WALK_MAX ? (int)nw : CTA_WALK_MAX;
 }
 
-__host__ __device__ inline size_t align16c(size_t x) { return (x + 15) & ~(size_t)15; }
+// warps that count windows at once: none where no class has the three windows of a walk; their bins
+// share the repair flags' bytes, and a small instance has room for 16
+__host__ __device__ inline int cta_count_warps(int32_t max_n, int32_t max_class, int W, int BS)
+{
+    const int nwm = cta_walk_windows(max_class, W);
+    const int fit = max_n / 1024 > 16 ? max_n / 1024 : 16;
+    const int nw = nwm < BS / 32 ? nwm : BS / 32;
+    return nwm < 3 ? 0 : (nw < fit ? nw : fit);
+}
 
-// Shared-memory layout of the sorted CTA kernel, one function for the kernel's carving and the
-// host's size: the common part (reductions, G, table row, spins, repair flags), then the class
+// Shared-memory layout of the counting CTA kernel, one function for the kernel's carving and the
+// host's size: the common part (reductions, G, table rows, spins, repair flags), then the class
 // buffers.  Every array starts on a 16-byte boundary.
 struct CtaSortedLayout {
-    size_t red64, red32, G, row, sig, flag, gam, rel, s0, narrow, fbits, fm, bins, maps, wmaps, tin, total;
+    size_t red64, red32, G, row, sig, flag, gam, es, s0, wmaps, tin, rofs, cbuf, total;
+    int row_stride;
 };
 
-__host__ __device__ inline CtaSortedLayout cta_sorted_layout(int32_t max_n, int32_t max_class, int32_t max_row,
-                                                             int W, int BS)
+__host__ __device__ inline CtaSortedLayout cta_sorted_layout(const GdiDevProblem &P, int32_t max_row, int BS, int opts,
+                                                             int32_t stage)
 {
     CtaSortedLayout L;
-    const size_t mc = (size_t)max_class + 8;
+    const size_t mc = (size_t)P.max_class + 8;
     size_t o = 0;
     L.red64 = o; o = align16c(o + sizeof(int64_t) * (BS / 32 + 2));
     L.red32 = o; o = align16c(o + sizeof(int32_t) * (BS / 32 + 2));
     L.G = o; o = align16c(o + 16);
-    L.row = o; o = align16c(o + sizeof(uint32_t) * (size_t)(max_row + 4));
-    L.sig = o; o = align16c(o + (size_t)max_n + 16);
-    L.flag = o; o = align16c(o + (size_t)max_n + 16);
+    L.row_stride = (max_row + 4 + 3) & ~3;
+    L.row = o; o = align16c(o + sizeof(uint32_t) * (size_t)L.row_stride * ((opts & CTA_OPT_ROWS2) ? 2 : 1));
+    L.sig = o; o = align16c(o + (size_t)P.max_n + 16);
+    // the repair flags and, during the sweeps, the counting warps' bins share their bytes
+    const size_t bins = 4 * (size_t)win::WBINS * cta_count_warps(P.max_n, P.max_class, P.W, BS);
+    const size_t fl = (size_t)P.max_n + 16;
+    L.flag = o; o = align16c(o + (fl > bins ? fl : bins));
     L.gam = o; o = align16c(o + 4 * mc);
-    L.rel = o; o = align16c(o + 2 * mc);
+    L.es = o; o = align16c(o + 4 * mc);
     L.s0 = o; o = align16c(o + mc);
-    L.narrow = o; o = align16c(o + (size_t)((max_class + W - 1) / W) + 4);
-    L.fbits = o; o = align16c(o + 2 * 4 * (mc / 32 + 2));
-    L.fm = o; o = align16c(o + 2 * 4 * (mc / 4 + 2));
-    L.bins = o; o = align16c(o + 4 * (size_t)win::HA);
-    L.maps = o; o = align16c(o + sizeof(StageMap) * 2 * (size_t)(BS / 32));
-    const int nwm = cta_walk_windows(max_class, W);
+    const int nwm = cta_walk_windows(P.max_class, P.W);
     L.wmaps = o; o = align16c(o + sizeof(StageMap) * 2 * (size_t)nwm);
     L.tin = o; o = align16c(o + sizeof(int32_t) * (size_t)(nwm + 2));
+    L.rofs = o; o = align16c(o + (stage ? 4 * mc : 0));
+    L.cbuf = o; o = align16c(o + 2 * (size_t)stage);
     L.total = o;
     return L;
 }
 
-__host__ __device__ inline size_t cta_sorted_smem(int32_t max_n, int32_t max_class, int32_t max_row, int W, int BS)
-{
-    return cta_sorted_layout(max_n, max_class, max_row, W, BS).total;
-}
-
 // PAIR: a cluster of two blocks anneals each item.  Both keep all spins and G; a class of 3 to
-// nwm windows is split in two halves of windows (thresholds, sorts and replays each block's own),
+// nwm windows is split in two halves of windows (thresholds, counts and replays each block's own),
 // each block copies the other's stage maps in through distributed shared memory and walks all of
-// them, and each block applies the whole class's flips from both blocks' bitmaps.  Other classes
-// are done by block 0 alone.  Flip bitmaps alternate between two buffers from class to class, so a block may clear
-// the next class's buffer while its partner still reads the current one.
+// them, and each replay writes its flips to both blocks' spins.  Other classes are done by block 0
+// alone.
 template <int BS, int SL, bool PAIR>
 __global__ void __launch_bounds__(BS, 1024 / BS) gdi_cta_sorted_kernel(GdiDevProblem P, GdiDevRun R)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Smem S = {};
     SortedCta C;
+    const bool rows2 = (R.cta_opts & CTA_OPT_ROWS2) != 0, staged = R.cta_stage > 0;
+    int row_stride;
+    int scratch_words;
     {
-        const CtaSortedLayout L = cta_sorted_layout(P.max_n, P.max_class, R.max_row, P.W, BS);
+        const CtaSortedLayout L = cta_sorted_layout(P, R.max_row, BS, R.cta_opts, R.cta_stage);
         S.red64 = reinterpret_cast<int64_t *>(smem_raw + L.red64);
         S.red32 = reinterpret_cast<int32_t *>(smem_raw + L.red32);
         S.G = reinterpret_cast<int32_t *>(smem_raw + L.G);
@@ -506,15 +908,15 @@ __global__ void __launch_bounds__(BS, 1024 / BS) gdi_cta_sorted_kernel(GdiDevPro
         S.sig = reinterpret_cast<int8_t *>(smem_raw + L.sig);
         S.flag = reinterpret_cast<int8_t *>(smem_raw + L.flag);
         C.gam = reinterpret_cast<int32_t *>(smem_raw + L.gam);
-        C.rel = reinterpret_cast<int16_t *>(smem_raw + L.rel);
+        C.es = reinterpret_cast<int32_t *>(smem_raw + L.es);
         C.s0 = smem_raw + L.s0;
-        C.narrow = smem_raw + L.narrow;
-        C.fbits = reinterpret_cast<uint32_t *>(smem_raw + L.fbits);
-        C.fm = reinterpret_cast<uint32_t *>(smem_raw + L.fm);
-        C.bins = reinterpret_cast<int32_t *>(smem_raw + L.bins);
-        C.maps = reinterpret_cast<StageMap *>(smem_raw + L.maps);
+        C.bins = reinterpret_cast<uint32_t *>(smem_raw + L.flag);
         C.wmaps = reinterpret_cast<StageMap *>(smem_raw + L.wmaps);
         C.tin = reinterpret_cast<int32_t *>(smem_raw + L.tin);
+        C.rofs = reinterpret_cast<int32_t *>(smem_raw + L.rofs);
+        C.cbuf = reinterpret_cast<uint16_t *>(smem_raw + L.cbuf);
+        row_stride = L.row_stride;
+        scratch_words = (int)((L.total - L.gam) / 4);
         // the launch must have given the whole layout (the host sizes it with the same function)
         uint32_t dyn;
         asm volatile("mov.u32 %0, %%dynamic_smem_size;" : "=r"(dyn));
@@ -526,9 +928,14 @@ __global__ void __launch_bounds__(BS, 1024 / BS) gdi_cta_sorted_kernel(GdiDevPro
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int W = P.W;
     const int nwm = cta_walk_windows(P.max_class, W);
+    const int cwarps = cta_count_warps(P.max_n, P.max_class, W, BS);
+    const int a_shift = (P.A > 0 && (P.A & (P.A - 1)) == 0) ? 2 + __ffs(P.A) - 1 : -1;   // log2(4A)
     const int32_t items = P.num_instances * P.replicas;
-    const size_t fbw = ((size_t)P.max_class + 8) / 32 + 2, fmw = ((size_t)P.max_class + 8) / 4 + 2;
     __shared__ int32_t next_item;
+    // class bounds, windows, team sizes and (staged) my own row range's entries, for the first CB classes
+    constexpr int CB = 64;
+    __shared__ int32_t c_lo[CB + 1], c_nw[CB], c_eb[CB], c_ee[CB];
+    __shared__ uint8_t c_tl[CB];
     unsigned crank = 0;                                  // block rank in the cluster
     if constexpr (PAIR) crank = cooperative_groups::this_cluster().block_rank();
     // the partner block's copy of a shared-memory object (same layout in both blocks)
@@ -555,8 +962,59 @@ __global__ void __launch_bounds__(BS, 1024 / BS) gdi_cta_sorted_kernel(GdiDevPro
         const int32_t *cls = P.class_ptr + P.class_off[q];
         const int32_t ncls = P.class_off[q + 1] - P.class_off[q] - 1;
         int8_t *gsig = R.spins + (int64_t)rep * P.N + base;
-        const int64_t nnz_item = P.row_ptr[base + n] - P.row_ptr[base];
+        const int64_t row0 = P.row_ptr[base];
+        const int64_t nnz_item = P.row_ptr[base + n] - row0;
         const int32_t mean_deg = n > 0 ? (int32_t)min((nnz_item + n - 1) / n, (int64_t)64) : 1;
+
+        // one class as this block sees it: a class of 3 to nwm windows keeps every window's stage
+        // maps for the walk; a pair splits such a class: windows [0, kmid) are block 0's, the rest
+        // block 1's; other classes are block 0's
+        struct Span {
+            int32_t lo, ns, nwin, kmid, kb, ke, rb, re;
+            bool walk;
+        };
+        auto span_of = [&](int32_t lo, int32_t hi, int32_t nwin) {
+            Span s;
+            s.lo = lo;
+            s.ns = hi - lo;
+            s.nwin = nwin;
+            s.walk = nwin >= 3 && nwin <= nwm;
+            s.kmid = PAIR && s.walk ? (nwin + 1) / 2 : nwin;
+            s.kb = crank ? s.kmid : 0;
+            s.ke = crank ? nwin : s.kmid;
+            s.rb = min(s.kb * W, s.ns);
+            s.re = min(s.ke * W, s.ns);
+            return s;
+        };
+        auto span = [&](int c) {
+            if (c < CB) return span_of(c_lo[c], c_lo[c + 1], c_nw[c]);
+            return span_of(cls[c], cls[c + 1], (cls[c + 1] - cls[c] + W - 1) / W);
+        };
+        for (int c = threadIdx.x; c < ncls && c < CB; c += BS) {
+            const int32_t lo = cls[c], hi = cls[c + 1], nw = (hi - lo + W - 1) / W;
+            c_lo[c] = lo;
+            if (c + 1 == ncls || c + 1 == CB) c_lo[c + 1] = hi;
+            c_nw[c] = nw;
+            const Span s = span_of(lo, hi, nw);
+            c_tl[c] = (uint8_t)team_log2<BS>(s.re - s.rb, mean_deg);
+            c_eb[c] = (int32_t)(P.row_ptr[base + lo + s.rb] - row0);
+            c_ee[c] = (int32_t)(P.row_ptr[base + lo + s.re] - row0);
+        }
+        auto draw = [&](const Span &s, int32_t sw, const uint32_t *row, int32_t rlen, float Tsw, int t, int nth) {
+            draw_estar(R, s.lo + s.rb, s.lo + s.re, s.lo, q, rep, sw, row, rlen, Tsw, C.es, t, nth);
+        };
+        auto stage = [&](const Span &s, int c, int t, int nth) {
+            if (s.re <= s.rb) return;
+            const int64_t *rp = P.row_ptr + base + s.lo + s.rb;
+            const int32_t nown = s.re - s.rb;
+            const int64_t eb = c < CB ? row0 + c_eb[c] : rp[0], ee = c < CB ? row0 + c_ee[c] : rp[nown];
+            if (stage_fits(eb, ee, R.cta_stage)) stage_rows(P, rp, nown, eb, ee, C.rofs, C.cbuf, t, nth);
+        };
+        auto is_staged = [&](const Span &s, int c) {
+            if (!staged || s.re <= s.rb) return false;
+            const int64_t *rp = P.row_ptr + base + s.lo;
+            return stage_fits(c < CB ? row0 + c_eb[c] : rp[s.rb], c < CB ? row0 + c_ee[c] : rp[s.re], R.cta_stage);
+        };
 
         int32_t g = 0;
         for (int32_t r = threadIdx.x; r < n; r += BS) {
@@ -564,132 +1022,101 @@ __global__ void __launch_bounds__(BS, 1024 / BS) gdi_cta_sorted_kernel(GdiDevPro
             S.sig[r] = sv;
             g += sv;
         }
+        {
+            const int32_t roff = R.tab_off[R.s_begin], rlen = R.tab_off[R.s_begin + 1] - roff;
+            uint32_t *row = S.row + (rows2 && (R.s_begin & 1) ? row_stride : 0);
+            for (int32_t k = threadIdx.x; k < rlen; k += BS) row[k] = R.tab[roff + k];
+        }
         g = block_sum<BS, int32_t>(g, S.red32);
         if (threadIdx.x == 0) *S.G = g;
         __syncthreads();
-        uint32_t cc = 0;                                 // classes annealed so far (buffer parity)
+        if (R.s_begin < R.s_end) {
+            const Span s = span(0);
+            const int32_t rlen = R.tab_off[R.s_begin + 1] - R.tab_off[R.s_begin];
+            if (staged) stage(s, 0, threadIdx.x, BS);
+            draw(s, R.s_begin, S.row + (rows2 && (R.s_begin & 1) ? row_stride : 0), rlen,
+                 R.temp ? R.temp[R.s_begin] : 0.f, threadIdx.x, BS);
+            cp_async_wait_all();
+        }
+        __syncthreads();
 
         for (int32_t sw = R.s_begin; sw < R.s_end; ++sw) {
             const int32_t roff = R.tab_off[sw];
             const int32_t rlen = R.tab_off[sw + 1] - roff;
-            for (int32_t k = threadIdx.x; k < rlen; k += BS) S.row[k] = R.tab[roff + k];
+            const uint32_t *row = S.row + (rows2 && (sw & 1) ? row_stride : 0);
+            // this sweep's row (its first class was drawn before), or the next sweep's beside it; the
+            // first class's barrier makes it visible to the draws that follow
+            if (!rows2 && sw > R.s_begin)
+                for (int32_t k = threadIdx.x; k < rlen; k += BS) S.row[k] = R.tab[roff + k];
+            const int32_t roff1 = sw + 1 < R.s_end ? roff + rlen : 0;
+            const int32_t rlen1 = sw + 1 < R.s_end ? R.tab_off[sw + 2] - roff1 : 0;
+            uint32_t *row1 = S.row + (sw & 1 ? 0 : row_stride);
+            if (rows2)
+                for (int32_t k = threadIdx.x; k < rlen1; k += BS) row1[k] = R.tab[roff1 + k];
             const float Tsw = R.temp ? R.temp[sw] : 0.f;
             const bool plus_first = (sw & 1) == 0;
-            __syncthreads();
             for (int32_t c = 0; c < ncls; ++c) {
-                const int32_t lo = cls[c], hi = cls[c + 1];
-                const int32_t ns = hi - lo;
-                const int32_t nwin = (ns + W - 1) / W;
+                const Span s = span(c);
+                const int32_t lo = s.lo, ns = s.ns;
                 const int32_t c0 = *S.G;                 // G at class start (the reference c)
-                uint32_t *fb = C.fbits + (PAIR ? (cc & 1u) * fbw : 0);
-                uint32_t *fmm = C.fm + (PAIR ? (cc & 1u) * fmw : 0);
-                ++cc;
-                // a class of 3 to nwm windows keeps every window's stage maps for the walk below
-                // (one or two windows replay in order at the cost of the walk's extra barrier);
-                // a pair splits such a class: windows [0, kmid) are block 0's, the rest block 1's
-                const bool walk = nwin >= 3 && nwin <= nwm;
-                const bool split = PAIR && walk;
-                const int32_t kmid = split ? (nwin + 1) / 2 : nwin;
-                const int32_t kb = crank ? kmid : 0, ke = crank ? nwin : kmid;
-                const int32_t rb = min(kb * W, ns), re = min(ke * W, ns);     // my ranks in the class
-                const int32_t nown = re - rb;
-                // the field sums' longest chain of dependent reads decides the layout: one thread
-                // per aligned quad of ranks (one Philox call per quad; per round 4 rows), or a team
-                // of T lanes per rank (T a power of two; per round a row / T); a round also costs
-                // about 4 reads of draw and reduction latency, and the team layout, which draws
-                // per rank, must shorten the chain by a quarter
-                int T = 0;
-                {
-                    const int32_t nq = (nown + 3) / 4 + 1;
-                    int32_t best = ((nq + BS - 1) / BS) * (4 * mean_deg + 4) * 3 / 4;
-                    for (int t = 1; t <= 32; t <<= 1) {
-                        const int32_t chain = ((nown * t + BS - 1) / BS) * ((mean_deg + t - 1) / t + 4);
-                        if (chain < best) { best = chain; T = t; }
-                    }
-                }
-                if (T == 0) {
-                    for (int32_t qd = ((lo + rb) >> 2) + threadIdx.x; nown > 0 && qd <= ((lo + re - 1) >> 2); qd += BS) {
-                        const uint4 u4 = philox4x32_10(
-                            make_uint4((uint32_t)qd, (uint32_t)sw, (uint32_t)q, (uint32_t)rep), R.key0, R.key1);
+                // ---- thresholds of my ranks
+                team_thresholds<BS>(P, S.sig, base, lo, s.rb, s.re, c < CB ? c_tl[c] : team_log2<BS>(s.re - s.rb, mean_deg),
+                                    is_staged(s, c) ? C.rofs : nullptr, C.cbuf, C.es, a_shift,
+                                    [&](int32_t i, int sg, int32_t gm) {
+                                        C.gam[i] = gm;
+                                        C.s0[i] = sg < 0 ? 1 : 0;
+                                    });
+                if (PAIR && !s.walk) pair_sync(); else __syncthreads();
+                // the next class: its E* and columns do not depend on the spins
+                const bool same = c + 1 < ncls;
+                const bool more = same || sw + 1 < R.s_end;
+                auto ahead = [&](int t, int nth) {
+                    if (!more) return;
+                    const Span nx = span(same ? c + 1 : 0);
+                    if (staged) stage(nx, same ? c + 1 : 0, t, nth);
+                    draw(nx, same ? sw : sw + 1, same ? row : (rows2 ? row1 : R.tab + roff1), same ? rlen : rlen1,
+                         same ? Tsw : (R.temp ? R.temp[sw + 1] : 0.f), t, nth);
+                };
+                // the flips of a window straight into the spins (of both blocks of a pair)
+                auto flip = [&](int32_t ws, int32_t we, const uint8_t *s0, const uint32_t (&wb)[SL]) {
 #pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            const int32_t r = 4 * qd + j;
-                            if (r < lo + rb || r >= lo + re) continue;
-                            const int sg = S.sig[r];
-                            const int32_t h = P.col16 ? local_field16(P, base, r, S.sig) : local_field(P, base, r, S.sig);
-                            const int32_t es = estar_of(S.row, rlen, R.mode, word_of(u4, j), Tsw);
-                            C.gam[r - lo] = gamma_of(sg, h, es, P.A, P.B);
-                            C.s0[r - lo] = sg < 0 ? 1 : 0;
+                    for (int k = 0; k < SL; ++k) {
+                        const int32_t i = ws + 32 * k + lane;
+                        if (i < we && ((wb[k] >> lane) & 1u)) {
+                            const int8_t v = s0[i] ? 1 : -1;
+                            S.sig[lo + i] = v;
+                            if constexpr (PAIR) peer(S.sig)[lo + i] = v;
                         }
                     }
-                } else {
-                    // teams are aligned lane groups of one warp; every lane takes part in every
-                    // round's shuffles (the round count is the same for the whole block)
-                    const int sub = threadIdx.x & (T - 1);
-                    for (int32_t k0 = rb; k0 < re; k0 += BS / T) {
-                        const int32_t i = k0 + (int32_t)threadIdx.x / T;
-                        int32_t h = 0;
-                        if (i < re) {
-                            const int64_t e0 = P.row_ptr[base + lo + i], e1 = P.row_ptr[base + lo + i + 1];
-                            if (P.col16) {
-                                for (int64_t e = e0 + sub; e < e1; e += T) {
-                                    const uint32_t cc = __ldg(P.col16 + e);
-                                    const int32_t sv = S.sig[cc & 0x7FFFu];
-                                    h += (cc >> 15) ? -sv : sv;
-                                }
-                            } else {
-                                for (int64_t e = e0 + sub; e < e1; e += T) {
-                                    const uint32_t cc = __ldg(P.col + e);
-                                    const int32_t sv = S.sig[cc & 0x7FFFFFFFu];
-                                    h += (cc >> 31) ? -sv : sv;
-                                }
-                            }
+                };
+                int32_t k_seq = 0;                       // first window replayed in order
+                if (s.walk) {
+                    // ---- every window of mine counted by one warp
+                    if (warp < cwarps)
+                        for (int32_t kk = s.kb + warp; kk < s.ke; kk += cwarps) {
+                            const int32_t ws = kk * W, wlen = min(W, ns - ws);
+                            window_maps<SL>(C.gam, C.s0, ws, wlen, 0, c0, C.bins + (size_t)warp * WBINS,
+                                            C.wmaps + 2 * kk);
                         }
-                        for (int o = T >> 1; o >= 1; o >>= 1) h += __shfl_xor_sync(0xFFFFFFFFu, h, o);
-                        if (i < re && sub == 0) {
-                            const int32_t r = lo + i;
-                            const uint4 u4 = philox4x32_10(
-                                make_uint4((uint32_t)(r >> 2), (uint32_t)sw, (uint32_t)q, (uint32_t)rep), R.key0,
-                                R.key1);
-                            const int sg = S.sig[r];
-                            const int32_t es = estar_of(S.row, rlen, R.mode, word_of(u4, r & 3), Tsw);
-                            C.gam[i] = gamma_of(sg, h, es, P.A, P.B);
-                            C.s0[i] = sg < 0 ? 1 : 0;
-                        }
+                    pair_sync();
+                    if constexpr (PAIR) {
+                        // the partner's stage maps copied in at once (one remote round trip), into the
+                        // slots of its windows, which this block does not use itself
+                        const int32_t pkb = crank ? 0 : s.kmid, pke = crank ? s.kmid : s.nwin;
+                        const uint4 *src = reinterpret_cast<const uint4 *>(peer(C.wmaps) + 2 * pkb);
+                        uint4 *dst = reinterpret_cast<uint4 *>(C.wmaps + 2 * pkb);
+                        for (int32_t i = threadIdx.x; i < 2 * (pke - pkb); i += BS) dst[i] = src[i];
+                        __syncthreads();
                     }
-                }
-                for (int32_t i = threadIdx.x; i < ns / 32 + 2; i += BS) fb[i] = 0;
-                for (int32_t i = threadIdx.x; i < ns / 4 + 2; i += BS) fmm[i] = 0;
-                __syncthreads();
-                // every window of mine sorted by one warp
-                for (int32_t kk = kb + warp; kk < ke; kk += BS / 32) {
-                    const int32_t ws = kk * W, wlen = min(W, ns - ws);
-                    StageMap *o = walk ? C.wmaps + 2 * kk : C.maps + 2 * warp;
-                    window_maps<SL>(C.gam, C.s0, C.rel, ws, wlen, 0, c0, o);
-                    __syncwarp();
-                    if (lane == 0) C.narrow[kk] = (uint8_t)o[0].narrow;
-                }
-                // (a pair meets here for every class: the tail below may write the partner's G,
-                // which the partner must have read as this class's c0 first)
-                pair_sync();
-                int32_t k_seq = 0;                       // first window the ordered tail replays
-                if (split) {
-                    // the partner's stage maps copied in at once (one remote round trip), into the
-                    // slots of its windows, which this block does not use itself
-                    const int32_t pkb = crank ? 0 : kmid, pke = crank ? kmid : nwin;
-                    const uint4 *src = reinterpret_cast<const uint4 *>(peer(C.wmaps) + 2 * pkb);
-                    uint4 *dst = reinterpret_cast<uint4 *>(C.wmaps + 2 * pkb);
-                    for (int32_t i = threadIdx.x; i < 2 * (pke - pkb); i += BS) dst[i] = src[i];
-                    __syncthreads();
-                }
-                if (walk) {
-                    // one thread follows x = G - c0 from 0 through the windows' stage maps (lattice
+                    // ---- one thread follows x = G - c0 from 0 through the windows' stage maps (lattice
                     // index t: x = 2 t - NT) up to the first window that leaves the lattice (in a
-                    // pair both blocks walk, to the same result)
-                    if (threadIdx.x == 0) {
+                    // pair both blocks walk, to the same result); the other warps work ahead
+                    if (warp > 0) {
+                        ahead(threadIdx.x - 32, BS - 32);
+                    } else if (lane == 0) {
                         int t = NT / 2;
-                        int32_t kf = nwin;
-                        for (int32_t kk = 0; kk < nwin; ++kk) {
+                        int32_t kf = s.nwin;
+                        for (int32_t kk = 0; kk < s.nwin; ++kk) {
                             C.tin[kk] = t;
                             const StageMap *wm = C.wmaps;
                             const int u = stage_apply(wm[2 * kk + (plus_first ? 1 : 0)],
@@ -699,56 +1126,40 @@ __global__ void __launch_bounds__(BS, 1024 / BS) gdi_cta_sorted_kernel(GdiDevPro
                         }
                         C.tin[nwm] = kf;
                         C.tin[nwm + 1] = t;
-                        if (kf == nwin) *S.G = c0 + 2 * t - NT;
+                        if (kf == s.nwin) *S.G = c0 + 2 * t - NT;
                     }
                     __syncthreads();
                     k_seq = C.tin[nwm];
-                    // my windows before it were entered on the lattice: all replayed at once
-                    for (int32_t kk = kb + warp; kk < min(ke, k_seq); kk += BS / 32) {
-                        const int32_t ws = kk * W, we = min(ws + W, ns);
-                        replay_window<SL>(C.rel, C.s0, 0, ws, we, 2 * C.tin[kk] - NT, plus_first, fb, W);
+                    // ---- my windows before it were entered on the lattice: all replayed at once
+                    for (int32_t kk = s.kb + warp; kk < min(s.ke, k_seq); kk += BS / 32) {
+                        const int32_t ws = kk * W, we = min(ws + W, ns), t = C.tin[kk];
+                        replay_mapped<SL>(C.gam, C.s0, 0, ws, we, c0 + 2 * t - NT, plus_first, t, C.wmaps + 2 * kk,
+                                          [&](const uint32_t (&wb)[SL]) { flip(ws, we, C.s0, wb); });
                     }
+                } else if (warp > 0) {
+                    ahead(threadIdx.x - 32, BS - 32);
                 }
-                // the rest in rank order by one warp of block 0, each window entered with the G its
-                // predecessors left; a window of block 1 is read, and its flips written, remotely
-                if (crank == 0 && warp == 0 && k_seq < nwin) {
-                    int32_t x = walk ? 2 * C.tin[k_seq] - NT : 0;
-                    for (int32_t kk = k_seq; kk < nwin; ++kk) {
-                        const bool mine = kk < kmid;
-                        const int16_t *rel = C.rel;
-                        const uint8_t *s0 = C.s0, *nar = C.narrow;
+                // ---- the rest in rank order by one warp of block 0, each window entered with the G its
+                // predecessors left; a window of block 1 is read remotely
+                if (crank == 0 && warp == 0 && k_seq < s.nwin) {
+                    int32_t gr = s.walk ? c0 + 2 * C.tin[nwm + 1] - NT : c0;
+                    for (int32_t kk = k_seq; kk < s.nwin; ++kk) {
+                        const uint8_t *s0 = C.s0;
                         const int32_t *gam = C.gam;
-                        uint32_t *fbo = fb, *fmo = fmm;
                         if constexpr (PAIR) {
-                            if (!mine) {
-                                rel = peer(C.rel); s0 = peer(C.s0); nar = peer(C.narrow);
-                                gam = peer(C.gam); fbo = peer(fb); fmo = peer(fmm);
-                            }
+                            if (kk >= s.kmid) { s0 = peer(C.s0); gam = peer(C.gam); }
                         }
                         const int32_t ws = kk * W, we = min(ws + W, ns);
-                        const bool on = nar[kk] ? (x >= -NT && x <= NT - 2) : (x >= -FAST_X && x <= FAST_X);
-                        x = on ? replay_window<SL>(rel, s0, 0, ws, we, x, plus_first, fbo, W)
-                               : window_replay_exact(gam, s0, 0, ws, we, c0 + x, plus_first, C.bins, fmo) - c0;
+                        gr = replay_window<SL>(gam, s0, 0, ws, we, gr, plus_first, -1, -1,
+                                               [&](const uint32_t (&wb)[SL]) { flip(ws, we, s0, wb); });
                     }
                     if (lane == 0) {
-                        *S.G = c0 + x;
-                        if constexpr (PAIR) *peer(S.G) = c0 + x;
+                        *S.G = gr;
+                        if constexpr (PAIR) *peer(S.G) = gr;
                     }
                 }
-                if constexpr (PAIR) pair_sync(); else __syncthreads();
-                // every block applies the whole class's flips to its copy of the spins
-                for (int part = 0; part < (PAIR ? 2 : 1); ++part) {
-                    const int32_t i0 = part == 0 ? 0 : min(kmid * W, ns), i1 = part == 0 ? min(kmid * W, ns) : ns;
-                    const uint32_t *fbr = fb, *fmr = fmm;
-                    if constexpr (PAIR) {
-                        if ((unsigned)part != crank) { fbr = peer(fb); fmr = peer(fmm); }
-                    }
-                    for (int32_t i = i0 + threadIdx.x; i < i1; i += BS) {
-                        const uint32_t f = ((fbr[i >> 5] >> (i & 31)) | (fmr[i >> 2] >> (8 * (i & 3)))) & 1u;
-                        if (f) S.sig[lo + i] = (int8_t)-S.sig[lo + i];
-                    }
-                }
-                __syncthreads();
+                if (staged) cp_async_wait_all();
+                pair_sync();
             }
             if (R.flags & GDI_DEV_TRACE) {
                 uint64_t dg = 0;
@@ -757,31 +1168,19 @@ __global__ void __launch_bounds__(BS, 1024 / BS) gdi_cta_sorted_kernel(GdiDevPro
                         dg += splitmix64_fin((uint64_t)(uint32_t)r | ((uint64_t)(sw & 0xFFFF) << 32) |
                                              ((uint64_t)(rep & 0xFFFF) << 48));
                 dg = block_sum<BS, uint64_t>(dg, reinterpret_cast<uint64_t *>(S.red64));
-                const int64_t ct = item_cut<BS>(P, base, n, S);
+                const int64_t ct = item_fields<BS>(P, base, n, mean_deg, S, 0, 0, nullptr, 0);
                 if (threadIdx.x == 0 && crank == 0) {
                     const int64_t o = (int64_t)item * R.sweeps + sw;
                     R.tr_digest[o] = dg;
                     R.tr_G[o] = *S.G;
                     R.tr_cut[o] = ct;
                 }
+                pair_sync();
             }
-            __syncthreads();
         }
-        const int64_t raw_cut = item_cut<BS>(P, base, n, S);
-        __syncthreads();
-        const int32_t raw_G = *S.G;
-        if (!(R.flags & GDI_DEV_NO_REPAIR)) repair<BS>(P, base, n, S);
-        const int64_t fin_cut = item_cut<BS>(P, base, n, S);
-        __syncthreads();
-        if (crank == 0) {
-            if (threadIdx.x == 0) {
-                R.raw_G[item] = raw_G;
-                R.raw_cut[item] = raw_cut;
-                R.final_G[item] = *S.G;
-                R.final_cut[item] = fin_cut;
-            }
+        finish_item<BS>(P, R, base, n, mean_deg, S, C.gam, scratch_words, item, crank == 0);
+        if (crank == 0)
             for (int32_t r = threadIdx.x; r < n; r += BS) gsig[r] = S.sig[r];
-        }
         __syncthreads();
     }
 }
@@ -834,35 +1233,64 @@ __global__ void gdi_gather_kernel(GdiDevProblem P, const int8_t *spins, int8_t *
     }
 }
 
-size_t cta_smem(const GdiDevProblem &P, const GdiDevRun &R, int BS, int H)
-{
-    size_t b = sizeof(int64_t) * (BS / 32 + 2) + sizeof(int32_t) * (BS / 32 + 2) + 16;
-    b += sizeof(int32_t) * (size_t)H;
-    b += sizeof(int32_t) * (size_t)((P.max_window + 3) & ~3);
-    b += sizeof(uint32_t) * (size_t)((R.max_row + 3) & ~3);
-    b += (size_t)((P.max_window + 15) & ~15);
-    b += (size_t)((P.max_n + 15) & ~15);
-    b += (size_t)P.max_n;
-    return b;
-}
-
-int hist_bins(const GdiDevProblem &P)
-{
-    int H = 64;
-    while (H < 2 * P.max_window + 2 && H < 256) H <<= 1;
-    return H;
-}
-
 // the sorted-window kernel serves every window size 1 .. 256 (one instantiation per members per
 // lane) of the running-G method when its whole-class buffers fit in a block's shared memory;
 // Algorithm 2 (GDI_DEV_STANDARD), larger windows and larger classes take gdi_cta_anneal_kernel
+constexpr size_t CTA_STATIC_SMEM = 2048;     // the kernel's class bounds and single words, rounded up
+
 inline bool cta_sorted(const GdiDevProblem &P, const GdiDevRun &R, int BS)
 {
     if (P.W < 1 || P.W > 256 || (R.flags & GDI_DEV_STANDARD)) return false;
     int dev = 0, optin = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    return cta_sorted_smem(P.max_n, P.max_class, R.max_row, P.W, BS) <= (size_t)optin;
+    return cta_sorted_layout(P, R.max_row, BS, 0, 0).total + CTA_STATIC_SMEM <= (size_t)optin;
+}
+
+// shared memory of the kernel that takes this call (counted windows, else whole-block windows)
+inline size_t cta_smem(const GdiDevProblem &P, const GdiDevRun &R, int BS, bool counted)
+{
+    return counted ? cta_sorted_layout(P, R.max_row, BS, R.cta_opts, R.cta_stage).total
+                   : cta_block_layout(P, R.max_row, BS, R.cta_opts, R.cta_stage).total;
+}
+
+// What the launch keeps in shared memory beyond the necessary (R.cta_opts, R.cta_stage): an option is
+// taken when it fits a block and leaves as many items resident on an SM as there are without it (never
+// more than the SM's share of the items, or than its 1024 threads at 64 registers); the staging buffer
+// takes what is then left, up to the largest class.  Returns whether the counting kernel takes the call.
+inline bool cta_options(const GdiDevProblem &P, GdiDevRun &R, int BS)
+{
+    int dev = 0, optin = 0, per_sm = 0, sms = 1;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int64_t items = (int64_t)P.num_instances * P.replicas;
+    const bool counted = cta_sorted(P, R, BS);
+    R.cta_opts = 0;
+    R.cta_stage = 0;
+    auto resident = [&]() {
+        const size_t need = cta_smem(P, R, BS, counted) + CTA_STATIC_SMEM;
+        if (need > (size_t)optin) return (int64_t)0;
+        return std::min<int64_t>((int64_t)((size_t)per_sm / (need + 1024)), 1024 / BS);
+    };
+    const int64_t want = std::max<int64_t>(1, std::min<int64_t>(resident(), (items + sms - 1) / sms));
+    auto take = [&](int opt) {
+        R.cta_opts |= opt;
+        if (resident() < want) R.cta_opts &= ~opt;
+    };
+    if (!counted) take(CTA_OPT_BINS);
+    if (!counted) take(CTA_OPT_ES);
+    take(CTA_OPT_ROWS2);
+    if (P.col16 && P.max_class_nnz > 0) {
+        // (the first 8 columns stand for the row offsets, which any staging needs)
+        R.cta_stage = 8;
+        const int64_t room = std::min<int64_t>(optin, (int64_t)per_sm / want - 1024) - (int64_t)CTA_STATIC_SMEM -
+                             (int64_t)cta_smem(P, R, BS, counted);
+        const int64_t cap = std::min<int64_t>(P.max_class_nnz + 24, room / 2 + 8 - 16);
+        R.cta_stage = cap >= std::min(512, P.max_class_nnz + 16) ? (int32_t)(cap & ~(int64_t)7) : 0;
+    }
+    return counted;
 }
 
 // a pair of blocks per item when the items fill at most half of the SMs and the largest class
@@ -890,23 +1318,18 @@ const void *cta_sorted_kernel_for(int W)
 template <int BS>
 const void *cta_kernel(const GdiDevProblem &P, const GdiDevRun &R)
 {
-    if (!cta_sorted(P, R, BS)) return (const void *)gdi_cta_anneal_kernel<BS>;
+    if (!cta_sorted(P, R, BS)) return (const void *)gdi_cta_block_kernel<BS>;
     return cta_pair(P, R, BS) ? cta_sorted_kernel_for<BS, true>(P.W) : cta_sorted_kernel_for<BS, false>(P.W);
 }
 
 template <int BS>
-size_t cta_kernel_smem(const GdiDevProblem &P, const GdiDevRun &R)
-{
-    return cta_sorted(P, R, BS) ? cta_sorted_smem(P.max_n, P.max_class, R.max_row, P.W, BS)
-                         : cta_smem(P, R, BS, hist_bins(P));
-}
-
-template <int BS>
-int launch_cta(const GdiDevProblem &P, const GdiDevRun &R, int grid_limit, cudaStream_t st,
+int launch_cta(const GdiDevProblem &P, const GdiDevRun &R0, int grid_limit, cudaStream_t st,
                int *grid_used, size_t *smem_used)
 {
+    GdiDevRun R = R0;
+    const bool counted = cta_options(P, R, BS);
     const void *kern = cta_kernel<BS>(P, R);
-    const size_t smem = cta_kernel_smem<BS>(P, R);
+    const size_t smem = cta_smem(P, R, BS, counted);
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return (int)e;
     int dev = 0, sms = 0, per_sm = 0;
@@ -921,7 +1344,7 @@ int launch_cta(const GdiDevProblem &P, const GdiDevRun &R, int grid_limit, cudaS
     if (grid_limit > 0 && grid > grid_limit) grid = grid_limit;
     if (cta_pair(P, R, BS)) {
         // clusters of two blocks, one item per cluster
-        void *args[] = {const_cast<GdiDevProblem *>(&P), const_cast<GdiDevRun *>(&R)};
+        void *args[] = {const_cast<GdiDevProblem *>(&P), &R};
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeClusterDimension;
         attr[0].val.clusterDim.x = 2;
@@ -943,12 +1366,10 @@ int launch_cta(const GdiDevProblem &P, const GdiDevRun &R, int grid_limit, cudaS
         cfg.gridDim = dim3(grid);
         e = cudaLaunchKernelExC(&cfg, kern, args);
         if (e != cudaSuccess) return (int)e;
-    } else if (cta_sorted(P, R, BS)) {
-        void *args[] = {const_cast<GdiDevProblem *>(&P), const_cast<GdiDevRun *>(&R)};
+    } else {
+        void *args[] = {const_cast<GdiDevProblem *>(&P), &R};
         e = cudaLaunchKernel(kern, dim3(grid), dim3(BS), args, smem, st);
         if (e != cudaSuccess) return (int)e;
-    } else {
-        gdi_cta_anneal_kernel<BS><<<grid, BS, smem, st>>>(P, R, hist_bins(P));
     }
     if (grid_used) *grid_used = grid;
     if (smem_used) *smem_used = smem;
@@ -956,10 +1377,12 @@ int launch_cta(const GdiDevProblem &P, const GdiDevRun &R, int grid_limit, cudaS
 }
 
 template <int BS>
-int cta_occupancy(const GdiDevProblem &P, const GdiDevRun &R, int *per_sm)
+int cta_occupancy(const GdiDevProblem &P, const GdiDevRun &R0, int *per_sm)
 {
+    GdiDevRun R = R0;
+    const bool counted = cta_options(P, R, BS);
     const void *kern = cta_kernel<BS>(P, R);
-    const size_t smem = cta_kernel_smem<BS>(P, R);
+    const size_t smem = cta_smem(P, R, BS, counted);
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, kern, BS, smem);
     return (int)e;
@@ -979,12 +1402,11 @@ int gdi_cta_blocks_per_sm(const GdiDevProblem &P, const GdiDevRun &R, int block,
     }
 }
 
-int gdi_cta_smem_bytes(const GdiDevProblem &P, const GdiDevRun &R, int block, size_t *bytes, int *hist)
+int gdi_cta_smem_bytes(const GdiDevProblem &P, const GdiDevRun &R0, int block, size_t *bytes)
 {
-    const int H = hist_bins(P);
-    if (hist) *hist = H;
-    if (bytes) *bytes = cta_sorted(P, R, block) ? cta_sorted_smem(P.max_n, P.max_class, R.max_row, P.W, block)
-                                      : cta_smem(P, R, block, H);
+    GdiDevRun R = R0;
+    const bool counted = cta_options(P, R, block);
+    *bytes = cta_smem(P, R, block, counted) + (counted ? CTA_STATIC_SMEM : 64);
     return 0;
 }
 

@@ -186,9 +186,11 @@ extern "C" int gdi_anneal_static(int32_t n, const int64_t *row_ptr, const uint32
     P.max_window = W < max_class ? W : max_class;
     P.max_degree = max_degree;
     P.max_class = max_class;
+    P.max_class_nnz = 0;
     int spc = 0, wpc = 0;
     size_t smem = 0;
-    if (gdi_grid_plan(P, max_row, nblk, (size_t)optin, &spc, &wpc, &smem) != 0)
+    bool counted = false;
+    if (gdi_grid_plan(P, max_row, nblk, (size_t)optin, &spc, &wpc, &smem, &counted) != 0)
         return gdi_set_error(GDI_ERR_TOO_LARGE, "gdi_anneal_static: the plan needs " + std::to_string(smem) +
                                                     " bytes of shared memory per block; use a smaller W");
 
@@ -245,7 +247,7 @@ extern "C" int gdi_anneal_static(int32_t n, const int64_t *row_ptr, const uint32
         static_rows_check_kernel<<<cb, 256, 0, st>>>(n, row_ptr, max_degree, X.err);
         static_cols_check_kernel<<<cb, 256, 0, st>>>(n, row_ptr, col, class_ptr, num_classes, X.err);
     }
-    const int ke = gdi_launch_grid_anneal(P, R, X, spins, nblk, spc, wpc, smem, nullptr, nullptr, st);
+    const int ke = gdi_launch_grid_anneal(P, R, X, spins, nblk, spc, wpc, smem, counted, nullptr, nullptr, st);
     if (ke) return gdi_set_error(GDI_ERR_CUDA, std::string("gdi_anneal_static launch: ") +
                                                    cudaGetErrorString((cudaError_t)ke));
     return GDI_OK;

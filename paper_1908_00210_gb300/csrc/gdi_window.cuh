@@ -1,12 +1,12 @@
-// gdi_window.cuh -- sorted-window building blocks of libgdi.so, shared by the grid-scale kernels
-// (gdi_grid.cu) and the CTA-resident sorted-window kernel (gdi_kernels.cu).
+// gdi_window.cuh -- window building blocks of libgdi.so, shared by the grid-scale kernels
+// (gdi_grid.cu) and the CTA-resident counting kernel (gdi_kernels.cu).
 //
 // A window is W consecutive ranks of one colour class.  Inside it the +1 group, in order of flip
 // threshold gamma ascending (then position), and the -1 group, by gamma descending, each see the
-// exact running G (reading R2 of Algorithm 3).  Sorting a group once gives every member k the value
-// rel = a_k - c (+1: a_k = gamma_(k) + 2k; -1: b_k = gamma_(k) - 2k) relative to a reference G c,
-// after which member k flips iff rel <= x (+1) or rel >= x (-1) for the x = G - c entering the
-// group: one comparison per member.  Stage maps summarise a window on the lattice x = -64 .. 62.
+// exact running G (reading R2 of Algorithm 3).  The k-th member of the +1 group flips iff
+// a_k = gamma_(k) + 2k <= G (-1: gamma_(k) - 2k >= G), so all that matters of a group is how many
+// members have their threshold on either side of a value: windows are counted, not sorted.  Stage
+// maps summarise a window on the lattice x = G - c = -64 .. 62 around a reference G c.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -20,15 +20,13 @@ namespace win {
 constexpr int KC = 31;                  // flips per group the exact counting histogram covers at once
 constexpr int HA = 2 * KC + 1;          // histogram bins of the exact counting replay
 constexpr int NT = 64;                  // lattice points of a stage map
-constexpr int32_t KEY_D = 1 << 22;      // threshold distances are clamped to [-KEY_D, KEY_D)
-constexpr int32_t REL_CAP = 32767;      // rel values are stored clamped to +-REL_CAP
-constexpr int32_t FAST_X = 32000;       // |G - c| up to which the stored rel values decide exactly
+constexpr int WBINS = 256;              // words a warp counts a window's distances in
 constexpr unsigned long long STEP_MASK = (1ull << (NT - 1)) - 1ull;
 
 struct StageMap {
     unsigned long long mask;            // bit j: the step from lattice point j to j + 1 rises
     int32_t ylo;                        // output index of lattice point 0
-    int32_t narrow;                     // 1: the window's rel values are exact on the lattice only
+    int32_t pad;
 };
 
 // In-place cumulative counts of bins[0, nb) by one warp: forward (bins[x] = base + sum_{b <= x})
@@ -199,260 +197,135 @@ __device__ inline int32_t warp_group(const int32_t *gam, int gs, int gc, const u
     return K;
 }
 
-// ascending sort of 32 * S keys held as key[s] of lane l = element l * S + s: a bitonic network in
-// its all-ascending form (every merge starts with a "flip" stage that pairs element e with
-// e ^ (size - 1), then half-cleaners pair e with e ^ j), so that a compare-exchange always sends
-// the minimum to the lower element -- in-register steps are a plain min/max pair
-template <int S>
-__device__ __forceinline__ void warp_bitonic(uint32_t (&key)[S])
+// The two stage maps of a window from its histogram, by one warp: lane l holds the counts of the PER
+// bins d = PER l - L ... (v[i]: +1 group low 16 bits, -1 group high 16).  The members of a group in
+// flip order are the bins in d order, so a bin with h members of which C come before it in the group
+// holds a_k = d + 2C, d + 2C + 2, ...: h consecutive lattice intervals, one run of mask bits.
+// out[0] = +1 group (flips iff a_k <= x), out[1] = -1 group (flips iff a_k <= -x).
+template <int PER>
+__device__ __forceinline__ void stage_maps_of(const uint32_t (&v)[PER], int L, StageMap *out)
 {
     const int lane = threadIdx.x & 31;
+    uint32_t tot = 0;
 #pragma unroll
-    for (int size = 2; size <= 32 * S; size <<= 1) {
-        if (size <= S) {
+    for (int i = 0; i < PER; ++i) tot += v[i];
+    uint32_t run = tot;
 #pragma unroll
-            for (int s = 0; s < S; ++s) {
-                if ((s & (size >> 1)) == 0) {
-                    const int q = s ^ (size - 1);
-                    const uint32_t a = key[s], b = key[q];
-                    key[s] = min(a, b);
-                    key[q] = max(a, b);
-                }
-            }
-        } else {
-            const bool lower = ((lane * S) & (size >> 1)) == 0;
-            uint32_t o[S];
-#pragma unroll
-            for (int s = 0; s < S; ++s) o[s] = __shfl_xor_sync(0xFFFFFFFFu, key[S - 1 - s], size / S - 1);
-#pragma unroll
-            for (int s = 0; s < S; ++s) key[s] = lower ? min(key[s], o[s]) : max(key[s], o[s]);
-        }
-#pragma unroll
-        for (int j = size >> 2; j >= 1; j >>= 1) {
-            if (j >= S) {
-                const bool keep_min = ((lane * S) & j) == 0;
-#pragma unroll
-                for (int s = 0; s < S; ++s) {
-                    const uint32_t o = __shfl_xor_sync(0xFFFFFFFFu, key[s], j / S);
-                    key[s] = keep_min ? min(key[s], o) : max(key[s], o);
-                }
-            } else {
-#pragma unroll
-                for (int s = 0; s < S; ++s) {
-                    if ((s & j) == 0) {
-                        const uint32_t a = key[s], b = key[s + j];
-                        key[s] = min(a, b);
-                        key[s + j] = max(a, b);
-                    }
-                }
-            }
-        }
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, run, o);
+        if (lane >= o) run += y;
     }
-}
-
-// The same ascending network on 16-bit keys packed two to a register: register t of a lane holds
-// its element t (low half) and element t + S/2 (high half), so a compare-exchange of two registers
-// in the same half does two element pairs at once (__vminu2 / __vmaxu2) and a cross-lane stage
-// moves two keys per shuffle.  Pairs that meet inside one register (the top bit of the in-lane
-// index) are swapped into place with a byte permute.  S >= 2.
-static __device__ __forceinline__ uint32_t swap16(uint32_t v) { return __byte_perm(v, 0, 0x1032); }
-
-// compare-exchange of the two halves of v: the minimum to the low half
-static __device__ __forceinline__ uint32_t ce_halves(uint32_t v)
-{
-    const uint32_t w = swap16(v);
-    return __byte_perm(__vminu2(v, w), __vmaxu2(v, w), 0x7610);
-}
-
-template <int S>
-__device__ __forceinline__ void warp_bitonic16(uint32_t (&P)[S / 2])
-{
-    constexpr int H = S / 2;
-    const int lane = threadIdx.x & 31;
-#pragma unroll
-    for (int size = 2; size <= 32 * S; size <<= 1) {
-        // flip stage: element e meets e ^ (size - 1), the minimum goes to the lower one
-        if (size <= H) {
-#pragma unroll
-            for (int t = 0; t < H; ++t) {
-                if ((t & (size >> 1)) == 0) {
-                    const int q = t ^ (size - 1);
-                    const uint32_t a = P[t], b = P[q];
-                    P[t] = __vminu2(a, b);
-                    P[q] = __vmaxu2(a, b);
-                }
-            }
-        } else if (size == S) {
-            // element t (low half of P[t]) meets S-1-t (high half of P[H-1-t]), and element t + H
-            // (high half of P[t]) meets H-1-t (low half of P[H-1-t])
-#pragma unroll
-            for (int t = 0; t < H; ++t) {
-                const int q = H - 1 - t;
-                if (q == t) {
-                    P[t] = ce_halves(P[t]);
-                } else if (t < q) {
-                    const uint32_t a = P[t], b = swap16(P[q]);
-                    const uint32_t mn = __vminu2(a, b), mx = __vmaxu2(a, b);
-                    P[t] = __byte_perm(mn, mx, 0x7610);
-                    P[q] = __byte_perm(mn, mx, 0x5432);
-                }
-            }
-        } else {
-            const bool lower = ((lane * S) & (size >> 1)) == 0;
-            uint32_t o[H];
-#pragma unroll
-            for (int t = 0; t < H; ++t) o[t] = swap16(__shfl_xor_sync(0xFFFFFFFFu, P[H - 1 - t], size / S - 1));
-#pragma unroll
-            for (int t = 0; t < H; ++t) P[t] = lower ? __vminu2(P[t], o[t]) : __vmaxu2(P[t], o[t]);
-        }
-        // half-cleaners: element e meets e ^ j
-#pragma unroll
-        for (int j = size >> 2; j >= 1; j >>= 1) {
-            if (j >= S) {
-                const bool keep_min = ((lane * S) & j) == 0;
-#pragma unroll
-                for (int t = 0; t < H; ++t) {
-                    const uint32_t o = __shfl_xor_sync(0xFFFFFFFFu, P[t], j / S);
-                    P[t] = keep_min ? __vminu2(P[t], o) : __vmaxu2(P[t], o);
-                }
-            } else if (j == H) {
-#pragma unroll
-                for (int t = 0; t < H; ++t) P[t] = ce_halves(P[t]);
-            } else {
-#pragma unroll
-                for (int t = 0; t < H; ++t) {
-                    if ((t & j) == 0) {
-                        const uint32_t a = P[t], b = P[t + j];
-                        P[t] = __vminu2(a, b);
-                        P[t + j] = __vmaxu2(a, b);
-                    }
-                }
-            }
-        }
-    }
-}
-
-// rel values and the two stage maps of one window (positions [ws, ws + wlen), wlen <= 32 * S) for
-// replica r, by one warp.  out[0] = +1 group, out[1] = -1 group.
-//
-// Narrow keys: when every member has d >= -62 (d = the threshold's distance from c in sort
-// direction), the window sorts 16-bit keys (group, d clamped to [-62, 65] in 7 bits, position).
-// With d >= -62 a window entered at x = G - c in the lattice [-64, 62] keeps x in [-64, 64]
-// through both of its groups (the +1 group cannot take x below -64, the -1 group not above 64), and
-// a member clamped at the top cannot flip at any such x (+1: rel = d + 2k >= 65 > 64; -1:
-// rel = -d - 2k <= -65 < -64) and sorts after every other member of its group either way.  So the
-// stage maps and the replay of a window entered on the lattice are exact; the stored rel values of
-// clamped members are not, so the replay uses a narrow window's rel values only when it is entered
-// on the lattice (StageMap.narrow) and replays it exactly otherwise.
-template <int S>
-__device__ __forceinline__ void window_maps(const int32_t *gam_r, const uint8_t *s0, int16_t *rel_r, int ws,
-                                            int wlen, int r, int32_t c, StageMap *out)
-{
-    const int lane = threadIdx.x & 31;
-    int32_t dv[S];
-    uint32_t ng = 0;                      // bit s: member s is in the -1 group
-    int32_t np = 0;
-    bool wide = false;
-#pragma unroll
-    for (int s = 0; s < S; ++s) {
-        const int pos = s * 32 + lane;
-        dv[s] = 0;
-        if (pos < wlen) {
-            const int32_t g = gam_r[ws + pos];
-            const uint32_t neg = (s0[ws + pos] >> r) & 1u;
-            int32_t d = neg ? c - g : g - c;
-            d = min(max(d, -KEY_D), KEY_D - 1);
-            dv[s] = d;
-            ng |= neg << s;
-            np += neg ? 0 : 1;
-            wide |= d < -62;
-        }
-    }
-    np = __reduce_add_sync(0xFFFFFFFFu, np);
-    const bool narrow = S >= 2 && !__any_sync(0xFFFFFFFFu, wide);
+    run -= tot;
     unsigned long long kp = 0, km = 0;
     int32_t cle = 0, cge = 0;
-    // element e of the sorted order: group, d and position -> rel value and lattice bits, without
-    // branches (the lanes of a warp hold members of both groups at every distance)
-    auto take = [&](int e, bool neg, int32_t d, int pos) {
-        const int32_t rel = neg ? -d - 2 * (e - np) : d + 2 * e;
-        rel_r[ws + pos] = (int16_t)min(max(rel, -REL_CAP), REL_CAP);
-        // +1 group: an a_k at or below the lattice start counts into ylo, one in (-64, 62] clears
-        // the step of its lattice interval; -1 group: b_k >= -64 counts, b_k in [-64, 61] clears
-        const bool pos_grp = !neg;
-        cle += (pos_grp && rel <= -NT) ? 1 : 0;
-        const bool p_in = pos_grp && rel > -NT && rel <= NT - 2;
-        kp |= p_in ? 1ull << (((uint32_t)(rel + NT - 1) >> 1) & 63u) : 0ull;
-        const bool m_ge = neg && rel >= -NT;
-        cge += m_ge ? 1 : 0;
-        km |= (m_ge && rel <= NT - 3) ? 1ull << (((uint32_t)(rel + NT) >> 1) & 63u) : 0ull;
-    };
-    if constexpr (S >= 2) {
-        if (narrow) {
-            constexpr int H = S / 2;
-            uint32_t P[H];
+    if (tot) {
 #pragma unroll
-            for (int t = 0; t < H; ++t) {
-                uint32_t k2[2];
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const int s = t + h * H;
-                    const int pos = s * 32 + lane;
-                    uint32_t k = 0xFFFFu;
-                    if (pos < wlen) {
-                        const uint32_t neg = (ng >> s) & 1u;
-                        const int32_t dq = min(dv[s], 65) + 62;
-                        k = (neg << 15) | ((uint32_t)dq << 8) | (uint32_t)pos;
-                    }
-                    k2[h] = k;
-                }
-                P[t] = k2[0] | (k2[1] << 16);
+        for (int i = 0; i < PER; ++i) {
+            const int32_t d = lane * PER + i - L;
+            const int32_t hp = (int32_t)(v[i] & 0xFFFFu), hm = (int32_t)(v[i] >> 16);
+            if (hp) {
+                // a in (x_j, x_j + 2] clears step j; a <= -NT (j < 0) counts into ylo
+                const int32_t j0 = (d + 2 * (int32_t)(run & 0xFFFFu) + NT - 1) >> 1;
+                const int32_t lo = max(j0, 0), cnt = hp - (lo - j0);
+                cle += hp - max(cnt, 0);
+                if (cnt > 0 && lo < NT) kp |= (cnt >= NT ? ~0ull : (1ull << cnt) - 1ull) << lo;
             }
-            warp_bitonic16<S>(P);
-#pragma unroll
-            for (int s = 0; s < S; ++s) {
-                const int e = lane * S + s;
-                if (e < wlen) {
-                    const uint32_t k = (s < H ? P[s] : (P[s - H] >> 16)) & 0xFFFFu;
-                    const bool neg = (k >> 15) != 0;
-                    const int32_t d = (int32_t)((k >> 8) & 0x7Fu) - 62;
-                    take(e, neg, d, (int)(k & 0xFFu));
-                }
+            if (hm) {
+                // b = -a in [x_j, x_j + 2) clears step j; b >= -NT (j >= 0) counts into ylo
+                const int32_t jt = (NT - (d + 2 * (int32_t)(run >> 16))) >> 1;
+                const int32_t lo = max(jt - hm + 1, 0), cnt = jt - lo + 1;
+                cge += max(cnt, 0);
+                if (cnt > 0 && lo < NT) km |= (cnt >= NT ? ~0ull : (1ull << cnt) - 1ull) << lo;
             }
-        }
-    }
-    if (!narrow) {
-        uint32_t key[S];
-#pragma unroll
-        for (int s = 0; s < S; ++s) {
-            const int pos = s * 32 + lane;
-            key[s] = pos < wlen ? (((ng >> s) & 1u) << 31) | ((uint32_t)(dv[s] + KEY_D) << 8) | (uint32_t)pos
-                                : 0xFFFFFFFFu;
-        }
-        warp_bitonic<S>(key);
-#pragma unroll
-        for (int s = 0; s < S; ++s) {
-            const int e = lane * S + s;
-            if (e < wlen) {
-                const uint32_t k = key[s];
-                take(e, (k >> 31) != 0, (int32_t)((k >> 8) & 0x7FFFFFu) - KEY_D, (int)(k & 0xFFu));
-            }
+            run += v[i];
         }
     }
     const uint32_t kp0 = __reduce_or_sync(0xFFFFFFFFu, (uint32_t)kp);
     const uint32_t kp1 = __reduce_or_sync(0xFFFFFFFFu, (uint32_t)(kp >> 32));
     const uint32_t km0 = __reduce_or_sync(0xFFFFFFFFu, (uint32_t)km);
     const uint32_t km1 = __reduce_or_sync(0xFFFFFFFFu, (uint32_t)(km >> 32));
-    cle = __reduce_add_sync(0xFFFFFFFFu, cle);
-    cge = __reduce_add_sync(0xFFFFFFFFu, cge);
+    const uint32_t cc = __reduce_add_sync(0xFFFFFFFFu, (uint32_t)cle | ((uint32_t)cge << 16));
     if (lane == 0) {
         out[0].mask = ~(((unsigned long long)kp1 << 32) | kp0) & STEP_MASK;
-        out[0].ylo = -cle;
-        out[0].narrow = narrow ? 1 : 0;
+        out[0].ylo = -(int32_t)(cc & 0xFFFFu);
         out[1].mask = ~(((unsigned long long)km1 << 32) | km0) & STEP_MASK;
-        out[1].ylo = cge;
-        out[1].narrow = narrow ? 1 : 0;
+        out[1].ylo = (int32_t)(cc >> 16);
     }
+}
+
+// The two stage maps of one window (positions [ws, ws + wlen), wlen <= 32 * S) for replica r, by one
+// warp.  Nothing is sorted: the lattice sees thresholds only through the histogram of their distance d
+// from c (d in the group's flip direction), so one shared atomic per member and one scan of the bins
+// replace a sorting network of 36 stages.
+//   * d > NT never flips on the lattice and is left out (+1: a_k >= d > 62; -1: a_k > 64).
+//   * No member below -62 (the common case): 128 bins, four per lane.  Otherwise 256 bins from -190
+//     on, the first taking everything below: with at most 64 members there, each has a_k <= -64 and
+//     flips at every lattice point whatever its distance; with more, at least 64 flip at every lattice
+//     point and the window leaves the lattice from each, which is also what the counts then say.
+// bins: WBINS words of this warp's own, 16-byte aligned.
+template <int S>
+__device__ __forceinline__ void window_maps(const int32_t *gam_r, const uint8_t *s0, int ws, int wlen, int r,
+                                            int32_t c, uint32_t *bins, StageMap *out)
+{
+    const int lane = threadIdx.x & 31;
+    int32_t dv[S];
+    uint32_t ng = 0;                      // bit s: member s is in the -1 group
+    bool wide = false;
+#pragma unroll
+    for (int s = 0; s < S; ++s) {
+        const int pos = s * 32 + lane;
+        dv[s] = NT + 1;
+        if (pos < wlen) {
+            const int32_t g = gam_r[ws + pos];
+            const uint32_t neg = (s0[ws + pos] >> r) & 1u;
+            dv[s] = neg ? c - g : g - c;
+            ng |= neg << s;
+            wide |= dv[s] < -62;
+        }
+    }
+    const bool w = __any_sync(0xFFFFFFFFu, wide);
+    uint4 *b4 = reinterpret_cast<uint4 *>(bins);
+    b4[lane] = make_uint4(0u, 0u, 0u, 0u);
+    if (w) b4[lane + 32] = make_uint4(0u, 0u, 0u, 0u);
+    __syncwarp();
+    const int L = w ? 190 : 62;
+#pragma unroll
+    for (int s = 0; s < S; ++s)
+        if (dv[s] <= NT) atomicAdd(&bins[max(dv[s] + L, 0)], (ng >> s) & 1u ? 0x10000u : 1u);
+    __syncwarp();
+    if (!w) {
+        const uint4 q = b4[lane];
+        const uint32_t v[4] = {q.x, q.y, q.z, q.w};
+        stage_maps_of<4>(v, 62, out);
+    } else {
+        const uint4 q = b4[2 * lane], p = b4[2 * lane + 1];
+        const uint32_t v[8] = {q.x, q.y, q.z, q.w, p.x, p.y, p.z, p.w};
+        stage_maps_of<8>(v, 190, out);
+    }
+    __syncwarp();
+}
+
+// The same for windows of any size (up to 32,767: counts share words), members read from shared memory:
+// positions [p0, p1) of a window counted into its WBINS bins (zeroed) by one warp; several warps may
+// count parts of one window.  bins_to_maps then reads the maps off them.
+__device__ __forceinline__ void count_members(const int32_t *gam_r, const uint8_t *s0, int p0, int p1, int r, int32_t c,
+                                              uint32_t *bins)
+{
+    for (int i = p0 + (int)(threadIdx.x & 31); i < p1; i += 32) {
+        const int32_t g = gam_r[i];
+        const bool neg = (s0[i] >> r) & 1u;
+        const int32_t d = neg ? c - g : g - c;
+        if (d <= NT) atomicAdd(&bins[max(d + 190, 0)], neg ? 0x10000u : 1u);
+    }
+}
+
+__device__ __forceinline__ void bins_to_maps(const uint32_t *bins, StageMap *out)
+{
+    const uint4 *b4 = reinterpret_cast<const uint4 *>(bins);
+    const int lane = threadIdx.x & 31;
+    const uint4 q = b4[2 * lane], p = b4[2 * lane + 1];
+    const uint32_t v[8] = {q.x, q.y, q.z, q.w, p.x, p.y, p.z, p.w};
+    stage_maps_of<8>(v, 190, out);
 }
 
 static __device__ __forceinline__ int stage_apply(const StageMap &m, int t)
@@ -462,35 +335,29 @@ static __device__ __forceinline__ int stage_apply(const StageMap &m, int t)
     return (y >= 0 && y < NT) ? y : -1;
 }
 
-// the exact replay of one window by counting (|G - c| beyond the stored values), kept out of line
-static __device__ __noinline__ int32_t window_replay_exact(const int32_t *gr, const uint8_t *s0, int r, int ws, int we,
-                                                    int32_t g, bool plus_first, int32_t *bins, uint32_t *fm)
+// Replay of one window (positions [ws, we)) of replica r from the exact entering G g, by one warp: both
+// groups in order; emit(wbits) takes the flips, bit l of wbits[s] for position ws + 32 s + l.  With e = the distance of a member's threshold
+// on the flipping side of G, the members flip in e order and the k-th (from 0) flips iff e >= 2k, so with
+// N(y) = #{e >= y} the number of flips is K = max{k : N(2k - 2) >= k}, and as N(2K) <= K <= N(2K - 2)
+// the last of them has e >= 2K, = 2K - 1 or = 2K - 2: three counts give the threshold, and equal
+// members flip in position order.  K1, K2: the flips of the first and second group when the stage
+// maps gave them (the window was entered on the lattice), else -1: searched, four-way, three counts
+// to a reduction.  Returns G after the window.
+template <int SL, class Emit>
+__device__ __forceinline__ int32_t replay_window(const int32_t *gr, const uint8_t *s0, int r, int ws, int we,
+                                                 int32_t g, bool plus_first, int K1, int K2, const Emit &emit)
 {
-    const int32_t K1 = warp_group(gr, 1, 0, s0, r, ws, we, g, plus_first, bins, fm);
-    g = plus_first ? g - 2 * K1 : g + 2 * K1;
-    const int32_t K2 = warp_group(gr, 1, 0, s0, r, ws, we, g, !plus_first, bins, fm);
-    return plus_first ? g + 2 * K2 : g - 2 * K2;
-}
-
-// Replay of one window (positions [ws, we)) of replica r from x = G - c with its rel values, by one
-// warp: both groups in order, each member deciding by one comparison; the flips go into the
-// replica's flip bitmap fb.  With W a multiple of 32 every window owns whole words; otherwise
-// windows share words and OR their bits in atomically, so windows may be replayed concurrently.
-// Returns x after the window.
-template <int SL>
-__device__ __forceinline__ int32_t replay_window(const int16_t *rr, const uint8_t *s0, int r, int ws, int we,
-                                                 int32_t x, bool plus_first, uint32_t *fb, int W)
-{
+    static_assert(32 * SL < 1024, "three counts share a word");
     const int lane = threadIdx.x & 31;
     // members of the window in registers (slot s = positions ws + 32 s + lane)
-    int32_t rv[SL];
+    int32_t gv[SL];
     uint32_t ng = 0, vd = 0;            // bit s: member is -1 / exists
 #pragma unroll
     for (int s = 0; s < SL; ++s) {
         const int i = ws + 32 * s + lane;
-        rv[s] = 0;
+        gv[s] = 0;
         if (i < we) {
-            rv[s] = rr[i];
+            gv[s] = gr[i];
             vd |= 1u << s;
             ng |= ((uint32_t)(s0[i] >> r) & 1u) << s;
         }
@@ -501,18 +368,68 @@ __device__ __forceinline__ int32_t replay_window(const int16_t *rr, const uint8_
 #pragma unroll
     for (int ph = 0; ph < 2; ++ph) {
         const bool plus = plus_first == (ph == 0);
-        int32_t cnt = 0;
+        const uint32_t mem = vd & (plus ? ~ng : ng);
+        int32_t e[SL];
 #pragma unroll
-        for (int s = 0; s < SL; ++s) {
-            const bool mem = ((vd >> s) & 1u) && (((ng >> s) & 1u) != (plus ? 1u : 0u));
-            const bool f = mem && (plus ? rv[s] <= x : rv[s] >= x);
-            const unsigned bm = __ballot_sync(0xFFFFFFFFu, f);
-            cnt += __popc(bm);
-            wbits[s] |= bm;
+        for (int s = 0; s < SL; ++s) e[s] = (mem >> s) & 1u ? (plus ? g - gv[s] : gv[s] - g) : -1;
+        // #{e >= y0}, #{e >= y1}, #{e >= y2} in bits 0, 10 and 20
+        auto count3 = [&](int32_t y0, int32_t y1, int32_t y2) {
+            uint32_t n = 0;
+#pragma unroll
+            for (int s = 0; s < SL; ++s)
+                n += (e[s] >= y0 ? 1u : 0u) + (e[s] >= y1 ? 1u << 10 : 0u) + (e[s] >= y2 ? 1u << 20 : 0u);
+            return __reduce_add_sync(0xFFFFFFFFu, n);
+        };
+        int32_t K = ph == 0 ? K1 : K2;
+        if (K < 0) {
+            int32_t n0 = 0;
+#pragma unroll
+            for (int s = 0; s < SL; ++s) n0 += e[s] >= 0 ? 1 : 0;
+            n0 = __reduce_add_sync(0xFFFFFFFFu, n0);
+            int32_t lo = min(n0, 1), hi = n0;
+            while (lo < hi) {
+                const int32_t sp = hi - lo;
+                const int32_t m1 = lo + ((sp + 3) >> 2), m2 = lo + ((2 * sp + 3) >> 2), m3 = lo + ((3 * sp + 3) >> 2);
+                const uint32_t n = count3(2 * m1 - 2, 2 * m2 - 2, 2 * m3 - 2);
+                if ((int32_t)(n >> 20) >= m3) lo = m3;
+                else if ((int32_t)((n >> 10) & 1023u) >= m2) { lo = m2; hi = m3 - 1; }
+                else if ((int32_t)(n & 1023u) >= m1) { lo = m1; hi = m2 - 1; }
+                else hi = m1 - 1;
+            }
+            K = lo;
         }
-        x = plus ? x - 2 * cnt : x + 2 * cnt;
+        if (K == 0) continue;
+        const uint32_t n = count3(2 * K, 2 * K - 1, 2 * K - 2);
+        const int32_t n0 = n & 1023u, n1 = (n >> 10) & 1023u, n2 = n >> 20;
+        // ties at y flip up to `left`; everything above flips
+        const int32_t y = n0 == K ? 2 * K : (n1 >= K ? 2 * K - 1 : 2 * K - 2);
+        const int32_t at = n0 == K ? n0 : (n1 >= K ? n1 : n2);
+        if (at == K) {
+#pragma unroll
+            for (int s = 0; s < SL; ++s) wbits[s] |= __ballot_sync(0xFFFFFFFFu, e[s] >= y);
+        } else {
+            int32_t left = K - (n1 >= K ? n0 : n1);
+#pragma unroll
+            for (int s = 0; s < SL; ++s) {
+                const unsigned tm = __ballot_sync(0xFFFFFFFFu, e[s] == y);
+                const int32_t idx = __popc(tm & ((1u << lane) - 1u));
+                wbits[s] |= __ballot_sync(0xFFFFFFFFu, e[s] > y || (e[s] == y && idx < left));
+                left -= __popc(tm);
+            }
+        }
+        g = plus ? g - 2 * K : g + 2 * K;
     }
-    // flip words: slot s covers positions [ws + 32 s, ws + 32 s + 32)
+    emit(wbits);
+    return g;
+}
+
+// the flips of a window (positions [ws, we)) into a flip bitmap.  With W a multiple of 32 every window
+// owns whole words; otherwise windows share words and OR their bits in atomically, so windows may be
+// replayed concurrently.
+template <int SL>
+__device__ __forceinline__ void flips_to_bitmap(const uint32_t (&wbits)[SL], int ws, int we, uint32_t *fb, int W)
+{
+    const int lane = threadIdx.x & 31;
     if ((W & 31) == 0) {
 #pragma unroll
         for (int s = 0; s < SL; ++s)
@@ -527,9 +444,81 @@ __device__ __forceinline__ int32_t replay_window(const int16_t *rr, const uint8_
             if (sh) atomicOr(&fb[q + 1], wbits[s] >> (32 - sh));
         }
     }
-    return x;
 }
 
+// The same for windows of any size, members read from shared memory in each pass; emit(i0, bits) takes the
+// flips of positions i0 .. i0 + 31 (once per group).
+template <class Emit>
+__device__ __noinline__ int32_t replay_large(const int32_t *gr, const uint8_t *s0, int r, int ws, int we, int32_t g,
+                                             bool plus_first, int K1, int K2, const Emit &emit)
+{
+    const int lane = threadIdx.x & 31;
+    for (int ph = 0; ph < 2; ++ph) {
+        const bool plus = plus_first == (ph == 0);
+        auto margin = [&](int i) {
+            const bool neg = (s0[i] >> r) & 1u;
+            return plus == neg ? -1 : (plus ? g - gr[i] : gr[i] - g);
+        };
+        auto count = [&](int32_t y) {
+            int32_t n = 0;
+            for (int i = ws + lane; i < we; i += 32) n += margin(i) >= y ? 1 : 0;
+            return (int32_t)__reduce_add_sync(0xFFFFFFFFu, n);
+        };
+        int32_t K = ph == 0 ? K1 : K2;
+        if (K < 0) {
+            int32_t hi = count(0), lo = min(hi, 1);
+            while (lo < hi) {
+                const int32_t mid = (lo + hi + 1) >> 1;
+                if (count(2 * mid - 2) >= mid) lo = mid; else hi = mid - 1;
+            }
+            K = lo;
+        }
+        if (K == 0) continue;
+        int32_t n0 = 0, n1 = 0;
+        for (int i = ws + lane; i < we; i += 32) {
+            const int32_t e = margin(i);
+            n0 += e >= 2 * K ? 1 : 0;
+            n1 += e >= 2 * K - 1 ? 1 : 0;
+        }
+        n0 = __reduce_add_sync(0xFFFFFFFFu, n0);
+        n1 = __reduce_add_sync(0xFFFFFFFFu, n1);
+        const int32_t y = n0 == K || n1 >= K ? 2 * K - 1 : 2 * K - 2;
+        int32_t left = n0 == K ? 0 : (n1 >= K ? K - n0 : K - n1);
+        for (int i0 = ws; i0 < we; i0 += 32) {
+            const int32_t e = i0 + lane < we ? margin(i0 + lane) : -1;
+            const unsigned tm = __ballot_sync(0xFFFFFFFFu, e == y);
+            const int32_t idx = __popc(tm & ((1u << lane) - 1u));
+            const unsigned bits = __ballot_sync(0xFFFFFFFFu, e > y || (e == y && idx < left));
+            left -= min(left, __popc(tm));
+            if (bits) emit(i0, bits);
+        }
+        g = plus ? g - 2 * K : g + 2 * K;
+    }
+    return g;
+}
+
+// flips of both groups of a window entered at lattice index t (-1: off the lattice), in order: -1 from
+// where its stage maps leave the lattice
+__device__ __forceinline__ void mapped_flips(bool plus_first, int t, const StageMap *maps, int &K1, int &K2)
+{
+    K1 = K2 = -1;
+    const int u = stage_apply(maps[plus_first ? 0 : 1], t);
+    if (u >= 0) {
+        K1 = plus_first ? t - u : u - t;
+        const int v = stage_apply(maps[plus_first ? 1 : 0], u);
+        if (v >= 0) K2 = plus_first ? v - u : u - v;
+    }
+}
+
+// replay_window for a window entered at lattice index t with its stage maps
+template <int SL, class Emit>
+__device__ __forceinline__ int32_t replay_mapped(const int32_t *gr, const uint8_t *s0, int r, int ws, int we, int32_t g,
+                                                 bool plus_first, int t, const StageMap *maps, const Emit &emit)
+{
+    int K1, K2;
+    mapped_flips(plus_first, t, maps, K1, K2);
+    return replay_window<SL>(gr, s0, r, ws, we, g, plus_first, K1, K2, emit);
+}
 
 }  // namespace win
 }  // namespace gdi

@@ -211,3 +211,24 @@ def test_cta_sorted_32bit_columns(gdi):
     ann.close()
     ref = oracle.anneal(g, replicas=2, **kw)
     assert_parity(res, spins, tr, ref)
+
+
+@pytest.mark.parametrize("path", ["cta", "grid"])
+@pytest.mark.parametrize("W,t0,mode", [(256, 60.0, 0), (256, 400.0, 0), (250, 1000.0, 0), (64, 400.0, 0),
+                                       (32, 1000.0, 0), (256, 1.0, 1), (5, 400.0, 0)])
+def test_counted_windows_with_thresholds_far_from_g(gdi, path, W, t0, mode):
+    """Windows whose thresholds spread far to either side of G: counted in the wide bins, with fewer and
+    with more than 64 members below them (a hot start, and flips forced by the draw in the P_f mode),
+    from a balanced and from a one-sided start, bit-exact."""
+    g = barabasi_albert(3000, 5, 77)
+    init = np.where(np.random.default_rng(5).random((2, g.n)) < 0.8, 1, -1).astype(np.int8)
+    sch = gdi.Schedule(sweeps=6, t0=t0, t1=t0 / 2 if mode == 0 else 0.1, mode=mode, pf0=0.45, pf1=0.05)
+    for start in (None, init):
+        ann = gdi.Annealer(g, A=1, B=1, W=W, replicas=2)
+        ann.configure(path=gdi.GDI_PATH_GRID if path == "grid" else gdi.GDI_PATH_CTA)
+        ann.anneal(sch, 3, init=start, flags=gdi.GDI_FLAG_TRACE)
+        res, spins, tr = ann.results(), ann.spins(), ann.trace()
+        ann.close()
+        ref = oracle.anneal(g, A=1, B=1, W=W, mode=mode, t0=t0, t1=sch.t1, pf0=0.45, pf1=0.05, sweeps=6, seed=3,
+                            replicas=2, init=start, trace=True)
+        assert_parity(res, spins, tr, ref)
