@@ -58,11 +58,11 @@ extern "C" {
                              above a few thousand vertices, or whenever the CTA path's shared
                              memory does not fit; CTA-resident otherwise                         */
 #define GDI_PATH_CTA  1   /* one thread block anneals one (instance, replica), spins in shared
-                             memory; with 1 <= W <= 256, when the items fill at most half of the
-                             SMs and the largest class has 8 to 128 windows, a cluster of two
-                             blocks anneals each item (gdi_last_launch counts both blocks)       */
+                             memory; with 1 <= W <= 256, when the items leave SMs idle and the
+                             largest class has at least four windows for each block, a cluster of
+                             2, 4 or 8 blocks anneals each item (gdi_last_launch counts them all) */
 #define GDI_PATH_GRID 2   /* one instance over every SM (needs W >= 1); up to 8 replicas per pass;
-                             W <= 256: sorted-window kernel, W > 256: tabulated-window kernel */
+                             windows counted, or tabulated (W > 256 where that fits alone)       */
 
 /* gdi_run.flags */
 #define GDI_FLAG_TRACE     1  /* record per-sweep G, cut and state digest (slower; for parity)     */
@@ -171,7 +171,8 @@ int gdi_balance(gdi_ctx *ctx, int32_t instance, int32_t replica, int32_t *raw_G,
 int gdi_get_trace(gdi_ctx *ctx, uint64_t *digest, int32_t *G, int64_t *cut);
 
 /* Launch configuration of later gdi_anneal calls: kernel path (GDI_PATH_*), threads per block of
- * the CTA-resident path (0 = keep, else 128/256/512/1024) and a cap on the number of blocks
+ * the CTA-resident path (0 = keep, at first chosen by size; else 128/256/512/1024) and a cap on the
+ * number of blocks
  * (0 = one wave on every SM).  Results do not depend on any of these (the autotuner relies on it). */
 int gdi_configure(gdi_ctx *ctx, int32_t path, int32_t block, int32_t grid_limit);
 

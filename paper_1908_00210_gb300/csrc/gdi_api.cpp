@@ -73,7 +73,7 @@ struct gdi_ctx {
     int device = 0;
     int32_t Q = 0, R = 1, A = 0, B = 1, W = 0;
     int64_t N = 0, nnz = 0;
-    int32_t max_n = 0, max_window = 0, max_degree = 0, max_class = 0, max_class_nnz = 0;
+    int32_t max_n = 0, max_window = 0, max_degree = 0, max_class = 0, max_class_nnz = 0, max_item_nnz = 0;
     int32_t path = 0;                        // GDI_PATH_*
     DevBuf<uint8_t> g_packed, g_rflags;
     DevBuf<int16_t> g_tables;
@@ -116,7 +116,7 @@ struct gdi_ctx {
     int32_t last_sweeps = 0, last_flags = 0, ecap = 0;
     bool annealed = false;
     cudaStream_t stream = nullptr;
-    int block = 256;
+    int block = 0;                           // 0: chosen per call (gdi_cta_default_block)
     int grid_limit = 0;
     int last_grid = 0;
     size_t last_smem = 0;
@@ -142,6 +142,7 @@ struct gdi_ctx {
         P.max_degree = max_degree;
         P.max_class = max_class;
         P.max_class_nnz = max_class_nnz;
+        P.max_item_nnz = max_item_nnz;
         return P;
     }
     void release()
@@ -491,6 +492,9 @@ int gdi_create(gdi_ctx **out, const gdi_graph *g, const gdi_model *m)
     c->max_class = H.max_class;
     c->max_degree = H.max_degree;
     c->max_class_nnz = H.max_class_nnz <= (1 << 20) ? (int32_t)H.max_class_nnz : 0;
+    int64_t most = 0;
+    for (int32_t q = 0; q < Q; ++q) most = std::max(most, rp[(size_t)inst[(size_t)q + 1]] - rp[(size_t)inst[(size_t)q]]);
+    c->max_item_nnz = most <= (1 << 20) ? (int32_t)most : 0;
     // window costs for the grid path's weighted split: a rank costs its degree plus a constant for
     // its threshold and its share of the window sort (both measured as about 12 neighbour reads)
     if (Q == 1 && c->W >= 1) {
@@ -735,10 +739,12 @@ int gdi_anneal(gdi_ctx *c, const gdi_schedule *S, const gdi_run *run)
     R.item_order = c->item_order.p;
     R.item_counter = c->item_counter.p;
 
-    size_t need = 0;
-    gdi_cta_smem_bytes(P, R, c->block, &need);
     int max_optin = 0, sms = 0;
     cudaDeviceGetAttribute(&max_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device);
+    int block = c->block ? c->block : gdi_cta_default_block(P, R);
+    size_t need = 0;
+    gdi_cta_smem_bytes(P, R, block, &need);
+    if (!c->block && need > (size_t)max_optin) gdi_cta_smem_bytes(P, R, block = 256, &need);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
     bool grid = false;
     if ((run->flags & GDI_FLAG_STANDARD) && ((run->flags & GDI_FLAG_RACY) || c->path == GDI_PATH_GRID))
@@ -751,19 +757,26 @@ int gdi_anneal(gdi_ctx *c, const gdi_schedule *S, const gdi_run *run)
         // 10; 1 to 152 replicas; 100 sweeps).  Per sweep, a CTA-resident block costs about 2 us
         // per colour class + 1.8 ns (blocks of 128 or 256 threads) or 1.2 ns (512, 1024) per
         // (vertex + directed edge), per wave of resident blocks; a grid-scale launch costs about
-        // 13 us per colour class (thresholds, sort, chain and barrier) + 0.02 ns per (vertex +
-        // edge), per group of 8 replicas.
+        // 13 us per colour class (thresholds, counts, chain and barrier) + 0.02 ns per (vertex +
+        // edge), per group of 8 replicas.  A cluster of blocks per replica costs about 5.5 us a
+        // class (9 with windows above 128) + 0.55 ns per (vertex + edge) of a block's share; the
+        // figures behind it (ms, cluster against grid): one replica of BA 20,000 and 30,000 at
+        // W = 64 13.9 / 21.4 and 5.3 / 7.5, 8 of 8,000 11.2 / 25.7, 3 of 30,000 at W = 256 7.3 / 8.3.
+        // The model is good to about a fifth, so the cluster has to win by that much.
         int per_sm = 0;
-        if (need > (size_t)max_optin || gdi_cta_blocks_per_sm(P, R, c->block, &per_sm) != 0 || per_sm < 1) {
+        if (need > (size_t)max_optin || gdi_cta_blocks_per_sm(P, R, block, &per_sm) != 0 || per_sm < 1) {
             grid = true;
         } else {
             const double work = (double)c->N + (double)c->nnz;
             const double ncls = (double)c->num_classes[0];
             const int64_t slots = (int64_t)sms * per_sm;
-            const double per_work = c->block >= 512 ? 1.2e-9 : 1.8e-9;
+            const double per_work = block >= 512 ? 1.2e-9 : 1.8e-9;
             const double cta_s = (double)((c->R + slots - 1) / slots) * (2e-6 * ncls + per_work * work);
             const double grid_s = (double)((c->R + 7) / 8) * (13e-6 * ncls + 0.02e-9 * work);
             grid = grid_s < cta_s;
+            const int cl = gdi_cta_cluster_size(P, R, block);
+            if (cl > 1 && P.col16)
+                grid = 0.8 * grid_s < (c->W > 128 ? 9e-6 : 5.5e-6) * ncls + 0.55e-9 * work / cl;
         }
     }
     // kernel timing events (not while the stream is being captured into a graph)
@@ -790,7 +803,7 @@ int gdi_anneal(gdi_ctx *c, const gdi_schedule *S, const gdi_run *run)
                                                " bytes of shared memory per block (limit " +
                                                std::to_string(max_optin) + "); use one instance with W > 0");
         if (timer.ev) cudaEventRecord(timer.ev[0], st);
-        int ke = gdi_launch_cta_anneal(P, R, c->block, c->grid_limit, st, &c->last_grid, &c->last_smem);
+        int ke = gdi_launch_cta_anneal(P, R, block, c->grid_limit, st, &c->last_grid, &c->last_smem);
         if (ke) return cuda_fail((cudaError_t)ke, "anneal kernel launch");
         if (timer.ev) {
             cudaEventRecord(timer.ev[1], st);
@@ -1046,7 +1059,7 @@ int gdi_autotune(gdi_ctx *c, const gdi_schedule *S, int32_t probe_sweeps, int32_
     if (rc != GDI_OK) { c->block = keep_block; c->grid_limit = keep_grid; return rc; }
     c->block = best_b;
     c->grid_limit = best_g;
-    if (block_out) *block_out = best_b;
+    if (block_out) *block_out = best_b ? best_b : 256;   // (the grid path ignores the block size)
     if (grid_out) *grid_out = best_g;
     if (ms_out) *ms_out = best;
     return GDI_OK;

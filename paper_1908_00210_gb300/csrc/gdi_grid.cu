@@ -9,13 +9,13 @@
 // counters); every block owns a contiguous run of windows of each class; the map "G at window
 // start -> G at window end" is monotone and is tabulated around c, the G at class start.
 //
-// Sorted-window variant (W <= 256, gdi_grid_sorted_kernel): a warp sorts each (window, replica)
-// group once, after which every member decides its own flip by one comparison; block tables are
-// published with the class parity in every byte and each block finds its entering G by looking
-// them up, so only one grid barrier per class remains (described before the kernel).  The local
-// fields are kept across classes and updated by the flips (atomic adds to the neighbours).
+// Counted-window variant (gdi_grid_sorted_kernel): the counts of a window's threshold distances give its
+// map and later its flips (gdi_window.cuh); block tables are published with the class parity in every
+// byte and each block finds its entering G by looking them up, so only one grid barrier per class remains
+// (described before the kernel).  The local fields are kept across classes and updated by the flips
+// (atomic adds to the neighbours).
 //
-// Tabulated variant (W > 256, gdi_grid_anneal_kernel):
+// Tabulated variant (gdi_grid_anneal_kernel; W > 256 where the counted variant's buffers do not fit):
 //   * every window tabulates its map for G in [c - RT, c + RT] from two small histograms of its
 //     thresholds, and each block composes the maps of its consecutive windows;
 //   * after a grid barrier one block per replica walks the P block maps (a few hundred
@@ -96,7 +96,9 @@ struct GridArgs {
     int spc, wpc;
     const int32_t *wbnd;    // [classes][blocks + 1] first window of every block, or null (even split)
     unsigned long long *hf; // maintained fields (X.hfield) when this kernel keeps them, else null
-    bool es_pre;            // sorted path: E* of the next class drawn ahead into shared memory
+    bool es_pre;            // counted path: E* of the next class drawn ahead into shared memory
+    bool tables;            // counted path: window maps composed as tables, windows replayed by all warps
+    bool binned;            // counted path: thresholds counted into their window's bins as they are made
 };
 
 // ---------------------------------------------------------------------------------------------
@@ -374,11 +376,15 @@ __device__ void estar_ahead(const GridArgs &A, const uint32_t *row, int32_t a0, 
 // warp).  Otherwise only replica `one`, stored at gam_out[i * gis] with fields [i] (thread-serial
 // rows; used by the rare exact fallback).  gam_out must hold 8 ints per rank either way (the
 // long-row partial sums live there before the thresholds are written).
+// seen(i, r, negative, threshold) is called once per threshold (after gc_out is visible).
+struct NoThreshold { __device__ void operator()(int32_t, int, bool, int32_t) const {} };
+
+template <class Seen = NoThreshold>
 __device__ void range_thresholds(const GridArgs &A, const GSmem &S, int32_t a0, int32_t a1, int sw,
                                  bool all_reps, int one, int32_t *gam_out, int gis, int grs, uint8_t *s0_out,
                                  int16_t *hbuf, int32_t rlen, float Tsw, bool quad_rows = false,
                                  const int16_t *es_in = nullptr, int es_s = 0, int32_t *gc_out = nullptr,
-                                 int32_t gc_val = 0)
+                                 int32_t gc_val = 0, const Seen &seen = Seen())
 {
     const GdiDevProblem &P = A.P;
     const int64_t base = P.node_off[0];
@@ -490,8 +496,9 @@ __device__ void range_thresholds(const GridArgs &A, const GSmem &S, int32_t a0, 
                 const int sg = ((s0_out[i] >> r) & 1) ? -1 : 1;
                 const int32_t h = hbuf[(size_t)i * hs + (all_reps ? r : 0)];
                 const int32_t es = estar_of(S.row, rlen, A.R.mode, word_of(u4, j), Tsw);
-                gam_out[(size_t)i * gis + (size_t)(all_reps ? r : 0) * grs] =
-                    a_shift >= 0 ? gamma_of_shift(sg, h, es, P.A, P.B, a_shift) : gamma_of(sg, h, es, P.A, P.B);
+                const int32_t gm = a_shift >= 0 ? gamma_of_shift(sg, h, es, P.A, P.B, a_shift) : gamma_of(sg, h, es, P.A, P.B);
+                gam_out[(size_t)i * gis + (size_t)(all_reps ? r : 0) * grs] = gm;
+                seen(i, r, sg < 0, gm);
             }
         };
         const int32_t nq = q1 - q0 + 1;
@@ -528,6 +535,7 @@ __device__ void range_thresholds(const GridArgs &A, const GSmem &S, int32_t a0, 
                     const int32_t h = hbuf[(size_t)i * 8 + r];
                     const int32_t es = ev[j];
                     g[j] = a_shift >= 0 ? gamma_of_shift(sg, h, es, P.A, P.B, a_shift) : gamma_of(sg, h, es, P.A, P.B);
+                    seen(i, r, sg < 0, g[j]);
                 }
                 *reinterpret_cast<int4 *>(row + 4 * qq) = make_int4(g[0], g[1], g[2], g[3]);
             }
@@ -884,16 +892,14 @@ __global__ void __launch_bounds__(GB, 1) gdi_grid_anneal_kernel(GridArgs A)
 }
 
 // =============================================================================================
-// Sorted-window path (1 <= W <= 256).
+// Counted-window path.
 //
-// One warp takes one (window, replica): lanes hold the window's members (up to 8 per lane) with
-// keys (group, threshold distance from the class-start G c, position), and a bitonic sort puts
-// each group in its flip order.  The k-th member of the +1 group (gamma ascending) flips iff
-// G - 2k >= gamma_(k), i.e. iff a_k = gamma_(k) + 2k <= G; a_k is strictly increasing, so for any
-// entering G the flips are exactly the members with a_k <= G -- one comparison per member, no
-// histogram.  The -1 group likewise flips iff b_k = gamma'_(k) - 2k >= G.  Every member keeps
-// rel = a_k - c (or b_k - c) in shared memory; the exact replay of a window is then two warp
-// counts.
+// Every threshold is counted into its (window, replica)'s 128 bins of distances from the class-start G c as
+// it is made; one warp per (window, replica) turns the bins into prefix counts, the window's two stage maps
+// and a byte table of both composed over 64 lattice points.  Where a distance lies below the bins, or they
+// do not fit shared memory, the warp counts the window's members itself.  Sorting the members instead
+// (36 stages of a 256-key network, then a comparison value per member) took 45 of 180 us of a sweep of
+// 10^6 vertices x 8 replicas; counting them takes about 18.
 //
 // Block maps: on the lattice x = G - c in {-64, -62, ..., 62} (64 points; G - c is always even) a
 // group is a staircase: index j -> ylo + popcount(mask & bits below j), read from where the a_k
@@ -902,8 +908,10 @@ __global__ void __launch_bounds__(GB, 1) gdi_grid_anneal_kernel(GridArgs A)
 // parity in every byte, so a reader needs no flag.  The last block of every run of 16 blocks also
 // composes the run's tables into a run table.  Every block then fetches the run tables before it
 // and the block tables of its own run (one poll of all of them per round trip) and looks its exact
-// entering G up from c: at most 160 / 16 + 15 byte lookups, without a grid barrier.  Where the walk leaves the lattice, the block whose table failed publishes its exact
-// outgoing G (it knows its own entering G and replays exactly), and the walk continues from it.
+// entering G up from c: at most 160 / 16 + 15 byte lookups, without a grid barrier.  It looks the entering point of each of its own
+// windows up the same way, and all warps replay the windows at once: K from the stage maps, the cut from
+// the prefix counts, one pass over the members.  Where the walk leaves the lattice, the block whose table
+// failed publishes its exact outgoing G (it knows its own entering G and replays exactly), and the walk continues from it.
 // One grid barrier per class remains: the next class reads this class's spins.
 constexpr int SMAXW = 256;              // windows a warp holds in registers
 constexpr int CMAXW = 32767;            // windows whose counts fit 16 bits
@@ -914,13 +922,19 @@ __host__ __device__ inline int walk_slots(int P) { return nruns(P) + 2 * RUN; }
 
 
 struct SortedLayout {
-    size_t off_h, off_gam, off_es, off_s0, off_fm, off_fbits, off_longq, off_smap, off_walk, off_row, off_misc, total;
+    size_t off_h, off_gam, off_es, off_s0, off_fm, off_fbits, off_longq, off_smap, off_wtab, off_tin, off_walk, off_row, off_bins, off_misc, total;
     int fw;                             // words of one replica's flip bitmap
     int gs;                             // threshold row stride (ints): >= spc + 7, 4 mod 32
     int es;                             // E* row stride (int16): >= spc + 7, 16 mod 32; 0 = no E* rows
 };
 
-__host__ __device__ inline SortedLayout sorted_layout(int spc, int wpc, int max_row, int P, bool es_rows)
+// bins of one (window, replica): 128 counts, the word that says a distance lay below them, padding that
+// sets the replicas' bins four banks apart
+constexpr int GBINS = 132;
+constexpr int GB_WIDE = 128;
+constexpr int GB_L = 62;                // distance of the first bin
+
+__host__ __device__ inline SortedLayout sorted_layout(int spc, int wpc, int max_row, int P, bool es_rows, bool tables, bool binned)
 {
     SortedLayout L;
     size_t o = 0;
@@ -940,8 +954,11 @@ __host__ __device__ inline SortedLayout sorted_layout(int spc, int wpc, int max_
     L.off_fbits = o; o = align16(o + (size_t)8 * L.fw * sizeof(uint32_t));
     L.off_longq = o; o = align16(o + (size_t)2 * spc * sizeof(int32_t));   // long rows, chunk counts
     L.off_smap = o; o = align16(o + (size_t)wpc * 8 * 2 * sizeof(StageMap));
+    L.off_wtab = o; o = align16(o + (tables ? (size_t)wpc * 8 * NT : 0));   // both maps of a window composed
+    L.off_tin = o; o = align16(o + (tables ? (size_t)wpc * 8 : 0));         // its entering lattice index, or -1
     L.off_walk = o; o = align16(o + (size_t)8 * walk_slots(P) * NT);
     L.off_row = o; o = align16(o + (size_t)(max_row + 4) * sizeof(uint32_t));
+    L.off_bins = o; o = align16(o + (binned ? (size_t)wpc * 8 * GBINS * sizeof(uint32_t) : 0));
     L.off_misc = o; o = align16(o + 64 * sizeof(int64_t));
     L.total = o;
     return L;
@@ -1062,6 +1079,25 @@ __device__ bool fetch_valid(const int8_t *a, int na, int8_t *da, const int8_t *b
     return ok;
 }
 
+// one window's replay into its replica's flip bitmap (SL as below)
+template <int SL>
+__device__ __forceinline__ int32_t grid_replay(const int32_t *gr, const uint8_t *s0, int r, int ws, int we, int32_t g,
+                                               bool plus_first, int K1, int K2, const WindowCounts &wc, uint32_t *fb, int W)
+{
+    if constexpr (SL > 0) {
+        return replay_window<SL>(gr, s0, r, ws, we, g, plus_first, K1, K2, wc,
+                                 [&](const uint32_t (&wb)[SL]) { flips_to_bitmap<SL>(wb, ws, we, fb, W); });
+    } else {
+        return replay_large(gr, s0, r, ws, we, g, plus_first, K1, K2, wc, [&](int i0, unsigned bits) {
+            if ((threadIdx.x & 31) == 0) {
+                const int sh = i0 & 31;
+                atomicOr(&fb[i0 >> 5], bits << sh);
+                if (sh && bits >> (32 - sh)) atomicOr(&fb[(i0 >> 5) + 1], bits >> (32 - sh));
+            }
+        });
+    }
+}
+
 // SL = members per lane of a window (1, 2, 4 or 8; 0: windows above 256, members read from shared
 // memory): one instantiation per window size class
 template <int SL>
@@ -1074,7 +1110,7 @@ __global__ void __launch_bounds__(GB, 1) gdi_grid_sorted_kernel(GridArgs A)
     const int Pb = gridDim.x, p = blockIdx.x;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int spc = A.spc;
-    const SortedLayout L = sorted_layout(spc, A.wpc, R.max_row, Pb, A.es_pre);
+    const SortedLayout L = sorted_layout(spc, A.wpc, R.max_row, Pb, A.es_pre, A.tables, A.binned);
     int16_t *hb = reinterpret_cast<int16_t *>(smem_raw + L.off_h);   // fields [i*8 + r], then the counting warps' bins
     int32_t *gam = reinterpret_cast<int32_t *>(smem_raw + L.off_gam);
     int16_t *esb = reinterpret_cast<int16_t *>(smem_raw + L.off_es);   // E* drawn ahead [r][L.es]
@@ -1082,6 +1118,10 @@ __global__ void __launch_bounds__(GB, 1) gdi_grid_sorted_kernel(GridArgs A)
     StageMap *smap = reinterpret_cast<StageMap *>(smem_raw + L.off_smap);
     uint32_t *hist = reinterpret_cast<uint32_t *>(smem_raw + L.off_h);
     int8_t *walk = reinterpret_cast<int8_t *>(smem_raw + L.off_walk);
+    int8_t *wtab = reinterpret_cast<int8_t *>(smem_raw + L.off_wtab);   // [window][replica][NT]
+    int8_t *tin = reinterpret_cast<int8_t *>(smem_raw + L.off_tin);     // [window][replica]
+    uint32_t *gbins = reinterpret_cast<uint32_t *>(smem_raw + L.off_bins);   // [window][replica][GBINS]
+    const int w_shift = (P.W & (P.W - 1)) == 0 ? __ffs(P.W) - 1 : -1;
     uint32_t *fbits = reinterpret_cast<uint32_t *>(smem_raw + L.off_fbits);   // [r][fw] fast-path flips
     GSmem S = {};
     S.longq = reinterpret_cast<int32_t *>(smem_raw + L.off_longq);
@@ -1104,6 +1144,8 @@ __global__ void __launch_bounds__(GB, 1) gdi_grid_sorted_kernel(GridArgs A)
     const int nrep = A.nrep;
 
     if (!plan_fits(A)) return;
+    if (A.binned)
+        for (int i = threadIdx.x; i < A.wpc * 8 * GBINS; i += GB) gbins[i] = 0;
     init_G(A, p, Pb, n, base);
     if (A.hf) init_fields(A, p, Pb, n, base);
     if (!grid_sync(X)) return;
@@ -1164,35 +1206,41 @@ __global__ void __launch_bounds__(GB, 1) gdi_grid_sorted_kernel(GridArgs A)
             // thresholds of rank a0 + i for replica r at gamc[r * gs + i]
             int32_t *gamc = gam + (a0 & 3);
             range_thresholds(A, S, a0, a1, sw, true, 0, gamc, 1, L.gs, s0, hb, rlen, Tsw, true,
-                             have_es ? esb : nullptr, L.es, threadIdx.x < nrep ? Gc : nullptr, gcl);
+                             have_es ? esb : nullptr, L.es, threadIdx.x < nrep ? Gc : nullptr, gcl,
+                             [&](int32_t i, int r, bool neg, int32_t gm) {
+                                 if (!A.binned) return;
+                                 const int kk = w_shift >= 0 ? i >> w_shift : i / W;
+                                 uint32_t *b = gbins + (size_t)(kk * 8 + r) * GBINS;
+                                 const int32_t d = neg ? Gc[r] - gm : gm - Gc[r];
+                                 if (d < -GB_L) b[GB_WIDE] = 1;
+                                 else if (d <= NT) atomicAdd(&b[d + GB_L], neg ? 0x10000u : 1u);
+                             });
             // ---- counts and stage maps of every (window, replica)
-            if constexpr (SL > 0) {
-                for (int task = warp; task < nwin * nrep; task += NWARP) {
-                    const int kk = task / nrep, r = task % nrep;
-                    const int ws = kk * W, wlen = min(W, ns - ws);
-                    window_maps<SL>(gamc + (size_t)r * L.gs, s0, ws, wlen, r, Gc[r], hist + (size_t)warp * WBINS,
-                                    smap + ((size_t)kk * 8 + r) * 2);
+            // (counted with their thresholds, or here where the bins do not fit or a distance lay below them)
+            for (int task = warp; task < nwin * nrep; task += NWARP) {
+                const int kk = task / nrep, r = task % nrep;
+                const int ws = kk * W, wlen = min(W, ns - ws);
+                StageMap *o = smap + ((size_t)kk * 8 + r) * 2;
+                uint32_t *b = gbins + (size_t)(kk * 8 + r) * GBINS;
+                if (A.binned && !b[GB_WIDE]) {
+                    bins_to_prefix<4>(b, GB_L, o);
+                } else if constexpr (SL > 0) {
+                    window_maps<SL>(gamc + (size_t)r * L.gs, s0, ws, wlen, r, Gc[r], hist + (size_t)warp * WBINS, o);
+                } else {
+                    uint32_t *wb = hist + (size_t)warp * WBINS;
+                    for (int i = lane; i < WBINS; i += 32) wb[i] = 0;
+                    __syncwarp();
+                    count_members(gamc + (size_t)r * L.gs, s0, ws, ws + wlen, r, Gc[r], wb);
+                    __syncwarp();
+                    bins_to_maps(wb, o);
                 }
-            } else {
-                // large windows are few: several warps count the parts of one (window, replica)
-                const int ntask = nwin * nrep;
-                const int parts = ntask > 0 && ntask < NWARP ? NWARP / ntask : 1;
-                const int per = NWARP / parts, grp = warp / parts, part = warp % parts;
-                for (int t0 = 0; t0 < ntask; t0 += per) {
-                    const int task = t0 + grp;
-                    const bool mine = grp < per && task < ntask;
-                    const int kk = task / nrep, r = task % nrep;
-                    uint32_t *bins = hist + (size_t)grp * WBINS;
-                    if (mine && part == 0)
-                        for (int b = lane; b < WBINS; b += 32) bins[b] = 0;
-                    __syncthreads();
-                    if (mine) {
-                        const int ws = kk * W, we = min(ws + W, ns), len = ((we - ws + parts - 1) / parts + 31) & ~31;
-                        count_members(gamc + (size_t)r * L.gs, s0, min(ws + part * len, we), min(ws + (part + 1) * len, we), r,
-                                      Gc[r], bins);
-                    }
-                    __syncthreads();
-                    if (mine && part == 0) bins_to_maps(bins, smap + ((size_t)kk * 8 + r) * 2);
+                __syncwarp();
+                if (A.tables) {
+                    const StageMap m0 = o[plus_first ? 0 : 1], m1 = o[plus_first ? 1 : 0];
+                    int8_t *wt = wtab + (size_t)(kk * 8 + r) * NT;
+                    wt[lane] = (int8_t)stage_apply(m1, stage_apply(m0, lane));
+                    wt[lane + 32] = (int8_t)stage_apply(m1, stage_apply(m0, lane + 32));
+                    __syncwarp();
                 }
             }
             for (int i = threadIdx.x; i < 8 * L.fw; i += GB) fbits[i] = 0;
@@ -1203,11 +1251,17 @@ __global__ void __launch_bounds__(GB, 1) gdi_grid_sorted_kernel(GridArgs A)
             if (warp < nrep) {
                 const int r = warp;
                 for (int kk = 0; kk < nwin; ++kk) {
+                    if (A.tables) {
+                        const int8_t *wt = wtab + (size_t)(kk * 8 + r) * NT;
+                        if (t0 >= 0) t0 = wt[t0];
+                        if (t1 >= 0) t1 = wt[t1];
+                    } else {
 #pragma unroll
-                    for (int ph = 0; ph < 2; ++ph) {
-                        const StageMap m = smap[((size_t)kk * 8 + r) * 2 + (plus_first ? ph : 1 - ph)];
-                        t0 = stage_apply(m, t0);
-                        t1 = stage_apply(m, t1);
+                        for (int ph = 0; ph < 2; ++ph) {
+                            const StageMap m = smap[((size_t)kk * 8 + r) * 2 + (plus_first ? ph : 1 - ph)];
+                            t0 = stage_apply(m, t0);
+                            t1 = stage_apply(m, t1);
+                        }
                     }
                 }
                 int8_t *dst = tabs + ((size_t)p * 8 + r) * NT;
@@ -1271,7 +1325,22 @@ __global__ void __launch_bounds__(GB, 1) gdi_grid_sorted_kernel(GridArgs A)
                     const int32_t xr = gx - c0;
                     idx = (xr >= -NT && xr <= NT - 2) ? (xr + NT) >> 1 : -1;
                 };
-                for (int q = 0; q < run && ok; ++q) {
+                // on the lattice: one dependent read per table
+                int q = 0, kb = 0;
+                if (ok) {
+                    for (; q < run; ++q) {
+                        const int nx = ws_run[q * NT + idx];
+                        if (nx < 0) break;
+                        idx = nx;
+                    }
+                    if (q == run)
+                        for (; kb < nown; ++kb) {
+                            const int nx = ws_own[kb * NT + idx];
+                            if (nx < 0) break;
+                            idx = nx;
+                        }
+                }
+                for (; q < run && ok; ++q) {
                     const int nidx = idx >= 0 ? (int)ws_run[q * NT + idx] : -1;
                     if (nidx >= 0) { idx = nidx; continue; }
                     // the run table cannot map the running G: walk the run block by block
@@ -1280,34 +1349,35 @@ __global__ void __launch_bounds__(GB, 1) gdi_grid_sorted_kernel(GridArgs A)
                     for (int k = 0; k < RUN && ok; ++k) block_step(ws_dsc + k * NT, q * RUN + k);
                     __syncwarp();
                 }
-                for (int k = 0; k < nown && ok; ++k) block_step(ws_own + k * NT, run0 + k);
+                for (; kb < nown && ok; ++kb) block_step(ws_own + kb * NT, run0 + kb);
                 ok = __all_sync(0xFFFFFFFFu, ok);
+                // ---- my windows: looked up from the entering point on, replayed by all warps below; from the
+                // first that leaves the lattice on, replayed here in order from the exact G
+                for (int kk = lane; kk < nwin && A.tables; kk += 32) tin[kk * 8 + r] = -1;
+                __syncwarp();
                 if (ok) {
-                    const int32_t gin = idx >= 0 ? c0 - NT + 2 * idx : gx;
                     const int own = __shfl_sync(0xFFFFFFFFu, (idx >= 0 && idx < 32) ? t0 : t1, idx & 31);
                     const bool need_exact = idx < 0 || own < 0;
-                    uint32_t *fb = fbits + (size_t)r * L.fw;
-                    int32_t gout = gin;
-                    const int32_t *gr = gamc + (size_t)r * L.gs;
-                    for (int kk = 0; kk < nwin; ++kk) {
-                        const int ws = kk * W, we = min(ws + W, ns);
-                        const int32_t x = gout - c0;
-                        const int t = x >= -NT && x <= NT - 2 ? (x + NT) >> 1 : -1;
-                        const StageMap *maps = smap + ((size_t)kk * 8 + r) * 2;
-                        if constexpr (SL > 0) {
-                            gout = replay_mapped<SL>(gr, s0, r, ws, we, gout, plus_first, t, maps,
-                                                     [&](const uint32_t (&wb)[SL]) { flips_to_bitmap<SL>(wb, ws, we, fb, W); });
-                        } else {
-                            int K1, K2;
-                            mapped_flips(plus_first, t, maps, K1, K2);
-                            gout = replay_large(gr, s0, r, ws, we, gout, plus_first, K1, K2, [&](int i0, unsigned bits) {
-                                if (lane == 0) {
-                                    const int sh = i0 & 31;
-                                    fb[i0 >> 5] |= bits << sh;
-                                    if (sh && bits >> (32 - sh)) fb[(i0 >> 5) + 1] |= bits >> (32 - sh);
-                                }
-                            });
+                    int kk = 0;
+                    if (A.tables && idx >= 0)
+                        for (; kk < nwin; ++kk) {
+                            const int nx = wtab[(size_t)(kk * 8 + r) * NT + idx];
+                            if (nx < 0) break;
+                            if (lane == 0) tin[kk * 8 + r] = (int8_t)idx;
+                            idx = nx;
                         }
+                    int32_t gout = idx >= 0 ? c0 - NT + 2 * idx : gx;
+                    uint32_t *fb = fbits + (size_t)r * L.fw;
+                    const int32_t *gr = gamc + (size_t)r * L.gs;
+                    for (; kk < nwin; ++kk) {
+                        const int ws = kk * W, we = min(ws + W, ns);
+                        const uint32_t *bw = gbins + (size_t)(kk * 8 + r) * GBINS;
+                        const WindowCounts wc{A.binned && !bw[GB_WIDE] ? bw : nullptr, c0, GB_L, true};
+                        int K1 = -1, K2 = -1;
+                        const int32_t x = gout - c0;
+                        if (x >= -NT && x <= NT - 2)
+                            mapped_flips(plus_first, (x + NT) >> 1, smap + ((size_t)kk * 8 + r) * 2, K1, K2);
+                        gout = grid_replay<SL>(gr, s0, r, ws, we, gout, plus_first, K1, K2, wc, fb, W);
                     }
                     if (lane == 0) {
                         if (need_exact) {
@@ -1333,9 +1403,25 @@ __global__ void __launch_bounds__(GB, 1) gdi_grid_sorted_kernel(GridArgs A)
             }
             have_es = A.es_pre && (c + 1 < ncls || sw + 1 < R.s_end);
             __syncthreads();
+            // ---- the windows entered on the lattice, replayed at once
+            for (int task = warp; task < nwin * nrep && A.tables; task += NWARP) {
+                const int kk = task / nrep, r = task % nrep;
+                const int ti = tin[kk * 8 + r];
+                if (ti < 0) continue;
+                const int ws = kk * W, we = min(ws + W, ns);
+                const uint32_t *bw = gbins + (size_t)(kk * 8 + r) * GBINS;
+                const WindowCounts wc{A.binned && !bw[GB_WIDE] ? bw : nullptr, Gc[r], GB_L, true};
+                int K1, K2;
+                mapped_flips(plus_first, ti, smap + ((size_t)kk * 8 + r) * 2, K1, K2);
+                grid_replay<SL>(gamc + (size_t)r * L.gs, s0, r, ws, we, Gc[r] + 2 * ti - NT, plus_first, K1, K2, wc,
+                                fbits + (size_t)r * L.fw, W);
+            }
+            __syncthreads();
             // ---- write the flips; with maintained fields, push their field changes to the
             // neighbours: a warp takes 32 consecutive ranks and walks the concatenated rows of its
             // flipping ones lane by lane (rows longer than LONG_ROW go to a block queue instead)
+            if (A.binned)
+                for (int i = threadIdx.x; i < nwin * 8 * GBINS; i += GB) gbins[i] = 0;
             uint32_t *pq = reinterpret_cast<uint32_t *>(S.longq);
             // row bounds of the next chunk are loaded while the current one is pushed
             int64_t nrow0 = 0, nrow1 = 0;
@@ -1455,7 +1541,7 @@ __global__ void __launch_bounds__(GB, 1) gdi_grid_racy_kernel(GridArgs A)
     const GdiGridScratch &X = A.X;
     const int Pb = gridDim.x, p = blockIdx.x;
     const int spc = A.spc;
-    const SortedLayout L = sorted_layout(spc, A.wpc, R.max_row, Pb, A.es_pre);
+    const SortedLayout L = sorted_layout(spc, A.wpc, R.max_row, Pb, A.es_pre, A.tables, A.binned);
     int16_t *hb = reinterpret_cast<int16_t *>(smem_raw + L.off_h);
     int32_t *gam = reinterpret_cast<int32_t *>(smem_raw + L.off_gam);
     uint8_t *s0 = smem_raw + L.off_s0;
@@ -1544,37 +1630,60 @@ __global__ void unpack_kernel(int8_t *spins, int64_t N, int rep_base, int nrep, 
 // cut of every replica of a group from the packed spins, in one pass over the CSR: for an entry
 // (i, j > i), d = b_i ^ b_j has bit r set where replica r cuts the edge; SWAR byte lanes count the
 // cut weights (flushed before they can overflow)
+// A warp takes 32 consecutive rows and walks their concatenated entries lane by lane, four in flight: a
+// row of a power-law graph's hub (thousands of entries) costs its share of entries, where a thread per
+// row waited for it alone (0.8 ms of 10^6 vertices' cut).
 __global__ void packed_cut_kernel(GdiDevProblem P, const uint8_t *packed, int nrep, int64_t *cut)
 {
     const int64_t base = P.node_off[0];
     const int64_t n = P.node_off[1] - base;
+    const int lane = threadIdx.x & 31;
     int64_t acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const uint8_t b = packed[base + i];
-        uint64_t aP = 0, aN = 0;
-        int cnt = 0;
-        const int64_t e1 = P.row_ptr[base + i + 1];
-        for (int64_t e = P.row_ptr[base + i]; e < e1; ++e) {
-            const uint32_t c = __ldg(P.col + e);
-            const uint32_t j = c & 0x7FFFFFFFu;
-            if ((int64_t)j <= i) continue;
-            const uint64_t sv = spread8((uint32_t)(b ^ packed[base + j]));
-            if (c >> 31) aN += sv; else aP += sv;
-            if (++cnt == 255) {
-#pragma unroll
-                for (int k = 0; k < 8; ++k)
-                    acc[k] += (int64_t)((aP >> (8 * k)) & 0xFF) - (int64_t)((aN >> (8 * k)) & 0xFF);
-                aP = aN = 0;
-                cnt = 0;
-            }
-        }
+    uint64_t aP = 0, aN = 0;             // eight byte counts each, folded into acc before they overflow
+    int cnt = 0;
+    auto fold = [&]() {
 #pragma unroll
         for (int k = 0; k < 8; ++k) acc[k] += (int64_t)((aP >> (8 * k)) & 0xFF) - (int64_t)((aN >> (8 * k)) & 0xFF);
+        aP = aN = 0;
+        cnt = 0;
+    };
+    const int64_t warps = (int64_t)gridDim.x * blockDim.x / 32;
+    for (int64_t i0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32 * 32; i0 < n; i0 += 32 * warps) {
+        const int64_t i = i0 + lane;
+        const int64_t e0 = P.row_ptr[base + min(i, n)], e1 = P.row_ptr[base + min(i + 1, n)];
+        const uint32_t b = i < n ? packed[base + i] : 0u;
+        const int64_t f0 = __shfl_sync(0xFFFFFFFFu, e0, 0), f1 = __shfl_sync(0xFFFFFFFFu, e1, 31);
+        for (int64_t eb = f0; eb < f1; eb += 4 * 32) {
+            uint32_t cc[4], ow[4], nb[4];
+            int src[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                // owner of entry e: the last lane whose row starts at or before it
+                const int64_t e = eb + 32 * u + lane;
+                src[u] = 0;
+#pragma unroll
+                for (int st = 16; st > 0; st >>= 1)
+                    if (__shfl_sync(0xFFFFFFFFu, e0, src[u] + st) <= e) src[u] += st;
+                ow[u] = __shfl_sync(0xFFFFFFFFu, b, src[u]);
+                cc[u] = e < f1 ? __ldg(P.col + e) : 0u;
+                if (e >= f1) src[u] = 32;
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) nb[u] = packed[base + (cc[u] & 0x7FFFFFFFu)];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                if (src[u] == 32 || (int64_t)(cc[u] & 0x7FFFFFFFu) <= i0 + src[u]) continue;
+                const uint64_t sv = spread8(ow[u] ^ nb[u]);
+                if (cc[u] >> 31) aN += sv; else aP += sv;
+            }
+            if ((cnt += 4) > 251) fold();
+        }
     }
+    fold();
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
         const int64_t v = warp_sum(acc[k]);
-        if (k < nrep && (threadIdx.x & 31) == 0 && v) atomicAdd((unsigned long long *)(cut + k), (unsigned long long)v);
+        if (k < nrep && lane == 0 && v) atomicAdd((unsigned long long *)(cut + k), (unsigned long long)v);
     }
 }
 
@@ -1723,6 +1832,12 @@ __global__ void repair_apply_kernel(int8_t *spins, int64_t N, int nrep, const ui
 }  // namespace
 
 // ---------------------------------------------------------------------------------------------
+// what the counted kernel keeps beyond the necessary: 1 E* rows, 2 also tables, 3 also bins
+static SortedLayout planned_layout(int spc, int wpc, int max_row, int sms, int level)
+{
+    return sorted_layout(spc, wpc, max_row, sms, level >= 1, level >= 2, level >= 3);
+}
+
 int gdi_grid_plan(const GdiDevProblem &P, int max_row, int sms, size_t smem_limit, int *spc, int *wpc,
                   size_t *smem, bool *counted)
 {
@@ -1738,11 +1853,11 @@ int gdi_grid_plan(const GdiDevProblem &P, int max_row, int sms, size_t smem_limi
     if (P.W <= CMAXW) {
         // the cost-weighted split stays within the even share of windows per block: more shared
         // memory per block (less L1) costs more than the finer balance gains
-        // with rows for the E* drawn ahead when they fit, else without
-        *smem = sorted_layout(*spc, *wpc, max_row, sms, true).total;
-        if (*smem <= smem_limit) return 0;
-        *smem = sorted_layout(*spc, *wpc, max_row, sms, false).total;
-        if (*smem <= smem_limit) return 0;
+        // with rows for the E* drawn ahead, tables and bins for every window while they fit
+        for (int level = 3; level >= 0; --level) {
+            *smem = planned_layout(*spc, *wpc, max_row, sms, level).total;
+            if (*smem <= smem_limit) return 0;
+        }
         if (P.W <= SMAXW) return -1;
     }
     // larger windows whose buffers do not fit the counted path (its E* and push queue take about 10 bytes
@@ -1803,7 +1918,7 @@ int gdi_launch_grid_anneal(const GdiDevProblem &P, const GdiDevRun &R, const Gdi
     cudaStream_t st = (cudaStream_t)stream;
     const bool racy = (R.flags & GDI_DEV_RACY) != 0;
     const bool sorted = counted && !racy;
-    if (racy) smem = sorted_layout(spc, wpc, R.max_row, sms, false).total;
+    if (racy) smem = planned_layout(spc, wpc, R.max_row, sms, 0).total;
     const void *kern = racy ? (const void *)gdi_grid_racy_kernel
                      : !sorted ? (const void *)gdi_grid_anneal_kernel
                      : P.W <= 32 ? (const void *)gdi_grid_sorted_kernel<1>
@@ -1837,7 +1952,12 @@ int gdi_launch_grid_anneal(const GdiDevProblem &P, const GdiDevRun &R, const Gdi
         A.wpc = wpc;
         A.wbnd = (sorted || racy) ? wbnd : nullptr;
         A.hf = sorted ? X.hfield : nullptr;
-        A.es_pre = sorted && R.max_row < 32000 && smem >= sorted_layout(spc, wpc, R.max_row, sms, true).total;
+        // the level the plan's size stands for
+        int level = 3;
+        while (level > 0 && smem < planned_layout(spc, wpc, R.max_row, sms, level).total) --level;
+        A.es_pre = sorted && level >= 1 && R.max_row < 32000;
+        A.tables = sorted && level >= 2;
+        A.binned = sorted && level >= 3;
         void *args[] = {&A};
         const bool timed = timer && timer->ev && timer->n < timer->cap;
         if (timed) cudaEventRecord(timer->ev[2 * timer->n], st);

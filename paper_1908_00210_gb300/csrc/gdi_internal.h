@@ -28,6 +28,7 @@ struct GdiDevProblem {
     int32_t max_degree;
     int32_t max_class;               // largest colour class
     int32_t max_class_nnz;           // most row entries of one colour class (0: not known, or above 2^20)
+    int32_t max_item_nnz;            // of one instance (0: not known, or above 2^20)
 };
 
 // Global scratch of the grid-scale path (single large instance).
@@ -71,7 +72,7 @@ struct GdiDevRun {
     int32_t *err;                    // device error word (0 = ok)
     const int32_t *item_order;       // [Q*R] items, largest instance first (CTA path)
     int32_t *item_counter;           // [1] next item to take (zeroed before the launch)
-    int32_t cta_opts, cta_stage;     // CTA path's shared-memory options (gdi_kernels.cu), set by the launch
+    int32_t cta_opts, cta_stage, cta_rofs, cta_bins, cta_cluster;   // CTA path's shared-memory options (gdi_kernels.cu), set by the launch
 };
 
 // record a failure for gdi_last_error() (gdi_api.cpp); returns code
@@ -86,6 +87,10 @@ int gdi_launch_init(const GdiDevProblem &P, int8_t *spins, const int8_t *init_or
 int gdi_launch_cta_anneal(const GdiDevProblem &P, const GdiDevRun &R, int block, int grid_limit,
                           void *stream, int *grid_used, size_t *smem_used);
 int gdi_cta_smem_bytes(const GdiDevProblem &P, const GdiDevRun &R, int block, size_t *bytes);
+// threads per CTA-path block where the caller has set none
+int gdi_cta_default_block(const GdiDevProblem &P, const GdiDevRun &R);
+// blocks per item of a CTA-path launch (a cluster of 1, 2, 4 or 8)
+int gdi_cta_cluster_size(const GdiDevProblem &P, const GdiDevRun &R, int block);
 // resident CTA-path blocks per SM for this problem and block size (0 when the block does not fit)
 int gdi_cta_blocks_per_sm(const GdiDevProblem &P, const GdiDevRun &R, int block, int *per_sm);
 // Grid plan for `sms` blocks: spans of ranks (spc) and windows (wpc) per block and per class, and

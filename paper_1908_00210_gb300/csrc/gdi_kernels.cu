@@ -296,8 +296,9 @@ __host__ __device__ inline size_t align16c(size_t x) { return (x + 15) & ~(size_
 constexpr int CTA_OPT_ROWS2 = 1;    // the next sweep's table row beside the current one
 constexpr int CTA_OPT_ES = 2;       // whole-block windows: the next window's E* (else drawn in place)
 constexpr int CTA_OPT_BINS = 4;     // whole-block windows: 512 bins of margins (else 16)
-// GdiDevRun::cta_stage: columns the staging buffer of the next class (window) holds; a class with more
-// is read from global memory
+// GdiDevRun::cta_stage: columns the staging buffer holds (rows beyond are read from global memory);
+// cta_rofs: row offsets beside it.  Where a block's rows of all classes fit both, they are staged once per
+// item, else the next class's (window's) while the current one is decided.
 
 // lanes per rank of a field sum: the layout whose longest chain of dependent reads is shortest
 // (rounds x (row / T + about 4 reads' worth of reduction and threshold latency per round))
@@ -328,74 +329,118 @@ __device__ __forceinline__ void draw_estar(const GdiDevRun &R, int32_t r0, int32
 {
     if (r1 <= r0) return;
     for (int32_t qd = (r0 >> 2) + t; qd <= ((r1 - 1) >> 2); qd += nth) {
-        const uint4 u4 = philox4x32_10(make_uint4((uint32_t)qd, (uint32_t)sw, (uint32_t)q, (uint32_t)rep), R.key0, R.key1);
-#pragma unroll
+        uint4 u4 = philox4x32_10(make_uint4((uint32_t)qd, (uint32_t)sw, (uint32_t)q, (uint32_t)rep), R.key0, R.key1);
+        // (rolled: a class is short, so straight-line code is fetched more often than it is reused)
+#pragma unroll 1
         for (int j = 0; j < 4; ++j) {
             const int32_t r = 4 * qd + j;
-            if (r >= r0 && r < r1) es[r - org] = estar_of(row, rlen, R.mode, word_of(u4, j), Tsw);
+            if (r >= r0 && r < r1) es[r - org] = estar_of(row, rlen, R.mode, u4.x, Tsw);
+            u4.x = u4.y;
+            u4.y = u4.z;
+            u4.z = u4.w;
         }
     }
 }
 
-// whether columns [eb, ee), staged in whole 16-byte pieces, fit a buffer of cap columns
-__device__ __forceinline__ bool stage_fits(int64_t eb, int64_t ee, int32_t cap)
-{
-    return ((ee - (eb & ~(int64_t)7) + 7) & ~(int64_t)7) <= cap;
-}
-
-// Columns [eb, ee) and the offsets of nrows rows (bounds rp) into shared memory, by threads t of nth:
-// whole 16-byte pieces from the boundary at or before the first column (the column array is padded).
-// The caller waits (cp_async_wait_all) before its block barrier.
-__device__ __forceinline__ void stage_rows(const GdiDevProblem &P, const int64_t *rp, int32_t nrows, int64_t eb, int64_t ee,
+// Columns from entry al on (a 16-byte boundary; whole pieces, the column array is padded), `pieces` of
+// them, and the offsets from al of nrows rows (bounds rp) into shared memory, by threads t of nth.  The
+// caller waits (cp_async_wait_all) before its block barrier.
+__device__ __forceinline__ void stage_rows(const GdiDevProblem &P, const int64_t *rp, int32_t nrows, int64_t al, int32_t pieces,
                                            int32_t *rofs, uint16_t *cbuf, int t, int nth)
 {
-    const int64_t al = eb & ~(int64_t)7;
-    const int32_t pieces = (int32_t)((ee - al + 7) >> 3);
     for (int32_t k = t; k < pieces; k += nth) cp_async16(cbuf + 8 * k, P.col16 + al + 8 * (int64_t)k);
     for (int32_t i = t; i <= nrows; i += nth) rofs[i] = (int32_t)(rp[i] - al);
 }
 
-// Flip thresholds of ranks [lo + rb, lo + re) of an item from the shared spins and E* (es[i], i counted from
-// lo), a team of 2^tl lanes per rank; put(i, sign, threshold) by each team's first lane.  rofs != null:
-// rows staged in shared memory (row i at rofs[i - rb]).  Teams are aligned lane groups of one warp; every
-// lane takes part in every round's shuffles (the round count is the block's).
-template <int BS, class Put>
-__device__ __forceinline__ void team_thresholds(const GdiDevProblem &P, const int8_t *sig, int64_t base, int32_t lo, int32_t rb,
-                                                int32_t re, int tl, const int32_t *rofs, const uint16_t *cbuf,
-                                                const int32_t *es, int a_shift, const Put &put)
+// Both preparations of a class (window) by warps w of nw: the first few draw (about 250 instructions a
+// quad), the others stage, so that neither waits for the other's latency
+template <class Draw, class Stage>
+__device__ __forceinline__ void split_ahead(int32_t nranks, int w, int nw, const Draw &draw, const Stage &stage, bool both)
 {
-    const int T = 1 << tl, sub = threadIdx.x & (T - 1);
-    for (int32_t k0 = rb; k0 < re; k0 += BS >> tl) {
+    const int lane = threadIdx.x & 31;
+    if (!both) {
+        draw(w * 32 + lane, nw * 32);
+        return;
+    }
+    const int quads = (nranks + 3) / 4 + 1;
+    const int dw = min((quads + 31) / 32, max(1, 3 * nw / 4));
+    if (w < dw) draw(w * 32 + lane, dw * 32);
+    if (dw == nw) stage(w * 32 + lane, nw * 32);
+    else if (w >= dw) stage((w - dw) * 32 + lane, (nw - dw) * 32);
+}
+
+// Flip thresholds of ranks [lo, lo + nr) of an item from the shared spins and E* (es[i], i counted from lo),
+// a team of 2^tl lanes per rank; put(i, sign, threshold) by each team's first lane.  rofs != null: row i
+// is entries rofs[i] ... from gcol on, the first `lim` of them staged in shared memory.  Teams are
+// aligned lane groups of one warp; every lane takes part in every round's shuffles (the round count is the
+// block's).  A row of more than `longrow` entries per lane is summed by the whole warp: a power-law
+// graph's class holds hubs of hundreds of entries, which one team would keep the block waiting for.
+template <int BS, class Put>
+__device__ __forceinline__ void team_thresholds(const GdiDevProblem &P, const int8_t *sig, int64_t base, int32_t lo, int32_t nr,
+                                                int tl, int32_t longrow, const int32_t *rofs, const uint16_t *cbuf,
+                                                int32_t lim, const uint16_t *gcol, const int32_t *es, int a_shift,
+                                                const Put &put)
+{
+    const int T = 1 << tl, sub = threadIdx.x & (T - 1), lane = threadIdx.x & 31;
+    const int32_t limit = longrow << tl;
+    const bool has_long = P.max_degree > limit;
+    // spin of an entry, signed by its weight
+    auto spin16 = [&](uint32_t cc) {
+        const int32_t sv = sig[cc & 0x7FFFu];
+        return (cc >> 15) ? -sv : sv;
+    };
+    auto spin32 = [&](uint32_t cc) {
+        const int32_t sv = sig[cc & 0x7FFFFFFFu];
+        return (cc >> 31) ? -sv : sv;
+    };
+    for (int32_t k0 = 0; k0 < nr; k0 += BS >> tl) {
         const int32_t i = k0 + ((int32_t)threadIdx.x >> tl);
         int32_t h = 0;
-        if (i < re) {
+        int64_t g0 = 0;                 // rows read from the whole CSR: entries g0 + [e0, e1)
+        int32_t e0 = 0, e1 = 0;
+        if (i < nr) {
             if (rofs) {
-                const int32_t e1 = rofs[i - rb + 1];
-#pragma unroll 4
-                for (int32_t e = rofs[i - rb] + sub; e < e1; e += T) {
-                    const uint32_t cc = cbuf[e];
-                    const int32_t sv = sig[cc & 0x7FFFu];
-                    h += (cc >> 15) ? -sv : sv;
-                }
+                e0 = rofs[i];
+                e1 = rofs[i + 1];
             } else {
-                const int64_t e0 = P.row_ptr[base + lo + i], e1 = P.row_ptr[base + lo + i + 1];
-                if (P.col16) {
-                    for (int64_t e = e0 + sub; e < e1; e += T) {
-                        const uint32_t cc = __ldg(P.col16 + e);
-                        const int32_t sv = sig[cc & 0x7FFFu];
-                        h += (cc >> 15) ? -sv : sv;
-                    }
-                } else {
-                    for (int64_t e = e0 + sub; e < e1; e += T) {
-                        const uint32_t cc = __ldg(P.col + e);
-                        const int32_t sv = sig[cc & 0x7FFFFFFFu];
-                        h += (cc >> 31) ? -sv : sv;
-                    }
-                }
+                g0 = P.row_ptr[base + lo + i];
+                e1 = (int32_t)(P.row_ptr[base + lo + i + 1] - g0);
             }
         }
+        // entries first, first + step, ... of a row
+        auto sum = [&](int64_t g, int32_t first, int32_t end, int32_t step) {
+            int32_t x = 0;
+            if (rofs) {
+                if (end <= lim) {
+#pragma unroll 4
+                    for (int32_t e = first; e < end; e += step) x += spin16(cbuf[e]);
+                } else {
+#pragma unroll 4
+                    for (int32_t e = first; e < end; e += step) x += spin16(__ldg(gcol + e));
+                }
+            } else if (P.col16) {
+                for (int32_t e = first; e < end; e += step) x += spin16(__ldg(P.col16 + g + e));
+            } else {
+#pragma unroll 4
+                for (int32_t e = first; e < end; e += step) x += spin32(__ldg(P.col + g + e));
+            }
+            return x;
+        };
+        const bool lng = e1 - e0 > limit;
+        if (!lng) h = sum(g0, e0 + sub, e1, T);
         for (int o = T >> 1; o >= 1; o >>= 1) h += __shfl_xor_sync(0xFFFFFFFFu, h, o);
-        if (i < re && sub == 0) {
+        if (has_long) {
+            unsigned m = __ballot_sync(0xFFFFFFFFu, lng && sub == 0);
+            while (m) {
+                const int src = __ffs(m) - 1;
+                m &= m - 1;
+                const int64_t g = __shfl_sync(0xFFFFFFFFu, g0, src);
+                const int32_t b = __shfl_sync(0xFFFFFFFFu, e0, src), e = __shfl_sync(0xFFFFFFFFu, e1, src);
+                const int32_t x = __reduce_add_sync(0xFFFFFFFFu, sum(g, b + lane, e, 32));
+                if (lane == src) h = x;
+            }
+        }
+        if (i < nr && sub == 0) {
             const int sg = sig[lo + i];
             const int32_t e = es[i];
             put(i, sg, a_shift >= 0 ? gamma_of_shift(sg, h, e, P.A, P.B, a_shift) : gamma_of(sg, h, e, P.A, P.B));
@@ -562,12 +607,21 @@ __global__ void __launch_bounds__(BS, 1024 / BS) gdi_cta_block_kernel(GdiDevProb
         const int64_t nnz_item = P.row_ptr[base + n] - P.row_ptr[base];
         const int32_t mean_deg = n > 0 ? (int32_t)min((nnz_item + n - 1) / n, (int64_t)64) : 1;
 
-        // the window at ranks [wlo, whi): its E* and rows, by threads t of nth
-        auto prepare = [&](int32_t wlo, int32_t whi, int32_t sw, const uint32_t *row, int32_t rlen, float Tsw, int t, int nth) {
+        // the window at ranks [wlo, whi): its E* and rows, by warps w of nw
+        auto prepare = [&](int32_t wlo, int32_t whi, int32_t sw, const uint32_t *row, int32_t rlen, float Tsw, int w, int nw) {
             const int64_t *rp = P.row_ptr + base + wlo;
-            if (staged && stage_fits(rp[0], rp[whi - wlo], R.cta_stage))
-                stage_rows(P, rp, whi - wlo, rp[0], rp[whi - wlo], rofs, cbuf, t, nth);
-            if (pre) draw_estar(R, wlo, whi, wlo, q, rep, sw, row, rlen, Tsw, es, t, nth);
+            const int32_t ns = whi - wlo;
+            split_ahead(
+                ns, w, nw,
+                [&](int t, int nth) {
+                    if (pre) draw_estar(R, wlo, whi, wlo, q, rep, sw, row, rlen, Tsw, es, t, nth);
+                },
+                [&](int t, int nth) {
+                    const int64_t al = rp[0] & ~(int64_t)7;
+                    const int32_t pieces = (int32_t)((min(rp[ns] - al, (int64_t)R.cta_stage) + 7) >> 3);
+                    stage_rows(P, rp, ns, al, pieces, rofs, cbuf, t, nth);
+                },
+                staged);
         };
 
         int32_t g = 0;
@@ -589,7 +643,7 @@ __global__ void __launch_bounds__(BS, 1024 / BS) gdi_cta_block_kernel(GdiDevProb
         if (R.s_begin < R.s_end && ncls > 0) {
             prepare(cls[0], P.W > 0 ? min(cls[0] + P.W, cls[1]) : cls[1], R.s_begin,
                     S.row + (rows2 && (R.s_begin & 1) ? L.row_stride : 0),
-                    R.tab_off[R.s_begin + 1] - R.tab_off[R.s_begin], R.temp ? R.temp[R.s_begin] : 0.f, threadIdx.x, BS);
+                    R.tab_off[R.s_begin + 1] - R.tab_off[R.s_begin], R.temp ? R.temp[R.s_begin] : 0.f, warp, BS / 32);
             cp_async_wait_all();
         }
         __syncthreads();
@@ -621,10 +675,9 @@ __global__ void __launch_bounds__(BS, 1024 / BS) gdi_cta_block_kernel(GdiDevProb
                         __syncthreads();
                     }
                     // ---- thresholds, counted by margin
-                    const int64_t *wrp = P.row_ptr + base + wlo;
-                    const bool st = staged && stage_fits(wrp[0], wrp[Wn], R.cta_stage);
+                    const uint16_t *gcol = staged ? P.col16 + (P.row_ptr[base + wlo] & ~(int64_t)7) : nullptr;
                     int32_t ge1 = 0, ge2 = 0;
-                    team_thresholds<BS>(P, S.sig, base, wlo, 0, Wn, tl, st ? rofs : nullptr, cbuf, es, a_shift,
+                    team_thresholds<BS>(P, S.sig, base, wlo, Wn, tl, max(32, 2 * mean_deg), staged ? rofs : nullptr, cbuf, R.cta_stage, gcol, es, a_shift,
                                         [&](int32_t i, int sg, int32_t gm) {
                                             gam[i] = gm;
                                             s0[i] = (int8_t)sg;
@@ -646,7 +699,7 @@ __global__ void __launch_bounds__(BS, 1024 / BS) gdi_cta_block_kernel(GdiDevProb
                     }
                     __syncthreads();
                     // the next window: its E* and rows do not depend on the spins
-                    auto ahead = [&](int t, int nth) {
+                    auto ahead = [&](int w, int nw) {
                         int32_t nlo = whi, nhi, nsw = sw;
                         if (whi < chi) {
                             nhi = min(whi + Wn0, chi);
@@ -661,11 +714,11 @@ __global__ void __launch_bounds__(BS, 1024 / BS) gdi_cta_block_kernel(GdiDevProb
                         }
                         const bool same = nsw == sw;
                         prepare(nlo, nhi, nsw, same ? row : (rows2 ? row1 : R.tab + roff1), same ? rlen : rlen1,
-                                same ? Tsw : (R.temp ? R.temp[nsw] : 0.f), t, nth);
+                                same ? Tsw : (R.temp ? R.temp[nsw] : 0.f), w, nw);
                     };
                     if (standard) {
                         standard_window<BS>(S, gam, s0, wlo, Wn, n);
-                        ahead(threadIdx.x, BS);
+                        ahead(warp, BS / 32);
                         if (staged) cp_async_wait_all();
                         __syncthreads();
                         continue;
@@ -691,7 +744,7 @@ __global__ void __launch_bounds__(BS, 1024 / BS) gdi_cta_block_kernel(GdiDevProb
                             }
                         }
                     } else {
-                        ahead(threadIdx.x - 32, BS - 32);
+                        ahead(warp - 1, BS / 32 - 1);
                     }
                     __syncthreads();
                     if (dec.slow) {
@@ -804,11 +857,13 @@ __global__ void __launch_bounds__(BS, 1024 / BS) gdi_cta_block_kernel(GdiDevProb
 // CTA-resident counting kernel (1 <= W <= 256): the same results as gdi_cta_anneal_kernel with far
 // fewer block barriers per window.  Per colour class:
 //   1. thresholds of the class's ranks: a team of T lanes sums a rank's row over the shared spins;
-//   2. a class of three or more windows: every warp counts whole windows into their stage maps on the
-//      lattice (gdi_window.cuh), one thread walks the maps from the class-start G, and every window
-//      entered on the lattice is replayed at once by its own warp; the rest, and classes of one or two
-//      windows, are replayed in rank order from the exact G by one warp.  A replay writes its flips
-//      to the spins itself: nothing reads them again before the class ends.
+//   2. a class of three or more windows: the counts of each window's threshold distances give its stage
+//      maps on the lattice (gdi_window.cuh) and both composed as a byte table of 64 lattice points; each
+//      replaying warp looks its window's entering lattice point up from the class-start G (a read per
+//      window before it; following the maps themselves costs ten times that), and all windows are
+//      replayed at once.  A window whose map leaves the lattice, and all after it, are
+//      replayed in rank order from the exact G by one warp, as are classes of one or two windows.  A
+//      replay writes its flips to the spins itself: nothing reads them again before the class ends.
 // The windows of a class share no edge, so only the running G passes from one window to the next.
 // SL = members per lane of a window.
 //
@@ -818,50 +873,57 @@ __global__ void __launch_bounds__(BS, 1024 / BS) gdi_cta_block_kernel(GdiDevProb
 // next class's columns and row offsets there (cp.async: contiguous in rank order), so that a threshold
 // is a few shared loads.
 struct SortedCta {
-    int32_t *gam;       // [max_class] flip thresholds of the class
-    int32_t *es;        // [max_class] E* of the next class's ranks, drawn ahead
-    uint8_t *s0;        // [max_class] 1 = the member was -1 at window start
-    uint32_t *bins;     // [warps that count][WBINS]
-    StageMap *wmaps;    // [nwm][2] stage maps of every window (classes of 3 to nwm windows)
-    int32_t *tin;       // [nwm + 2] entering lattice index of every window; then the walk's
-                        // first failing window and its last lattice index
-    int32_t *rofs;      // [max_class + 1] row offsets of the next class's ranks in cbuf
-    uint16_t *cbuf;     // [cta_stage] its columns
+    int32_t *gam;       // [own ranks] flip thresholds of my share of the class
+    int32_t *es;        // [own ranks] E* of the next class's, drawn ahead
+    uint8_t *s0;        // [own ranks] 1 = the member was -1 at window start
+    uint32_t *bins;     // [cta_bins windows, or warps that count][WBINS]
+    StageMap *wmaps;    // [nwm][2] stage maps of my windows (classes of 3 windows and more)
+    int8_t *wtab;       // [nwm][NT] both maps composed (-1: leaves the lattice)
+    int32_t *rofs;      // row offsets of the staged rows
+    uint16_t *cbuf;     // [cta_stage] their columns
 };
 
-// windows per class whose stage maps are kept for the walk (more: one warp replays them in order)
+// windows of one block whose stage maps are kept (a class with more is replayed in order)
 constexpr int CTA_WALK_MAX = 128;
-static_assert(sizeof(StageMap) == 16, "a pair copies stage maps as 16-byte words");
 
-__host__ __device__ inline int cta_walk_windows(int32_t max_class, int W)
+// windows a block of a cluster of cl (1: alone) has of the largest class: a class of one or two windows
+// is the first block's
+__host__ __device__ inline int cta_own_windows(int32_t max_class, int W, int cl)
 {
-    const int32_t nw = (max_class + W - 1) / W;
-    return nw < CTA_WALK_MAX ? (int)nw : CTA_WALK_MAX;
+    const int nw = (max_class + W - 1) / W;
+    return cl > 1 ? ((nw + cl - 1) / cl > 2 ? (nw + cl - 1) / cl : 2) : nw;
 }
 
-// warps that count windows at once: none where no class has the three windows of a walk; their bins
-// share the repair flags' bytes, and a small instance has room for 16
-__host__ __device__ inline int cta_count_warps(int32_t max_n, int32_t max_class, int W, int BS)
+__host__ __device__ inline int cta_walk_windows(int32_t max_class, int W, int cl)
 {
-    const int nwm = cta_walk_windows(max_class, W);
+    const int nw = cta_own_windows(max_class, W, cl);
+    return nw < CTA_WALK_MAX ? nw : CTA_WALK_MAX;
+}
+
+// warps that count windows at once where the windows have no bins of their own: none where no class has
+// three windows; their bins share the repair flags' bytes, and a small instance has room for 16
+__host__ __device__ inline int cta_count_warps(int32_t max_n, int32_t max_class, int W, int BS, int cl)
+{
+    const int nwm = cta_walk_windows(max_class, W, cl);
     const int fit = max_n / 1024 > 16 ? max_n / 1024 : 16;
     const int nw = nwm < BS / 32 ? nwm : BS / 32;
-    return nwm < 3 ? 0 : (nw < fit ? nw : fit);
+    return (max_class + W - 1) / W < 3 ? 0 : (nw < fit ? nw : fit);
 }
 
 // Shared-memory layout of the counting CTA kernel, one function for the kernel's carving and the
 // host's size: the common part (reductions, G, table rows, spins, repair flags), then the class
 // buffers.  Every array starts on a 16-byte boundary.
 struct CtaSortedLayout {
-    size_t red64, red32, G, row, sig, flag, gam, es, s0, wmaps, tin, rofs, cbuf, total;
+    size_t red64, red32, G, row, sig, flag, gam, es, s0, wmaps, wtab, rofs, cbuf, total;
     int row_stride;
 };
 
 __host__ __device__ inline CtaSortedLayout cta_sorted_layout(const GdiDevProblem &P, int32_t max_row, int BS, int opts,
-                                                             int32_t stage)
+                                                             int32_t stage, int32_t rofs, int nbw, int cl)
 {
     CtaSortedLayout L;
-    const size_t mc = (size_t)P.max_class + 8;
+    const size_t own = cl > 1 ? (size_t)cta_own_windows(P.max_class, P.W, cl) * P.W : (size_t)P.max_class;
+    const size_t mc = own + 8;
     size_t o = 0;
     L.red64 = o; o = align16c(o + sizeof(int64_t) * (BS / 32 + 2));
     L.red32 = o; o = align16c(o + sizeof(int32_t) * (BS / 32 + 2));
@@ -869,38 +931,45 @@ __host__ __device__ inline CtaSortedLayout cta_sorted_layout(const GdiDevProblem
     L.row_stride = (max_row + 4 + 3) & ~3;
     L.row = o; o = align16c(o + sizeof(uint32_t) * (size_t)L.row_stride * ((opts & CTA_OPT_ROWS2) ? 2 : 1));
     L.sig = o; o = align16c(o + (size_t)P.max_n + 16);
-    // the repair flags and, during the sweeps, the counting warps' bins share their bytes
-    const size_t bins = 4 * (size_t)win::WBINS * cta_count_warps(P.max_n, P.max_class, P.W, BS);
+    // the repair flags and, during the sweeps, the windows' or counting warps' bins share their bytes
+    const int cw = cta_count_warps(P.max_n, P.max_class, P.W, BS, cl);
+    const size_t bins = 4 * (size_t)win::WBINS * (cw > nbw ? cw : nbw);
     const size_t fl = (size_t)P.max_n + 16;
     L.flag = o; o = align16c(o + (fl > bins ? fl : bins));
     L.gam = o; o = align16c(o + 4 * mc);
     L.es = o; o = align16c(o + 4 * mc);
     L.s0 = o; o = align16c(o + mc);
-    const int nwm = cta_walk_windows(P.max_class, P.W);
+    const int nwm = cta_walk_windows(P.max_class, P.W, cl);
     L.wmaps = o; o = align16c(o + sizeof(StageMap) * 2 * (size_t)nwm);
-    L.tin = o; o = align16c(o + sizeof(int32_t) * (size_t)(nwm + 2));
-    L.rofs = o; o = align16c(o + (stage ? 4 * mc : 0));
+    L.wtab = o; o = align16c(o + (size_t)NT * nwm);
+    L.rofs = o; o = align16c(o + (stage ? 4 * (mc > (size_t)rofs ? mc : (size_t)rofs) : 0));
     L.cbuf = o; o = align16c(o + 2 * (size_t)stage);
     L.total = o;
     return L;
 }
 
-// PAIR: a cluster of two blocks anneals each item.  Both keep all spins and G; a class of 3 to
-// nwm windows is split in two halves of windows (thresholds, counts and replays each block's own),
-// each block copies the other's stage maps in through distributed shared memory and walks all of
-// them, and each replay writes its flips to both blocks' spins.  Other classes are done by block 0
-// alone.
-template <int BS, int SL, bool PAIR>
+// CLUS: a cluster of 2, 4 or 8 blocks anneals each item (few items, many windows).  Every block keeps all
+// spins and G; a class of three windows and more is split into contiguous runs of windows, each block's
+// thresholds, counts and replays its own.  The blocks exchange one composed 64-entry table each through
+// distributed shared memory, every replay writes its flips to every block's spins, and two cluster
+// barriers a class remain (after the tables, after the flips).  Classes of one or two windows are the
+// first block's alone.
+template <int BS, int SL, bool CLUS>
 __global__ void __launch_bounds__(BS, 1024 / BS) gdi_cta_sorted_kernel(GdiDevProblem P, GdiDevRun R)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Smem S = {};
     SortedCta C;
     const bool rows2 = (R.cta_opts & CTA_OPT_ROWS2) != 0, staged = R.cta_stage > 0;
+    unsigned crank = 0, CL = 1;                          // block rank in the cluster, cluster size
+    if constexpr (CLUS) {
+        crank = cooperative_groups::this_cluster().block_rank();
+        CL = cooperative_groups::this_cluster().num_blocks();
+    }
     int row_stride;
     int scratch_words;
     {
-        const CtaSortedLayout L = cta_sorted_layout(P, R.max_row, BS, R.cta_opts, R.cta_stage);
+        const CtaSortedLayout L = cta_sorted_layout(P, R.max_row, BS, R.cta_opts, R.cta_stage, R.cta_rofs, R.cta_bins, (int)CL);
         S.red64 = reinterpret_cast<int64_t *>(smem_raw + L.red64);
         S.red32 = reinterpret_cast<int32_t *>(smem_raw + L.red32);
         S.G = reinterpret_cast<int32_t *>(smem_raw + L.G);
@@ -912,7 +981,7 @@ __global__ void __launch_bounds__(BS, 1024 / BS) gdi_cta_sorted_kernel(GdiDevPro
         C.s0 = smem_raw + L.s0;
         C.bins = reinterpret_cast<uint32_t *>(smem_raw + L.flag);
         C.wmaps = reinterpret_cast<StageMap *>(smem_raw + L.wmaps);
-        C.tin = reinterpret_cast<int32_t *>(smem_raw + L.tin);
+        C.wtab = reinterpret_cast<int8_t *>(smem_raw + L.wtab);
         C.rofs = reinterpret_cast<int32_t *>(smem_raw + L.rofs);
         C.cbuf = reinterpret_cast<uint16_t *>(smem_raw + L.cbuf);
         row_stride = L.row_stride;
@@ -926,32 +995,43 @@ __global__ void __launch_bounds__(BS, 1024 / BS) gdi_cta_sorted_kernel(GdiDevPro
         }
     }
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    constexpr int NW = BS / 32;
     const int W = P.W;
-    const int nwm = cta_walk_windows(P.max_class, W);
-    const int cwarps = cta_count_warps(P.max_n, P.max_class, W, BS);
+    const int cwarps = cta_count_warps(P.max_n, P.max_class, W, BS, (int)CL);
+    const int w_shift = (W & (W - 1)) == 0 ? __ffs(W) - 1 : -1;
     const int a_shift = (P.A > 0 && (P.A & (P.A - 1)) == 0) ? 2 + __ffs(P.A) - 1 : -1;   // log2(4A)
     const int32_t items = P.num_instances * P.replicas;
     __shared__ int32_t next_item;
-    // class bounds, windows, team sizes and (staged) my own row range's entries, for the first CB classes
-    constexpr int CB = 64;
-    __shared__ int32_t c_lo[CB + 1], c_nw[CB], c_eb[CB], c_ee[CB];
-    __shared__ uint8_t c_tl[CB];
-    unsigned crank = 0;                                  // block rank in the cluster
-    if constexpr (PAIR) crank = cooperative_groups::this_cluster().block_rank();
-    // the partner block's copy of a shared-memory object (same layout in both blocks)
-    auto peer = [&](auto *ptr) { return cooperative_groups::this_cluster().map_shared_rank(ptr, crank ^ 1u); };
-    auto pair_sync = [&]() {
-        if constexpr (PAIR) cooperative_groups::this_cluster().sync();
+    // the first CB classes as this block sees them (a class starts without deriving them anew)
+    constexpr int CB = 48;
+    struct Span {
+        int32_t lo, ns;                 // my ranks [lo, lo + ns)
+        int32_t nwin, kq, kb, nk;       // windows [kb, kb + nk) of nwin are mine, kq to a block
+        int32_t clo, chi;               // the class's ranks
+        int32_t al, pieces;             // staging: first entry (from the item's, a 16-byte boundary), pieces,
+        int32_t cb, ro;                 // where its columns and row offsets start
+        int16_t tl, walk;               // log2 of the team size; three windows or more
+    };
+    __shared__ Span c_span[CB];
+    __shared__ bool all_staged;
+    __shared__ int8_t btab[8][NT];                       // composed tables of the cluster's blocks
+    __shared__ int32_t w_fail[2];                        // the class's first window off the lattice (or -1), its index
+    // another block's copy of a shared-memory object (same layout in all blocks)
+    auto remote = [&](auto *ptr, unsigned r) { return cooperative_groups::this_cluster().map_shared_rank(ptr, r); };
+    auto item_sync = [&]() {
+        if constexpr (CLUS) cooperative_groups::this_cluster().sync();
         else __syncthreads();
     };
+    if (threadIdx.x == 0) w_fail[0] = -1;
     while (true) {
-        pair_sync();
+        item_sync();
         if (crank == 0 && threadIdx.x == 0) {
             const int32_t t = atomicAdd(R.item_counter, 1);
             next_item = t;
-            if constexpr (PAIR) *peer(&next_item) = t;
+            if constexpr (CLUS)
+                for (unsigned r = 1; r < CL; ++r) *remote(&next_item, r) = t;
         }
-        pair_sync();
+        item_sync();
         const int32_t slot = next_item;
         if (slot >= items) break;
         const int32_t item = R.item_order[slot];
@@ -966,56 +1046,73 @@ __global__ void __launch_bounds__(BS, 1024 / BS) gdi_cta_sorted_kernel(GdiDevPro
         const int64_t nnz_item = P.row_ptr[base + n] - row0;
         const int32_t mean_deg = n > 0 ? (int32_t)min((nnz_item + n - 1) / n, (int64_t)64) : 1;
 
-        // one class as this block sees it: a class of 3 to nwm windows keeps every window's stage
-        // maps for the walk; a pair splits such a class: windows [0, kmid) are block 0's, the rest
-        // block 1's; other classes are block 0's
-        struct Span {
-            int32_t lo, ns, nwin, kmid, kb, ke, rb, re;
-            bool walk;
-        };
-        auto span_of = [&](int32_t lo, int32_t hi, int32_t nwin) {
+        auto make_span = [&](int c) {
             Span s;
-            s.lo = lo;
-            s.ns = hi - lo;
-            s.nwin = nwin;
-            s.walk = nwin >= 3 && nwin <= nwm;
-            s.kmid = PAIR && s.walk ? (nwin + 1) / 2 : nwin;
-            s.kb = crank ? s.kmid : 0;
-            s.ke = crank ? nwin : s.kmid;
-            s.rb = min(s.kb * W, s.ns);
-            s.re = min(s.ke * W, s.ns);
+            s.clo = cls[c];
+            s.chi = cls[c + 1];
+            const int32_t size = s.chi - s.clo;
+            s.nwin = (size + W - 1) / W;
+            s.kq = CLUS ? (s.nwin + (int)CL - 1) / (int)CL : s.nwin;
+            s.walk = s.nwin >= 3 && s.kq <= CTA_WALK_MAX;
+            if (!s.walk) s.kq = s.nwin;
+            s.kb = min((int)crank * s.kq, s.nwin);
+            s.nk = min(s.kq, s.nwin - s.kb);
+            const int32_t rb = min(s.kb * W, size), re = min((s.kb + s.nk) * W, size);
+            s.lo = s.clo + rb;
+            s.ns = re - rb;
+            s.tl = (int16_t)team_log2<BS>(s.ns, mean_deg);
+            const int64_t eb = P.row_ptr[base + s.lo], ee = P.row_ptr[base + s.lo + s.ns], al = eb & ~(int64_t)7;
+            s.al = (int32_t)(al - row0);
+            s.pieces = (int32_t)((min(ee - al, (int64_t)R.cta_stage) + 7) >> 3);
+            s.cb = s.ro = 0;
             return s;
         };
-        auto span = [&](int c) {
-            if (c < CB) return span_of(c_lo[c], c_lo[c + 1], c_nw[c]);
-            return span_of(cls[c], cls[c + 1], (cls[c + 1] - cls[c] + W - 1) / W);
-        };
-        for (int c = threadIdx.x; c < ncls && c < CB; c += BS) {
-            const int32_t lo = cls[c], hi = cls[c + 1], nw = (hi - lo + W - 1) / W;
-            c_lo[c] = lo;
-            if (c + 1 == ncls || c + 1 == CB) c_lo[c + 1] = hi;
-            c_nw[c] = nw;
-            const Span s = span_of(lo, hi, nw);
-            c_tl[c] = (uint8_t)team_log2<BS>(s.re - s.rb, mean_deg);
-            c_eb[c] = (int32_t)(P.row_ptr[base + lo + s.rb] - row0);
-            c_ee[c] = (int32_t)(P.row_ptr[base + lo + s.re] - row0);
+        auto span = [&](int c) { return c < CB ? c_span[c] : make_span(c); };
+        for (int c = threadIdx.x; c < ncls && c < CB; c += BS) c_span[c] = make_span(c);
+        __syncthreads();
+        if (staged && warp == 0) {
+            // places of all classes side by side, if they fit
+            int32_t cb = 0, ro = 0;
+            for (int c0 = 0; c0 < CB && ncls <= CB; c0 += 32) {
+                const int c = c0 + lane;
+                const int32_t a = c < ncls ? 8 * c_span[c].pieces : 0, b = c < ncls ? c_span[c].ns + 1 : 0;
+                int32_t xa = a, xb = b;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int32_t ya = __shfl_up_sync(0xFFFFFFFFu, xa, o), yb = __shfl_up_sync(0xFFFFFFFFu, xb, o);
+                    if (lane >= o) { xa += ya; xb += yb; }
+                }
+                if (c < ncls) {
+                    c_span[c].cb = cb + xa - a;
+                    c_span[c].ro = ro + xb - b;
+                }
+                cb += __shfl_sync(0xFFFFFFFFu, xa, 31);
+                ro += __shfl_sync(0xFFFFFFFFu, xb, 31);
+            }
+            const bool all = ncls <= CB && cb < R.cta_stage && ro <= R.cta_rofs;
+            __syncwarp();
+            for (int c = lane; c < ncls && c < CB && !all; c += 32) c_span[c].cb = c_span[c].ro = 0;
+            if (lane == 0) all_staged = all;
         }
-        auto draw = [&](const Span &s, int32_t sw, const uint32_t *row, int32_t rlen, float Tsw, int t, int nth) {
-            draw_estar(R, s.lo + s.rb, s.lo + s.re, s.lo, q, rep, sw, row, rlen, Tsw, C.es, t, nth);
+        __syncthreads();
+        const bool whole = staged && all_staged;
+        // E* and rows of a class (span s) at sweep sw, by warps w of nw
+        auto prepare = [&](const Span &s, int32_t sw, const uint32_t *row, int32_t rlen, float Tsw, int w, int nw) {
+            if (s.ns == 0) return;
+            split_ahead(
+                s.ns, w, nw,
+                [&](int t, int nth) { draw_estar(R, s.lo, s.lo + s.ns, s.lo, q, rep, sw, row, rlen, Tsw, C.es, t, nth); },
+                [&](int t, int nth) {
+                    stage_rows(P, P.row_ptr + base + s.lo, s.ns, row0 + s.al, s.pieces, C.rofs, C.cbuf, t, nth);
+                },
+                staged && !whole);
         };
-        auto stage = [&](const Span &s, int c, int t, int nth) {
-            if (s.re <= s.rb) return;
-            const int64_t *rp = P.row_ptr + base + s.lo + s.rb;
-            const int32_t nown = s.re - s.rb;
-            const int64_t eb = c < CB ? row0 + c_eb[c] : rp[0], ee = c < CB ? row0 + c_ee[c] : rp[nown];
-            if (stage_fits(eb, ee, R.cta_stage)) stage_rows(P, rp, nown, eb, ee, C.rofs, C.cbuf, t, nth);
-        };
-        auto is_staged = [&](const Span &s, int c) {
-            if (!staged || s.re <= s.rb) return false;
-            const int64_t *rp = P.row_ptr + base + s.lo;
-            return stage_fits(c < CB ? row0 + c_eb[c] : rp[s.rb], c < CB ? row0 + c_ee[c] : rp[s.re], R.cta_stage);
-        };
+        if (whole)
+            for (int c = warp; c < ncls; c += NW)
+                stage_rows(P, P.row_ptr + base + c_span[c].lo, c_span[c].ns, row0 + c_span[c].al, c_span[c].pieces,
+                           C.rofs + c_span[c].ro, C.cbuf + c_span[c].cb, lane, 32);
 
+        for (int b = threadIdx.x; b < R.cta_bins * WBINS; b += BS) C.bins[b] = 0;
         int32_t g = 0;
         for (int32_t r = threadIdx.x; r < n; r += BS) {
             const int8_t sv = gsig[r];
@@ -1030,15 +1127,12 @@ __global__ void __launch_bounds__(BS, 1024 / BS) gdi_cta_sorted_kernel(GdiDevPro
         g = block_sum<BS, int32_t>(g, S.red32);
         if (threadIdx.x == 0) *S.G = g;
         __syncthreads();
-        if (R.s_begin < R.s_end) {
-            const Span s = span(0);
-            const int32_t rlen = R.tab_off[R.s_begin + 1] - R.tab_off[R.s_begin];
-            if (staged) stage(s, 0, threadIdx.x, BS);
-            draw(s, R.s_begin, S.row + (rows2 && (R.s_begin & 1) ? row_stride : 0), rlen,
-                 R.temp ? R.temp[R.s_begin] : 0.f, threadIdx.x, BS);
-            cp_async_wait_all();
+        if (R.s_begin < R.s_end && ncls > 0) {
+            prepare(span(0), R.s_begin, S.row + (rows2 && (R.s_begin & 1) ? row_stride : 0),
+                    R.tab_off[R.s_begin + 1] - R.tab_off[R.s_begin], R.temp ? R.temp[R.s_begin] : 0.f, warp, NW);
         }
-        __syncthreads();
+        cp_async_wait_all();
+        item_sync();
 
         for (int32_t sw = R.s_begin; sw < R.s_end; ++sw) {
             const int32_t roff = R.tab_off[sw];
@@ -1055,111 +1149,163 @@ __global__ void __launch_bounds__(BS, 1024 / BS) gdi_cta_sorted_kernel(GdiDevPro
                 for (int32_t k = threadIdx.x; k < rlen1; k += BS) row1[k] = R.tab[roff1 + k];
             const float Tsw = R.temp ? R.temp[sw] : 0.f;
             const bool plus_first = (sw & 1) == 0;
+            const int st0 = plus_first ? 0 : 1;          // the stage that goes first
             for (int32_t c = 0; c < ncls; ++c) {
                 const Span s = span(c);
                 const int32_t lo = s.lo, ns = s.ns;
                 const int32_t c0 = *S.G;                 // G at class start (the reference c)
+                // a class whose windows here all have bins counts its thresholds as they are made
+                const bool binned = s.nk <= R.cta_bins;
                 // ---- thresholds of my ranks
-                team_thresholds<BS>(P, S.sig, base, lo, s.rb, s.re, c < CB ? c_tl[c] : team_log2<BS>(s.re - s.rb, mean_deg),
-                                    is_staged(s, c) ? C.rofs : nullptr, C.cbuf, C.es, a_shift,
-                                    [&](int32_t i, int sg, int32_t gm) {
+                team_thresholds<BS>(P, S.sig, base, lo, ns, s.tl, max(32, 2 * mean_deg), staged ? C.rofs + s.ro : nullptr, C.cbuf + s.cb, 8 * s.pieces,
+                                    P.col16 + row0 + s.al, C.es, a_shift, [&](int32_t i, int sg, int32_t gm) {
                                         C.gam[i] = gm;
                                         C.s0[i] = sg < 0 ? 1 : 0;
+                                        if (binned) {
+                                            const int32_t d = sg < 0 ? c0 - gm : gm - c0;
+                                            const int k = w_shift >= 0 ? i >> w_shift : i / W;
+                                            if (d <= NT)
+                                                atomicAdd(&C.bins[k * WBINS + max(d + BIN_L, 0)], sg < 0 ? 0x10000u : 1u);
+                                        }
                                     });
-                if (PAIR && !s.walk) pair_sync(); else __syncthreads();
+                // (the first block's replay of a small class writes the others' G and spins: they must
+                // have read this class's c0 first)
+                if (CLUS && !s.walk) item_sync(); else __syncthreads();
                 // the next class: its E* and columns do not depend on the spins
-                const bool same = c + 1 < ncls;
-                const bool more = same || sw + 1 < R.s_end;
-                auto ahead = [&](int t, int nth) {
-                    if (!more) return;
-                    const Span nx = span(same ? c + 1 : 0);
-                    if (staged) stage(nx, same ? c + 1 : 0, t, nth);
-                    draw(nx, same ? sw : sw + 1, same ? row : (rows2 ? row1 : R.tab + roff1), same ? rlen : rlen1,
-                         same ? Tsw : (R.temp ? R.temp[sw + 1] : 0.f), t, nth);
+                auto ahead = [&](int w, int nw) {
+                    const bool same = c + 1 < ncls;
+                    if (!same && sw + 1 >= R.s_end) return;
+                    prepare(span(same ? c + 1 : 0), same ? sw : sw + 1, same ? row : (rows2 ? row1 : R.tab + roff1),
+                            same ? rlen : rlen1, same ? Tsw : (R.temp ? R.temp[sw + 1] : 0.f), w, nw);
                 };
-                // the flips of a window straight into the spins (of both blocks of a pair)
-                auto flip = [&](int32_t ws, int32_t we, const uint8_t *s0, const uint32_t (&wb)[SL]) {
+                // the flips of a window (ranks from r0 on) straight into the spins of every block
+                auto flip = [&](int32_t r0, int32_t ws, int32_t we, const uint8_t *s0, const uint32_t (&wb)[SL]) {
 #pragma unroll
                     for (int k = 0; k < SL; ++k) {
                         const int32_t i = ws + 32 * k + lane;
                         if (i < we && ((wb[k] >> lane) & 1u)) {
                             const int8_t v = s0[i] ? 1 : -1;
-                            S.sig[lo + i] = v;
-                            if constexpr (PAIR) peer(S.sig)[lo + i] = v;
+                            S.sig[r0 + i] = v;
+                            if constexpr (CLUS)
+                                for (unsigned r = 0; r < CL; ++r)
+                                    if (r != crank) remote(S.sig, r)[r0 + i] = v;
                         }
                     }
                 };
-                int32_t k_seq = 0;                       // first window replayed in order
+                auto zero_bins = [&](uint32_t *bins) {
+                    __syncwarp();
+                    reinterpret_cast<uint4 *>(bins)[lane] = make_uint4(0u, 0u, 0u, 0u);
+                    reinterpret_cast<uint4 *>(bins)[lane + 32] = make_uint4(0u, 0u, 0u, 0u);
+                };
+                // *p of every block, by lane 0 of a warp
+                auto set_all = [&](int32_t *p, int32_t v) {
+                    if (lane == 0) {
+                        *p = v;
+                        if constexpr (CLUS)
+                            for (unsigned r = 0; r < CL; ++r)
+                                if (r != crank) *remote(p, r) = v;
+                    }
+                };
                 if (s.walk) {
-                    // ---- every window of mine counted by one warp
-                    if (warp < cwarps)
-                        for (int32_t kk = s.kb + warp; kk < s.ke; kk += cwarps) {
-                            const int32_t ws = kk * W, wlen = min(W, ns - ws);
-                            window_maps<SL>(C.gam, C.s0, ws, wlen, 0, c0, C.bins + (size_t)warp * WBINS,
-                                            C.wmaps + 2 * kk);
-                        }
-                    pair_sync();
-                    if constexpr (PAIR) {
-                        // the partner's stage maps copied in at once (one remote round trip), into the
-                        // slots of its windows, which this block does not use itself
-                        const int32_t pkb = crank ? 0 : s.kmid, pke = crank ? s.kmid : s.nwin;
-                        const uint4 *src = reinterpret_cast<const uint4 *>(peer(C.wmaps) + 2 * pkb);
-                        uint4 *dst = reinterpret_cast<uint4 *>(C.wmaps + 2 * pkb);
-                        for (int32_t i = threadIdx.x; i < 2 * (pke - pkb); i += BS) dst[i] = src[i];
-                        __syncthreads();
+                    // ---- the maps and the table of every window of mine, by one warp
+                    const int cw = binned ? NW : cwarps;
+                    for (int k = warp; k < s.nk && warp < cw; k += cw) {
+                        if (binned)
+                            bins_to_prefix<8>(C.bins + (size_t)k * WBINS, BIN_L, C.wmaps + 2 * k);
+                        else
+                            window_maps<SL>(C.gam, C.s0, k * W, min(W, ns - k * W), 0, c0, C.bins + (size_t)warp * WBINS,
+                                            C.wmaps + 2 * k);
+                        __syncwarp();
+                        const StageMap m0 = C.wmaps[2 * k + st0], m1 = C.wmaps[2 * k + (1 ^ st0)];
+                        C.wtab[k * NT + lane] = (int8_t)stage_apply(m1, stage_apply(m0, lane));
+                        C.wtab[k * NT + lane + 32] = (int8_t)stage_apply(m1, stage_apply(m0, lane + 32));
                     }
-                    // ---- one thread follows x = G - c0 from 0 through the windows' stage maps (lattice
-                    // index t: x = 2 t - NT) up to the first window that leaves the lattice (in a
-                    // pair both blocks walk, to the same result); the other warps work ahead
-                    if (warp > 0) {
-                        ahead(threadIdx.x - 32, BS - 32);
-                    } else if (lane == 0) {
-                        int t = NT / 2;
-                        int32_t kf = s.nwin;
-                        for (int32_t kk = 0; kk < s.nwin; ++kk) {
-                            C.tin[kk] = t;
-                            const StageMap *wm = C.wmaps;
-                            const int u = stage_apply(wm[2 * kk + (plus_first ? 1 : 0)],
-                                                      stage_apply(wm[2 * kk + (plus_first ? 0 : 1)], t));
-                            if (u < 0) { kf = kk; break; }
-                            t = u;
-                        }
-                        C.tin[nwm] = kf;
-                        C.tin[nwm + 1] = t;
-                        if (kf == s.nwin) *S.G = c0 + 2 * t - NT;
-                    }
+                    if (!binned && R.cta_bins && warp < cwarps) zero_bins(C.bins + (size_t)warp * WBINS);
                     __syncthreads();
-                    k_seq = C.tin[nwm];
-                    // ---- my windows before it were entered on the lattice: all replayed at once
-                    for (int32_t kk = s.kb + warp; kk < min(s.ke, k_seq); kk += BS / 32) {
-                        const int32_t ws = kk * W, we = min(ws + W, ns), t = C.tin[kk];
-                        replay_mapped<SL>(C.gam, C.s0, 0, ws, we, c0 + 2 * t - NT, plus_first, t, C.wmaps + 2 * kk,
-                                          [&](const uint32_t (&wb)[SL]) { flip(ws, we, C.s0, wb); });
+                    // the first warps replay, the others work ahead
+                    const int busy = min(s.nk, NW / 2);
+                    if constexpr (CLUS) {
+                        // my windows' tables composed (lanes hold lattice points lane and lane + 32), into
+                        // every block; only the replays wait for the others'
+                        if (warp == 0) {
+                            int t0 = lane, t1 = lane + 32;
+                            for (int k = 0; k < s.nk; ++k) {
+                                if (t0 >= 0) t0 = C.wtab[k * NT + t0];
+                                if (t1 >= 0) t1 = C.wtab[k * NT + t1];
+                            }
+                            for (unsigned r = 0; r < CL; ++r) {
+                                int8_t *d = r == crank ? btab[crank] : remote(btab[crank], r);
+                                d[lane] = (int8_t)t0;
+                                d[lane + 32] = (int8_t)t1;
+                            }
+                        }
+                        cooperative_groups::this_cluster().barrier_arrive();
+                        if (warp < busy) cooperative_groups::this_cluster().barrier_wait();
+                    }
+                    // ---- replays: each warp follows x = G - c0 from 0 (lattice index t: x = 2 t - NT) through the
+                    // blocks before mine and the windows before its own
+                    if (warp < busy) {
+                        int t = NT / 2, j = 0;
+                        if constexpr (CLUS)
+                            for (unsigned r = 0; r < crank && t >= 0; ++r) t = btab[r][t];
+                        for (int k = warp; k < s.nk; k += busy) {
+                            for (; j < k && t >= 0; ++j) t = C.wtab[j * NT + t];
+                            const int tk = t;
+                            uint32_t *pre = binned ? C.bins + (size_t)k * WBINS : nullptr;
+                            if (tk >= 0) {
+                                const int u = C.wtab[k * NT + tk];
+                                const int32_t ws = k * W, we = min(ws + W, ns);
+                                if (u < 0) {
+                                    // the first window off the lattice: it and the rest in rank order below
+                                    set_all(&w_fail[1], tk);
+                                    set_all(&w_fail[0], s.kb + k);
+                                } else {
+                                    replay_mapped<SL>(C.gam, C.s0, 0, ws, we, c0 + 2 * tk - NT, plus_first, tk, C.wmaps + 2 * k,
+                                                      WindowCounts{pre, c0, BIN_L, false},
+                                                      [&](const uint32_t (&wb)[SL]) { flip(lo, ws, we, C.s0, wb); });
+                                    if (s.kb + k == s.nwin - 1) set_all(S.G, c0 + 2 * u - NT);
+                                }
+                            }
+                            if (pre) zero_bins(pre);
+                        }
+                    } else {
+                        ahead(warp - busy, NW - busy);
+                        if constexpr (CLUS) cooperative_groups::this_cluster().barrier_wait();
                     }
                 } else if (warp > 0) {
-                    ahead(threadIdx.x - 32, BS - 32);
+                    ahead(warp - 1, NW - 1);
                 }
-                // ---- the rest in rank order by one warp of block 0, each window entered with the G its
-                // predecessors left; a window of block 1 is read remotely
-                if (crank == 0 && warp == 0 && k_seq < s.nwin) {
-                    int32_t gr = s.walk ? c0 + 2 * C.tin[nwm + 1] - NT : c0;
-                    for (int32_t kk = k_seq; kk < s.nwin; ++kk) {
+                // windows [k0, nwin) in rank order by one warp of block 0 from the exact G, each entered with the
+                // G its predecessors left; another block's windows are read remotely
+                auto in_order = [&](int k0, int32_t gr, bool bins) {
+                    for (int k = k0; k < s.nwin; ++k) {
                         const uint8_t *s0 = C.s0;
                         const int32_t *gam = C.gam;
-                        if constexpr (PAIR) {
-                            if (kk >= s.kmid) { s0 = peer(C.s0); gam = peer(C.gam); }
+                        const int b = k / s.kq;          // owner
+                        if constexpr (CLUS) {
+                            if (b > 0) { s0 = remote(C.s0, b); gam = remote(C.gam, b); }
                         }
-                        const int32_t ws = kk * W, we = min(ws + W, ns);
-                        gr = replay_window<SL>(gam, s0, 0, ws, we, gr, plus_first, -1, -1,
-                                               [&](const uint32_t (&wb)[SL]) { flip(ws, we, s0, wb); });
+                        const int32_t first = b * s.kq * W;              // the owner's first rank in the class
+                        const int32_t ws = k * W - first, we = min(ws + W, s.chi - s.clo - first);
+                        uint32_t *pre = bins ? C.bins + (size_t)k * WBINS : nullptr;
+                        if (pre) bins_to_prefix<8>(pre, BIN_L, nullptr);
+                        gr = replay_window<SL>(gam, s0, 0, ws, we, gr, plus_first, -1, -1, WindowCounts{pre, c0, BIN_L, false},
+                                               [&](const uint32_t (&wb)[SL]) { flip(s.clo + first, ws, we, s0, wb); });
+                        if (pre) zero_bins(pre);
                     }
-                    if (lane == 0) {
-                        *S.G = gr;
-                        if constexpr (PAIR) *peer(S.G) = gr;
-                    }
+                    set_all(S.G, gr);
+                };
+                if (!s.walk && crank == 0 && warp == 0) in_order(0, c0, binned);
+                cp_async_wait_all();
+                item_sync();
+                if (s.walk && w_fail[0] >= 0) {
+                    // rare: the lattice was left (every block sees the same flag)
+                    const int kf = w_fail[0];
+                    if (crank == 0 && warp == 0) in_order(kf, c0 + 2 * w_fail[1] - NT, false);
+                    item_sync();
+                    if (threadIdx.x == 0) w_fail[0] = -1;
+                    item_sync();
                 }
-                if (staged) cp_async_wait_all();
-                pair_sync();
             }
             if (R.flags & GDI_DEV_TRACE) {
                 uint64_t dg = 0;
@@ -1175,7 +1321,7 @@ __global__ void __launch_bounds__(BS, 1024 / BS) gdi_cta_sorted_kernel(GdiDevPro
                     R.tr_G[o] = *S.G;
                     R.tr_cut[o] = ct;
                 }
-                pair_sync();
+                item_sync();
             }
         }
         finish_item<BS>(P, R, base, n, mean_deg, S, C.gam, scratch_words, item, crank == 0);
@@ -1236,7 +1382,7 @@ __global__ void gdi_gather_kernel(GdiDevProblem P, const int8_t *spins, int8_t *
 // the sorted-window kernel serves every window size 1 .. 256 (one instantiation per members per
 // lane) of the running-G method when its whole-class buffers fit in a block's shared memory;
 // Algorithm 2 (GDI_DEV_STANDARD), larger windows and larger classes take gdi_cta_anneal_kernel
-constexpr size_t CTA_STATIC_SMEM = 2048;     // the kernel's class bounds and single words, rounded up
+constexpr size_t CTA_STATIC_SMEM = 3072;     // the kernel's class bounds and single words, rounded up
 
 inline bool cta_sorted(const GdiDevProblem &P, const GdiDevRun &R, int BS)
 {
@@ -1244,13 +1390,28 @@ inline bool cta_sorted(const GdiDevProblem &P, const GdiDevRun &R, int BS)
     int dev = 0, optin = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    return cta_sorted_layout(P, R.max_row, BS, 0, 0).total + CTA_STATIC_SMEM <= (size_t)optin;
+    return cta_sorted_layout(P, R.max_row, BS, 0, 0, 0, 0, 1).total + CTA_STATIC_SMEM <= (size_t)optin;
+}
+
+// Blocks per item (a cluster of 1, 2, 4 or 8): as many as leave every item its own SMs and four windows
+// of the largest class to each block.
+inline int cta_cluster(const GdiDevProblem &P, const GdiDevRun &R, int BS)
+{
+    if (!cta_sorted(P, R, BS)) return 1;
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int64_t items = (int64_t)P.num_instances * P.replicas;
+    const int64_t nw = (P.max_class + P.W - 1) / P.W;
+    int cl = 1;
+    while (cl < 8 && 2 * cl * items <= sms && 4 * 2 * cl <= nw) cl *= 2;
+    return nw <= (int64_t)cl * CTA_WALK_MAX ? cl : 1;
 }
 
 // shared memory of the kernel that takes this call (counted windows, else whole-block windows)
 inline size_t cta_smem(const GdiDevProblem &P, const GdiDevRun &R, int BS, bool counted)
 {
-    return counted ? cta_sorted_layout(P, R.max_row, BS, R.cta_opts, R.cta_stage).total
+    return counted ? cta_sorted_layout(P, R.max_row, BS, R.cta_opts, R.cta_stage, R.cta_rofs, R.cta_bins, R.cta_cluster).total
                    : cta_block_layout(P, R.max_row, BS, R.cta_opts, R.cta_stage).total;
 }
 
@@ -1258,7 +1419,7 @@ inline size_t cta_smem(const GdiDevProblem &P, const GdiDevRun &R, int BS, bool 
 // taken when it fits a block and leaves as many items resident on an SM as there are without it (never
 // more than the SM's share of the items, or than its 1024 threads at 64 registers); the staging buffer
 // takes what is then left, up to the largest class.  Returns whether the counting kernel takes the call.
-inline bool cta_options(const GdiDevProblem &P, GdiDevRun &R, int BS)
+inline bool cta_options(const GdiDevProblem &P, GdiDevRun &R, int BS, int max_cluster = 8)
 {
     int dev = 0, optin = 0, per_sm = 0, sms = 1;
     cudaGetDevice(&dev);
@@ -1269,57 +1430,63 @@ inline bool cta_options(const GdiDevProblem &P, GdiDevRun &R, int BS)
     const bool counted = cta_sorted(P, R, BS);
     R.cta_opts = 0;
     R.cta_stage = 0;
+    R.cta_rofs = 0;
+    R.cta_bins = 0;
+    R.cta_cluster = counted ? std::min(cta_cluster(P, R, BS), max_cluster) : 1;
     auto resident = [&]() {
         const size_t need = cta_smem(P, R, BS, counted) + CTA_STATIC_SMEM;
         if (need > (size_t)optin) return (int64_t)0;
         return std::min<int64_t>((int64_t)((size_t)per_sm / (need + 1024)), 1024 / BS);
     };
-    const int64_t want = std::max<int64_t>(1, std::min<int64_t>(resident(), (items + sms - 1) / sms));
+    const int64_t want = std::max<int64_t>(1, std::min<int64_t>(resident(), (items * R.cta_cluster + sms - 1) / sms));
     auto take = [&](int opt) {
         R.cta_opts |= opt;
         if (resident() < want) R.cta_opts &= ~opt;
     };
     if (!counted) take(CTA_OPT_BINS);
     if (!counted) take(CTA_OPT_ES);
+    if (counted) {
+        // bins for every window a block has of a class, up to 32, where a warp holds more than four members
+        // a lane: a count over eight costs more than the bins do (one replica of W = 64 windows runs 5 to
+        // 12 % faster without, 400 ER instances at W = 256 6 % slower)
+        if (P.W > 128) R.cta_bins = std::min(cta_own_windows(P.max_class, P.W, R.cta_cluster), 32);
+        if (resident() < want) R.cta_bins = 0;
+    }
     take(CTA_OPT_ROWS2);
     if (P.col16 && P.max_class_nnz > 0) {
         // (the first 8 columns stand for the row offsets, which any staging needs)
         R.cta_stage = 8;
         const int64_t room = std::min<int64_t>(optin, (int64_t)per_sm / want - 1024) - (int64_t)CTA_STATIC_SMEM -
                              (int64_t)cta_smem(P, R, BS, counted);
-        const int64_t cap = std::min<int64_t>(P.max_class_nnz + 24, room / 2 + 8 - 16);
-        R.cta_stage = cap >= std::min(512, P.max_class_nnz + 16) ? (int32_t)(cap & ~(int64_t)7) : 0;
+        // all rows of a block's share (a quarter above the even share), else one class's
+        const int cl = R.cta_cluster;
+        const int64_t rows = (int64_t)P.max_n / cl + (cl > 1 ? P.max_n / (4 * cl) : 0) + 64;
+        const int64_t cols = (P.max_item_nnz / cl + (cl > 1 ? P.max_item_nnz / (4 * cl) : 0) + 48 * 16) & ~(int64_t)7;
+        if (counted && P.max_item_nnz > 0 && 2 * cols + 4 * rows + 64 <= room) {
+            R.cta_stage = (int32_t)cols;
+            R.cta_rofs = (int32_t)rows;
+        } else {
+            const int64_t cap = std::min<int64_t>(P.max_class_nnz + 24, room / 2 + 8 - 16);
+            R.cta_stage = cap >= std::min(512, P.max_class_nnz + 16) ? (int32_t)(cap & ~(int64_t)7) : 0;
+        }
     }
     return counted;
 }
 
-// a pair of blocks per item when the items fill at most half of the SMs and the largest class
-// has enough windows (8 to the walk's limit) for two halves
-inline bool cta_pair(const GdiDevProblem &P, const GdiDevRun &R, int BS)
-{
-    if (!cta_sorted(P, R, BS)) return false;
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int64_t items = (int64_t)P.num_instances * P.replicas;
-    const int32_t nw = (P.max_class + P.W - 1) / P.W;
-    return 2 * items <= sms && nw >= 8 && nw <= CTA_WALK_MAX;
-}
-
-template <int BS, bool PAIR>
+template <int BS, bool CLUS>
 const void *cta_sorted_kernel_for(int W)
 {
-    return W <= 32 ? (const void *)gdi_cta_sorted_kernel<BS, 1, PAIR>
-         : W <= 64 ? (const void *)gdi_cta_sorted_kernel<BS, 2, PAIR>
-         : W <= 128 ? (const void *)gdi_cta_sorted_kernel<BS, 4, PAIR>
-                    : (const void *)gdi_cta_sorted_kernel<BS, 8, PAIR>;
+    return W <= 32 ? (const void *)gdi_cta_sorted_kernel<BS, 1, CLUS>
+         : W <= 64 ? (const void *)gdi_cta_sorted_kernel<BS, 2, CLUS>
+         : W <= 128 ? (const void *)gdi_cta_sorted_kernel<BS, 4, CLUS>
+                    : (const void *)gdi_cta_sorted_kernel<BS, 8, CLUS>;
 }
 
 template <int BS>
 const void *cta_kernel(const GdiDevProblem &P, const GdiDevRun &R)
 {
     if (!cta_sorted(P, R, BS)) return (const void *)gdi_cta_block_kernel<BS>;
-    return cta_pair(P, R, BS) ? cta_sorted_kernel_for<BS, true>(P.W) : cta_sorted_kernel_for<BS, false>(P.W);
+    return R.cta_cluster > 1 ? cta_sorted_kernel_for<BS, true>(P.W) : cta_sorted_kernel_for<BS, false>(P.W);
 }
 
 template <int BS>
@@ -1327,31 +1494,41 @@ int launch_cta(const GdiDevProblem &P, const GdiDevRun &R0, int grid_limit, cuda
                int *grid_used, size_t *smem_used)
 {
     GdiDevRun R = R0;
-    const bool counted = cta_options(P, R, BS);
-    const void *kern = cta_kernel<BS>(P, R);
-    const size_t smem = cta_smem(P, R, BS, counted);
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return (int)e;
-    int dev = 0, sms = 0, per_sm = 0;
+    const int items = P.num_instances * P.replicas;
+    int dev = 0, sms = 0, grid = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, BS, smem);
-    if (e != cudaSuccess) return (int)e;
-    if (per_sm < 1) return (int)cudaErrorInvalidConfiguration;
-    const int items = P.num_instances * P.replicas;
-    int grid = sms * per_sm;
-    if (grid > items) grid = items;
-    if (grid_limit > 0 && grid > grid_limit) grid = grid_limit;
-    if (cta_pair(P, R, BS)) {
-        // clusters of two blocks, one item per cluster
-        void *args[] = {const_cast<GdiDevProblem *>(&P), &R};
+    void *args[] = {const_cast<GdiDevProblem *>(&P), &R};
+    size_t smem = 0;
+    cudaError_t e = cudaSuccess;
+    for (int cap = grid_limit > 0 && grid_limit < 8 ? grid_limit : 8;;) {
+        // (a grid limit below a cluster's size, or a GPU partition that holds no such cluster, halves it)
+        int mc = 1;
+        while (2 * mc <= cap) mc *= 2;
+        const bool counted = cta_options(P, R, BS, mc);
+        const void *kern = cta_kernel<BS>(P, R);
+        smem = cta_smem(P, R, BS, counted);
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return (int)e;
+        if (R.cta_cluster == 1) {
+            int per_sm = 0;
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, BS, smem);
+            if (e != cudaSuccess) return (int)e;
+            if (per_sm < 1) return (int)cudaErrorInvalidConfiguration;
+            grid = std::min(sms * per_sm, items);
+            if (grid_limit > 0) grid = std::min(grid, grid_limit);
+            e = cudaLaunchKernel(kern, dim3(grid), dim3(BS), args, smem, st);
+            break;
+        }
+        // clusters of blocks, one item per cluster
+        const int cl = R.cta_cluster;
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = 2;
+        attr[0].val.clusterDim.x = cl;
         attr[0].val.clusterDim.y = 1;
         attr[0].val.clusterDim.z = 1;
         cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(2 * items);
+        cfg.gridDim = dim3(cl * items);
         cfg.blockDim = dim3(BS);
         cfg.dynamicSmemBytes = smem;
         cfg.stream = st;
@@ -1360,17 +1537,17 @@ int launch_cta(const GdiDevProblem &P, const GdiDevRun &R0, int grid_limit, cuda
         int ncl = 0;
         e = cudaOccupancyMaxActiveClusters(&ncl, kern, &cfg);
         if (e != cudaSuccess) return (int)e;
-        if (ncl < 1) return (int)cudaErrorInvalidConfiguration;
-        grid = 2 * (items < ncl ? items : ncl);
-        if (grid_limit > 0 && grid > grid_limit) grid = grid_limit >= 2 ? (grid_limit & ~1) : 2;
+        if (ncl < 1) {
+            cap = cl / 2;
+            continue;
+        }
+        grid = cl * std::min(items, ncl);
+        if (grid_limit > 0) grid = std::min(grid, grid_limit / cl * cl);
         cfg.gridDim = dim3(grid);
         e = cudaLaunchKernelExC(&cfg, kern, args);
-        if (e != cudaSuccess) return (int)e;
-    } else {
-        void *args[] = {const_cast<GdiDevProblem *>(&P), &R};
-        e = cudaLaunchKernel(kern, dim3(grid), dim3(BS), args, smem, st);
-        if (e != cudaSuccess) return (int)e;
+        break;
     }
+    if (e != cudaSuccess) return (int)e;
     if (grid_used) *grid_used = grid;
     if (smem_used) *smem_used = smem;
     return (int)cudaGetLastError();
@@ -1389,6 +1566,30 @@ int cta_occupancy(const GdiDevProblem &P, const GdiDevRun &R0, int *per_sm)
 }
 
 }  // namespace
+
+// Threads per block where the caller has set none.  Items that leave SMs idle take 512 (ms at 256 / 512 /
+// 1024: 8 replicas of 1500 vertices, W = 64: 32.0 / 27.8 / 31.8; whole-class windows 7.4 / 6.9 / 8.6), 1024
+// where a block's share of the largest class passes 800 ranks (BA 20,000 on one cluster: 19.4 / 15.1 /
+// 13.9; 64 replicas of a 100 x 100 torus: 26.2 / 15.8 / 10.8), 256 where no class reaches 128 (ER-800: 42.7 /
+// 44.1 / 51.7: barriers, not work).  Three items an SM still gain from 512 (400 ER instances: 15.6 / 15.0 /
+// 25.3); more take 256 (1024 short anneals: 4.4 / 6.0 / 10.2).
+int gdi_cta_default_block(const GdiDevProblem &P, const GdiDevRun &R)
+{
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int64_t items = (int64_t)P.num_instances * P.replicas;
+    if (items > 3LL * sms) return 256;
+    const int cl = cta_cluster(P, R, 512);
+    if (items * cl <= sms && cta_sorted(P, R, 512)) {
+        const int64_t own = cl > 1 ? (int64_t)cta_own_windows(P.max_class, P.W, cl) * P.W : P.max_class;
+        if (own > 800) return 1024;
+        if (P.max_class < 128) return 256;
+    }
+    return 512;
+}
+
+int gdi_cta_cluster_size(const GdiDevProblem &P, const GdiDevRun &R, int block) { return cta_cluster(P, R, block); }
 
 int gdi_cta_blocks_per_sm(const GdiDevProblem &P, const GdiDevRun &R, int block, int *per_sm)
 {

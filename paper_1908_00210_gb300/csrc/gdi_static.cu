@@ -187,6 +187,7 @@ extern "C" int gdi_anneal_static(int32_t n, const int64_t *row_ptr, const uint32
     P.max_degree = max_degree;
     P.max_class = max_class;
     P.max_class_nnz = 0;
+    P.max_item_nnz = 0;
     int spc = 0, wpc = 0;
     size_t smem = 0;
     bool counted = false;

@@ -20,7 +20,8 @@ namespace win {
 constexpr int KC = 31;                  // flips per group the exact counting histogram covers at once
 constexpr int HA = 2 * KC + 1;          // histogram bins of the exact counting replay
 constexpr int NT = 64;                  // lattice points of a stage map
-constexpr int WBINS = 256;              // words a warp counts a window's distances in
+constexpr int WBINS = 256;              // words a window's distances are counted in
+constexpr int BIN_L = 190;              // distance -BIN_L is bin 0 (everything below too) in 256 bins
 constexpr unsigned long long STEP_MASK = (1ull << (NT - 1)) - 1ull;
 
 struct StageMap {
@@ -197,13 +198,9 @@ __device__ inline int32_t warp_group(const int32_t *gam, int gs, int gc, const u
     return K;
 }
 
-// The two stage maps of a window from its histogram, by one warp: lane l holds the counts of the PER
-// bins d = PER l - L ... (v[i]: +1 group low 16 bits, -1 group high 16).  The members of a group in
-// flip order are the bins in d order, so a bin with h members of which C come before it in the group
-// holds a_k = d + 2C, d + 2C + 2, ...: h consecutive lattice intervals, one run of mask bits.
-// out[0] = +1 group (flips iff a_k <= x), out[1] = -1 group (flips iff a_k <= -x).
+// counts of all bins before this lane's PER, by one warp
 template <int PER>
-__device__ __forceinline__ void stage_maps_of(const uint32_t (&v)[PER], int L, StageMap *out)
+__device__ __forceinline__ uint32_t bins_before(const uint32_t (&v)[PER])
 {
     const int lane = threadIdx.x & 31;
     uint32_t tot = 0;
@@ -216,9 +213,22 @@ __device__ __forceinline__ void stage_maps_of(const uint32_t (&v)[PER], int L, S
         if (lane >= o) run += y;
     }
     run -= tot;
+    return run;
+}
+
+// The two stage maps of a window from its histogram, by one warp: lane l holds the counts of the PER
+// bins d = PER l - L ... (v[i]: +1 group low 16 bits, -1 group high 16; run: the counts of the bins
+// before).  The members of a group in
+// flip order are the bins in d order, so a bin with h members of which C come before it in the group
+// holds a_k = d + 2C, d + 2C + 2, ...: h consecutive lattice intervals, one run of mask bits.
+// out[0] = +1 group (flips iff a_k <= x), out[1] = -1 group (flips iff a_k <= -x).
+template <int PER>
+__device__ __forceinline__ void stage_maps_of(const uint32_t (&v)[PER], uint32_t run, int L, StageMap *out)
+{
+    const int lane = threadIdx.x & 31;
     unsigned long long kp = 0, km = 0;
     int32_t cle = 0, cge = 0;
-    if (tot) {
+    {
 #pragma unroll
         for (int i = 0; i < PER; ++i) {
             const int32_t d = lane * PER + i - L;
@@ -288,7 +298,7 @@ __device__ __forceinline__ void window_maps(const int32_t *gam_r, const uint8_t 
     b4[lane] = make_uint4(0u, 0u, 0u, 0u);
     if (w) b4[lane + 32] = make_uint4(0u, 0u, 0u, 0u);
     __syncwarp();
-    const int L = w ? 190 : 62;
+    const int L = w ? BIN_L : 62;
 #pragma unroll
     for (int s = 0; s < S; ++s)
         if (dv[s] <= NT) atomicAdd(&bins[max(dv[s] + L, 0)], (ng >> s) & 1u ? 0x10000u : 1u);
@@ -296,11 +306,11 @@ __device__ __forceinline__ void window_maps(const int32_t *gam_r, const uint8_t 
     if (!w) {
         const uint4 q = b4[lane];
         const uint32_t v[4] = {q.x, q.y, q.z, q.w};
-        stage_maps_of<4>(v, 62, out);
+        stage_maps_of<4>(v, bins_before<4>(v), 62, out);
     } else {
         const uint4 q = b4[2 * lane], p = b4[2 * lane + 1];
         const uint32_t v[8] = {q.x, q.y, q.z, q.w, p.x, p.y, p.z, p.w};
-        stage_maps_of<8>(v, 190, out);
+        stage_maps_of<8>(v, bins_before<8>(v), BIN_L, out);
     }
     __syncwarp();
 }
@@ -315,7 +325,7 @@ __device__ __forceinline__ void count_members(const int32_t *gam_r, const uint8_
         const int32_t g = gam_r[i];
         const bool neg = (s0[i] >> r) & 1u;
         const int32_t d = neg ? c - g : g - c;
-        if (d <= NT) atomicAdd(&bins[max(d + 190, 0)], neg ? 0x10000u : 1u);
+        if (d <= NT) atomicAdd(&bins[max(d + BIN_L, 0)], neg ? 0x10000u : 1u);
     }
 }
 
@@ -325,7 +335,7 @@ __device__ __forceinline__ void bins_to_maps(const uint32_t *bins, StageMap *out
     const int lane = threadIdx.x & 31;
     const uint4 q = b4[2 * lane], p = b4[2 * lane + 1];
     const uint32_t v[8] = {q.x, q.y, q.z, q.w, p.x, p.y, p.z, p.w};
-    stage_maps_of<8>(v, 190, out);
+    stage_maps_of<8>(v, bins_before<8>(v), BIN_L, out);
 }
 
 static __device__ __forceinline__ int stage_apply(const StageMap &m, int t)
@@ -335,6 +345,78 @@ static __device__ __forceinline__ int stage_apply(const StageMap &m, int t)
     return (y >= 0 && y < NT) ? y : -1;
 }
 
+// a window's 32 * PER bins (distance -L first) to inclusive prefix counts in place, by one warp; its stage
+// maps too (out != null)
+template <int PER>
+__device__ __forceinline__ void bins_to_prefix(uint32_t *bins, int L, StageMap *out)
+{
+    uint4 *b4 = reinterpret_cast<uint4 *>(bins);
+    const int lane = threadIdx.x & 31;
+    uint32_t v[PER], c[PER];
+#pragma unroll
+    for (int i = 0; i < PER / 4; ++i) {
+        const uint4 q = b4[PER / 4 * lane + i];
+        v[4 * i] = q.x; v[4 * i + 1] = q.y; v[4 * i + 2] = q.z; v[4 * i + 3] = q.w;
+    }
+    const uint32_t run = bins_before<PER>(v);
+    c[0] = run + v[0];
+#pragma unroll
+    for (int i = 1; i < PER; ++i) c[i] = c[i - 1] + v[i];
+#pragma unroll
+    for (int i = 0; i < PER / 4; ++i)
+        b4[PER / 4 * lane + i] = make_uint4(c[4 * i], c[4 * i + 1], c[4 * i + 2], c[4 * i + 3]);
+    if (out) stage_maps_of<PER>(v, run, L, out);
+    __syncwarp();
+}
+
+// prefix counts of one window: bin i holds the members with distance <= i - L; full: none lies below -L
+struct WindowCounts {
+    const uint32_t *pre;                // null: none kept
+    int32_t c;                          // reference G of the distances
+    int L;
+    bool full;
+};
+
+// A group's flips off a window's prefix counts (shift sh: 0 = +1 group, 16 = -1 group), by one warp.
+// z = the entering G's distance from the bins' reference on the group's flipping side, so that a member
+// with distance d has margin e = z - d and #{e >= y} = C(z - y).  K: known, or -1 and found.  Members with
+// e > y flip, and of those with e == y the first `left`.  False when the bins do not reach that far.
+__device__ __forceinline__ bool binned_flips(const WindowCounts &wc, int sh, int32_t z, int32_t &K, int32_t &y, int32_t &left)
+{
+    if (z > NT) return false;
+    const int lane = threadIdx.x & 31;
+    const int i0 = z + wc.L;
+    auto at = [&](int i) { return i < 0 ? 0 : (int32_t)((wc.pre[i] >> sh) & 0xFFFFu); };
+    if (K < 0) {
+        for (int k0 = 0; K < 0; k0 += 32) {
+            const int i = i0 - 2 * (k0 + lane);
+            const unsigned hit = __ballot_sync(0xFFFFFFFFu, (i >= 0 || wc.full) && at(i) <= k0 + lane);
+            if (hit) K = k0 + __ffs(hit) - 1;
+            else if (i0 - 2 * (k0 + 32) < 0) return false;
+        }
+    }
+    y = INT32_MAX;
+    left = 0;
+    if (K == 0) return true;
+    const int i = i0 - 2 * K;
+    if (i < 0 && !wc.full) return false;
+    const int32_t n0 = at(i), n1 = at(i + 1), n2 = at(i + 2);
+    int32_t ties = 0;
+    y = 2 * K - 1;
+    if (n0 != K) {
+        if (n1 >= K) {
+            left = K - n0;
+            ties = n1 - n0;
+        } else {
+            y = 2 * K - 2;
+            left = K - n1;
+            ties = n2 - n1;
+        }
+        if (left == ties) { --y; left = 0; }
+    }
+    return true;
+}
+
 // Replay of one window (positions [ws, we)) of replica r from the exact entering G g, by one warp: both
 // groups in order; emit(wbits) takes the flips, bit l of wbits[s] for position ws + 32 s + l.  With e = the distance of a member's threshold
 // on the flipping side of G, the members flip in e order and the k-th (from 0) flips iff e >= 2k, so with
@@ -342,10 +424,12 @@ static __device__ __forceinline__ int stage_apply(const StageMap &m, int t)
 // the last of them has e >= 2K, = 2K - 1 or = 2K - 2: three counts give the threshold, and equal
 // members flip in position order.  K1, K2: the flips of the first and second group when the stage
 // maps gave them (the window was entered on the lattice), else -1: searched, four-way, three counts
-// to a reduction.  Returns G after the window.
+// to a reduction.  wc: the window's prefix counts, which answer all of this in a few reads where
+// they reach.  Returns G after the window.
 template <int SL, class Emit>
 __device__ __forceinline__ int32_t replay_window(const int32_t *gr, const uint8_t *s0, int r, int ws, int we,
-                                                 int32_t g, bool plus_first, int K1, int K2, const Emit &emit)
+                                                 int32_t g, bool plus_first, int K1, int K2, const WindowCounts &wc,
+                                                 const Emit &emit)
 {
     static_assert(32 * SL < 1024, "three counts share a word");
     const int lane = threadIdx.x & 31;
@@ -362,10 +446,42 @@ __device__ __forceinline__ int32_t replay_window(const int32_t *gr, const uint8_
             ng |= ((uint32_t)(s0[i] >> r) & 1u) << s;
         }
     }
+    // both groups off the counts: one pass over the members, each against its group's cut
+    if (wc.pre) {
+        int32_t Ka = K1, Kb = K2, ya, yb, la, lb;
+        const int32_t xa = plus_first ? g - wc.c : wc.c - g;             // on the first group's side
+        if (binned_flips(wc, plus_first ? 0 : 16, xa, Ka, ya, la)) {
+            const int32_t xb = 2 * Ka - xa;                              // on the second's, after it
+            if (binned_flips(wc, plus_first ? 16 : 0, xb, Kb, yb, lb)) {
+                // members at distance d < c* flip, and of those at c* the first l*
+                const int32_t ca = Ka ? xa - ya : INT32_MIN, cb = Kb ? xb - yb : INT32_MIN;
+                const int32_t cp = plus_first ? ca : cb, cm = plus_first ? cb : ca;
+                int32_t lp = plus_first ? la : lb, lm = plus_first ? lb : la;
+                uint32_t wbits[SL];
+                const unsigned before = (1u << lane) - 1u;
+#pragma unroll
+                for (int s = 0; s < SL; ++s) {
+                    const bool neg = (ng >> s) & 1u, in = (vd >> s) & 1u;
+                    const int32_t d = neg ? wc.c - gv[s] : gv[s] - wc.c, cut = neg ? cm : cp;
+                    bool f = in && d < cut;
+                    if (lp | lm) {
+                        const bool tie = in && d == cut;
+                        const unsigned tn = __ballot_sync(0xFFFFFFFFu, tie && neg), tp = __ballot_sync(0xFFFFFFFFu, tie && !neg);
+                        f |= tie && __popc((neg ? tn : tp) & before) < (neg ? lm : lp);
+                        lp = max(lp - __popc(tp), 0);
+                        lm = max(lm - __popc(tn), 0);
+                    }
+                    wbits[s] = __ballot_sync(0xFFFFFFFFu, f);
+                }
+                emit(wbits);
+                return g + (plus_first ? 2 * (Kb - Ka) : 2 * (Ka - Kb));
+            }
+        }
+    }
     uint32_t wbits[SL];
 #pragma unroll
     for (int s = 0; s < SL; ++s) wbits[s] = 0;
-#pragma unroll
+#pragma unroll 1
     for (int ph = 0; ph < 2; ++ph) {
         const bool plus = plus_first == (ph == 0);
         const uint32_t mem = vd & (plus ? ~ng : ng);
@@ -380,7 +496,7 @@ __device__ __forceinline__ int32_t replay_window(const int32_t *gr, const uint8_
                 n += (e[s] >= y0 ? 1u : 0u) + (e[s] >= y1 ? 1u << 10 : 0u) + (e[s] >= y2 ? 1u << 20 : 0u);
             return __reduce_add_sync(0xFFFFFFFFu, n);
         };
-        int32_t K = ph == 0 ? K1 : K2;
+        int32_t K = ph == 0 ? K1 : K2, y, left;
         if (K < 0) {
             int32_t n0 = 0;
 #pragma unroll
@@ -398,17 +514,22 @@ __device__ __forceinline__ int32_t replay_window(const int32_t *gr, const uint8_
             }
             K = lo;
         }
+        y = 2 * K - 1;
+        left = 0;
+        if (K > 0) {
+            const uint32_t n = count3(2 * K, 2 * K - 1, 2 * K - 2);
+            const int32_t n0 = n & 1023u, n1 = (n >> 10) & 1023u, n2 = n >> 20;
+            if (n0 != K) {
+                if (n1 < K) --y;
+                left = n1 >= K ? K - n0 : K - n1;
+                if (left == (n1 >= K ? n1 - n0 : n2 - n1)) { --y; left = 0; }
+            }
+        }
         if (K == 0) continue;
-        const uint32_t n = count3(2 * K, 2 * K - 1, 2 * K - 2);
-        const int32_t n0 = n & 1023u, n1 = (n >> 10) & 1023u, n2 = n >> 20;
-        // ties at y flip up to `left`; everything above flips
-        const int32_t y = n0 == K ? 2 * K : (n1 >= K ? 2 * K - 1 : 2 * K - 2);
-        const int32_t at = n0 == K ? n0 : (n1 >= K ? n1 : n2);
-        if (at == K) {
+        if (left == 0) {
 #pragma unroll
-            for (int s = 0; s < SL; ++s) wbits[s] |= __ballot_sync(0xFFFFFFFFu, e[s] >= y);
+            for (int s = 0; s < SL; ++s) wbits[s] |= __ballot_sync(0xFFFFFFFFu, e[s] > y);
         } else {
-            int32_t left = K - (n1 >= K ? n0 : n1);
 #pragma unroll
             for (int s = 0; s < SL; ++s) {
                 const unsigned tm = __ballot_sync(0xFFFFFFFFu, e[s] == y);
@@ -450,7 +571,7 @@ __device__ __forceinline__ void flips_to_bitmap(const uint32_t (&wbits)[SL], int
 // flips of positions i0 .. i0 + 31 (once per group).
 template <class Emit>
 __device__ __noinline__ int32_t replay_large(const int32_t *gr, const uint8_t *s0, int r, int ws, int we, int32_t g,
-                                             bool plus_first, int K1, int K2, const Emit &emit)
+                                             bool plus_first, int K1, int K2, const WindowCounts &wc, const Emit &emit)
 {
     const int lane = threadIdx.x & 31;
     for (int ph = 0; ph < 2; ++ph) {
@@ -464,28 +585,27 @@ __device__ __noinline__ int32_t replay_large(const int32_t *gr, const uint8_t *s
             for (int i = ws + lane; i < we; i += 32) n += margin(i) >= y ? 1 : 0;
             return (int32_t)__reduce_add_sync(0xFFFFFFFFu, n);
         };
-        int32_t K = ph == 0 ? K1 : K2;
-        if (K < 0) {
-            int32_t hi = count(0), lo = min(hi, 1);
-            while (lo < hi) {
-                const int32_t mid = (lo + hi + 1) >> 1;
-                if (count(2 * mid - 2) >= mid) lo = mid; else hi = mid - 1;
+        int32_t K = ph == 0 ? K1 : K2, y, left;
+        if (!wc.pre || !binned_flips(wc, plus ? 0 : 16, plus ? g - wc.c : wc.c - g, K, y, left)) {
+            if (K < 0) {
+                int32_t hi = count(0), lo = min(hi, 1);
+                while (lo < hi) {
+                    const int32_t mid = (lo + hi + 1) >> 1;
+                    if (count(2 * mid - 2) >= mid) lo = mid; else hi = mid - 1;
+                }
+                K = lo;
             }
-            K = lo;
+            y = 2 * K - 1;
+            left = 0;
+            if (K > 0) {
+                const int32_t n0 = count(2 * K), n1 = count(2 * K - 1);
+                if (n0 != K && n1 < K) --y;
+                left = n0 == K ? 0 : (n1 >= K ? K - n0 : K - n1);
+            }
         }
         if (K == 0) continue;
-        int32_t n0 = 0, n1 = 0;
-        for (int i = ws + lane; i < we; i += 32) {
-            const int32_t e = margin(i);
-            n0 += e >= 2 * K ? 1 : 0;
-            n1 += e >= 2 * K - 1 ? 1 : 0;
-        }
-        n0 = __reduce_add_sync(0xFFFFFFFFu, n0);
-        n1 = __reduce_add_sync(0xFFFFFFFFu, n1);
-        const int32_t y = n0 == K || n1 >= K ? 2 * K - 1 : 2 * K - 2;
-        int32_t left = n0 == K ? 0 : (n1 >= K ? K - n0 : K - n1);
         for (int i0 = ws; i0 < we; i0 += 32) {
-            const int32_t e = i0 + lane < we ? margin(i0 + lane) : -1;
+            const int32_t e = i0 + lane < we ? margin(i0 + lane) : INT32_MIN;
             const unsigned tm = __ballot_sync(0xFFFFFFFFu, e == y);
             const int32_t idx = __popc(tm & ((1u << lane) - 1u));
             const unsigned bits = __ballot_sync(0xFFFFFFFFu, e > y || (e == y && idx < left));
@@ -513,11 +633,12 @@ __device__ __forceinline__ void mapped_flips(bool plus_first, int t, const Stage
 // replay_window for a window entered at lattice index t with its stage maps
 template <int SL, class Emit>
 __device__ __forceinline__ int32_t replay_mapped(const int32_t *gr, const uint8_t *s0, int r, int ws, int we, int32_t g,
-                                                 bool plus_first, int t, const StageMap *maps, const Emit &emit)
+                                                 bool plus_first, int t, const StageMap *maps,
+                                                 const WindowCounts &wc, const Emit &emit)
 {
     int K1, K2;
     mapped_flips(plus_first, t, maps, K1, K2);
-    return replay_window<SL>(gr, s0, r, ws, we, g, plus_first, K1, K2, emit);
+    return replay_window<SL>(gr, s0, r, ws, we, g, plus_first, K1, K2, wc, emit);
 }
 
 }  // namespace win

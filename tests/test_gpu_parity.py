@@ -232,3 +232,18 @@ def test_counted_windows_with_thresholds_far_from_g(gdi, path, W, t0, mode):
         ref = oracle.anneal(g, A=1, B=1, W=W, mode=mode, t0=t0, t1=sch.t1, pf0=0.45, pf1=0.05, sweeps=6, seed=3,
                             replicas=2, init=start, trace=True)
         assert_parity(res, spins, tr, ref)
+
+
+@pytest.mark.parametrize("n,W,replicas", [(5000, 64, 1), (6001, 256, 3), (9000, 32, 20), (2500, 7, 2), (33000, 128, 2)])
+def test_cta_cluster_sizes(gdi, n, W, replicas):
+    """Clusters of two to eight blocks per item (uneven window counts, 16- and 32-bit columns, several
+    waves of items), bit-exact after every sweep."""
+    g = barabasi_albert(n, 5, 91)
+    sch = gdi.Schedule(sweeps=12, t0=12.0, t1=0.2)
+    ann = gdi.Annealer(g, A=1, B=4, W=W, replicas=replicas)
+    ann.configure(path=gdi.GDI_PATH_CTA)
+    ann.anneal(sch, 11, flags=gdi.GDI_FLAG_TRACE)
+    res, spins, tr = ann.results(), ann.spins(), ann.trace()
+    ann.close()
+    ref = oracle.anneal(g, A=1, B=4, W=W, t0=12.0, t1=0.2, sweeps=12, seed=11, replicas=replicas, trace=True)
+    assert_parity(res, spins, tr, ref)
