@@ -925,6 +925,7 @@ __host__ __device__ inline int walk_slots(int P) { return nruns(P) + 2 * RUN; }
 struct SortedLayout {
     size_t off_h, off_gam, off_es, off_s0, off_fm, off_fbits, off_longq, off_smap, off_wtab, off_tin, off_walk, off_row, off_bins, off_misc, total;
     int fw;                             // words of one replica's flip bitmap
+    int cw;                             // warps that count windows
     int gs;                             // threshold row stride (ints): >= spc + 7, 4 mod 32
     int es;                             // E* row stride (int16): >= spc + 7, 16 mod 32; 0 = no E* rows
 };
@@ -939,9 +940,7 @@ __host__ __device__ inline SortedLayout sorted_layout(int spc, int wpc, int max_
 {
     SortedLayout L;
     size_t o = 0;
-    // the fields; once the thresholds are made, the counting warps' bins
-    const size_t fields = (size_t)spc * 8 * sizeof(int16_t), bins = (size_t)NWARP * WBINS * sizeof(uint32_t);
-    L.off_h = o; o = align16(o + (fields > bins ? fields : bins));
+    L.off_h = o; o = align16(o + (size_t)spc * 8 * sizeof(int16_t));      // fields
     // thresholds [r][gs]: a row starts 4 words (16 banks' worth of bytes) after the previous
     // one's bank, so the 8 replicas' 16-byte stores of one quad of ranks hit disjoint banks
     L.gs = ((spc + 3 + 31) & ~31) + 4;
@@ -957,7 +956,12 @@ __host__ __device__ inline SortedLayout sorted_layout(int spc, int wpc, int max_
     L.off_smap = o; o = align16(o + (size_t)wpc * 8 * 2 * sizeof(StageMap));
     L.off_wtab = o; o = align16(o + (tables ? (size_t)wpc * 8 * NT : 0));   // both maps of a window composed
     L.off_tin = o; o = align16(o + (tables ? (size_t)wpc * 8 : 0));         // its entering lattice index, or -1
-    L.off_walk = o; o = align16(o + (size_t)8 * walk_slots(P) * NT);
+    // the walk's tables and, before it, the counting warps' bins: all warps count where anything beyond the
+    // necessary is kept, else as many as the tables' bytes hold
+    const size_t wk = (size_t)8 * walk_slots(P) * NT, wbin = WBINS * sizeof(uint32_t);
+    const bool grow = es_rows || tables || binned;
+    L.cw = grow || wk >= NWARP * wbin ? NWARP : (int)(wk / wbin);
+    L.off_walk = o; o = align16(o + (L.cw * wbin > wk ? L.cw * wbin : wk));
     L.off_row = o; o = align16(o + (size_t)(max_row + 4) * sizeof(uint32_t));
     L.off_bins = o; o = align16(o + (binned ? (size_t)wpc * 8 * GBINS * sizeof(uint32_t) : 0));
     L.off_misc = o; o = align16(o + 64 * sizeof(int64_t));
@@ -1112,12 +1116,12 @@ __global__ void __launch_bounds__(GB, 1) gdi_grid_sorted_kernel(GridArgs A)
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int spc = A.spc;
     const SortedLayout L = sorted_layout(spc, A.wpc, R.max_row, Pb, A.es_pre, A.tables, A.binned);
-    int16_t *hb = reinterpret_cast<int16_t *>(smem_raw + L.off_h);   // fields [i*8 + r], then the counting warps' bins
+    int16_t *hb = reinterpret_cast<int16_t *>(smem_raw + L.off_h);   // fields [i*8 + r]
     int32_t *gam = reinterpret_cast<int32_t *>(smem_raw + L.off_gam);
     int16_t *esb = reinterpret_cast<int16_t *>(smem_raw + L.off_es);   // E* drawn ahead [r][L.es]
     uint8_t *s0 = smem_raw + L.off_s0;
     StageMap *smap = reinterpret_cast<StageMap *>(smem_raw + L.off_smap);
-    uint32_t *hist = reinterpret_cast<uint32_t *>(smem_raw + L.off_h);
+    uint32_t *hist = reinterpret_cast<uint32_t *>(smem_raw + L.off_walk);   // counting warps' bins
     int8_t *walk = reinterpret_cast<int8_t *>(smem_raw + L.off_walk);
     int8_t *wtab = reinterpret_cast<int8_t *>(smem_raw + L.off_wtab);   // [window][replica][NT]
     int8_t *tin = reinterpret_cast<int8_t *>(smem_raw + L.off_tin);     // [window][replica]
@@ -1218,7 +1222,7 @@ __global__ void __launch_bounds__(GB, 1) gdi_grid_sorted_kernel(GridArgs A)
                              });
             // ---- counts and stage maps of every (window, replica)
             // (counted with their thresholds, or here where the bins do not fit or a distance lay below them)
-            for (int task = warp; task < nwin * nrep; task += NWARP) {
+            for (int task = warp; task < nwin * nrep && warp < L.cw; task += L.cw) {
                 const int kk = task / nrep, r = task % nrep;
                 const int ws = kk * W, wlen = min(W, ns - ws);
                 StageMap *o = smap + ((size_t)kk * 8 + r) * 2;
