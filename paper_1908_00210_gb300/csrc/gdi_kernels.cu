@@ -1398,9 +1398,11 @@ inline bool cta_sorted(const GdiDevProblem &P, const GdiDevRun &R, int BS)
     return cta_sorted_layout(P, R.max_row, BS, 0, 0, 0, 0, 1).total + CTA_STATIC_SMEM <= (size_t)optin;
 }
 
-// Blocks per item (a cluster of 1, 2, 4 or 8): as many as leave every item its own SMs and four windows
-// of the largest class to each block.
-inline int cta_cluster(const GdiDevProblem &P, const GdiDevRun &R, int BS)
+// Blocks per item (a cluster of 1, 2, 4 or 8, at most `most`): as many as leave every item its own SMs and four
+// windows of the largest class to each block.  A block's share of the largest class has to stay within the
+// windows whose maps are kept: cta_sorted_layout sizes a cluster's class buffers for the shares, and a class
+// beyond that would be the first block's alone.
+inline int cta_cluster(const GdiDevProblem &P, const GdiDevRun &R, int BS, int most)
 {
     if (!cta_sorted(P, R, BS)) return 1;
     int dev = 0, sms = 0;
@@ -1409,7 +1411,7 @@ inline int cta_cluster(const GdiDevProblem &P, const GdiDevRun &R, int BS)
     const int64_t items = (int64_t)P.num_instances * P.replicas;
     const int64_t nw = (P.max_class + P.W - 1) / P.W;
     int cl = 1;
-    while (cl < 8 && 2 * cl * items <= sms && 4 * 2 * cl <= nw) cl *= 2;
+    while (2 * cl <= std::min(most, 8) && 2 * cl * items <= sms && 4 * 2 * cl <= nw) cl *= 2;
     return nw <= (int64_t)cl * CTA_WALK_MAX ? cl : 1;
 }
 
@@ -1437,7 +1439,7 @@ inline bool cta_options(const GdiDevProblem &P, GdiDevRun &R, int BS, int max_cl
     R.cta_stage = 0;
     R.cta_rofs = 0;
     R.cta_bins = 0;
-    R.cta_cluster = counted ? std::min(cta_cluster(P, R, BS), max_cluster) : 1;
+    R.cta_cluster = cta_cluster(P, R, BS, max_cluster);
     auto resident = [&]() {
         const size_t need = cta_smem(P, R, BS, counted) + CTA_STATIC_SMEM;
         if (need > (size_t)optin) return (int64_t)0;
@@ -1508,9 +1510,7 @@ int launch_cta(const GdiDevProblem &P, const GdiDevRun &R0, int grid_limit, cuda
     cudaError_t e = cudaSuccess;
     for (int cap = grid_limit > 0 && grid_limit < 8 ? grid_limit : 8;;) {
         // (a grid limit below a cluster's size, or a GPU partition that holds no such cluster, halves it)
-        int mc = 1;
-        while (2 * mc <= cap) mc *= 2;
-        const bool counted = cta_options(P, R, BS, mc);
+        const bool counted = cta_options(P, R, BS, cap);
         const void *kern = cta_kernel<BS>(P, R);
         smem = cta_smem(P, R, BS, counted);
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -1585,7 +1585,7 @@ int gdi_cta_default_block(const GdiDevProblem &P, const GdiDevRun &R)
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int64_t items = (int64_t)P.num_instances * P.replicas;
     if (items > 3LL * sms) return 256;
-    const int cl = cta_cluster(P, R, 512);
+    const int cl = cta_cluster(P, R, 512, 8);
     if (items * cl <= sms && cta_sorted(P, R, 512)) {
         const int64_t own = cl > 1 ? (int64_t)cta_own_windows(P.max_class, P.W, cl) * P.W : P.max_class;
         if (own > 800) return 1024;
@@ -1594,7 +1594,7 @@ int gdi_cta_default_block(const GdiDevProblem &P, const GdiDevRun &R)
     return 512;
 }
 
-int gdi_cta_cluster_size(const GdiDevProblem &P, const GdiDevRun &R, int block) { return cta_cluster(P, R, block); }
+int gdi_cta_cluster_size(const GdiDevProblem &P, const GdiDevRun &R, int block) { return cta_cluster(P, R, block, 8); }
 
 int gdi_cta_blocks_per_sm(const GdiDevProblem &P, const GdiDevRun &R, int block, int *per_sm)
 {

@@ -247,3 +247,24 @@ def test_cta_cluster_sizes(gdi, n, W, replicas):
     ann.close()
     ref = oracle.anneal(g, A=1, B=4, W=W, t0=12.0, t1=0.2, sweeps=12, seed=11, replicas=replicas, trace=True)
     assert_parity(res, spins, tr, ref)
+
+
+@pytest.mark.parametrize("grid_limit", [1, 2, 3, 4, 7, 16])
+@pytest.mark.parametrize("W", [1, 3, 5, 9])
+def test_cta_cluster_capped_by_grid_limit(gdi, W, grid_limit):
+    """A grid limit below the cluster that the sizes ask for: classes of more than 128 windows a block at two and
+    at four blocks (W = 5 and 3 of 2,186 ranks), at every cluster size (W = 1), and within them (W = 9).
+    Results do not depend on the limit: bit-exact after every sweep."""
+    g = barabasi_albert(9000, 5, 92)
+    windows = -(-gdi.rank_space(g).max_class // W)
+    assert windows > {1: 1024, 3: 512, 5: 256, 9: 128}[W]
+    sch = gdi.Schedule(sweeps=5, t0=12.0, t1=0.2)
+    ann = gdi.Annealer(g, A=1, B=4, W=W, replicas=2)
+    ann.configure(path=gdi.GDI_PATH_CTA, grid_limit=grid_limit)
+    ann.anneal(sch, 13, flags=gdi.GDI_FLAG_TRACE)
+    res, spins, tr = ann.results(), ann.spins(), ann.trace()
+    launch = ann.last_launch()
+    ann.close()
+    assert launch["grid"] <= grid_limit
+    ref = oracle.anneal(g, A=1, B=4, W=W, t0=12.0, t1=0.2, sweeps=5, seed=13, replicas=2, trace=True)
+    assert_parity(res, spins, tr, ref)
