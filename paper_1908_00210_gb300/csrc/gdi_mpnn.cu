@@ -642,7 +642,9 @@ __global__ void feat_init_kernel(int64_t N, int G, const int64_t *graph_ptr, con
 // eighth slice each; the runs live in the caller's X and scratch, which hold 128 bytes per vertex and
 // are free until the result is written (run r of a graph of n vertices: X for r < n, then the two
 // halves of the scratch), so a graph whose runs exceed 2 n, or of more than `cap` vertices, is left
-// to walk_rest_kernel.  The sums run in CSR order whatever the renumbering.
+// to walk_rest_kernel.  The sums run in CSR order whatever the renumbering.  Only columns inside the graph have
+// a rank: one that leads to another graph is laid out as the number n, and the batch is marked for
+// walk_rest_kernel.
 //
 // Bound by the random shared-memory reads: 32 random words take 3.5 passes on average.  Inference on
 // 128 graphs of 1,000 to 5,000 vertices (256 steps): 120 ms with one launch per step (470 us each), 18.6 ms
@@ -690,6 +692,7 @@ diffuse_kernel(const int64_t *graph_ptr, const uint32_t *graph_id, const int64_t
     extern __shared__ __align__(16) unsigned char sm_raw[];
     __shared__ int hist[DF_BINS];
     __shared__ int nruns;
+    __shared__ int leaves;                                             // block 0's: a column leads out of the graph
     const int g = blockIdx.x / DF_CL, ch = blockIdx.x % DF_CL;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t v0 = graph_ptr[g];
@@ -711,6 +714,7 @@ diffuse_kernel(const int64_t *graph_ptr, const uint32_t *graph_id, const int64_t
     runs.r0 = reinterpret_cast<uint16_t *>(R0 + v0 * NRAND);
     runs.r1 = reinterpret_cast<uint16_t *>(R1 + v0 * NRAND);
     runs.n = n;
+    if (threadIdx.x == 0) leaves = 0;
     if (fits && ch == 0) {
         // ranks by falling degree (degrees from DF_BINS - 1 on share a bin), by block 0 for the cluster:
         // the atomics rank equal degrees in any order
@@ -782,6 +786,7 @@ diffuse_kernel(const int64_t *graph_ptr, const uint32_t *graph_id, const int64_t
         cluster.sync();
     }
     if (fits) {
+        bool out = false;
         for (int s = warp * DF_CL + ch; s < ns; s += DF_CL * (DF_T / 32)) {
             const int r = 32 * s + lane;
             const int64_t e0 = r < n ? rp[perm[r]] : 0;
@@ -789,9 +794,16 @@ diffuse_kernel(const int64_t *graph_ptr, const uint32_t *graph_id, const int64_t
             for (int k = 0; k < len; ++k) {
                 int room;
                 uint16_t *o = runs.at((int)slice[s] + k, room);
-                o[lane] = k < d ? rank[col[e0 + k] - v0] : (uint16_t)n;
+                uint16_t at = (uint16_t)n;
+                if (k < d) {
+                    const int64_t j = col[e0 + k] - v0;
+                    if (j >= 0 && j < n) at = rank[j];
+                    else out = true;
+                }
+                o[lane] = at;
             }
         }
+        if (out) *cluster.map_shared_rank(&leaves, 0) = 1;
         // all runs written (and seen by the whole cluster) before the first step reads them
         __threadfence();
         cluster.sync();
@@ -838,29 +850,59 @@ diffuse_kernel(const int64_t *graph_ptr, const uint32_t *graph_id, const int64_t
     } else {
         for (int64_t i = threadIdx.x; i < n64; i += DF_T) res[i * NRAND] = noise_sign((uint32_t)i, ch, id, k0, k1);
     }
-    // which graphs walk_rest_kernel has to take (X is free again)
-    if (ch == 0 && threadIdx.x == 0 && n64 > 0) X[v0 * FIN] = fits ? 0.f : 1.f;
+    // what walk_rest_kernel has to take (X is free again): 1 = this graph, 2 = the whole batch, since a column
+    // leads from this graph to another (written above before the cluster's barriers)
+    if (ch == 0 && threadIdx.x == 0 && n64 > 0) {
+        X[v0 * FIN] = !fits ? 1.f : (leaves ? 2.f : 0.f);
+        X[v0 * FIN + 1] = 0.f;                                         // walk_rest_kernel's own mark
+    }
 }
 
 // The walk steps of the graphs that diffuse_kernel marked, whose noise it left in R0: one cooperative
 // launch, a warp per row as in aggregate_vec_kernel<8>, a grid barrier per step.  Without marked
 // graphs it returns at once.  (One launch per step over all vertices would cost every batch `steps`
-// launches for the rare graph that does not fit.)
-__global__ void __launch_bounds__(256) walk_rest_kernel(int64_t N, int G, const int64_t *graph_ptr, const int64_t *row_ptr,
-                                                        const int32_t *col, int steps, const float *X, float *R0, float *R1)
+// launches for the rare graph that does not fit.)  A batch in which a column leads from one graph to another
+// walks as a whole, from the noise on: every vertex's value is then read at its own step.
+__global__ void __launch_bounds__(256) walk_rest_kernel(int64_t N, int G, const int64_t *graph_ptr, const uint32_t *graph_id,
+                                                        const int64_t *row_ptr, const int32_t *col, uint32_t k0, uint32_t k1,
+                                                        int steps, float *X, float *R0, float *R1)
 {
-    int any = 0;
-    for (int g = threadIdx.x; g < G; g += 256)
-        any |= graph_ptr[g + 1] > graph_ptr[g] && X[graph_ptr[g] * FIN] != 0.f;
-    if (!__syncthreads_or(any)) return;
+    // a mark of any graph: word 0 (diffuse_kernel's) at least v, or word 1 (set below)
+    auto marked = [&](float v) {
+        int any = 0;
+        for (int g = threadIdx.x; g < G; g += 256) {
+            if (graph_ptr[g + 1] <= graph_ptr[g]) continue;
+            const float *m = X + graph_ptr[g] * FIN;
+            any |= m[0] >= v || m[1] != 0.f;
+        }
+        return __syncthreads_or(any) != 0;
+    };
+    if (!marked(1.f)) return;
     cooperative_groups::grid_group grid = cooperative_groups::this_grid();
     const int lane = threadIdx.x & 31, sub = lane >> 1, c4 = lane & 1;
     const int64_t wglob = ((int64_t)blockIdx.x * 256 + threadIdx.x) >> 5, nw = ((int64_t)gridDim.x * 256) >> 5;
     float4 *in = reinterpret_cast<float4 *>(R0), *out = reinterpret_cast<float4 *>(R1);
+    // diffuse_kernel has looked at the columns of the graphs that fit it; here the others'
+    for (int64_t i = wglob; i < N; i += nw) {
+        const int64_t g = graph_of(graph_ptr, G, i), v0 = graph_ptr[g], v1 = graph_ptr[g + 1];
+        if (X[v0 * FIN] != 1.f) continue;
+        for (int64_t e = row_ptr[i] + lane; e < row_ptr[i + 1]; e += 32)
+            if (col[e] < v0 || col[e] >= v1) X[v0 * FIN + 1] = 1.f;
+    }
+    grid.sync();
+    const bool all = marked(2.f);
+    if (all) {
+        for (int64_t t = (int64_t)blockIdx.x * 256 + threadIdx.x; t < N * NRAND; t += (int64_t)gridDim.x * 256) {
+            const int64_t i = t / NRAND;
+            const int g = (int)graph_of(graph_ptr, G, i);
+            R0[t] = noise_sign((uint32_t)(i - graph_ptr[g]), (int)(t % NRAND), graph_id[g], k0, k1);
+        }
+        grid.sync();
+    }
     // the last round copies the result back to R0 when it ended in R1
     for (int s = 0; s < steps + (steps & 1); ++s) {
         for (int64_t i = wglob; i < N; i += nw) {
-            if (X[graph_ptr[graph_of(graph_ptr, G, i)] * FIN] == 0.f) continue;
+            if (!all && X[graph_ptr[graph_of(graph_ptr, G, i)] * FIN] == 0.f) continue;
             if (s == steps) {
                 if (lane < 2) out[i * 2 + lane] = in[i * 2 + lane];
                 continue;
@@ -1067,7 +1109,8 @@ int gdi_mpnn_features(int64_t N, int32_t G, const int64_t *graph_ptr, const uint
             return GDI_ERR_CUDA;
         diffuse_kernel<<<G * DF_CL, DF_T, smem, st>>>(graph_ptr, graph_id, row_ptr, col, (uint32_t)seed,
                                                       (uint32_t)(seed >> 32), steps, DF_CAP, X, R0, R1);
-        void *args[] = {&N, &G, &graph_ptr, &row_ptr, &col, &steps, &X, &R0, &R1};
+        uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32);
+        void *args[] = {&N, &G, &graph_ptr, &graph_id, &row_ptr, &col, &k0, &k1, &steps, &X, &R0, &R1};
         if (cudaLaunchCooperativeKernel((const void *)walk_rest_kernel, dim3(152 * 4), dim3(256), args, 0, st) != cudaSuccess)
             return GDI_ERR_CUDA;
     } else {

@@ -270,3 +270,28 @@ def test_features_one_launch_and_the_rest(gdi, steps):
                 continue                       # one vertex: centred to 0, scaled by 1e-12
             s = slice(gp[q], gp[q + 1])
             assert np.max(np.abs(X[s] - Xr[s])) < 1e-4, (q, np.max(np.abs(X[s] - Xr[s])))
+
+
+@pytest.mark.parametrize("steps", [1, 4, 5])
+@pytest.mark.parametrize("cut", [(0, 700, 1999, 2000), (0, 300, 300, 1500, 2000), (0, 9400, 9600), (0, 200, 9600)])
+def test_features_of_graphs_with_columns_between_them(gdi, cut, steps):
+    """graph_ptr cuts connected graphs, so columns lead from one to another: walked as one graph, as the
+    definition says, with every piece small (an empty and a one-vertex one among them) and with one too large
+    for a block.  Float32 sums of at most some 2,000 terms, scaled to unit RMS: 1e-4."""
+    import ctypes as C
+    import torch
+    from paper_1908_00210_gb300 import learn
+    g = _ring_graph(cut[-1], 4 * cut[-1], len(cut))
+    gp = np.array(cut, dtype=np.int64)
+    ids = np.arange(9, 9 + len(cut) - 1, dtype=np.uint32)
+    dev = [torch.from_numpy(a).cuda() for a in (gp, ids.view(np.int32), g.row_ptr, g.col)]
+    X, scratch = torch.empty(g.n, 16, device="cuda"), torch.empty(16 * g.n, device="cuda")
+    for _ in range(2):
+        rc = learn.lib().gdi_mpnn_features(g.n, len(ids), *[a.data_ptr() for a in dev], 77, steps, 0, X.data_ptr(),
+                                           scratch.data_ptr(), C.c_void_p(torch.cuda.current_stream().cuda_stream))
+        assert rc == 0
+        Xr = ref.features(gp, ids, g.row_ptr, g.col, 77, steps)
+        got = X.cpu().numpy()
+        for a, b in zip(gp[:-1], gp[1:]):
+            if b - a > 1:                  # (one vertex: centred to 0, scaled by 1e-12)
+                assert np.max(np.abs(got[a:b] - Xr[a:b])) < 1e-4, (a, b)
