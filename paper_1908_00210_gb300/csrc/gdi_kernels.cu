@@ -888,28 +888,34 @@ struct SortedCta {
     uint16_t *cbuf;     // [cta_stage] their columns
 };
 
-// windows of one block whose stage maps are kept (a class with more is replayed in order)
+// Windows of one block whose stage maps are kept.  A class of more than so many for each of its blocks is
+// taken in pieces of that size, one after another like classes: its vertices share no edge, so a piece's
+// thresholds do not see the flips of the pieces before it, and only G passes on.  (One warp that replayed such a
+// class window by window took 0.47 us a window.  A sweep of 40 replicas of 3,000 vertices, W = 1: 1,399 -> 314 us;
+// 300 of a 100 x 100 torus, W = 32: 257 -> 118.)
 constexpr int CTA_WALK_MAX = 128;
+__host__ __device__ inline int32_t cta_piece(int W, int cl) { return CTA_WALK_MAX * cl * W; }
 
-// windows a block of a cluster of cl (1: alone) has of the largest class: a class of one or two windows
-// is the first block's
+// windows a block of a cluster of cl (1: alone) has of the largest piece: one or two windows are the first
+// block's
 __host__ __device__ inline int cta_own_windows(int32_t max_class, int W, int cl)
 {
-    const int nw = (max_class + W - 1) / W;
+    const int all = (max_class + W - 1) / W, nw = all < CTA_WALK_MAX * cl ? all : CTA_WALK_MAX * cl;
     return cl > 1 ? ((nw + cl - 1) / cl > 2 ? (nw + cl - 1) / cl : 2) : nw;
 }
 
-__host__ __device__ inline int cta_walk_windows(int32_t max_class, int W, int cl)
+// its ranks
+__host__ __device__ inline int32_t cta_own_ranks(int32_t max_class, int W, int cl)
 {
-    const int nw = cta_own_windows(max_class, W, cl);
-    return nw < CTA_WALK_MAX ? nw : CTA_WALK_MAX;
+    const int32_t own = cta_own_windows(max_class, W, cl) * W;
+    return own < max_class ? own : max_class;
 }
 
 // warps that count windows at once where the windows have no bins of their own: none where no class has
 // three windows; their bins share the repair flags' bytes, and a small instance has room for 16
 __host__ __device__ inline int cta_count_warps(int32_t max_n, int32_t max_class, int W, int BS, int cl)
 {
-    const int nwm = cta_walk_windows(max_class, W, cl);
+    const int nwm = cta_own_windows(max_class, W, cl);
     const int fit = max_n / 1024 > 16 ? max_n / 1024 : 16;
     const int nw = nwm < BS / 32 ? nwm : BS / 32;
     return (max_class + W - 1) / W < 3 ? 0 : (nw < fit ? nw : fit);
@@ -927,8 +933,7 @@ __host__ __device__ inline CtaSortedLayout cta_sorted_layout(const GdiDevProblem
                                                              int32_t stage, int32_t rofs, int nbw, int cl)
 {
     CtaSortedLayout L;
-    const size_t own = cl > 1 ? (size_t)cta_own_windows(P.max_class, P.W, cl) * P.W : (size_t)P.max_class;
-    const size_t mc = own + 8;
+    const size_t mc = (size_t)cta_own_ranks(P.max_class, P.W, cl) + 8;
     size_t o = 0;
     L.red64 = o; o = align16c(o + sizeof(int64_t) * (BS / 32 + 2));
     L.red32 = o; o = align16c(o + sizeof(int32_t) * (BS / 32 + 2));
@@ -944,7 +949,7 @@ __host__ __device__ inline CtaSortedLayout cta_sorted_layout(const GdiDevProblem
     L.gam = o; o = align16c(o + 4 * mc);
     L.es = o; o = align16c(o + 4 * mc);
     L.s0 = o; o = align16c(o + mc);
-    const int nwm = cta_walk_windows(P.max_class, P.W, cl);
+    const int nwm = cta_own_windows(P.max_class, P.W, cl);
     L.wmaps = o; o = align16c(o + sizeof(StageMap) * 2 * (size_t)nwm);
     L.wtab = o; o = align16c(o + (size_t)NT * nwm);
     L.rofs = o; o = align16c(o + (stage ? 4 * (mc > (size_t)rofs ? mc : (size_t)rofs) : 0));
@@ -1045,7 +1050,15 @@ __global__ void __launch_bounds__(BS, 1024 / BS) gdi_cta_sorted_kernel(GdiDevPro
         const int64_t base = P.node_off[q];
         const int32_t n = (int32_t)(P.node_off[q + 1] - base);
         const int32_t *cls = P.class_ptr + P.class_off[q];
-        const int32_t ncls = P.class_off[q + 1] - P.class_off[q] - 1;
+        // the item's classes, or the pieces of all of them (both "class" below)
+        const int32_t piece = cta_piece(W, (int)CL);
+        const bool pieces = P.max_class > piece;
+        int32_t ncls = P.class_off[q + 1] - P.class_off[q] - 1;
+        if (pieces) {
+            int32_t np = 0;
+            for (int c = 0; c < ncls; ++c) np += (cls[c + 1] - cls[c] + piece - 1) / piece;
+            ncls = np;
+        }
         int8_t *gsig = R.spins + (int64_t)rep * P.N + base;
         const int64_t row0 = P.row_ptr[base];
         const int64_t nnz_item = P.row_ptr[base + n] - row0;
@@ -1053,12 +1066,23 @@ __global__ void __launch_bounds__(BS, 1024 / BS) gdi_cta_sorted_kernel(GdiDevPro
 
         auto make_span = [&](int c) {
             Span s;
-            s.clo = cls[c];
-            s.chi = cls[c + 1];
+            int32_t at = 0;                          // ranks of the class before this piece
+            if (pieces) {
+                int cc = 0;
+                for (;; ++cc) {
+                    const int32_t np = (cls[cc + 1] - cls[cc] + piece - 1) / piece;
+                    if (c < np) break;
+                    c -= np;
+                }
+                at = c * piece;
+                c = cc;
+            }
+            s.clo = cls[c] + at;
+            s.chi = pieces ? min(s.clo + piece, cls[c + 1]) : cls[c + 1];
             const int32_t size = s.chi - s.clo;
             s.nwin = (size + W - 1) / W;
             s.kq = CLUS ? (s.nwin + (int)CL - 1) / (int)CL : s.nwin;
-            s.walk = s.nwin >= 3 && s.kq <= CTA_WALK_MAX;
+            s.walk = s.nwin >= 3;
             if (!s.walk) s.kq = s.nwin;
             s.kb = min((int)crank * s.kq, s.nwin);
             s.nk = min(s.kq, s.nwin - s.kb);
@@ -1399,9 +1423,7 @@ inline bool cta_sorted(const GdiDevProblem &P, const GdiDevRun &R, int BS)
 }
 
 // Blocks per item (a cluster of 1, 2, 4 or 8, at most `most`): as many as leave every item its own SMs and four
-// windows of the largest class to each block.  A block's share of the largest class has to stay within the
-// windows whose maps are kept: cta_sorted_layout sizes a cluster's class buffers for the shares, and a class
-// beyond that would be the first block's alone.
+// windows of the largest class to each block.
 inline int cta_cluster(const GdiDevProblem &P, const GdiDevRun &R, int BS, int most)
 {
     if (!cta_sorted(P, R, BS)) return 1;
@@ -1412,7 +1434,7 @@ inline int cta_cluster(const GdiDevProblem &P, const GdiDevRun &R, int BS, int m
     const int64_t nw = (P.max_class + P.W - 1) / P.W;
     int cl = 1;
     while (2 * cl <= std::min(most, 8) && 2 * cl * items <= sms && 4 * 2 * cl <= nw) cl *= 2;
-    return nw <= (int64_t)cl * CTA_WALK_MAX ? cl : 1;
+    return cl;
 }
 
 // shared memory of the kernel that takes this call (counted windows, else whole-block windows)
@@ -1587,8 +1609,7 @@ int gdi_cta_default_block(const GdiDevProblem &P, const GdiDevRun &R)
     if (items > 3LL * sms) return 256;
     const int cl = cta_cluster(P, R, 512, 8);
     if (items * cl <= sms && cta_sorted(P, R, 512)) {
-        const int64_t own = cl > 1 ? (int64_t)cta_own_windows(P.max_class, P.W, cl) * P.W : P.max_class;
-        if (own > 800) return 1024;
+        if (cta_own_ranks(P.max_class, P.W, cl) > 800) return 1024;
         if (P.max_class < 128) return 256;
     }
     return 512;

@@ -268,3 +268,44 @@ def test_cta_cluster_capped_by_grid_limit(gdi, W, grid_limit):
     assert launch["grid"] <= grid_limit
     ref = oracle.anneal(g, A=1, B=4, W=W, t0=12.0, t1=0.2, sweeps=5, seed=13, replicas=2, trace=True)
     assert_parity(res, spins, tr, ref)
+
+
+@pytest.mark.parametrize("n,W,replicas", [(3000, 1, 160), (3000, 5, 160), (12000, 2, 1), (9000, 1, 19), (2500, 1, 400)])
+def test_cta_classes_in_pieces(gdi, n, W, replicas):
+    """Classes of more than 128 windows a block, alone (160 and 400 items) and in clusters of two to eight, with
+    pieces that end inside a class: bit-exact after every sweep."""
+    g = barabasi_albert(n, 5, 93)
+    sch = gdi.Schedule(sweeps=4, t0=12.0, t1=0.2)
+    ann = gdi.Annealer(g, A=1, B=4, W=W, replicas=replicas)
+    ann.configure(path=gdi.GDI_PATH_CTA)
+    ann.anneal(sch, 17, flags=gdi.GDI_FLAG_TRACE)
+    res, spins, tr = ann.results(), ann.spins(), ann.trace()
+    blocks = ann.last_launch()["grid"]
+    ann.close()
+    most = gdi.rank_space(g).max_class
+    assert most > 128 * W * max(1, min(8, blocks // replicas))
+    ref = oracle.anneal(g, A=1, B=4, W=W, t0=12.0, t1=0.2, sweeps=4, seed=17, replicas=replicas, trace=True)
+    assert_parity(res, spins, tr, ref)
+
+
+def sweep_us(gdi, ann, sweeps=20):
+    """Device time of a sweep, the least of five anneals."""
+    sch = gdi.Schedule(sweeps=sweeps, t0=12.0, t1=0.2)
+    ms = []
+    for _ in range(5):
+        ann.anneal(sch, 3)
+        ms.append(ann.kernel_ms()[0])
+    return 1e3 * min(ms) / sweeps
+
+
+def test_cta_small_windows_cost_no_more_than_their_number(gdi):
+    """40 replicas of 3,000 vertices: W = 1 has 32 times the windows of W = 32, most of whose time is not the
+    windows'.  It took 8 times as long (and 33 times when one warp replayed the windows of a large class)."""
+    g = barabasi_albert(3000, 5, 3000)
+    us = {}
+    for W in (1, 32):
+        ann = gdi.Annealer(g, A=1, B=4, W=W, replicas=40)
+        ann.configure(path=gdi.GDI_PATH_CTA)
+        us[W] = sweep_us(gdi, ann)
+        ann.close()
+    assert us[1] < 16 * us[32], us
