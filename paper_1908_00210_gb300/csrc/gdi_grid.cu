@@ -97,7 +97,7 @@ struct GridArgs {
     const int32_t *wbnd;    // [classes][blocks + 1] first window of every block, or null (even split)
     unsigned long long *hf; // maintained fields (X.hfield) when this kernel keeps them, else null
     bool es_pre;            // counted path: E* of the next class drawn ahead into shared memory
-    bool tables;            // counted path: window maps composed as tables, windows replayed by all warps
+    bool tables;            // counted path: window maps composed as tables
     bool binned;            // counted path: thresholds counted into their window's bins as they are made
 };
 
@@ -910,8 +910,10 @@ __global__ void __launch_bounds__(GB, 1) gdi_grid_anneal_kernel(GridArgs A)
 // composes the run's tables into a run table.  Every block then fetches the run tables before it
 // and the block tables of its own run (one poll of all of them per round trip) and looks its exact
 // entering G up from c: at most 160 / 16 + 15 byte lookups, without a grid barrier.  It looks the entering point of each of its own
-// windows up the same way, and all warps replay the windows at once: K from the stage maps, the cut from
-// the prefix counts, one pass over the members.  Where the walk leaves the lattice, the block whose table
+// windows up the same way (where their tables do not fit shared memory, through the stage maps), and all warps replay
+// the windows at once: K from the stage maps, the cut from the prefix counts, one pass over the members.  One warp
+// replaying them in order, which blocks without tables did, took 1,583 us a sweep of 300,000 vertices at W = 1; 854
+// now (1,108 when windows were sorted).  Where the walk leaves the lattice, the block whose table
 // failed publishes its exact outgoing G (it knows its own entering G and replays exactly), and the walk continues from it.
 // One grid barrier per class remains: the next class reads this class's spins.
 constexpr int SMAXW = 256;              // windows a warp holds in registers
@@ -923,7 +925,7 @@ __host__ __device__ inline int walk_slots(int P) { return nruns(P) + 2 * RUN; }
 
 
 struct SortedLayout {
-    size_t off_h, off_gam, off_es, off_s0, off_fm, off_fbits, off_longq, off_smap, off_wtab, off_tin, off_walk, off_row, off_bins, off_misc, total;
+    size_t off_h, off_gam, off_es, off_s0, off_fm, off_fbits, off_longq, off_smap, off_wtab, off_walk, off_row, off_bins, off_misc, total;
     int fw;                             // words of one replica's flip bitmap
     int cw;                             // warps that count windows
     int gs;                             // threshold row stride (ints): >= spc + 7, 4 mod 32
@@ -940,7 +942,8 @@ __host__ __device__ inline SortedLayout sorted_layout(int spc, int wpc, int max_
 {
     SortedLayout L;
     size_t o = 0;
-    L.off_h = o; o = align16(o + (size_t)spc * 8 * sizeof(int16_t));      // fields
+    // the fields; once the thresholds are made, the entering lattice index of each (window, replica), or -1
+    L.off_h = o; o = align16(o + (size_t)spc * 8 * sizeof(int16_t));
     // thresholds [r][gs]: a row starts 4 words (16 banks' worth of bytes) after the previous
     // one's bank, so the 8 replicas' 16-byte stores of one quad of ranks hit disjoint banks
     L.gs = ((spc + 3 + 31) & ~31) + 4;
@@ -955,7 +958,6 @@ __host__ __device__ inline SortedLayout sorted_layout(int spc, int wpc, int max_
     L.off_longq = o; o = align16(o + (size_t)2 * spc * sizeof(int32_t));   // long rows, chunk counts
     L.off_smap = o; o = align16(o + (size_t)wpc * 8 * 2 * sizeof(StageMap));
     L.off_wtab = o; o = align16(o + (tables ? (size_t)wpc * 8 * NT : 0));   // both maps of a window composed
-    L.off_tin = o; o = align16(o + (tables ? (size_t)wpc * 8 : 0));         // its entering lattice index, or -1
     // the walk's tables and, before it, the counting warps' bins: all warps count where anything beyond the
     // necessary is kept, else as many as the tables' bytes hold
     const size_t wk = (size_t)8 * walk_slots(P) * NT, wbin = WBINS * sizeof(uint32_t);
@@ -1116,7 +1118,7 @@ __global__ void __launch_bounds__(GB, 1) gdi_grid_sorted_kernel(GridArgs A)
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int spc = A.spc;
     const SortedLayout L = sorted_layout(spc, A.wpc, R.max_row, Pb, A.es_pre, A.tables, A.binned);
-    int16_t *hb = reinterpret_cast<int16_t *>(smem_raw + L.off_h);   // fields [i*8 + r]
+    int16_t *hb = reinterpret_cast<int16_t *>(smem_raw + L.off_h);   // fields [i*8 + r], until the thresholds are made
     int32_t *gam = reinterpret_cast<int32_t *>(smem_raw + L.off_gam);
     int16_t *esb = reinterpret_cast<int16_t *>(smem_raw + L.off_es);   // E* drawn ahead [r][L.es]
     uint8_t *s0 = smem_raw + L.off_s0;
@@ -1124,7 +1126,7 @@ __global__ void __launch_bounds__(GB, 1) gdi_grid_sorted_kernel(GridArgs A)
     uint32_t *hist = reinterpret_cast<uint32_t *>(smem_raw + L.off_walk);   // counting warps' bins
     int8_t *walk = reinterpret_cast<int8_t *>(smem_raw + L.off_walk);
     int8_t *wtab = reinterpret_cast<int8_t *>(smem_raw + L.off_wtab);   // [window][replica][NT]
-    int8_t *tin = reinterpret_cast<int8_t *>(smem_raw + L.off_tin);     // [window][replica]
+    int8_t *tin = reinterpret_cast<int8_t *>(smem_raw + L.off_h);       // [window][replica], on the fields' bytes
     uint32_t *gbins = reinterpret_cast<uint32_t *>(smem_raw + L.off_bins);   // [window][replica][GBINS]
     const int w_shift = (P.W & (P.W - 1)) == 0 ? __ffs(P.W) - 1 : -1;
     uint32_t *fbits = reinterpret_cast<uint32_t *>(smem_raw + L.off_fbits);   // [r][fw] fast-path flips
@@ -1251,6 +1253,7 @@ __global__ void __launch_bounds__(GB, 1) gdi_grid_sorted_kernel(GridArgs A)
             for (int i = threadIdx.x; i < 8 * L.fw; i += GB) fbits[i] = 0;
             if (threadIdx.x == 0) npush = 0;
             __syncthreads();
+            const bool spread = nwin > 1;                // more than one window: replayed by all warps
             // ---- block table per replica: lanes hold lattice points lane and lane + 32
             int t0 = lane, t1 = lane + 32;
             if (warp < nrep) {
@@ -1356,21 +1359,31 @@ __global__ void __launch_bounds__(GB, 1) gdi_grid_sorted_kernel(GridArgs A)
                 }
                 for (; kb < nown && ok; ++kb) block_step(ws_own + kb * NT, run0 + kb);
                 ok = __all_sync(0xFFFFFFFFu, ok);
-                // ---- my windows: looked up from the entering point on, replayed by all warps below; from the
-                // first that leaves the lattice on, replayed here in order from the exact G
-                for (int kk = lane; kk < nwin && A.tables; kk += 32) tin[kk * 8 + r] = -1;
+                // ---- my windows: looked up from the entering point on (without tables: followed through the
+                // stage maps, a tenth of a replay each), replayed by all warps below; from the first that leaves
+                // the lattice on, and a window that is alone, replayed here in order from the exact G
+                for (int kk = lane; kk < nwin && spread; kk += 32) tin[kk * 8 + r] = -1;
                 __syncwarp();
                 if (ok) {
                     const int own = __shfl_sync(0xFFFFFFFFu, (idx >= 0 && idx < 32) ? t0 : t1, idx & 31);
                     const bool need_exact = idx < 0 || own < 0;
                     int kk = 0;
-                    if (A.tables && idx >= 0)
+                    if (spread && idx >= 0 && A.tables) {
                         for (; kk < nwin; ++kk) {
                             const int nx = wtab[(size_t)(kk * 8 + r) * NT + idx];
                             if (nx < 0) break;
                             if (lane == 0) tin[kk * 8 + r] = (int8_t)idx;
                             idx = nx;
                         }
+                    } else if (spread && idx >= 0) {
+                        for (; kk < nwin; ++kk) {
+                            const StageMap *o = smap + ((size_t)kk * 8 + r) * 2;
+                            const int nx = stage_apply(o[plus_first ? 1 : 0], stage_apply(o[plus_first ? 0 : 1], idx));
+                            if (nx < 0) break;
+                            if (lane == 0) tin[kk * 8 + r] = (int8_t)idx;
+                            idx = nx;
+                        }
+                    }
                     int32_t gout = idx >= 0 ? c0 - NT + 2 * idx : gx;
                     uint32_t *fb = fbits + (size_t)r * L.fw;
                     const int32_t *gr = gamc + (size_t)r * L.gs;
@@ -1409,7 +1422,7 @@ __global__ void __launch_bounds__(GB, 1) gdi_grid_sorted_kernel(GridArgs A)
             have_es = A.es_pre && (c + 1 < ncls || sw + 1 < R.s_end);
             __syncthreads();
             // ---- the windows entered on the lattice, replayed at once
-            for (int task = warp; task < nwin * nrep && A.tables; task += NWARP) {
+            for (int task = warp; task < nwin * nrep && spread; task += NWARP) {
                 const int kk = task / nrep, r = task % nrep;
                 const int ti = tin[kk * 8 + r];
                 if (ti < 0) continue;
@@ -1421,7 +1434,7 @@ __global__ void __launch_bounds__(GB, 1) gdi_grid_sorted_kernel(GridArgs A)
                 grid_replay<SL>(gamc + (size_t)r * L.gs, s0, r, ws, we, Gc[r] + 2 * ti - NT, plus_first, K1, K2, wc,
                                 fbits + (size_t)r * L.fw, W);
             }
-            __syncthreads();
+            if (spread) __syncthreads();
             // ---- write the flips; with maintained fields, push their field changes to the
             // neighbours: a warp takes 32 consecutive ranks and walks the concatenated rows of its
             // flipping ones lane by lane (rows longer than LONG_ROW go to a block queue instead)

@@ -125,3 +125,30 @@ def test_bounded_waits_report_timeout_and_context_recovers(gdi):
     ref = oracle.anneal(g, A=1, B=4, W=64, t0=12.0, t1=0.2, sweeps=6, seed=3, replicas=2)
     assert np.array_equal(spins, ref.spins)
     assert np.array_equal(res["final_cut"][0], ref.final_cut)
+
+
+@pytest.mark.parametrize("W,blocks", [(1, 8), (2, 3), (4, 2), (64, 1), (300, 1), (16, 2)])
+@pytest.mark.parametrize("start", ["random", "one-sided"])
+def test_grid_windows_without_tables(gdi, W, blocks, start):
+    """So many windows a block that their tables (the last: their bins) do not fit shared memory: followed through
+    the stage maps and replayed by all warps, bit-exact; from the one-sided start in order from the exact G."""
+    g = barabasi_albert(12000, 5, 61)
+    init = np.ones((3, g.n), dtype=np.int8) if start == "one-sided" else None
+    grid_vs_oracle(gdi, g, W=W, sweeps=4, replicas=3, grid_limit=blocks, init=init)
+
+
+def test_grid_small_windows_replayed_by_all_warps(gdi):
+    """One replica of 300,000 vertices at W = 1, where a block's windows have no tables, against W = 4, where they
+    have: 5 times as long (and 9 times when one warp replayed the windows)."""
+    g = barabasi_albert(300_000, 5, 62)
+    us = {}
+    for W in (1, 4):
+        ann = gdi.Annealer(g, A=1, B=4, W=W, replicas=1)
+        ann.configure(path=gdi.GDI_PATH_GRID)
+        ms = []
+        for _ in range(5):
+            ann.anneal(gdi.Schedule(sweeps=10, t0=12.0, t1=0.2), 7)
+            ms.append(ann.kernel_ms()[0])
+        us[W] = 1e3 * min(ms)
+        ann.close()
+    assert us[1] < 7 * us[4], us
