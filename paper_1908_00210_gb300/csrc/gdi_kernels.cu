@@ -1598,8 +1598,10 @@ int cta_occupancy(const GdiDevProblem &P, const GdiDevRun &R0, int *per_sm)
 // 1024: 8 replicas of 1500 vertices, W = 64: 32.0 / 27.8 / 31.8; whole-class windows 7.4 / 6.9 / 8.6), 1024
 // where a block's share of the largest class passes 800 ranks (BA 20,000 on one cluster: 19.4 / 15.1 /
 // 13.9; 64 replicas of a 100 x 100 torus: 26.2 / 15.8 / 10.8), 256 where no class reaches 128 (ER-800: 42.7 /
-// 44.1 / 51.7: barriers, not work).  Three items an SM still gain from 512 (400 ER instances: 15.6 / 15.0 /
-// 25.3); more take 256 (1024 short anneals: 4.4 / 6.0 / 10.2).
+// 44.1 / 51.7: barriers, not work).  Two blocks of 512 fit an SM: of items of one size a third on the SM would wait
+// for a wave as long as the first (400 replicas of 64, 1,000 and 2,000 vertices, W = 64, us a sweep 15.5 / 28.9, 32.4 /
+// 50.1, 51.4 / 60.8 at 256 / 512), while among unequal ones, the largest first, it fills in behind small ones (400 ER
+// instances: 15.6 / 15.0 / 25.3 ms); more than three take 256 (1024 short anneals: 4.4 / 6.0 / 10.2).
 int gdi_cta_default_block(const GdiDevProblem &P, const GdiDevRun &R)
 {
     int dev = 0, sms = 0;
@@ -1607,6 +1609,7 @@ int gdi_cta_default_block(const GdiDevProblem &P, const GdiDevRun &R)
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int64_t items = (int64_t)P.num_instances * P.replicas;
     if (items > 3LL * sms) return 256;
+    if (items > 2LL * sms && 4 * P.N >= 3LL * P.max_n * P.num_instances) return 256;
     const int cl = cta_cluster(P, R, 512, 8);
     if (items * cl <= sms && cta_sorted(P, R, 512)) {
         if (cta_own_ranks(P.max_class, P.W, cl) > 800) return 1024;

@@ -309,3 +309,15 @@ def test_cta_small_windows_cost_no_more_than_their_number(gdi):
         us[W] = sweep_us(gdi, ann)
         ann.close()
     assert us[1] < 16 * us[32], us
+
+
+@pytest.mark.parametrize("n,W", [(64, 64), (1000, 64), (300, 0)])
+def test_cta_third_block_of_an_sm_needs_no_second_wave(gdi, n, W):
+    """400 equal items, three to an SM, take about as long as 300, not twice as long."""
+    g = barabasi_albert(n, 5, n)
+    us = {}
+    for replicas in (300, 400):
+        ann = gdi.Annealer(g, A=1, B=4, W=W, replicas=replicas)
+        us[replicas] = sweep_us(gdi, ann)
+        ann.close()
+    assert us[400] < 1.35 * us[300], us
