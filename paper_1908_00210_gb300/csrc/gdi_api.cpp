@@ -741,10 +741,10 @@ int gdi_anneal(gdi_ctx *c, const gdi_schedule *S, const gdi_run *run)
 
     int max_optin = 0, sms = 0;
     cudaDeviceGetAttribute(&max_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device);
-    int block = c->block ? c->block : gdi_cta_default_block(P, R);
+    int block = c->block ? c->block : gdi_cta_default_block(P, R, c->grid_limit);
     size_t need = 0;
-    gdi_cta_smem_bytes(P, R, block, &need);
-    if (!c->block && need > (size_t)max_optin) gdi_cta_smem_bytes(P, R, block = 256, &need);
+    gdi_cta_smem_bytes(P, R, block, c->grid_limit, &need);
+    if (!c->block && need > (size_t)max_optin) gdi_cta_smem_bytes(P, R, block = 256, c->grid_limit, &need);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
     bool grid = false;
     if ((run->flags & GDI_FLAG_STANDARD) && ((run->flags & GDI_FLAG_RACY) || c->path == GDI_PATH_GRID))
@@ -752,31 +752,46 @@ int gdi_anneal(gdi_ctx *c, const gdi_schedule *S, const gdi_run *run)
     if (c->path == GDI_PATH_GRID || (run->flags & GDI_FLAG_RACY)) grid = true;
     else if (run->flags & GDI_FLAG_STANDARD) grid = false;
     else if (c->path == GDI_PATH_AUTO && c->Q == 1 && c->W >= 1 && c->max_degree <= 32767) {
-        // one instance: the cheaper path by a cost model fitted on GB300 (BA graphs, m = 5, of
-        // 2*10^3 to 6.4*10^4 vertices; ER graphs of 800 vertices at mean degree 49 and 1.6*10^4 at
-        // 10; 1 to 152 replicas; 100 sweeps).  Per sweep, a CTA-resident block costs about 2 us
-        // per colour class + 1.8 ns (blocks of 128 or 256 threads) or 1.2 ns (512, 1024) per
-        // (vertex + directed edge), per wave of resident blocks; a grid-scale launch costs about
-        // 13 us per colour class (thresholds, counts, chain and barrier) + 0.02 ns per (vertex +
-        // edge), per group of 8 replicas.  A cluster of blocks per replica costs about 5.5 us a
-        // class (9 with windows above 128) + 0.55 ns per (vertex + edge) of a block's share; the
-        // figures behind it (ms, cluster against grid): one replica of BA 20,000 and 30,000 at
-        // W = 64 13.9 / 21.4 and 5.3 / 7.5, 8 of 8,000 11.2 / 25.7, 3 of 30,000 at W = 256 7.3 / 8.3.
-        // The model is good to about a fifth, so the cluster has to win by that much.
-        int per_sm = 0;
-        if (need > (size_t)max_optin || gdi_cta_blocks_per_sm(P, R, block, &per_sm) != 0 || per_sm < 1) {
+        // One instance: the cheaper path by a cost model fitted on GB300 (least squares of the relative error over
+        // 380 pairs of both paths: BA, ER and torus graphs of 800 to 32,000 vertices, mean degree 4 to 200, W = 1 to
+        // 256, 1 to 100 replicas, 20 to 30 sweeps, and with 1 to 76 blocks).  Per sweep, in microseconds:
+        //   CTA path, per wave of resident items: 2.1 a colour class (0.5 more with windows above 128) + 2.4e-3 a
+        //   vertex, 0.16e-3 a directed edge and 0.2 a window; in a cluster 4.5 a class + 0.19e-3 a vertex and
+        //   edge and 0.22 a window of a block's share;
+        //   grid path, per group of up to 8 replicas: 12.1 a class + 0.41 a class and further replica + 0.42e-3 a
+        //   vertex and edge, 0.05e-3 more and 0.105 a window for each replica, of a block's share.
+        // (us a sweep, CTA / grid: BA 20,000, one replica, W = 64 57 / 76, W = 4 187 / 81, W = 1 566 / 95; 8 on 4
+        // blocks, W = 64 601 / 212; ER 3,000 of mean degree 200, W = 64 196 / 557.)
+        // Clusters with windows above 128, whose cost scatters most, keep the older and more careful estimate: 9 a
+        // class + 0.55e-3 a vertex and edge, which has to undercut the grid path's 13 and 0.02e-3 by a fifth.
+        // Without 16-bit columns nothing is staged, and the whole-block kernel sums its rows more slowly: 2 a class
+        // and 1.2e-3 (1.8e-3 with blocks of 128 or 256) a vertex and edge.
+        GdiCtaPlan plan;
+        int spc, wpc;
+        size_t grid_need;
+        bool counted;
+        const int nblk = c->grid_limit > 0 ? std::min(c->grid_limit, sms) : sms;
+        if (need > (size_t)max_optin || gdi_cta_plan(P, R, block, c->grid_limit, &plan) != 0 || plan.at_once < 1) {
             grid = true;
-        } else {
-            const double work = (double)c->N + (double)c->nnz;
-            const double ncls = (double)c->num_classes[0];
-            const int64_t slots = (int64_t)sms * per_sm;
-            const double per_work = block >= 512 ? 1.2e-9 : 1.8e-9;
-            const double cta_s = (double)((c->R + slots - 1) / slots) * (2e-6 * ncls + per_work * work);
-            const double grid_s = (double)((c->R + 7) / 8) * (13e-6 * ncls + 0.02e-9 * work);
-            grid = grid_s < cta_s;
-            const int cl = gdi_cta_cluster_size(P, R, block);
-            if (cl > 1 && P.col16)
-                grid = 0.8 * grid_s < (c->W > 128 ? 9e-6 : 5.5e-6) * ncls + 0.55e-9 * work / cl;
+        } else if (gdi_grid_plan(P, max_row, nblk, (size_t)max_optin, &spc, &wpc, &grid_need, &counted) == 0) {
+            const double N = (double)c->N, nnz = (double)c->nnz, ncls = (double)c->num_classes[0];
+            const double windows = N / c->W;
+            const int nrep = std::min(c->R, 8), cl = plan.cluster;
+            const double waves = (double)((c->R + plan.at_once - 1) / plan.at_once), groups = (double)((c->R + 7) / 8);
+            double grid_us = (12.1 + 0.41 * (nrep - 1)) * ncls +
+                             ((0.42e-3 + 0.05e-3 * nrep) * (N + nnz) + 0.105 * windows * nrep) / nblk;
+            double cta_us;
+            if (!plan.counted || !P.col16) {
+                cta_us = 2.0 * ncls + (block >= 512 ? 1.2e-3 : 1.8e-3) * (N + nnz);
+            } else if (cl == 1) {
+                cta_us = (c->W > 128 ? 2.6 : 2.1) * ncls + 2.4e-3 * N + 0.16e-3 * nnz + 0.2 * windows;
+            } else if (c->W > 128) {
+                cta_us = 9.0 * ncls + 0.55e-3 * (N + nnz) / cl;
+                grid_us = 0.8 * (13.0 * ncls + 0.02e-3 * (N + nnz));
+            } else {
+                cta_us = 4.5 * ncls + (0.19e-3 * (N + nnz) + 0.22 * windows) / cl;
+            }
+            grid = groups * grid_us < waves * cta_us;
         }
     }
     // kernel timing events (not while the stream is being captured into a graph)

@@ -86,13 +86,16 @@ int gdi_launch_init(const GdiDevProblem &P, int8_t *spins, const int8_t *init_or
                     uint32_t key0, uint32_t key1, void *stream);
 int gdi_launch_cta_anneal(const GdiDevProblem &P, const GdiDevRun &R, int block, int grid_limit,
                           void *stream, int *grid_used, size_t *smem_used);
-int gdi_cta_smem_bytes(const GdiDevProblem &P, const GdiDevRun &R, int block, size_t *bytes);
+int gdi_cta_smem_bytes(const GdiDevProblem &P, const GdiDevRun &R, int block, int grid_limit, size_t *bytes);
 // threads per CTA-path block where the caller has set none
-int gdi_cta_default_block(const GdiDevProblem &P, const GdiDevRun &R);
-// blocks per item of a CTA-path launch (a cluster of 1, 2, 4 or 8)
-int gdi_cta_cluster_size(const GdiDevProblem &P, const GdiDevRun &R, int block);
-// resident CTA-path blocks per SM for this problem and block size (0 when the block does not fit)
-int gdi_cta_blocks_per_sm(const GdiDevProblem &P, const GdiDevRun &R, int block, int *per_sm);
+int gdi_cta_default_block(const GdiDevProblem &P, const GdiDevRun &R, int grid_limit);
+// what a CTA-path launch of this problem, block size and block limit (0: none) is
+struct GdiCtaPlan {
+    bool counted;                    // the counting kernel (else the whole-block one)
+    int cluster;                     // blocks per item: 1, 2, 4 or 8
+    int at_once;                     // items resident at once (0 when a block does not fit)
+};
+int gdi_cta_plan(const GdiDevProblem &P, const GdiDevRun &R, int block, int grid_limit, GdiCtaPlan *plan);
 // Grid plan for `sms` blocks: spans of ranks (spc) and windows (wpc) per block and per class, and
 // the dynamic shared memory; counted: the counted-window kernel runs it (else the tabulated one); -1 if
 // the instance does not fit smem_limit.

@@ -1422,18 +1422,24 @@ inline bool cta_sorted(const GdiDevProblem &P, const GdiDevRun &R, int BS)
     return cta_sorted_layout(P, R.max_row, BS, 0, 0, 0, 0, 1).total + CTA_STATIC_SMEM <= (size_t)optin;
 }
 
-// Blocks per item (a cluster of 1, 2, 4 or 8, at most `most`): as many as leave every item its own SMs and four
-// windows of the largest class to each block.
-inline int cta_cluster(const GdiDevProblem &P, const GdiDevRun &R, int BS, int most)
+// blocks of a launch that are to run at once: one per SM, or the caller's limit
+inline int cta_blocks(int grid_limit)
 {
-    if (!cta_sorted(P, R, BS)) return 1;
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return grid_limit > 0 ? std::min(grid_limit, sms) : sms;
+}
+
+// Blocks per item (a cluster of 1, 2, 4 or 8, at most `most`): as many as leave every item its own of `blocks`
+// and four windows of the largest class to each block.
+inline int cta_cluster(const GdiDevProblem &P, const GdiDevRun &R, int BS, int blocks, int most)
+{
+    if (!cta_sorted(P, R, BS)) return 1;
     const int64_t items = (int64_t)P.num_instances * P.replicas;
     const int64_t nw = (P.max_class + P.W - 1) / P.W;
     int cl = 1;
-    while (2 * cl <= std::min(most, 8) && 2 * cl * items <= sms && 4 * 2 * cl <= nw) cl *= 2;
+    while (2 * cl <= std::min(most, 8) && 2 * cl * items <= blocks && 4 * 2 * cl <= nw) cl *= 2;
     return cl;
 }
 
@@ -1448,7 +1454,7 @@ inline size_t cta_smem(const GdiDevProblem &P, const GdiDevRun &R, int BS, bool 
 // taken when it fits a block and leaves as many items resident on an SM as there are without it (never
 // more than the SM's share of the items, or than its 1024 threads at 64 registers); the staging buffer
 // takes what is then left, up to the largest class.  Returns whether the counting kernel takes the call.
-inline bool cta_options(const GdiDevProblem &P, GdiDevRun &R, int BS, int max_cluster = 8)
+inline bool cta_options(const GdiDevProblem &P, GdiDevRun &R, int BS, int grid_limit, int max_cluster = 8)
 {
     int dev = 0, optin = 0, per_sm = 0, sms = 1;
     cudaGetDevice(&dev);
@@ -1461,7 +1467,7 @@ inline bool cta_options(const GdiDevProblem &P, GdiDevRun &R, int BS, int max_cl
     R.cta_stage = 0;
     R.cta_rofs = 0;
     R.cta_bins = 0;
-    R.cta_cluster = cta_cluster(P, R, BS, max_cluster);
+    R.cta_cluster = cta_cluster(P, R, BS, cta_blocks(grid_limit), max_cluster);
     auto resident = [&]() {
         const size_t need = cta_smem(P, R, BS, counted) + CTA_STATIC_SMEM;
         if (need > (size_t)optin) return (int64_t)0;
@@ -1518,6 +1524,23 @@ const void *cta_kernel(const GdiDevProblem &P, const GdiDevRun &R)
     return R.cta_cluster > 1 ? cta_sorted_kernel_for<BS, true>(P.W) : cta_sorted_kernel_for<BS, false>(P.W);
 }
 
+// a launch of clusters of cl blocks, one for each item (attr: storage of its attribute)
+inline cudaLaunchConfig_t cta_cluster_config(int cl, int items, int BS, size_t smem, cudaStream_t st, cudaLaunchAttribute *attr)
+{
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = cl;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(cl * items);
+    cfg.blockDim = dim3(BS);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cfg;
+}
+
 template <int BS>
 int launch_cta(const GdiDevProblem &P, const GdiDevRun &R0, int grid_limit, cudaStream_t st,
                int *grid_used, size_t *smem_used)
@@ -1530,9 +1553,9 @@ int launch_cta(const GdiDevProblem &P, const GdiDevRun &R0, int grid_limit, cuda
     void *args[] = {const_cast<GdiDevProblem *>(&P), &R};
     size_t smem = 0;
     cudaError_t e = cudaSuccess;
-    for (int cap = grid_limit > 0 && grid_limit < 8 ? grid_limit : 8;;) {
-        // (a grid limit below a cluster's size, or a GPU partition that holds no such cluster, halves it)
-        const bool counted = cta_options(P, R, BS, cap);
+    for (int cap = 8;;) {
+        // (a GPU partition that holds no such cluster halves it)
+        const bool counted = cta_options(P, R, BS, grid_limit, cap);
         const void *kern = cta_kernel<BS>(P, R);
         smem = cta_smem(P, R, BS, counted);
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -1550,17 +1573,7 @@ int launch_cta(const GdiDevProblem &P, const GdiDevRun &R0, int grid_limit, cuda
         // clusters of blocks, one item per cluster
         const int cl = R.cta_cluster;
         cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = cl;
-        attr[0].val.clusterDim.y = 1;
-        attr[0].val.clusterDim.z = 1;
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(cl * items);
-        cfg.blockDim = dim3(BS);
-        cfg.dynamicSmemBytes = smem;
-        cfg.stream = st;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
+        cudaLaunchConfig_t cfg = cta_cluster_config(cl, items, BS, smem, st, attr);
         int ncl = 0;
         e = cudaOccupancyMaxActiveClusters(&ncl, kern, &cfg);
         if (e != cudaSuccess) return (int)e;
@@ -1581,14 +1594,25 @@ int launch_cta(const GdiDevProblem &P, const GdiDevRun &R0, int grid_limit, cuda
 }
 
 template <int BS>
-int cta_occupancy(const GdiDevProblem &P, const GdiDevRun &R0, int *per_sm)
+int cta_occupancy(const GdiDevProblem &P, const GdiDevRun &R0, int grid_limit, GdiCtaPlan *plan)
 {
     GdiDevRun R = R0;
-    const bool counted = cta_options(P, R, BS);
+    plan->counted = cta_options(P, R, BS, grid_limit);
+    plan->cluster = R.cta_cluster;
     const void *kern = cta_kernel<BS>(P, R);
-    const size_t smem = cta_smem(P, R, BS, counted);
+    const size_t smem = cta_smem(P, R, BS, plan->counted);
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, kern, BS, smem);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&plan->at_once, kern, BS, smem);
+    plan->at_once *= sms;
+    if (e == cudaSuccess && plan->cluster > 1) {
+        cudaLaunchAttribute attr[1];
+        const cudaLaunchConfig_t cfg = cta_cluster_config(plan->cluster, P.num_instances * P.replicas, BS, smem, nullptr, attr);
+        e = cudaOccupancyMaxActiveClusters(&plan->at_once, kern, &cfg);
+    }
+    if (grid_limit > 0) plan->at_once = std::min(plan->at_once, grid_limit / plan->cluster);
     return (int)e;
 }
 
@@ -1602,7 +1626,7 @@ int cta_occupancy(const GdiDevProblem &P, const GdiDevRun &R0, int *per_sm)
 // for a wave as long as the first (400 replicas of 64, 1,000 and 2,000 vertices, W = 64, us a sweep 15.5 / 28.9, 32.4 /
 // 50.1, 51.4 / 60.8 at 256 / 512), while among unequal ones, the largest first, it fills in behind small ones (400 ER
 // instances: 15.6 / 15.0 / 25.3 ms); more than three take 256 (1024 short anneals: 4.4 / 6.0 / 10.2).
-int gdi_cta_default_block(const GdiDevProblem &P, const GdiDevRun &R)
+int gdi_cta_default_block(const GdiDevProblem &P, const GdiDevRun &R, int grid_limit)
 {
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
@@ -1610,7 +1634,7 @@ int gdi_cta_default_block(const GdiDevProblem &P, const GdiDevRun &R)
     const int64_t items = (int64_t)P.num_instances * P.replicas;
     if (items > 3LL * sms) return 256;
     if (items > 2LL * sms && 4 * P.N >= 3LL * P.max_n * P.num_instances) return 256;
-    const int cl = cta_cluster(P, R, 512, 8);
+    const int cl = cta_cluster(P, R, 512, cta_blocks(grid_limit), 8);
     if (items * cl <= sms && cta_sorted(P, R, 512)) {
         if (cta_own_ranks(P.max_class, P.W, cl) > 800) return 1024;
         if (P.max_class < 128) return 256;
@@ -1618,24 +1642,22 @@ int gdi_cta_default_block(const GdiDevProblem &P, const GdiDevRun &R)
     return 512;
 }
 
-int gdi_cta_cluster_size(const GdiDevProblem &P, const GdiDevRun &R, int block) { return cta_cluster(P, R, block, 8); }
-
-int gdi_cta_blocks_per_sm(const GdiDevProblem &P, const GdiDevRun &R, int block, int *per_sm)
+int gdi_cta_plan(const GdiDevProblem &P, const GdiDevRun &R, int block, int grid_limit, GdiCtaPlan *plan)
 {
-    *per_sm = 0;
+    *plan = GdiCtaPlan{};
     switch (block) {
-    case 128: return cta_occupancy<128>(P, R, per_sm);
-    case 256: return cta_occupancy<256>(P, R, per_sm);
-    case 512: return cta_occupancy<512>(P, R, per_sm);
-    case 1024: return cta_occupancy<1024>(P, R, per_sm);
+    case 128: return cta_occupancy<128>(P, R, grid_limit, plan);
+    case 256: return cta_occupancy<256>(P, R, grid_limit, plan);
+    case 512: return cta_occupancy<512>(P, R, grid_limit, plan);
+    case 1024: return cta_occupancy<1024>(P, R, grid_limit, plan);
     default: return (int)cudaErrorInvalidValue;
     }
 }
 
-int gdi_cta_smem_bytes(const GdiDevProblem &P, const GdiDevRun &R0, int block, size_t *bytes)
+int gdi_cta_smem_bytes(const GdiDevProblem &P, const GdiDevRun &R0, int block, int grid_limit, size_t *bytes)
 {
     GdiDevRun R = R0;
-    const bool counted = cta_options(P, R, block);
+    const bool counted = cta_options(P, R, block, grid_limit);
     *bytes = cta_smem(P, R, block, counted) + (counted ? CTA_STATIC_SMEM : 64);
     return 0;
 }

@@ -139,3 +139,22 @@ def test_autotune_under_auto_path(gdi):
     a.anneal(sch, 3, flags=gdi.GDI_FLAG_TRACE)
     assert np.array_equal(a.trace()[0], d0) and tuned["ms"] > 0
     a.close()
+
+
+@pytest.mark.parametrize("graph,W,replicas,limit,want", [
+    ("ba", 64, 1, 0, "cta"), ("ba", 4, 1, 0, "grid"), ("ba", 1, 8, 0, "grid"), ("ba", 64, 8, 0, "cta"),
+    ("ba", 64, 8, 4, "grid"), ("ba", 64, 8, 2, "grid"), ("ba", 64, 1, 1, "cta"), ("er", 64, 1, 0, "cta")])
+def test_auto_path_counts_windows_replicas_and_blocks(gdi, graph, W, replicas, limit, want):
+    """20,000 vertices on a cluster of eight a replica lose to the grid path where windows are small, or where a
+    block limit lets the replicas' clusters run one after another; with one block the grid path's plan does not
+    fit.  A dense graph of 50 classes pays the grid path's barrier 50 times."""
+    from gdi_synth import erdos_renyi
+    g = barabasi_albert(20000, 5, 20000) if graph == "ba" else erdos_renyi(3000, 200 / 2999, 2)
+    a = gdi.Annealer(g, A=1, B=4, W=W, replicas=replicas)
+    a.configure(grid_limit=limit)
+    a.anneal(gdi.Schedule(sweeps=2, t0=12.0, t1=0.2), 5)
+    a.results()
+    launch = a.last_launch()
+    a.close()
+    assert launch["path"] == (gdi.GDI_PATH_GRID if want == "grid" else gdi.GDI_PATH_CTA)
+    assert limit == 0 or launch["grid"] <= limit
