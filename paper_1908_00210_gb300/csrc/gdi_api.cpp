@@ -483,7 +483,8 @@ int gdi_create(gdi_ctx **out, const gdi_graph *g, const gdi_model *m)
     c->R = m->replicas;
     c->A = m->A;
     c->B = m->B;
-    c->W = m->W;
+    // (no class has 2^28 vertices, so a larger W is the same window; the kernels add it to ranks)
+    c->W = std::min(m->W, 1 << 28);
     c->N = N;
     c->nnz = g->row_ptr[N];
     c->num_classes = H.num_classes;

@@ -321,3 +321,27 @@ def test_cta_third_block_of_an_sm_needs_no_second_wave(gdi, n, W):
         us[replicas] = sweep_us(gdi, ann)
         ann.close()
     assert us[400] < 1.35 * us[300], us
+
+
+@pytest.mark.parametrize("W", [2**31 - 1, 2**31 - 200, 2**30])
+def test_window_of_any_size_is_the_whole_class(gdi, W):
+    """Ranks plus W stay below 2^31 for any W: one graph and a batch, against windows of n ranks."""
+    g = erdos_renyi(400, 0.03, 95)
+    gp, u = batch_union([erdos_renyi(150 + 30 * i, 0.05, 96 + i) for i in range(4)])
+    sch = gdi.Schedule(sweeps=8, t0=12.0, t1=0.2)
+    for graph, kw in ((g, {}), (u, dict(inst_ptr=gp))):
+        got = []
+        for w in (W, g.n):
+            ann = gdi.Annealer(graph, A=1, B=4, W=w, replicas=2, **kw)
+            ann.configure(path=gdi.GDI_PATH_CTA)
+            ann.anneal(sch, 19)
+            got.append((ann.spins(), ann.results()))
+            ann.close()
+        assert np.array_equal(got[0][0], got[1][0])
+        for k in ("raw_G", "final_G", "raw_cut", "final_cut"):
+            assert np.array_equal(got[0][1][k], got[1][1][k]), k
+    ref = oracle.anneal(g, A=1, B=4, W=g.n, t0=12.0, t1=0.2, sweeps=8, seed=19, replicas=2)
+    ann = gdi.Annealer(g, A=1, B=4, W=W, replicas=2)
+    ann.anneal(sch, 19)
+    assert np.array_equal(ann.spins(), ref.spins)
+    ann.close()
