@@ -1075,6 +1075,46 @@ int grid_for(int64_t work, int per_block)
 
 constexpr int DF_CAP = 8960;              // two blocks of 1,024 threads and this many vertices fit an SM
 
+// The one-launch walk's two launches: diffuse_kernel in clusters of DF_CL blocks, then walk_rest_kernel with at most
+// four blocks per SM and no more than the device, or the part of it that this process has, holds at once (a
+// cooperative launch of more is refused).  1: enqueued; 0: the device holds no such cluster, and nothing was
+// enqueued; else a negative error.
+int launch_walk(int64_t N, int32_t G, const int64_t *graph_ptr, const uint32_t *graph_id, const int64_t *row_ptr,
+                const int32_t *col, uint32_t k0, uint32_t k1, int32_t steps, float *X, float *R0, float *R1, cudaStream_t st)
+{
+    int dev = 0, sms = 0, rest = 0, clusters = 0;
+    const size_t smem = df_layout(DF_CAP).total;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = DF_CL;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)G * DF_CL);
+    cfg.blockDim = dim3(DF_T);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&rest, (const void *)walk_rest_kernel, 256, 0) != cudaSuccess ||
+        sms * rest < 1 ||
+        cudaFuncSetAttribute(diffuse_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&clusters, diffuse_kernel, &cfg) != cudaSuccess || clusters < 1) {
+        cudaGetLastError();                   // (a refused query is no error of the call)
+        return 0;
+    }
+    const int cap = DF_CAP;
+    if (cudaLaunchKernelEx(&cfg, diffuse_kernel, graph_ptr, graph_id, row_ptr, col, k0, k1, (int)steps, cap, X, R0, R1) !=
+        cudaSuccess)
+        return GDI_ERR_CUDA;
+    void *args[] = {&N, &G, &graph_ptr, &graph_id, &row_ptr, &col, &k0, &k1, &steps, &X, &R0, &R1};
+    if (cudaLaunchCooperativeKernel((const void *)walk_rest_kernel, dim3(sms * (rest < 4 ? rest : 4)), dim3(256), args, 0,
+                                    st) != cudaSuccess)
+        return GDI_ERR_CUDA;
+    return 1;
+}
+
 // 8-, 16- and 64-wide rows (the network's) on a 16-byte boundary take the vector kernel, other widths
 // and alignments the general one.
 void launch_aggregate(int64_t N, const int64_t *row_ptr, const int32_t *col, const float *X, int d, float *Y,
@@ -1102,18 +1142,14 @@ int gdi_mpnn_features(int64_t N, int32_t G, const int64_t *graph_ptr, const uint
     cudaStream_t st = (cudaStream_t)stream;
     float *R0 = scratch, *R1 = scratch + N * NRAND;
     // all steps in one launch where the mean graph fits a block, and one for the graphs that do not; else,
-    // and without steps, one launch per step over all vertices
+    // without steps, and on a device that holds no cluster, one launch per step over all vertices
+    int walked = 0;
     if (steps > 0 && N / G <= DF_CAP && aligned(scratch, 16)) {
-        const size_t smem = df_layout(DF_CAP).total;
-        if (cudaFuncSetAttribute(diffuse_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-            return GDI_ERR_CUDA;
-        diffuse_kernel<<<G * DF_CL, DF_T, smem, st>>>(graph_ptr, graph_id, row_ptr, col, (uint32_t)seed,
-                                                      (uint32_t)(seed >> 32), steps, DF_CAP, X, R0, R1);
-        uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32);
-        void *args[] = {&N, &G, &graph_ptr, &graph_id, &row_ptr, &col, &k0, &k1, &steps, &X, &R0, &R1};
-        if (cudaLaunchCooperativeKernel((const void *)walk_rest_kernel, dim3(152 * 4), dim3(256), args, 0, st) != cudaSuccess)
-            return GDI_ERR_CUDA;
-    } else {
+        walked = launch_walk(N, G, graph_ptr, graph_id, row_ptr, col, (uint32_t)seed, (uint32_t)(seed >> 32), steps, X, R0,
+                             R1, st);
+        if (walked < 0) return walked;
+    }
+    if (!walked) {
         feat_init_kernel<<<grid_for(N * NRAND, 256), 256, 0, st>>>(N, G, graph_ptr, graph_id, (uint32_t)seed,
                                                                     (uint32_t)(seed >> 32), R0);
         for (int s = 0; s < steps; ++s) {
