@@ -93,7 +93,7 @@ struct gdi_ctx {
     long long inject_limit = 0;
     std::vector<int32_t> num_classes;       // per instance
     DevBuf<int64_t> node_off, row_ptr;
-    DevBuf<int32_t> class_off, class_ptr, rank_of;
+    DevBuf<int32_t> class_off, class_ptr, rank_of, piece_off[4], piece_ptr[4];
     DevBuf<uint32_t> col;
     DevBuf<uint16_t> col16;
     DevBuf<int8_t> spins, init_stage, out_stage;
@@ -130,6 +130,10 @@ struct gdi_ctx {
         P.node_off = node_off.p;
         P.class_off = class_off.p;
         P.class_ptr = class_ptr.p;
+        for (int k = 0; k < 4; ++k) {
+            P.piece_off[k] = piece_off[k].p;
+            P.piece_ptr[k] = piece_ptr[k].p;
+        }
         P.row_ptr = row_ptr.p;
         P.col = col.p;
         P.col16 = col16.p;
@@ -148,6 +152,7 @@ struct gdi_ctx {
     void release()
     {
         node_off.release(); row_ptr.release(); class_off.release(); class_ptr.release();
+        for (int k = 0; k < 4; ++k) { piece_off[k].release(); piece_ptr[k].release(); }
         rank_of.release(); col.release(); col16.release(); spins.release(); init_stage.release(); out_stage.release();
         tab.release(); tab_off.release(); temp.release(); raw_G.release(); final_G.release(); tr_G.release();
         err.release(); raw_cut.release(); final_cut.release(); tr_cut.release(); tr_digest.release();
@@ -537,6 +542,19 @@ int gdi_create(gdi_ctx **out, const gdi_graph *g, const gdi_model *m)
     }
     GDI_UP(c->class_off, class_off);
     GDI_UP(c->class_ptr, class_ptr);
+    // classes too large for the counting kernel's class buffers, in pieces
+    for (int k = 0; k < 4 && c->W >= 1 && c->W <= 256 && H.max_class > gdi_cta_piece(c->W, 1 << k); ++k) {
+        const int32_t piece = gdi_cta_piece(c->W, 1 << k);
+        std::vector<int32_t> off(1, 0), ptr;
+        for (int32_t q = 0; q < Q; ++q) {
+            for (int32_t i = class_off[(size_t)q]; i + 1 < class_off[(size_t)q + 1]; ++i)
+                for (int32_t r = class_ptr[(size_t)i]; r < class_ptr[(size_t)i + 1]; r += piece) ptr.push_back(r);
+            ptr.push_back(class_ptr[(size_t)class_off[(size_t)q + 1] - 1]);
+            off.push_back((int32_t)ptr.size());
+        }
+        GDI_UP(c->piece_off[k], off);
+        GDI_UP(c->piece_ptr[k], ptr);
+    }
     GDI_UP(c->rank_of, rank_of);
     {
         // work queue order for the CTA path: largest instance (vertices + CSR entries) first

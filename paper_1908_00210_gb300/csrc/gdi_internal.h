@@ -16,6 +16,8 @@ struct GdiDevProblem {
     const int64_t *node_off;         // [Q+1]
     const int32_t *class_off;        // [Q+1] offsets into class_ptr
     const int32_t *class_ptr;        // per instance: C_q + 1 class boundaries in local ranks
+    const int32_t *piece_off[4];     // the same for the classes in pieces of gdi_cta_piece(W, 1, 2, 4 and 8)
+    const int32_t *piece_ptr[4];     // ranks; null where no class is larger
     const int64_t *row_ptr;          // [N+1] rank-space CSR offsets
     const uint32_t *col;             // [nnz] local neighbour rank | (weight < 0) << 31
     const uint16_t *col16;           // [nnz] the same in 16 bits (rank | (weight < 0) << 15) when
@@ -95,6 +97,8 @@ struct GdiCtaPlan {
     int cluster;                     // blocks per item: 1, 2, 4 or 8
     int at_once;                     // items resident at once (0 when a block does not fit)
 };
+// most ranks of a class that the counting kernel takes at once with clusters of so many blocks
+int32_t gdi_cta_piece(int32_t W, int32_t cluster);
 int gdi_cta_plan(const GdiDevProblem &P, const GdiDevRun &R, int block, int grid_limit, GdiCtaPlan *plan);
 // Grid plan for `sms` blocks: spans of ranks (spc) and windows (wpc) per block and per class, and
 // the dynamic shared memory; counted: the counted-window kernel runs it (else the tabulated one); -1 if

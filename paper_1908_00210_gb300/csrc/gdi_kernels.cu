@@ -890,11 +890,12 @@ struct SortedCta {
 
 // Windows of one block whose stage maps are kept.  A class of more than so many for each of its blocks is
 // taken in pieces of that size, one after another like classes: its vertices share no edge, so a piece's
-// thresholds do not see the flips of the pieces before it, and only G passes on.  (One warp that replayed such a
+// thresholds do not see the flips of the pieces before it, and only G passes on.  gdi_create lays the pieces
+// out for every cluster size as it does the classes, and the launch hands the kernel those in their place (the
+// kernel finding them itself spilled 640 bytes and lost 8 % with windows above 128, pieces or not).  (One warp that replayed such a
 // class window by window took 0.47 us a window.  A sweep of 40 replicas of 3,000 vertices, W = 1: 1,399 -> 314 us;
 // 300 of a 100 x 100 torus, W = 32: 257 -> 118.)
 constexpr int CTA_WALK_MAX = 128;
-__host__ __device__ inline int32_t cta_piece(int W, int cl) { return CTA_WALK_MAX * cl * W; }
 
 // windows a block of a cluster of cl (1: alone) has of the largest piece: one or two windows are the first
 // block's
@@ -1050,15 +1051,7 @@ __global__ void __launch_bounds__(BS, 1024 / BS) gdi_cta_sorted_kernel(GdiDevPro
         const int64_t base = P.node_off[q];
         const int32_t n = (int32_t)(P.node_off[q + 1] - base);
         const int32_t *cls = P.class_ptr + P.class_off[q];
-        // the item's classes, or the pieces of all of them (both "class" below)
-        const int32_t piece = cta_piece(W, (int)CL);
-        const bool pieces = P.max_class > piece;
-        int32_t ncls = P.class_off[q + 1] - P.class_off[q] - 1;
-        if (pieces) {
-            int32_t np = 0;
-            for (int c = 0; c < ncls; ++c) np += (cls[c + 1] - cls[c] + piece - 1) / piece;
-            ncls = np;
-        }
+        const int32_t ncls = P.class_off[q + 1] - P.class_off[q] - 1;
         int8_t *gsig = R.spins + (int64_t)rep * P.N + base;
         const int64_t row0 = P.row_ptr[base];
         const int64_t nnz_item = P.row_ptr[base + n] - row0;
@@ -1066,19 +1059,8 @@ __global__ void __launch_bounds__(BS, 1024 / BS) gdi_cta_sorted_kernel(GdiDevPro
 
         auto make_span = [&](int c) {
             Span s;
-            int32_t at = 0;                          // ranks of the class before this piece
-            if (pieces) {
-                int cc = 0;
-                for (;; ++cc) {
-                    const int32_t np = (cls[cc + 1] - cls[cc] + piece - 1) / piece;
-                    if (c < np) break;
-                    c -= np;
-                }
-                at = c * piece;
-                c = cc;
-            }
-            s.clo = cls[c] + at;
-            s.chi = pieces ? min(s.clo + piece, cls[c + 1]) : cls[c + 1];
+            s.clo = cls[c];
+            s.chi = cls[c + 1];
             const int32_t size = s.chi - s.clo;
             s.nwin = (size + W - 1) / W;
             s.kq = CLUS ? (s.nwin + (int)CL - 1) / (int)CL : s.nwin;
@@ -1542,20 +1524,27 @@ inline cudaLaunchConfig_t cta_cluster_config(int cl, int items, int BS, size_t s
 }
 
 template <int BS>
-int launch_cta(const GdiDevProblem &P, const GdiDevRun &R0, int grid_limit, cudaStream_t st,
+int launch_cta(const GdiDevProblem &P0, const GdiDevRun &R0, int grid_limit, cudaStream_t st,
                int *grid_used, size_t *smem_used)
 {
     GdiDevRun R = R0;
-    const int items = P.num_instances * P.replicas;
+    const int items = P0.num_instances * P0.replicas;
     int dev = 0, sms = 0, grid = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    void *args[] = {const_cast<GdiDevProblem *>(&P), &R};
+    GdiDevProblem P = P0;
+    void *args[] = {&P, &R};
     size_t smem = 0;
     cudaError_t e = cudaSuccess;
     for (int cap = 8;;) {
         // (a GPU partition that holds no such cluster halves it)
-        const bool counted = cta_options(P, R, BS, grid_limit, cap);
+        const bool counted = cta_options(P0, R, BS, grid_limit, cap);
+        P = P0;
+        const int k = R.cta_cluster == 8 ? 3 : R.cta_cluster / 2;
+        if (counted && P.piece_ptr[k]) {
+            P.class_ptr = P.piece_ptr[k];
+            P.class_off = P.piece_off[k];
+        }
         const void *kern = cta_kernel<BS>(P, R);
         smem = cta_smem(P, R, BS, counted);
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -1641,6 +1630,8 @@ int gdi_cta_default_block(const GdiDevProblem &P, const GdiDevRun &R, int grid_l
     }
     return 512;
 }
+
+int32_t gdi_cta_piece(int32_t W, int32_t cluster) { return CTA_WALK_MAX * cluster * W; }
 
 int gdi_cta_plan(const GdiDevProblem &P, const GdiDevRun &R, int block, int grid_limit, GdiCtaPlan *plan)
 {
