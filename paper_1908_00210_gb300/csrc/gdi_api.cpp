@@ -784,33 +784,36 @@ int gdi_anneal(gdi_ctx *c, const gdi_schedule *S, const gdi_run *run)
         // Clusters with windows above 128, whose cost scatters most, keep the older and more careful estimate: 9 a
         // class + 0.55e-3 a vertex and edge, which has to undercut the grid path's 13 and 0.02e-3 by a fifth.
         // Without 16-bit columns nothing is staged, and the whole-block kernel sums its rows more slowly: 2 a class
-        // and 1.2e-3 (1.8e-3 with blocks of 128 or 256) a vertex and edge.
-        GdiCtaPlan plan;
-        int spc, wpc;
-        size_t grid_need;
-        bool counted;
-        const int nblk = c->grid_limit > 0 ? std::min(c->grid_limit, sms) : sms;
-        if (need > (size_t)max_optin || gdi_cta_plan(P, R, block, c->grid_limit, &plan) != 0 || plan.at_once < 1) {
-            grid = true;
-        } else if (gdi_grid_plan(P, max_row, nblk, (size_t)max_optin, &spc, &wpc, &grid_need, &counted) == 0) {
+        // and 1.2e-3 (1.8e-3 with blocks of 128 or 256) a vertex and edge, against 13 and 0.02e-3 too.
+        auto grid_wins = [&](int limit) {
+            GdiCtaPlan plan;
+            if (need > (size_t)max_optin || gdi_cta_plan(P, R, block, limit, &plan) != 0 || plan.at_once < 1) return true;
             const double N = (double)c->N, nnz = (double)c->nnz, ncls = (double)c->num_classes[0];
             const double windows = N / c->W;
-            const int nrep = std::min(c->R, 8), cl = plan.cluster;
+            const int nrep = std::min(c->R, 8), cl = plan.cluster, nblk = limit > 0 ? std::min(limit, sms) : sms;
             const double waves = (double)((c->R + plan.at_once - 1) / plan.at_once), groups = (double)((c->R + 7) / 8);
-            double grid_us = (12.1 + 0.41 * (nrep - 1)) * ncls +
-                             ((0.42e-3 + 0.05e-3 * nrep) * (N + nnz) + 0.105 * windows * nrep) / nblk;
-            double cta_us;
+            double cta_us, grid_us = 13.0 * ncls + 0.02e-3 * (N + nnz);
             if (!plan.counted || !P.col16) {
                 cta_us = 2.0 * ncls + (block >= 512 ? 1.2e-3 : 1.8e-3) * (N + nnz);
-            } else if (cl == 1) {
-                cta_us = (c->W > 128 ? 2.6 : 2.1) * ncls + 2.4e-3 * N + 0.16e-3 * nnz + 0.2 * windows;
-            } else if (c->W > 128) {
+            } else if (cl > 1 && c->W > 128) {
                 cta_us = 9.0 * ncls + 0.55e-3 * (N + nnz) / cl;
-                grid_us = 0.8 * (13.0 * ncls + 0.02e-3 * (N + nnz));
+                grid_us *= 0.8;
             } else {
-                cta_us = 4.5 * ncls + (0.19e-3 * (N + nnz) + 0.22 * windows) / cl;
+                cta_us = cl == 1 ? (c->W > 128 ? 2.6 : 2.1) * ncls + 2.4e-3 * N + 0.16e-3 * nnz + 0.2 * windows
+                                 : 4.5 * ncls + (0.19e-3 * (N + nnz) + 0.22 * windows) / cl;
+                grid_us = (12.1 + 0.41 * (nrep - 1)) * ncls +
+                          ((0.42e-3 + 0.05e-3 * nrep) * (N + nnz) + 0.105 * windows * nrep) / nblk;
             }
-            grid = groups * grid_us < waves * cta_us;
+            return groups * grid_us < waves * cta_us;
+        };
+        grid = grid_wins(c->grid_limit);
+        if (grid && c->grid_limit > 0) {
+            // a plan that does not fit so few blocks: as without the limit
+            int spc, wpc;
+            size_t grid_need;
+            bool counted;
+            if (gdi_grid_plan(P, max_row, std::min(c->grid_limit, sms), (size_t)max_optin, &spc, &wpc, &grid_need, &counted) != 0)
+                grid = grid_wins(0);
         }
     }
     // kernel timing events (not while the stream is being captured into a graph)
