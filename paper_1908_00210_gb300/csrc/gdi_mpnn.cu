@@ -850,27 +850,36 @@ diffuse_kernel(const int64_t *graph_ptr, const uint32_t *graph_id, const int64_t
     } else {
         for (int64_t i = threadIdx.x; i < n64; i += DF_T) res[i * NRAND] = noise_sign((uint32_t)i, ch, id, k0, k1);
     }
-    // what walk_rest_kernel has to take (X is free again): 1 = this graph, 2 = the whole batch, since a column
-    // leads from this graph to another (written above before the cluster's barriers)
-    if (ch == 0 && threadIdx.x == 0 && n64 > 0) {
-        X[v0 * FIN] = !fits ? 1.f : (leaves ? 2.f : 0.f);
-        X[v0 * FIN + 1] = 0.f;                                         // walk_rest_kernel's own mark
-    }
+    // what walk_rest_kernel has to take (X is free again), in word 0 of each of the graph's vertices: 1 = this
+    // graph, 2 = the whole batch, since a column leads from this graph to another (block 0's `leaves`, written
+    // before the cluster's barriers).  Word 1 is walk_rest_kernel's own.
+    if (fits && ch != 0) return;
+    const int64_t i0 = fits ? threadIdx.x : (int64_t)ch * DF_T + threadIdx.x, step = fits ? DF_T : DF_CL * DF_T;
+    const float mark = !fits ? 1.f : (leaves ? 2.f : 0.f);
+    for (int64_t i = i0; i < n64; i += step) X[(v0 + i) * FIN] = mark;
+    if (ch == 0 && threadIdx.x == 0 && n64 > 0) X[v0 * FIN + 1] = 0.f;
 }
 
 // The walk steps of the graphs that diffuse_kernel marked, whose noise it left in R0: one cooperative
 // launch, a warp per row as in aggregate_vec_kernel<8>, a grid barrier per step.  Without marked
 // graphs it returns at once.  (One launch per step over all vertices would cost every batch `steps`
-// launches for the rare graph that does not fit.)  A batch in which a column leads from one graph to another
+// launches for the rare graph that does not fit.)  Bound by the chain of dependent L2 reads of a row (bounds,
+// column, its bounds and value), so by rows in flight, and by the grid barrier: 32 registers leave 64 warps an SM, and
+// blocks of 1,024 threads keep the barrier to two arrivals an SM.  (us a step, 256 steps: a graph of 10^6 vertices of
+// degree 6 beside 400 of 1,000: one launch per step, one neighbour at a time, 720; four blocks of 256 and a search for
+// the row's graph in each step 1,120, without the search 951; this 285.  One of 12,000 beside one of 1,000: 12.9, 14.6,
+// 14.1, 7.8.  With the block size written as a constant the compiler spills differently and the first takes 500.)
+// A batch in which a column leads from one graph to another
 // walks as a whole, from the noise on: every vertex's value is then read at its own step.
-__global__ void __launch_bounds__(256) walk_rest_kernel(int64_t N, int G, const int64_t *graph_ptr, const uint32_t *graph_id,
+constexpr int WR_T = 1024;
+__global__ void __launch_bounds__(WR_T, 2) walk_rest_kernel(int64_t N, int G, const int64_t *graph_ptr, const uint32_t *graph_id,
                                                         const int64_t *row_ptr, const int32_t *col, uint32_t k0, uint32_t k1,
                                                         int steps, float *X, float *R0, float *R1)
 {
     // a mark of any graph: word 0 (diffuse_kernel's) at least v, or word 1 (set below)
     auto marked = [&](float v) {
         int any = 0;
-        for (int g = threadIdx.x; g < G; g += 256) {
+        for (int g = threadIdx.x; g < G; g += blockDim.x) {
             if (graph_ptr[g + 1] <= graph_ptr[g]) continue;
             const float *m = X + graph_ptr[g] * FIN;
             any |= m[0] >= v || m[1] != 0.f;
@@ -880,19 +889,19 @@ __global__ void __launch_bounds__(256) walk_rest_kernel(int64_t N, int G, const 
     if (!marked(1.f)) return;
     cooperative_groups::grid_group grid = cooperative_groups::this_grid();
     const int lane = threadIdx.x & 31, sub = lane >> 1, c4 = lane & 1;
-    const int64_t wglob = ((int64_t)blockIdx.x * 256 + threadIdx.x) >> 5, nw = ((int64_t)gridDim.x * 256) >> 5;
+    const int64_t wglob = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     float4 *in = reinterpret_cast<float4 *>(R0), *out = reinterpret_cast<float4 *>(R1);
     // diffuse_kernel has looked at the columns of the graphs that fit it; here the others'
     for (int64_t i = wglob; i < N; i += nw) {
+        if (X[i * FIN] != 1.f) continue;
         const int64_t g = graph_of(graph_ptr, G, i), v0 = graph_ptr[g], v1 = graph_ptr[g + 1];
-        if (X[v0 * FIN] != 1.f) continue;
         for (int64_t e = row_ptr[i] + lane; e < row_ptr[i + 1]; e += 32)
             if (col[e] < v0 || col[e] >= v1) X[v0 * FIN + 1] = 1.f;
     }
     grid.sync();
     const bool all = marked(2.f);
     if (all) {
-        for (int64_t t = (int64_t)blockIdx.x * 256 + threadIdx.x; t < N * NRAND; t += (int64_t)gridDim.x * 256) {
+        for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < N * NRAND; t += (int64_t)gridDim.x * blockDim.x) {
             const int64_t i = t / NRAND;
             const int g = (int)graph_of(graph_ptr, G, i);
             R0[t] = noise_sign((uint32_t)(i - graph_ptr[g]), (int)(t % NRAND), graph_id[g], k0, k1);
@@ -902,7 +911,7 @@ __global__ void __launch_bounds__(256) walk_rest_kernel(int64_t N, int G, const 
     // the last round copies the result back to R0 when it ended in R1
     for (int s = 0; s < steps + (steps & 1); ++s) {
         for (int64_t i = wglob; i < N; i += nw) {
-            if (!all && X[graph_ptr[graph_of(graph_ptr, G, i)] * FIN] == 0.f) continue;
+            if (!all && X[i * FIN] == 0.f) continue;
             if (s == steps) {
                 if (lane < 2) out[i * 2 + lane] = in[i * 2 + lane];
                 continue;
@@ -910,7 +919,7 @@ __global__ void __launch_bounds__(256) walk_rest_kernel(int64_t N, int G, const 
             const int64_t e0 = row_ptr[i], e1 = row_ptr[i + 1];
             const float degi = (float)(e1 - e0);
             float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 4
+#pragma unroll 1
             for (int64_t e = e0 + sub; e < e1; e += 16) {
                 const int64_t j = col[e];
                 const float w = edge_weight(2, row_ptr, j, degi);
@@ -1075,9 +1084,9 @@ int grid_for(int64_t work, int per_block)
 
 constexpr int DF_CAP = 8960;              // two blocks of 1,024 threads and this many vertices fit an SM
 
-// The one-launch walk's two launches: diffuse_kernel in clusters of DF_CL blocks, then walk_rest_kernel with at most
-// four blocks per SM and no more than the device, or the part of it that this process has, holds at once (a
-// cooperative launch of more is refused).  1: enqueued; 0: the device holds no such cluster, and nothing was
+// The one-launch walk's two launches: diffuse_kernel in clusters of DF_CL blocks, then walk_rest_kernel with as many
+// blocks as the device, or the part of it that this process has, holds at once (a cooperative
+// launch of more is refused).  1: enqueued; 0: the device holds no such cluster, and nothing was
 // enqueued; else a negative error.
 int launch_walk(int64_t N, int32_t G, const int64_t *graph_ptr, const uint32_t *graph_id, const int64_t *row_ptr,
                 const int32_t *col, uint32_t k0, uint32_t k1, int32_t steps, float *X, float *R0, float *R1, cudaStream_t st)
@@ -1097,7 +1106,7 @@ int launch_walk(int64_t N, int32_t G, const int64_t *graph_ptr, const uint32_t *
     cfg.numAttrs = 1;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&rest, (const void *)walk_rest_kernel, 256, 0) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&rest, (const void *)walk_rest_kernel, WR_T, 0) != cudaSuccess ||
         sms * rest < 1 ||
         cudaFuncSetAttribute(diffuse_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
         cudaOccupancyMaxActiveClusters(&clusters, diffuse_kernel, &cfg) != cudaSuccess || clusters < 1) {
@@ -1109,7 +1118,7 @@ int launch_walk(int64_t N, int32_t G, const int64_t *graph_ptr, const uint32_t *
         cudaSuccess)
         return GDI_ERR_CUDA;
     void *args[] = {&N, &G, &graph_ptr, &graph_id, &row_ptr, &col, &k0, &k1, &steps, &X, &R0, &R1};
-    if (cudaLaunchCooperativeKernel((const void *)walk_rest_kernel, dim3(sms * (rest < 4 ? rest : 4)), dim3(256), args, 0,
+    if (cudaLaunchCooperativeKernel((const void *)walk_rest_kernel, dim3(sms * rest), dim3(WR_T), args, 0,
                                     st) != cudaSuccess)
         return GDI_ERR_CUDA;
     return 1;

@@ -295,3 +295,39 @@ def test_features_of_graphs_with_columns_between_them(gdi, cut, steps):
         for a, b in zip(gp[:-1], gp[1:]):
             if b - a > 1:                  # (one vertex: centred to 0, scaled by 1e-12)
                 assert np.max(np.abs(got[a:b] - Xr[a:b])) < 1e-4, (a, b)
+
+
+@pytest.mark.parametrize("big,deg,small", [(300_000, 4, 40), (12_000, 6, 1)])
+def test_features_of_one_large_graph_among_small_ones(gdi, big, deg, small):
+    """The walk of a batch whose large graph does not fit a block takes no longer than a launch per step over all
+    its vertices (it took 1.3 to 2 times as long)."""
+    import torch
+    from gdi_synth import from_edges
+    from paper_1908_00210_gb300 import learn
+    rng = np.random.default_rng(big)
+
+    def graph(n, d):
+        u, v = rng.integers(0, n, (2, n * d // 2))
+        e = np.unique(np.minimum(u, v)[u != v].astype(np.int64) * n + np.maximum(u, v)[u != v])
+        return from_edges(n, e // n, e % n)
+    b = learn.GraphBatch.from_graphs([graph(big, deg)] + [graph(1000, 6)] * small)
+    m = learn.MPNN(seed=1, steps=256)
+    r = torch.empty(2, b.N, 8, device="cuda")
+
+    def one_launch_per_step():
+        for s in range(m.steps):
+            learn.lib().gdi_mpnn_aggregate(b.N, b.row_ptr.data_ptr(), b.col.data_ptr(), r[s & 1].data_ptr(), 8,
+                                           r[1 - (s & 1)].data_ptr(), 2, 0, m._st())
+
+    def ms(f):
+        f()
+        t = []
+        for _ in range(3):
+            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            e0.record()
+            f()
+            e1.record()
+            e1.synchronize()
+            t.append(e0.elapsed_time(e1))
+        return min(t)
+    assert ms(lambda: m.features(b)) < 1.1 * ms(one_launch_per_step)
