@@ -1124,6 +1124,18 @@ int launch_walk(int64_t N, int32_t G, const int64_t *graph_ptr, const uint32_t *
     return 1;
 }
 
+// Whether the one-launch walk saves more than it costs.  Few steps do not repay laying out the columns: a step in a
+// launch of its own costs about 3.5 us + N / 3000, in the one launch 0.4 + n / 800 (mean degree 12, n = the mean graph),
+// which costs 12 us + n / 200 + G / 4 more to begin with.  (us for 1 / 2 / 4 / 8 steps, one launch against one per step: one
+// graph of 300 vertices 51 53 54 56 / 43 44 50 67, of 2,000 75 74 83 95 / 53 58 65 80, of 5,000 120 126 141 165 / 84
+// 89 100 127; 64 of 2,000 115 123 143 178 / 95 134 211 367.)
+bool one_launch_walk(int64_t N, int32_t G, int32_t steps)
+{
+    if (steps >= 32) return true;
+    const double n = (double)N / G;
+    return steps * (3.1 + (double)N / 3000 - n / 800) > 12.0 + n / 200 + G / 4.0;
+}
+
 // 8-, 16- and 64-wide rows (the network's) on a 16-byte boundary take the vector kernel, other widths
 // and alignments the general one.
 void launch_aggregate(int64_t N, const int64_t *row_ptr, const int32_t *col, const float *X, int d, float *Y,
@@ -1151,9 +1163,9 @@ int gdi_mpnn_features(int64_t N, int32_t G, const int64_t *graph_ptr, const uint
     cudaStream_t st = (cudaStream_t)stream;
     float *R0 = scratch, *R1 = scratch + N * NRAND;
     // all steps in one launch where the mean graph fits a block, and one for the graphs that do not; else,
-    // without steps, and on a device that holds no cluster, one launch per step over all vertices
+    // for few steps, and on a device that holds no cluster, one launch per step over all vertices
     int walked = 0;
-    if (steps > 0 && N / G <= DF_CAP && aligned(scratch, 16)) {
+    if (one_launch_walk(N, G, steps) && N / G <= DF_CAP && aligned(scratch, 16)) {
         walked = launch_walk(N, G, graph_ptr, graph_id, row_ptr, col, (uint32_t)seed, (uint32_t)(seed >> 32), steps, X, R0,
                              R1, st);
         if (walked < 0) return walked;

@@ -272,7 +272,7 @@ def test_features_one_launch_and_the_rest(gdi, steps):
             assert np.max(np.abs(X[s] - Xr[s])) < 1e-4, (q, np.max(np.abs(X[s] - Xr[s])))
 
 
-@pytest.mark.parametrize("steps", [1, 4, 5])
+@pytest.mark.parametrize("steps", [1, 4, 5, 32, 33])
 @pytest.mark.parametrize("cut", [(0, 700, 1999, 2000), (0, 300, 300, 1500, 2000), (0, 9400, 9600), (0, 200, 9600)])
 def test_features_of_graphs_with_columns_between_them(gdi, cut, steps):
     """graph_ptr cuts connected graphs, so columns lead from one to another: walked as one graph, as the
@@ -331,3 +331,16 @@ def test_features_of_one_large_graph_among_small_ones(gdi, big, deg, small):
             t.append(e0.elapsed_time(e1))
         return min(t)
     assert ms(lambda: m.features(b)) < 1.1 * ms(one_launch_per_step)
+
+
+@pytest.mark.parametrize("steps", [1, 2, 3, 4, 5, 8, 31, 32, 33])
+@pytest.mark.parametrize("n,count", [(90, 1), (300, 40), (2000, 1), (2000, 20)])
+def test_features_of_few_steps(gdi, n, count, steps):
+    """Step counts on both sides of the line between a launch per step and the one-launch walk, and of 32.
+    Float32 sums of at most 30 terms a step, scaled to unit RMS: 1e-4."""
+    from paper_1908_00210_gb300 import learn
+    gs = [_ring_graph(n + 3 * (i % 5), 4 * n, i) for i in range(count)]
+    gp, u = batch_union(gs)
+    ids = np.arange(count, dtype=np.uint32)
+    X = learn.MPNN(seed=1, feat_seed=5, steps=steps).features(learn.GraphBatch.from_graphs(gs, graph_ids=ids))
+    assert np.max(np.abs(X.cpu().numpy() - ref.features(gp, ids, u.row_ptr, u.col, 5, steps))) < 1e-4
