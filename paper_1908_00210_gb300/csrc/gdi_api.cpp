@@ -93,7 +93,8 @@ struct gdi_ctx {
     long long inject_limit = 0;
     std::vector<int32_t> num_classes;       // per instance
     DevBuf<int64_t> node_off, row_ptr;
-    DevBuf<int32_t> class_off, class_ptr, rank_of, piece_off[4], piece_ptr[4];
+    DevBuf<int32_t> class_off, class_ptr, rank_of, pieces;
+    int64_t piece_at[4][2] = {};             // where a cluster size's offsets and boundaries start in pieces (0: none)
     DevBuf<uint32_t> col;
     DevBuf<uint16_t> col16;
     DevBuf<int8_t> spins, init_stage, out_stage;
@@ -130,10 +131,6 @@ struct gdi_ctx {
         P.node_off = node_off.p;
         P.class_off = class_off.p;
         P.class_ptr = class_ptr.p;
-        for (int k = 0; k < 4; ++k) {
-            P.piece_off[k] = piece_off[k].p;
-            P.piece_ptr[k] = piece_ptr[k].p;
-        }
         P.row_ptr = row_ptr.p;
         P.col = col.p;
         P.col16 = col16.p;
@@ -152,7 +149,7 @@ struct gdi_ctx {
     void release()
     {
         node_off.release(); row_ptr.release(); class_off.release(); class_ptr.release();
-        for (int k = 0; k < 4; ++k) { piece_off[k].release(); piece_ptr[k].release(); }
+        pieces.release();
         rank_of.release(); col.release(); col16.release(); spins.release(); init_stage.release(); out_stage.release();
         tab.release(); tab_off.release(); temp.release(); raw_G.release(); final_G.release(); tr_G.release();
         err.release(); raw_cut.release(); final_cut.release(); tr_cut.release(); tr_digest.release();
@@ -542,8 +539,10 @@ int gdi_create(gdi_ctx **out, const gdi_graph *g, const gdi_model *m)
     }
     GDI_UP(c->class_off, class_off);
     GDI_UP(c->class_ptr, class_ptr);
-    // classes too large for the counting kernel's class buffers, in pieces
-    for (int k = 0; k < 4 && c->W >= 1 && c->W <= 256 && H.max_class > gdi_cta_piece(c->W, 1 << k); ++k) {
+    // classes too large for the counting kernel's class buffers, in pieces (a block holds two bytes a vertex)
+    std::vector<int32_t> all;
+    for (int k = 0; k < 4 && c->W >= 1 && c->W <= 256 && H.max_n < (1 << 17) && H.max_class > gdi_cta_piece(c->W, 1 << k);
+         ++k) {
         const int32_t piece = gdi_cta_piece(c->W, 1 << k);
         std::vector<int32_t> off(1, 0), ptr;
         for (int32_t q = 0; q < Q; ++q) {
@@ -552,9 +551,12 @@ int gdi_create(gdi_ctx **out, const gdi_graph *g, const gdi_model *m)
             ptr.push_back(class_ptr[(size_t)class_off[(size_t)q + 1] - 1]);
             off.push_back((int32_t)ptr.size());
         }
-        GDI_UP(c->piece_off[k], off);
-        GDI_UP(c->piece_ptr[k], ptr);
+        c->piece_at[k][0] = (int64_t)all.size();
+        all.insert(all.end(), off.begin(), off.end());
+        c->piece_at[k][1] = (int64_t)all.size();
+        all.insert(all.end(), ptr.begin(), ptr.end());
     }
+    if (!all.empty()) GDI_UP(c->pieces, all);
     GDI_UP(c->rank_of, rank_of);
     {
         // work queue order for the CTA path: largest instance (vertices + CSR entries) first
@@ -840,7 +842,12 @@ int gdi_anneal(gdi_ctx *c, const gdi_schedule *S, const gdi_run *run)
                                                " bytes of shared memory per block (limit " +
                                                std::to_string(max_optin) + "); use one instance with W > 0");
         if (timer.ev) cudaEventRecord(timer.ev[0], st);
-        int ke = gdi_launch_cta_anneal(P, R, block, c->grid_limit, st, &c->last_grid, &c->last_smem);
+        GdiCtaPieces pieces = {};
+        for (int k = 0; k < 4 && c->piece_at[k][1]; ++k) {
+            pieces.off[k] = c->pieces.p + c->piece_at[k][0];
+            pieces.ptr[k] = c->pieces.p + c->piece_at[k][1];
+        }
+        int ke = gdi_launch_cta_anneal(P, R, pieces, block, c->grid_limit, st, &c->last_grid, &c->last_smem);
         if (ke) return cuda_fail((cudaError_t)ke, "anneal kernel launch");
         if (timer.ev) {
             cudaEventRecord(timer.ev[1], st);

@@ -16,8 +16,6 @@ struct GdiDevProblem {
     const int64_t *node_off;         // [Q+1]
     const int32_t *class_off;        // [Q+1] offsets into class_ptr
     const int32_t *class_ptr;        // per instance: C_q + 1 class boundaries in local ranks
-    const int32_t *piece_off[4];     // the same for the classes in pieces of gdi_cta_piece(W, 1, 2, 4 and 8)
-    const int32_t *piece_ptr[4];     // ranks; null where no class is larger
     const int64_t *row_ptr;          // [N+1] rank-space CSR offsets
     const uint32_t *col;             // [nnz] local neighbour rank | (weight < 0) << 31
     const uint16_t *col16;           // [nnz] the same in 16 bits (rank | (weight < 0) << 15) when
@@ -86,8 +84,13 @@ int gdi_set_error(int code, const std::string &msg);
 // kernel launch wrappers (gdi_kernels.cu); return a cudaError_t as int
 int gdi_launch_init(const GdiDevProblem &P, int8_t *spins, const int8_t *init_orig, int init_kind,
                     uint32_t key0, uint32_t key1, void *stream);
-int gdi_launch_cta_anneal(const GdiDevProblem &P, const GdiDevRun &R, int block, int grid_limit,
-                          void *stream, int *grid_used, size_t *smem_used);
+// class_off and class_ptr for the classes in pieces of gdi_cta_piece(W, 1, 2, 4 and 8) ranks; null where no class is
+// larger
+struct GdiCtaPieces {
+    const int32_t *off[4], *ptr[4];
+};
+int gdi_launch_cta_anneal(const GdiDevProblem &P, const GdiDevRun &R, const GdiCtaPieces &pieces, int block,
+                          int grid_limit, void *stream, int *grid_used, size_t *smem_used);
 int gdi_cta_smem_bytes(const GdiDevProblem &P, const GdiDevRun &R, int block, int grid_limit, size_t *bytes);
 // threads per CTA-path block where the caller has set none
 int gdi_cta_default_block(const GdiDevProblem &P, const GdiDevRun &R, int grid_limit);

@@ -891,32 +891,32 @@ struct SortedCta {
 // Windows of one block whose stage maps are kept.  A class of more than so many for each of its blocks is
 // taken in pieces of that size, one after another like classes: its vertices share no edge, so a piece's
 // thresholds do not see the flips of the pieces before it, and only G passes on.  gdi_create lays the pieces
-// out for every cluster size as it does the classes, and the launch hands the kernel those in their place (the
-// kernel finding them itself spilled 640 bytes and lost 8 % with windows above 128, pieces or not).  (One warp that replayed such a
+// out for every cluster size as it does the classes, and the launch hands the kernel those in their place, with
+// their size as that of the largest class (the kernel finding them itself spilled 640 bytes and lost 8 % with
+// windows above 128, pieces or not).  (One warp that replayed such a
 // class window by window took 0.47 us a window.  A sweep of 40 replicas of 3,000 vertices, W = 1: 1,399 -> 314 us;
 // 300 of a 100 x 100 torus, W = 32: 257 -> 118.)
 constexpr int CTA_WALK_MAX = 128;
 
-// windows a block of a cluster of cl (1: alone) has of the largest piece: one or two windows are the first
-// block's
+// windows a block of a cluster of cl (1: alone) has of the largest class: a class of one or two windows
+// is the first block's
 __host__ __device__ inline int cta_own_windows(int32_t max_class, int W, int cl)
 {
-    const int all = (max_class + W - 1) / W, nw = all < CTA_WALK_MAX * cl ? all : CTA_WALK_MAX * cl;
+    const int nw = (max_class + W - 1) / W;
     return cl > 1 ? ((nw + cl - 1) / cl > 2 ? (nw + cl - 1) / cl : 2) : nw;
 }
 
-// its ranks
-__host__ __device__ inline int32_t cta_own_ranks(int32_t max_class, int W, int cl)
+__host__ __device__ inline int cta_walk_windows(int32_t max_class, int W, int cl)
 {
-    const int32_t own = cta_own_windows(max_class, W, cl) * W;
-    return own < max_class ? own : max_class;
+    const int nw = cta_own_windows(max_class, W, cl);
+    return nw < CTA_WALK_MAX ? nw : CTA_WALK_MAX;
 }
 
 // warps that count windows at once where the windows have no bins of their own: none where no class has
 // three windows; their bins share the repair flags' bytes, and a small instance has room for 16
 __host__ __device__ inline int cta_count_warps(int32_t max_n, int32_t max_class, int W, int BS, int cl)
 {
-    const int nwm = cta_own_windows(max_class, W, cl);
+    const int nwm = cta_walk_windows(max_class, W, cl);
     const int fit = max_n / 1024 > 16 ? max_n / 1024 : 16;
     const int nw = nwm < BS / 32 ? nwm : BS / 32;
     return (max_class + W - 1) / W < 3 ? 0 : (nw < fit ? nw : fit);
@@ -934,7 +934,8 @@ __host__ __device__ inline CtaSortedLayout cta_sorted_layout(const GdiDevProblem
                                                              int32_t stage, int32_t rofs, int nbw, int cl)
 {
     CtaSortedLayout L;
-    const size_t mc = (size_t)cta_own_ranks(P.max_class, P.W, cl) + 8;
+    const size_t own = cl > 1 ? (size_t)cta_own_windows(P.max_class, P.W, cl) * P.W : (size_t)P.max_class;
+    const size_t mc = own + 8;
     size_t o = 0;
     L.red64 = o; o = align16c(o + sizeof(int64_t) * (BS / 32 + 2));
     L.red32 = o; o = align16c(o + sizeof(int32_t) * (BS / 32 + 2));
@@ -950,7 +951,7 @@ __host__ __device__ inline CtaSortedLayout cta_sorted_layout(const GdiDevProblem
     L.gam = o; o = align16c(o + 4 * mc);
     L.es = o; o = align16c(o + 4 * mc);
     L.s0 = o; o = align16c(o + mc);
-    const int nwm = cta_own_windows(P.max_class, P.W, cl);
+    const int nwm = cta_walk_windows(P.max_class, P.W, cl);
     L.wmaps = o; o = align16c(o + sizeof(StageMap) * 2 * (size_t)nwm);
     L.wtab = o; o = align16c(o + (size_t)NT * nwm);
     L.rofs = o; o = align16c(o + (stage ? 4 * (mc > (size_t)rofs ? mc : (size_t)rofs) : 0));
@@ -1064,7 +1065,7 @@ __global__ void __launch_bounds__(BS, 1024 / BS) gdi_cta_sorted_kernel(GdiDevPro
             const int32_t size = s.chi - s.clo;
             s.nwin = (size + W - 1) / W;
             s.kq = CLUS ? (s.nwin + (int)CL - 1) / (int)CL : s.nwin;
-            s.walk = s.nwin >= 3;
+            s.walk = s.nwin >= 3 && s.kq <= CTA_WALK_MAX;
             if (!s.walk) s.kq = s.nwin;
             s.kb = min((int)crank * s.kq, s.nwin);
             s.nk = min(s.kq, s.nwin - s.kb);
@@ -1395,13 +1396,20 @@ __global__ void gdi_gather_kernel(GdiDevProblem P, const int8_t *spins, int8_t *
 // Algorithm 2 (GDI_DEV_STANDARD), larger windows and larger classes take gdi_cta_anneal_kernel
 constexpr size_t CTA_STATIC_SMEM = 3072;     // the kernel's class bounds and single words, rounded up
 
+// the problem as the counting kernel with clusters of cl blocks sees it: no class larger than a piece
+inline GdiDevProblem in_pieces(GdiDevProblem P, int cl)
+{
+    P.max_class = std::min(P.max_class, CTA_WALK_MAX * cl * P.W);
+    return P;
+}
+
 inline bool cta_sorted(const GdiDevProblem &P, const GdiDevRun &R, int BS)
 {
     if (P.W < 1 || P.W > 256 || (R.flags & GDI_DEV_STANDARD)) return false;
     int dev = 0, optin = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    return cta_sorted_layout(P, R.max_row, BS, 0, 0, 0, 0, 1).total + CTA_STATIC_SMEM <= (size_t)optin;
+    return cta_sorted_layout(in_pieces(P, 1), R.max_row, BS, 0, 0, 0, 0, 1).total + CTA_STATIC_SMEM <= (size_t)optin;
 }
 
 // blocks of a launch that are to run at once: one per SM, or the caller's limit
@@ -1428,7 +1436,7 @@ inline int cta_cluster(const GdiDevProblem &P, const GdiDevRun &R, int BS, int b
 // shared memory of the kernel that takes this call (counted windows, else whole-block windows)
 inline size_t cta_smem(const GdiDevProblem &P, const GdiDevRun &R, int BS, bool counted)
 {
-    return counted ? cta_sorted_layout(P, R.max_row, BS, R.cta_opts, R.cta_stage, R.cta_rofs, R.cta_bins, R.cta_cluster).total
+    return counted ? cta_sorted_layout(in_pieces(P, R.cta_cluster), R.max_row, BS, R.cta_opts, R.cta_stage, R.cta_rofs, R.cta_bins, R.cta_cluster).total
                    : cta_block_layout(P, R.max_row, BS, R.cta_opts, R.cta_stage).total;
 }
 
@@ -1466,7 +1474,7 @@ inline bool cta_options(const GdiDevProblem &P, GdiDevRun &R, int BS, int grid_l
         // bins for every window a block has of a class, up to 32, where a warp holds more than four members
         // a lane: a count over eight costs more than the bins do (one replica of W = 64 windows runs 5 to
         // 12 % faster without, 400 ER instances at W = 256 6 % slower)
-        if (P.W > 128) R.cta_bins = std::min(cta_own_windows(P.max_class, P.W, R.cta_cluster), 32);
+        if (P.W > 128) R.cta_bins = std::min(cta_own_windows(in_pieces(P, R.cta_cluster).max_class, P.W, R.cta_cluster), 32);
         if (resident() < want) R.cta_bins = 0;
     }
     take(CTA_OPT_ROWS2);
@@ -1524,7 +1532,7 @@ inline cudaLaunchConfig_t cta_cluster_config(int cl, int items, int BS, size_t s
 }
 
 template <int BS>
-int launch_cta(const GdiDevProblem &P0, const GdiDevRun &R0, int grid_limit, cudaStream_t st,
+int launch_cta(const GdiDevProblem &P0, const GdiDevRun &R0, const GdiCtaPieces &pieces, int grid_limit, cudaStream_t st,
                int *grid_used, size_t *smem_used)
 {
     GdiDevRun R = R0;
@@ -1541,12 +1549,13 @@ int launch_cta(const GdiDevProblem &P0, const GdiDevRun &R0, int grid_limit, cud
         const bool counted = cta_options(P0, R, BS, grid_limit, cap);
         P = P0;
         const int k = R.cta_cluster == 8 ? 3 : R.cta_cluster / 2;
-        if (counted && P.piece_ptr[k]) {
-            P.class_ptr = P.piece_ptr[k];
-            P.class_off = P.piece_off[k];
+        if (counted) P = in_pieces(P0, R.cta_cluster);
+        if (counted && pieces.ptr[k]) {
+            P.class_ptr = pieces.ptr[k];
+            P.class_off = pieces.off[k];
         }
-        const void *kern = cta_kernel<BS>(P, R);
-        smem = cta_smem(P, R, BS, counted);
+        const void *kern = cta_kernel<BS>(P0, R);
+        smem = cta_smem(P0, R, BS, counted);
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return (int)e;
         if (R.cta_cluster == 1) {
@@ -1625,7 +1634,9 @@ int gdi_cta_default_block(const GdiDevProblem &P, const GdiDevRun &R, int grid_l
     if (items > 2LL * sms && 4 * P.N >= 3LL * P.max_n * P.num_instances) return 256;
     const int cl = cta_cluster(P, R, 512, cta_blocks(grid_limit), 8);
     if (items * cl <= sms && cta_sorted(P, R, 512)) {
-        if (cta_own_ranks(P.max_class, P.W, cl) > 800) return 1024;
+        const GdiDevProblem Q = in_pieces(P, cl);
+        const int64_t own = cl > 1 ? (int64_t)cta_own_windows(Q.max_class, P.W, cl) * P.W : Q.max_class;
+        if (own > 800) return 1024;
         if (P.max_class < 128) return 256;
     }
     return 512;
@@ -1653,15 +1664,15 @@ int gdi_cta_smem_bytes(const GdiDevProblem &P, const GdiDevRun &R0, int block, i
     return 0;
 }
 
-int gdi_launch_cta_anneal(const GdiDevProblem &P, const GdiDevRun &R, int block, int grid_limit,
-                          void *stream, int *grid_used, size_t *smem_used)
+int gdi_launch_cta_anneal(const GdiDevProblem &P, const GdiDevRun &R, const GdiCtaPieces &pieces, int block,
+                          int grid_limit, void *stream, int *grid_used, size_t *smem_used)
 {
     cudaStream_t st = (cudaStream_t)stream;
     switch (block) {
-    case 128: return launch_cta<128>(P, R, grid_limit, st, grid_used, smem_used);
-    case 256: return launch_cta<256>(P, R, grid_limit, st, grid_used, smem_used);
-    case 512: return launch_cta<512>(P, R, grid_limit, st, grid_used, smem_used);
-    case 1024: return launch_cta<1024>(P, R, grid_limit, st, grid_used, smem_used);
+    case 128: return launch_cta<128>(P, R, pieces, grid_limit, st, grid_used, smem_used);
+    case 256: return launch_cta<256>(P, R, pieces, grid_limit, st, grid_used, smem_used);
+    case 512: return launch_cta<512>(P, R, pieces, grid_limit, st, grid_used, smem_used);
+    case 1024: return launch_cta<1024>(P, R, pieces, grid_limit, st, grid_used, smem_used);
     default: return (int)cudaErrorInvalidValue;
     }
 }

@@ -168,7 +168,7 @@ extern "C" int gdi_anneal_static(int32_t n, const int64_t *row_ptr, const uint32
     cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     const int nblk = sms < (int)ST_MAX_BLOCKS ? sms : (int)ST_MAX_BLOCKS;
 
-    GdiDevProblem P = {};
+    GdiDevProblem P;
     P.num_instances = 1;
     P.replicas = replicas;
     P.N = n;
