@@ -791,16 +791,18 @@ diffuse_kernel(const int64_t *graph_ptr, const uint32_t *graph_id, const int64_t
             const int r = 32 * s + lane;
             const int64_t e0 = r < n ? rp[perm[r]] : 0;
             const int d = deg[r], len = (int)(slice[s + 1] - slice[s]);
-            for (int k = 0; k < len; ++k) {
-                int room;
-                uint16_t *o = runs.at((int)slice[s] + k, room);
-                uint16_t at = (uint16_t)n;
-                if (k < d) {
-                    const int64_t j = col[e0 + k] - v0;
-                    if (j >= 0 && j < n) at = rank[j];
-                    else out = true;
+            for (int k0 = 0; k0 < len; k0 += 4) {      // four columns in flight
+                uint32_t j[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) j[u] = k0 + u < d ? (uint32_t)col[e0 + k0 + u] - (uint32_t)v0 : 0xFFFFFFFFu;
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const bool in = j[u] < (uint32_t)n;
+                    out |= k0 + u < d && !in;
+                    if (k0 + u >= len) break;
+                    int room;
+                    runs.at((int)slice[s] + k0 + u, room)[lane] = in ? rank[j[u]] : (uint16_t)n;
                 }
-                o[lane] = at;
             }
         }
         if (out) *cluster.map_shared_rank(&leaves, 0) = 1;
@@ -850,14 +852,12 @@ diffuse_kernel(const int64_t *graph_ptr, const uint32_t *graph_id, const int64_t
     } else {
         for (int64_t i = threadIdx.x; i < n64; i += DF_T) res[i * NRAND] = noise_sign((uint32_t)i, ch, id, k0, k1);
     }
-    // what walk_rest_kernel has to take (X is free again), in word 0 of each of the graph's vertices: 1 = this
-    // graph, 2 = the whole batch, since a column leads from this graph to another (block 0's `leaves`, written
-    // before the cluster's barriers).  Word 1 is walk_rest_kernel's own.
-    if (fits && ch != 0) return;
-    const int64_t i0 = fits ? threadIdx.x : (int64_t)ch * DF_T + threadIdx.x, step = fits ? DF_T : DF_CL * DF_T;
-    const float mark = !fits ? 1.f : (leaves ? 2.f : 0.f);
-    for (int64_t i = i0; i < n64; i += step) X[(v0 + i) * FIN] = mark;
-    if (ch == 0 && threadIdx.x == 0 && n64 > 0) X[v0 * FIN + 1] = 0.f;
+    // what walk_rest_kernel has to take (X is free again): 1 = this graph, 2 = the whole batch, since a column
+    // leads from this graph to another (written above before the cluster's barriers)
+    if (ch == 0 && threadIdx.x == 0 && n64 > 0) {
+        X[v0 * FIN] = !fits ? 1.f : (leaves ? 2.f : 0.f);
+        X[v0 * FIN + 1] = 0.f;                                         // walk_rest_kernel's own mark
+    }
 }
 
 // The walk steps of the graphs that diffuse_kernel marked, whose noise it left in R0: one cooperative
@@ -891,10 +891,13 @@ __global__ void __launch_bounds__(WR_T, 2) walk_rest_kernel(int64_t N, int G, co
     const int lane = threadIdx.x & 31, sub = lane >> 1, c4 = lane & 1;
     const int64_t wglob = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     float4 *in = reinterpret_cast<float4 *>(R0), *out = reinterpret_cast<float4 *>(R1);
-    // diffuse_kernel has looked at the columns of the graphs that fit it; here the others'
+    // every row takes its graph's mark; diffuse_kernel has looked at the columns of the graphs that fit it, here
+    // the others'
     for (int64_t i = wglob; i < N; i += nw) {
-        if (X[i * FIN] != 1.f) continue;
         const int64_t g = graph_of(graph_ptr, G, i), v0 = graph_ptr[g], v1 = graph_ptr[g + 1];
+        const float mark = X[v0 * FIN];
+        if (i != v0 && lane == 0) X[i * FIN] = mark;
+        if (mark != 1.f) continue;
         for (int64_t e = row_ptr[i] + lane; e < row_ptr[i + 1]; e += 32)
             if (col[e] < v0 || col[e] >= v1) X[v0 * FIN + 1] = 1.f;
     }
