@@ -62,7 +62,7 @@ extern "C" {
                              largest class has at least four windows for each block, a cluster of
                              2, 4 or 8 blocks anneals each item (gdi_last_launch counts them all) */
 #define GDI_PATH_GRID 2   /* one instance over every SM (needs W >= 1); up to 8 replicas per pass;
-                             windows counted, or tabulated (W > 256 where that fits alone)       */
+                             windows of up to 32,767 ranks                                       */
 
 /* gdi_run.flags */
 #define GDI_FLAG_TRACE     1  /* record per-sweep G, cut and state digest (slower; for parity)     */
@@ -244,7 +244,7 @@ int gdi_build_table(const gdi_schedule *schedule, uint32_t *tab, int64_t tab_cap
  * first use; gdi_anneal_static calls no cudaMalloc, cudaFree or allocating library routine.  It
  * runs the grid-scale sweep kernel of GDI_PATH_GRID on one graph whose arrays the caller already
  * holds on the device, in the rank-space layout below, with its scratch in one fixed-size static
- * device array of about 1.4 MB that every GPU which loads libgdi.so keeps until the process exits.
+ * device array of about 1.15 MB that every GPU which loads libgdi.so keeps until the process exits.
  *
  * Inputs (device pointers, current device, read only):
  *   row_ptr   [n + 1] int64 CSR offsets of the graph relabelled in rank order (the order described

@@ -76,8 +76,8 @@ struct gdi_ctx {
     int32_t max_n = 0, max_window = 0, max_degree = 0, max_class = 0, max_class_nnz = 0, max_item_nnz = 0;
     int32_t path = 0;                        // GDI_PATH_*
     DevBuf<uint8_t> g_packed, g_rflags;
-    DevBuf<int16_t> g_tables;
-    DevBuf<int32_t> g_gin, g_Gcls, g_err, g_status, g_rhist, g_rties, g_rparams;
+    DevBuf<unsigned char> g_chain;
+    DevBuf<int32_t> g_Gcls, g_err, g_status, g_rhist, g_rties, g_rparams;
     DevBuf<unsigned int> g_bar;
     DevBuf<unsigned long long> g_hfield;
     bool used_grid = false;
@@ -153,7 +153,7 @@ struct gdi_ctx {
         rank_of.release(); col.release(); col16.release(); spins.release(); init_stage.release(); out_stage.release();
         tab.release(); tab_off.release(); temp.release(); raw_G.release(); final_G.release(); tr_G.release();
         err.release(); raw_cut.release(); final_cut.release(); tr_cut.release(); tr_digest.release();
-        g_packed.release(); g_rflags.release(); g_tables.release(); g_gin.release(); g_Gcls.release();
+        g_packed.release(); g_rflags.release(); g_chain.release(); g_Gcls.release();
         g_wbnd.release();
         for (cudaEvent_t ev : kev) cudaEventDestroy(ev);
         kev.clear();
@@ -170,8 +170,7 @@ struct gdi_ctx {
     {
         GdiGridScratch X;
         X.packed = g_packed.p;
-        X.tables = g_tables.p;
-        X.gin = g_gin.p;
+        X.chain = g_chain.p;
         X.Gcls = g_Gcls.p;
         X.bar = g_bar.p;
         X.err = g_err.p;
@@ -498,8 +497,8 @@ int gdi_create(gdi_ctx **out, const gdi_graph *g, const gdi_model *m)
     int64_t most = 0;
     for (int32_t q = 0; q < Q; ++q) most = std::max(most, rp[(size_t)inst[(size_t)q + 1]] - rp[(size_t)inst[(size_t)q]]);
     c->max_item_nnz = most <= (1 << 20) ? (int32_t)most : 0;
-    // window costs for the grid path's weighted split: a rank costs its degree plus a constant for
-    // its threshold and its share of the window sort (both measured as about 12 neighbour reads)
+    // window costs for the grid path's weighted split: a rank costs its degree plus a constant for its threshold
+    // and its share of the window (12 neighbour reads, measured when windows were still sorted)
     if (Q == 1 && c->W >= 1) {
         const int32_t nclass = c->num_classes[0];
         c->wcost_off.assign((size_t)nclass + 1, 0);
@@ -813,8 +812,7 @@ int gdi_anneal(gdi_ctx *c, const gdi_schedule *S, const gdi_run *run)
             // a plan that does not fit so few blocks: as without the limit
             int spc, wpc;
             size_t grid_need;
-            bool counted;
-            if (gdi_grid_plan(P, max_row, std::min(c->grid_limit, sms), (size_t)max_optin, &spc, &wpc, &grid_need, &counted) != 0)
+            if (gdi_grid_plan(P, max_row, std::min(c->grid_limit, sms), (size_t)max_optin, &spc, &wpc, &grid_need) != 0)
                 grid = grid_wins(0);
         }
     }
@@ -860,16 +858,14 @@ int gdi_anneal(gdi_ctx *c, const gdi_schedule *S, const gdi_run *run)
         if (c->max_degree > 32767) return fail(GDI_ERR_TOO_LARGE, "degree above 32767 on the grid-scale path");
         int spc = 0, wpc = 0;
         size_t smem = 0;
-        bool counted = false;
         const int nblk = c->grid_limit > 0 ? std::min(c->grid_limit, sms) : sms;
-        if (gdi_grid_plan(P, max_row, nblk, (size_t)max_optin, &spc, &wpc, &smem, &counted) != 0)
+        if (gdi_grid_plan(P, max_row, nblk, (size_t)max_optin, &spc, &wpc, &smem) != 0)
             return fail(GDI_ERR_TOO_LARGE, "grid-scale plan needs " + std::to_string(smem) +
                                                " bytes of shared memory per block; use a smaller W");
         const int D = c->max_degree;
         e = c->g_packed.alloc((size_t)c->N);
         if (e == cudaSuccess) e = c->g_rflags.alloc((size_t)c->N);
-        if (e == cudaSuccess) e = c->g_tables.alloc((size_t)nblk * 8 * GDI_GRID_TW);
-        if (e == cudaSuccess) e = c->g_gin.alloc((size_t)nblk * 8);
+        if (e == cudaSuccess) e = c->g_chain.alloc(GDI_GRID_CHAIN_BYTES(nblk));
         if (e == cudaSuccess) e = c->g_Gcls.alloc(8);
         if (e == cudaSuccess) e = c->g_err.alloc(4);
         if (e == cudaSuccess) e = c->g_status.alloc(16);
@@ -877,7 +873,7 @@ int gdi_anneal(gdi_ctx *c, const gdi_schedule *S, const gdi_run *run)
         if (e == cudaSuccess) e = c->g_rties.alloc((size_t)8 * 152 * 4);
         if (e == cudaSuccess) e = c->g_rparams.alloc(32);
         if (e == cudaSuccess) e = c->g_bar.alloc(4);
-        if (e == cudaSuccess && counted) e = c->g_hfield.alloc((size_t)2 * c->N);
+        if (e == cudaSuccess) e = c->g_hfield.alloc((size_t)2 * c->N);
         if (e != cudaSuccess) return fail(GDI_ERR_OOM, "device allocation failed (grid scratch)");
         cudaMemsetAsync(c->g_err.p, 0, sizeof(int32_t), st);
         cudaMemsetAsync(c->g_status.p, 0, 16 * sizeof(int32_t), st);
@@ -888,7 +884,7 @@ int gdi_anneal(gdi_ctx *c, const gdi_schedule *S, const gdi_run *run)
             c->inject_limit = 0;
         }
         const int32_t *wbnd = nullptr;
-        if (counted && !c->wcost_off.empty()) {
+        if (!c->wcost_off.empty()) {
             if (c->wbnd_blocks != nblk || c->wbnd_wpc != wpc) {
                 const int ncls = (int)c->wcost_off.size() - 1;
                 std::vector<int32_t> bnd((size_t)ncls * (nblk + 1));
@@ -902,7 +898,7 @@ int gdi_anneal(gdi_ctx *c, const gdi_schedule *S, const gdi_run *run)
             }
             wbnd = c->g_wbnd.p;
         }
-        int ke = gdi_launch_grid_anneal(P, R, X, c->spins.p, nblk, spc, wpc, smem, counted, wbnd, &timer, st);
+        int ke = gdi_launch_grid_anneal(P, R, X, c->spins.p, nblk, spc, wpc, smem, wbnd, &timer, st);
         if (ke) return cuda_fail((cudaError_t)ke, "grid anneal launch");
         ke = gdi_launch_grid_finish(P, R, X, c->spins.p, (run->flags & GDI_FLAG_NO_REPAIR) ? 0 : 1, st);
         if (ke) return cuda_fail((cudaError_t)ke, "grid finish kernels");

@@ -4,25 +4,13 @@
 // colour classes in order, windows of W ranks, inside a window the +1 group by threshold ascending
 // then the -1 group by threshold descending, each seeing the exact running G).  What changes is
 // how the chain of windows is evaluated when a class holds thousands of windows spread over every
-// SM.  Common to both variants below: up to 8 replicas share one byte per vertex (bit r set = spin
-// of replica r is -1), so one gather of a neighbour byte feeds all of them (SWAR byte-lane
-// counters); every block owns a contiguous run of windows of each class; the map "G at window
-// start -> G at window end" is monotone and is tabulated around c, the G at class start.
-//
-// Counted-window variant (gdi_grid_sorted_kernel): the counts of a window's threshold distances give its
-// map and later its flips (gdi_window.cuh); block tables are published with the class parity in every
-// byte and each block finds its entering G by looking them up, so only one grid barrier per class remains
-// (described before the kernel).  The local fields are kept across classes and updated by the flips
-// (atomic adds to the neighbours).
-//
-// Tabulated variant (gdi_grid_anneal_kernel; W > 256 where the counted variant's buffers do not fit):
-//   * every window tabulates its map for G in [c - RT, c + RT] from two small histograms of its
-//     thresholds, and each block composes the maps of its consecutive windows;
-//   * after a grid barrier one block per replica walks the P block maps (a few hundred
-//     shared-memory lookups) and publishes every block's exact input G; an entry that left the
-//     tabulated range is recomputed exactly from the spins (fallback);
-//   * after a second barrier every block replays its windows with the exact input, flips, and a
-//     third barrier makes the class's spins visible to the next class.
+// SM.  Up to 8 replicas share one byte per vertex (bit r set = spin of replica r is -1), so one gather of a
+// neighbour byte feeds all of them (SWAR byte-lane counters); every block owns a contiguous run of windows of
+// each class.  The map "G at window start -> G at window end" is monotone and is tabulated on a lattice around
+// c, the G at class start: the counts of a window's threshold distances give its map and later its flips
+// (gdi_window.cuh).  Block tables are published with the class parity in every byte and each block finds its
+// entering G by looking them up, so one grid barrier per class remains (described before the kernel).  The
+// local fields are kept across classes and updated by the flips (atomic adds to the neighbours).
 //
 // Grid barriers are sense/generation barriers on global counters with a bounded spin, and every
 // other wait (tables, exact G words) is bounded too: a block that waits too long sets the error word and the kernel returns
@@ -42,11 +30,6 @@ namespace {
 constexpr int GB = 768;                 // threads per block
 constexpr int NWARP = GB / 32;
 static_assert(GB % 32 == 0, "whole warps; the threshold loop keeps one replica per thread");
-constexpr int RT = 64;                  // tables cover G in [c - RT, c + RT]
-constexpr int TW = 2 * RT + 1;
-static_assert(TW == GDI_GRID_TW, "table width mismatch");
-constexpr int HB = 2 * RT + 4 * KC + 1; // histogram bins for building a window table (KC: gdi_window.cuh)
-constexpr int16_t TINV = INT16_MIN;
 constexpr int LONG_ROW = 48;
 
 __device__ __forceinline__ int warp_id() { return threadIdx.x >> 5; }
@@ -57,36 +40,7 @@ __device__ __forceinline__ uint64_t spread8(uint32_t b)
            ((uint64_t)(b >> 7) << 56);
 }
 
-struct GridLayout {
-    int spc, wpc, P, max_row;
-    size_t off_h, off_gam, off_s0, off_fm, off_longq, off_wtab, off_win, off_hist, off_ctab, off_row,
-        off_misc, total;
-};
-
 __host__ __device__ inline size_t align16(size_t x) { return (x + 15) & ~(size_t)15; }
-
-__host__ __device__ inline GridLayout grid_layout(int spc, int wpc, int P, int max_row)
-{
-    GridLayout L;
-    L.spc = spc;
-    L.wpc = wpc;
-    L.P = P;
-    L.max_row = max_row;
-    size_t o = 0;
-    L.off_h = o; o = align16(o + (size_t)spc * 8 * sizeof(int16_t));
-    L.off_gam = o; o = align16(o + (size_t)spc * 8 * sizeof(int32_t));
-    L.off_s0 = o; o = align16(o + (size_t)spc);
-    L.off_fm = o; o = align16(o + (size_t)((spc + 3) / 4) * sizeof(uint32_t));
-    L.off_longq = o; o = align16(o + (size_t)spc * sizeof(int32_t));
-    L.off_wtab = o; o = align16(o + (size_t)wpc * 8 * TW * sizeof(int16_t));
-    L.off_win = o; o = align16(o + (size_t)wpc * 8 * sizeof(int32_t));
-    L.off_hist = o; o = align16(o + (size_t)NWARP * 2 * HB * sizeof(int32_t));
-    L.off_ctab = o; o = align16(o + (size_t)P * TW * sizeof(int16_t));
-    L.off_row = o; o = align16(o + (size_t)(max_row + 4) * sizeof(uint32_t));
-    L.off_misc = o; o = align16(o + 64 * sizeof(int64_t));
-    L.total = o;
-    return L;
-}
 
 struct GridArgs {
     GdiDevProblem P;
@@ -96,9 +50,9 @@ struct GridArgs {
     int spc, wpc;
     const int32_t *wbnd;    // [classes][blocks + 1] first window of every block, or null (even split)
     unsigned long long *hf; // maintained fields (X.hfield) when this kernel keeps them, else null
-    bool es_pre;            // counted path: E* of the next class drawn ahead into shared memory
-    bool tables;            // counted path: window maps composed as tables
-    bool binned;            // counted path: thresholds counted into their window's bins as they are made
+    bool es_pre;            // E* of the next class drawn ahead into shared memory
+    bool tables;            // window maps composed as tables
+    bool binned;            // thresholds counted into their window's bins as they are made
 };
 
 // ---------------------------------------------------------------------------------------------
@@ -137,9 +91,9 @@ __device__ bool grid_sync(const GdiGridScratch &X)
 }
 
 // local fields of one rank (row entries [e0, e1)) for all 8 replicas, thread-serial over the row,
-// written to hout[0..7] (all replicas) or hout[0] (replica `one` only)
+// written to hout[0..7]
 __device__ __forceinline__ void field8_thread(const GdiDevProblem &P, int64_t base, int64_t e0, int64_t e1,
-                                              const uint8_t *packed, int16_t *hout, int one)
+                                              const uint8_t *packed, int16_t *hout)
 {
     uint64_t aP = 0, aN = 0;
     int32_t nN = 0, cnt = 0;
@@ -179,18 +133,10 @@ __device__ __forceinline__ void field8_thread(const GdiDevProblem &P, int64_t ba
 #undef GDI_FLUSH
     const int32_t sw = (int32_t)(e1 - e0) - 2 * nN;     // sum of weights
     // h = sum w (1 - 2 bit) = sum w - 2 sum w bit
-    if (one < 0) {
-        hout[0] = (int16_t)(sw - 2 * (cP0 - cN0)); hout[1] = (int16_t)(sw - 2 * (cP1 - cN1));
-        hout[2] = (int16_t)(sw - 2 * (cP2 - cN2)); hout[3] = (int16_t)(sw - 2 * (cP3 - cN3));
-        hout[4] = (int16_t)(sw - 2 * (cP4 - cN4)); hout[5] = (int16_t)(sw - 2 * (cP5 - cN5));
-        hout[6] = (int16_t)(sw - 2 * (cP6 - cN6)); hout[7] = (int16_t)(sw - 2 * (cP7 - cN7));
-    } else {
-        const int32_t cp = one == 0 ? cP0 : one == 1 ? cP1 : one == 2 ? cP2 : one == 3 ? cP3
-                         : one == 4 ? cP4 : one == 5 ? cP5 : one == 6 ? cP6 : cP7;
-        const int32_t cn = one == 0 ? cN0 : one == 1 ? cN1 : one == 2 ? cN2 : one == 3 ? cN3
-                         : one == 4 ? cN4 : one == 5 ? cN5 : one == 6 ? cN6 : cN7;
-        hout[0] = (int16_t)(sw - 2 * (cp - cn));
-    }
+    hout[0] = (int16_t)(sw - 2 * (cP0 - cN0)); hout[1] = (int16_t)(sw - 2 * (cP1 - cN1));
+    hout[2] = (int16_t)(sw - 2 * (cP2 - cN2)); hout[3] = (int16_t)(sw - 2 * (cP3 - cN3));
+    hout[4] = (int16_t)(sw - 2 * (cP4 - cN4)); hout[5] = (int16_t)(sw - 2 * (cP5 - cN5));
+    hout[6] = (int16_t)(sw - 2 * (cP6 - cN6)); hout[7] = (int16_t)(sw - 2 * (cP7 - cN7));
 }
 
 // Partial sums of one chunk [c0, c1) of a long row (c1 - c0 <= LCHUNK), by one warp: sw = sum of
@@ -268,16 +214,8 @@ __device__ __forceinline__ void flip_words(uint32_t f, uint32_t s, unsigned long
 
 // ---------------------------------------------------------------------------------------------
 struct GSmem {
-    int16_t *h;        // [spc][8]
-    int32_t *gam;      // [spc][8]
-    uint8_t *s0;       // [spc]
-    uint32_t *fm;      // [spc/4]
     int32_t *longq;    // [spc]
-    int16_t *wtab;     // [wpc][8][TW]
-    int32_t *win;      // [wpc][8]
-    int32_t *hist;     // [NWARP][2][HB] (tabulated path)
     int32_t *nchunk;   // [spc] chunk counts of the long rows
-    int16_t *ctab;     // [P][TW]
     uint32_t *row;     // [max_row]
     int64_t *misc;     // scratch
 };
@@ -371,17 +309,15 @@ __device__ void estar_ahead(const GridArgs &A, const uint32_t *row, int32_t a0, 
     }
 }
 
-// Thresholds of the spin range [a0, a1).  all_reps: every replica, threshold of (i, r) stored at
-// gam_out[i * gis + r * grs] (fields in hbuf [i*8 + r], rows longer than LONG_ROW summed by a
-// warp).  Otherwise only replica `one`, stored at gam_out[i * gis] with fields [i] (thread-serial
-// rows; used by the rare exact fallback).  gam_out must hold 8 ints per rank either way (the
+// Thresholds of the spin range [a0, a1): the threshold of (i, r) is stored at gam_out[i + r * grs] (fields in
+// hbuf [i*8 + r], rows longer than LONG_ROW summed by a warp).  gam_out must hold 8 ints per rank (the
 // long-row partial sums live there before the thresholds are written).
 // seen(i, r, negative, threshold) is called once per threshold (after gc_out is visible).
 struct NoThreshold { __device__ void operator()(int32_t, int, bool, int32_t) const {} };
 
 template <class Seen = NoThreshold>
 __device__ void range_thresholds(const GridArgs &A, const GSmem &S, int32_t a0, int32_t a1, int sw,
-                                 bool all_reps, int one, int32_t *gam_out, int gis, int grs, uint8_t *s0_out,
+                                 int32_t *gam_out, int grs, uint8_t *s0_out,
                                  int16_t *hbuf, int32_t rlen, float Tsw, bool quad_rows = false,
                                  const int16_t *es_in = nullptr, int es_s = 0, int32_t *gc_out = nullptr,
                                  int32_t gc_val = 0, const Seen &seen = Seen())
@@ -390,11 +326,10 @@ __device__ void range_thresholds(const GridArgs &A, const GSmem &S, int32_t a0, 
     const int64_t base = P.node_off[0];
     const uint8_t *packed = A.X.packed;
     const int32_t ns = a1 - a0;
-    const int hs = all_reps ? 8 : 1;
     __shared__ int nlong;
     if (threadIdx.x == 0) nlong = 0;
     __syncthreads();
-    const bool kept = all_reps && A.hf != nullptr;
+    const bool kept = A.hf != nullptr;
     if (kept) {
         // kept fields: the start signs and field words of up to KU ranks per thread are all in
         // flight before any is used (one L2 round trip instead of one per rank)
@@ -427,18 +362,15 @@ __device__ void range_thresholds(const GridArgs &A, const GSmem &S, int32_t a0, 
         const int32_t rk = a0 + i;
         s0_out[i] = __ldcg(packed + base + rk);
         const int64_t e0 = P.row_ptr[base + rk], e1 = P.row_ptr[base + rk + 1];
-        if (all_reps && e1 - e0 > LONG_ROW) {
-            S.longq[atomicAdd(&nlong, 1)] = i;
-        } else {
-            field8_thread(P, base, e0, e1, packed, all_reps ? hbuf + (size_t)i * 8 : hbuf + i, all_reps ? -1 : one);
-        }
+        if (e1 - e0 > LONG_ROW) S.longq[atomicAdd(&nlong, 1)] = i;
+        else field8_thread(P, base, e0, e1, packed, hbuf + (size_t)i * 8);
     }
     __syncthreads();
-    if (all_reps && !kept) {
+    if (!kept) {
         // long rows: chunks of LCHUNK entries are warp tasks; partial sums meet in shared memory.
         // acc[i*8 + k] = sum_j w_ij bit_k(j) lives in the threshold array (free until the
         // thresholds are written below); sum_j w_ij lives in the first 4 bytes of the row's
-        // field slots; the chunk count of long row t is kept in the histogram area.
+        // field slots.
         const int nl = nlong;
         int32_t *acc = gam_out;
         int32_t *nchunk = S.nchunk;              // [nl]
@@ -481,7 +413,7 @@ __device__ void range_thresholds(const GridArgs &A, const GSmem &S, int32_t a0, 
     }
     if (ns > 0) {
         const int32_t q0 = a0 >> 2, q1 = (a1 - 1) >> 2;
-        const int nr = all_reps ? A.nrep : 1;
+        const int nr = A.nrep;
         const int a_shift = (P.A > 0 && (P.A & (P.A - 1)) == 0) ? 2 + __ffs(P.A) - 1 : -1;   // log2(4A)
         // one Philox block per (quad of ranks, replica)
         auto quad = [&](int32_t qd, int r) {
@@ -494,10 +426,10 @@ __device__ void range_thresholds(const GridArgs &A, const GSmem &S, int32_t a0, 
                 if (rk < a0 || rk >= a1) continue;
                 const int32_t i = rk - a0;
                 const int sg = ((s0_out[i] >> r) & 1) ? -1 : 1;
-                const int32_t h = hbuf[(size_t)i * hs + (all_reps ? r : 0)];
+                const int32_t h = hbuf[(size_t)i * 8 + r];
                 const int32_t es = estar_of(S.row, rlen, A.R.mode, word_of(u4, j), Tsw);
                 const int32_t gm = a_shift >= 0 ? gamma_of_shift(sg, h, es, P.A, P.B, a_shift) : gamma_of(sg, h, es, P.A, P.B);
-                gam_out[(size_t)i * gis + (size_t)(all_reps ? r : 0) * grs] = gm;
+                gam_out[i + (size_t)r * grs] = gm;
                 seen(i, r, sg < 0, gm);
             }
         };
@@ -544,68 +476,10 @@ __device__ void range_thresholds(const GridArgs &A, const GSmem &S, int32_t a0, 
             const int r = threadIdx.x & 7;
             for (int32_t qq = threadIdx.x >> 3; qq < nq; qq += GB / 8) quad(q0 + qq, r);
         } else {
-            for (int32_t t = threadIdx.x; t < nq * nr; t += GB) quad(q0 + t / nr, all_reps ? t % nr : one);
+            for (int32_t t = threadIdx.x; t < nq * nr; t += GB) quad(q0 + t / nr, t % nr);
         }
     }
     __syncthreads();
-}
-
-// table of one window (positions [ws, we)) for replica r over G in [c - RT, c + RT], by one warp
-__device__ void window_table(const GSmem &S, int ws, int we, int r, int32_t c, bool plus_first,
-                             int32_t *hp, int32_t *hm, int16_t *tab)
-{
-    const int lane = threadIdx.x & 31;
-    const int64_t base = (int64_t)c - RT - 2 * KC;
-    for (int b = lane; b < HB; b += 32) { hp[b] = 0; hm[b] = 0; }
-    __syncwarp();
-    int32_t under = 0, over = 0;
-    for (int i = ws + lane; i < we; i += 32) {
-        const bool neg = (S.s0[i] >> r) & 1;
-        const int64_t b = (int64_t)S.gam[(size_t)i * 8 + r] - base;
-        if (!neg) {
-            if (b < 0) ++under;
-            else if (b < HB) atomicAdd(&hp[b], 1);
-        } else {
-            if (b >= HB) ++over;
-            else if (b >= 0) atomicAdd(&hm[b], 1);
-        }
-    }
-    under = warp_sum(under);
-    over = warp_sum(over);
-    __syncwarp();
-    warp_cumulate(hp, HB, under, true);     // C(base + b)
-    warp_cumulate(hm, HB, over, false);     // D(base + b)
-    for (int e = lane; e < TW; e += 32) {
-        int64_t g = (int64_t)c - RT + e;
-        bool valid = true;
-        for (int ph = 0; ph < 2 && valid; ++ph) {
-            const bool plus = plus_first ? (ph == 0) : (ph == 1);
-            // K = #{k in [0, KC] : count(g -/+ 2k) >= k + 1}; the predicate holds for a prefix of
-            // k, so K is found by binary search; K = KC + 1 means the table cannot represent it
-            int32_t lo = 0, hi = KC + 1;
-            while (lo < hi) {
-                const int32_t mid = (lo + hi + 1) >> 1;          // does k = mid - 1 hold?
-                const int64_t v = plus ? g - 2 * (mid - 1) : g + 2 * (mid - 1);
-                const int32_t cnt = plus ? hp[v - base] : hm[v - base];
-                if (cnt >= mid) lo = mid; else hi = mid - 1;
-            }
-            const int32_t K = lo;
-            if (K > KC) valid = false;
-            g = plus ? g - 2 * K : g + 2 * K;
-        }
-        tab[e] = valid ? (int16_t)(g - ((int64_t)c - RT)) : TINV;
-    }
-    __syncwarp();
-}
-
-// exact output G of a window (both groups), by one warp
-__device__ int32_t window_exact(const int32_t *gam, int gs, int gc, const uint8_t *s0, int r, int ws,
-                                int we, int32_t g, bool plus_first, int32_t *bins)
-{
-    const int32_t K1 = warp_group(gam, gs, gc, s0, r, ws, we, g, plus_first, bins, nullptr);
-    g = plus_first ? g - 2 * K1 : g + 2 * K1;
-    const int32_t K2 = warp_group(gam, gs, gc, s0, r, ws, we, g, !plus_first, bins, nullptr);
-    return plus_first ? g + 2 * K2 : g - 2 * K2;
 }
 
 // G of every replica: n - 2 #(-1), accumulated into X.Gcls (zeroed by the host)
@@ -629,7 +503,6 @@ __device__ __noinline__ void init_G(const GridArgs &A, int p, int Pb, int32_t n,
     if (p == 0 && threadIdx.x < nrep) atomicAdd(&X.Gcls[threadIdx.x], n);
 }
 
-// digest and cut of every replica after sweep sw (grid-wide atomics), and G after the sweep
 // maintained fields of every rank from the packed spins at launch start
 __device__ __noinline__ void init_fields(const GridArgs &A, int p, int Pb, int32_t n, int64_t base)
 {
@@ -639,7 +512,7 @@ __device__ __noinline__ void init_fields(const GridArgs &A, int p, int Pb, int32
         const int64_t e0 = P.row_ptr[base + rk], e1 = P.row_ptr[base + rk + 1];
         if (e1 - e0 > LONG_ROW) continue;
         int16_t h[8];
-        field8_thread(P, base, e0, e1, A.X.packed, h, -1);
+        field8_thread(P, base, e0, e1, A.X.packed, h);
         H[2 * (base + rk)] = field_word(h);
         H[2 * (base + rk) + 1] = field_word(h + 4);
     }
@@ -666,6 +539,7 @@ __device__ __noinline__ void init_fields(const GridArgs &A, int p, int Pb, int32
     }
 }
 
+// digest and cut of every replica after sweep sw (grid-wide atomics), and G after the sweep
 __device__ __noinline__ void sweep_trace(const GridArgs &A, int p, int Pb, int32_t n, int64_t base, int sw)
 {
     const GdiDevProblem &P = A.P;
@@ -712,187 +586,8 @@ __device__ __noinline__ void sweep_trace(const GridArgs &A, int p, int Pb, int32
             *(volatile int32_t *)&X.Gcls[threadIdx.x];
 }
 
-__global__ void __launch_bounds__(GB, 1) gdi_grid_anneal_kernel(GridArgs A)
-{
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ int chain_pp;
-    __shared__ int32_t chain_g;
-    const GdiDevProblem &P = A.P;
-    const GdiDevRun &R = A.R;
-    const GdiGridScratch &X = A.X;
-    const int Pb = gridDim.x, p = blockIdx.x;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const GridLayout L = grid_layout(A.spc, A.wpc, Pb, R.max_row);
-    GSmem S;
-    S.h = reinterpret_cast<int16_t *>(smem_raw + L.off_h);
-    S.gam = reinterpret_cast<int32_t *>(smem_raw + L.off_gam);
-    S.s0 = reinterpret_cast<uint8_t *>(smem_raw + L.off_s0);
-    S.fm = reinterpret_cast<uint32_t *>(smem_raw + L.off_fm);
-    S.longq = reinterpret_cast<int32_t *>(smem_raw + L.off_longq);
-    S.wtab = reinterpret_cast<int16_t *>(smem_raw + L.off_wtab);
-    S.win = reinterpret_cast<int32_t *>(smem_raw + L.off_win);
-    S.hist = reinterpret_cast<int32_t *>(smem_raw + L.off_hist);
-    S.nchunk = S.hist;   // spc <= NWARP * 2 * HB, checked by the plan
-    S.ctab = reinterpret_cast<int16_t *>(smem_raw + L.off_ctab);
-    S.row = reinterpret_cast<uint32_t *>(smem_raw + L.off_row);
-    S.misc = reinterpret_cast<int64_t *>(smem_raw + L.off_misc);
-    int32_t *Gc = reinterpret_cast<int32_t *>(S.misc);   // [8] class-start G of each replica
-    const int64_t base = P.node_off[0];
-    const int32_t n = (int32_t)(P.node_off[1] - base);
-    const int32_t *cls = P.class_ptr + P.class_off[0];
-    const int32_t ncls = P.class_off[1] - P.class_off[0] - 1;
-    const int W = P.W;
-    const int nrep = A.nrep;
-
-    if (!plan_fits(A)) return;
-    init_G(A, p, Pb, n, base);
-    if (!grid_sync(X)) return;
-
-    for (int sw = R.s_begin; sw < R.s_end; ++sw) {
-        const int32_t roff = R.tab_off[sw];
-        const int32_t rlen = R.tab_off[sw + 1] - roff;
-        for (int k = threadIdx.x; k < rlen; k += GB) S.row[k] = R.tab[roff + k];
-        const float Tsw = R.temp ? R.temp[sw] : 0.f;
-        const bool plus_first = (sw & 1) == 0;
-        __syncthreads();
-        for (int c = 0; c < ncls; ++c) {
-            const int32_t lo = cls[c], hi = cls[c + 1];
-            int32_t a0, a1;
-            int nwin;
-            class_partition(lo, hi, W, p, Pb, a0, a1, nwin);
-            if (threadIdx.x < nrep) Gc[threadIdx.x] = *(volatile int32_t *)&X.Gcls[threadIdx.x];
-            // ---- phase A: thresholds of my windows, window tables, block table
-            range_thresholds(A, S, a0, a1, sw, true, 0, S.gam, 8, 1, S.s0, S.h, rlen, Tsw);
-            for (int task = warp; task < nwin * nrep; task += NWARP) {
-                const int kk = task / nrep, r = task % nrep;
-                const int ws = kk * W, we = min(ws + W, a1 - a0);
-                window_table(S, ws, we, r, Gc[r], plus_first, S.hist + (size_t)warp * 2 * HB,
-                             S.hist + (size_t)warp * 2 * HB + HB, S.wtab + ((size_t)kk * 8 + r) * TW);
-            }
-            __syncthreads();
-            if (warp < nrep) {
-                const int r = warp;
-                for (int e = lane; e < TW; e += 32) {
-                    int32_t idx = e;
-                    for (int kk = 0; kk < nwin; ++kk) {
-                        if (idx < 0 || idx >= TW) { idx = TINV; break; }
-                        const int16_t v = S.wtab[((size_t)kk * 8 + r) * TW + idx];
-                        if (v == TINV) { idx = TINV; break; }
-                        idx = v;
-                    }
-                    X.tables[((size_t)p * 8 + r) * TW + e] = (int16_t)idx;
-                }
-            }
-            if (!grid_sync(X)) return;
-            // ---- phase C: one block per replica chains the block tables
-            if (p < nrep) {
-                const int r = p;
-                for (int pp = warp; pp < Pb; pp += NWARP) {
-                    const int16_t *src = X.tables + ((size_t)pp * 8 + r) * TW;
-                    int16_t v[(TW + 31) / 32];
-#pragma unroll
-                    for (int j = 0; j < (TW + 31) / 32; ++j)
-                        v[j] = (lane + 32 * j < TW) ? __ldcg(src + lane + 32 * j) : (int16_t)0;
-#pragma unroll
-                    for (int j = 0; j < (TW + 31) / 32; ++j)
-                        if (lane + 32 * j < TW) S.ctab[(size_t)pp * TW + lane + 32 * j] = v[j];
-                }
-                const int32_t c0 = Gc[r];
-                if (threadIdx.x == 0) { chain_pp = 0; chain_g = c0; }
-                __syncthreads();
-                while (true) {
-                    if (threadIdx.x == 0) {
-                        int pp = chain_pp;
-                        int32_t g = chain_g;
-                        while (pp < Pb) {
-                            const int64_t idx = (int64_t)g - ((int64_t)c0 - RT);
-                            if (idx < 0 || idx >= TW) break;
-                            const int16_t v = S.ctab[(size_t)pp * TW + idx];
-                            if (v == TINV) break;
-                            X.gin[(size_t)pp * 8 + r] = g;
-                            g = (int32_t)((int64_t)c0 - RT + v);
-                            ++pp;
-                        }
-                        chain_pp = pp;
-                        chain_g = g;
-                    }
-                    __syncthreads();
-                    const int pp = chain_pp;
-                    const int32_t g = chain_g;
-                    __syncthreads();
-                    if (pp >= Pb) break;
-                    // exact fallback for block pp: its thresholds for replica r, recomputed into the
-                    // histogram area (free during this phase)
-                    if (threadIdx.x == 0) X.gin[(size_t)pp * 8 + r] = g;
-                    int32_t b0, b1;
-                    int nw2;
-                    class_partition(lo, hi, W, pp, Pb, b0, b1, nw2);
-                    const int32_t nb = b1 - b0;
-                    int32_t *fg = S.hist;
-                    int16_t *fh = reinterpret_cast<int16_t *>(fg + nb);
-                    uint8_t *fs = reinterpret_cast<uint8_t *>(fh + ((nb + 7) & ~7));
-                    int32_t *fbins = reinterpret_cast<int32_t *>(fs + ((nb + 15) & ~15));
-                    range_thresholds(A, S, b0, b1, sw, false, r, fg, 1, 0, fs, fh, rlen, Tsw);
-                    if (warp == 0) {
-                        int32_t gg = g;
-                        for (int kk = 0; kk < nw2; ++kk) {
-                            const int ws = kk * W, we = min(ws + W, nb);
-                            gg = window_exact(fg, 1, 0, fs, r, ws, we, gg, plus_first, fbins);
-                        }
-                        if (lane == 0) {
-                            chain_pp = pp + 1;
-                            chain_g = gg;
-                            atomicAdd(X.status + r, 1);
-                        }
-                    }
-                    __syncthreads();
-                }
-                if (threadIdx.x == 0) X.Gcls[r] = chain_g;
-            }
-            if (!grid_sync(X)) return;
-            // ---- phase D: inputs of my windows, then the exact flips of every (window, replica)
-            for (int i = threadIdx.x; i < (a1 - a0 + 3) / 4; i += GB) S.fm[i] = 0;
-            if (warp < nrep) {
-                const int r = warp;
-                int32_t g = __ldcg(X.gin + (size_t)p * 8 + r);
-                const int32_t cbase = Gc[r] - RT;
-                int32_t *bins = S.hist + (size_t)warp * 2 * HB;
-                for (int kk = 0; kk < nwin; ++kk) {
-                    if (lane == 0) S.win[kk * 8 + r] = g;
-                    const int64_t idx = (int64_t)g - cbase;
-                    int16_t v = TINV;
-                    if (idx >= 0 && idx < TW) v = S.wtab[((size_t)kk * 8 + r) * TW + idx];
-                    if (v != TINV) {
-                        g = cbase + v;
-                    } else {
-                        const int ws = kk * W, we = min(ws + W, a1 - a0);
-                        g = window_exact(S.gam, 8, r, S.s0, r, ws, we, g, plus_first, bins);
-                    }
-                }
-            }
-            __syncthreads();
-            for (int task = warp; task < nwin * nrep; task += NWARP) {
-                const int kk = task / nrep, r = task % nrep;
-                const int ws = kk * W, we = min(ws + W, a1 - a0);
-                int32_t *bins = S.hist + (size_t)warp * 2 * HB;
-                int32_t g = S.win[kk * 8 + r];
-                const int32_t K1 = warp_group(S.gam, 8, r, S.s0, r, ws, we, g, plus_first, bins, S.fm);
-                g = plus_first ? g - 2 * K1 : g + 2 * K1;
-                warp_group(S.gam, 8, r, S.s0, r, ws, we, g, !plus_first, bins, S.fm);
-            }
-            __syncthreads();
-            for (int32_t i = threadIdx.x; i < a1 - a0; i += GB) {
-                const uint8_t f = (uint8_t)(S.fm[i >> 2] >> (8 * (i & 3)));
-                if (f) X.packed[base + a0 + i] = S.s0[i] ^ f;
-            }
-            if (!grid_sync(X)) return;
-        }
-        if (R.flags & GDI_DEV_TRACE) sweep_trace(A, p, Pb, n, base, sw);
-    }
-}
-
 // =============================================================================================
-// Counted-window path.
+// The sweep kernel.
 //
 // Every threshold is counted into its (window, replica)'s 128 bins of distances from the class-start G c as
 // it is made; one warp per (window, replica) turns the bins into prefix counts, the window's two stage maps
@@ -971,7 +666,7 @@ __host__ __device__ inline SortedLayout sorted_layout(int spc, int wpc, int max_
     return L;
 }
 
-// chain buffers carved from the scratch table area: exact outgoing G [P][8] (epoch << 32 | G),
+// chain buffers carved from X.chain: exact outgoing G [P][8] (epoch << 32 | G),
 // block tables [P][8][64], run tables [NR][8][64]
 __host__ __device__ inline size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 __host__ __device__ inline size_t chain_off_tab(int P) { return align256((size_t)P * 8 * sizeof(uint64_t)); }
@@ -1136,7 +831,7 @@ __global__ void __launch_bounds__(GB, 1) gdi_grid_sorted_kernel(GridArgs A)
     S.row = reinterpret_cast<uint32_t *>(smem_raw + L.off_row);
     S.misc = reinterpret_cast<int64_t *>(smem_raw + L.off_misc);
     int32_t *Gc = reinterpret_cast<int32_t *>(S.misc);   // [8] class-start G of each replica
-    unsigned char *cb = reinterpret_cast<unsigned char *>(X.tables);
+    unsigned char *cb = X.chain;
     unsigned long long *exg = reinterpret_cast<unsigned long long *>(cb);
     int8_t *tabs = reinterpret_cast<int8_t *>(cb + chain_off_tab(Pb));
     int8_t *rtabs = reinterpret_cast<int8_t *>(cb + chain_off_rtab(Pb));
@@ -1212,7 +907,7 @@ __global__ void __launch_bounds__(GB, 1) gdi_grid_sorted_kernel(GridArgs A)
             // ---- thresholds of my ranks (ends with a block barrier)
             // thresholds of rank a0 + i for replica r at gamc[r * gs + i]
             int32_t *gamc = gam + (a0 & 3);
-            range_thresholds(A, S, a0, a1, sw, true, 0, gamc, 1, L.gs, s0, hb, rlen, Tsw, true,
+            range_thresholds(A, S, a0, a1, sw, gamc, L.gs, s0, hb, rlen, Tsw, true,
                              have_es ? esb : nullptr, L.es, threadIdx.x < nrep ? Gc : nullptr, gcl,
                              [&](int32_t i, int r, bool neg, int32_t gm) {
                                  if (!A.binned) return;
@@ -1595,7 +1290,7 @@ __global__ void __launch_bounds__(GB, 1) gdi_grid_racy_kernel(GridArgs A)
                 class_partition(cls[c], cls[c + 1], P.W, p, Pb, a0, a1, nwin);
             }
             const int32_t ns = a1 - a0;
-            range_thresholds(A, S, a0, a1, sw, true, 0, gam, 1, spc, s0, hb, rlen, Tsw);
+            range_thresholds(A, S, a0, a1, sw, gam, spc, s0, hb, rlen, Tsw);
             for (int i = threadIdx.x; i < (ns + 3) / 4; i += GB) fm[i] = 0;
             __syncthreads();
             for (int r = 0; r < nrep; ++r) {
@@ -1850,14 +1545,14 @@ __global__ void repair_apply_kernel(int8_t *spins, int64_t N, int nrep, const ui
 }  // namespace
 
 // ---------------------------------------------------------------------------------------------
-// what the counted kernel keeps beyond the necessary: 1 E* rows, 2 also tables, 3 also bins
+// what the sweep kernel keeps beyond the necessary: 1 E* rows, 2 also tables, 3 also bins
 static SortedLayout planned_layout(int spc, int wpc, int max_row, int sms, int level)
 {
     return sorted_layout(spc, wpc, max_row, sms, level >= 1, level >= 2, level >= 3);
 }
 
 int gdi_grid_plan(const GdiDevProblem &P, int max_row, int sms, size_t smem_limit, int *spc, int *wpc,
-                  size_t *smem, bool *counted)
+                  size_t *smem)
 {
     if (P.num_instances != 1 || P.W < 1) return -1;
     // the kernels' static shared memory (class bounds, a few words) counts against the same limit
@@ -1866,27 +1561,17 @@ int gdi_grid_plan(const GdiDevProblem &P, int max_row, int sms, size_t smem_limi
     const int wp = (int)((P.max_class + P.W - 1) / P.W);
     const int w = (wp + sms - 1) / sms;
     *wpc = w < 1 ? 1 : w;
+    *smem = 0;
+    if (P.W > CMAXW) return -1;             // (32,768 ranks a block would not fit either)
     *spc = *wpc * P.W;
-    *counted = true;
-    if (P.W <= CMAXW) {
-        // the cost-weighted split stays within the even share of windows per block: more shared
-        // memory per block (less L1) costs more than the finer balance gains
-        // with rows for the E* drawn ahead, tables and bins for every window while they fit
-        for (int level = 3; level >= 0; --level) {
-            *smem = planned_layout(*spc, *wpc, max_row, sms, level).total;
-            if (*smem <= smem_limit) return 0;
-        }
-        if (P.W <= SMAXW) return -1;
+    // the cost-weighted split stays within the even share of windows per block: more shared
+    // memory per block (less L1) costs more than the finer balance gains
+    // with rows for the E* drawn ahead, tables and bins for every window while they fit
+    for (int level = 3; level >= 0; --level) {
+        *smem = planned_layout(*spc, *wpc, max_row, sms, level).total;
+        if (*smem <= smem_limit) return 0;
     }
-    // larger windows whose buffers do not fit the counted path (its E* and push queue take about 10 bytes
-    // a rank more): tabulated.  It keeps the long rows' chunk counts in the histogram area, and its exact
-    // chain fallback the thresholds, fields, start signs and bins of one block's windows (one
-    // replica)
-    *counted = false;
-    if ((size_t)*spc > (size_t)NWARP * 2 * HB) return -1;
-    if ((size_t)*spc * 7 + 64 + HA * sizeof(int32_t) > (size_t)NWARP * 2 * HB * sizeof(int32_t)) return -1;
-    *smem = grid_layout(*spc, *wpc, sms, max_row).total;
-    return *smem <= smem_limit ? 0 : -1;
+    return -1;
 }
 
 constexpr double LAST_SHARE = 0.6;
@@ -1930,15 +1615,13 @@ void gdi_grid_window_bounds(const int64_t *cost, const int64_t *cost_off, int nu
 }
 
 int gdi_launch_grid_anneal(const GdiDevProblem &P, const GdiDevRun &R, const GdiGridScratch &X,
-                           int8_t *spins, int sms, int spc, int wpc, size_t smem, bool counted,
+                           int8_t *spins, int sms, int spc, int wpc, size_t smem,
                            const int32_t *wbnd, GdiKernelTimer *timer, void *stream)
 {
     cudaStream_t st = (cudaStream_t)stream;
     const bool racy = (R.flags & GDI_DEV_RACY) != 0;
-    const bool sorted = counted && !racy;
     if (racy) smem = planned_layout(spc, wpc, R.max_row, sms, 0).total;
     const void *kern = racy ? (const void *)gdi_grid_racy_kernel
-                     : !sorted ? (const void *)gdi_grid_anneal_kernel
                      : P.W <= 32 ? (const void *)gdi_grid_sorted_kernel<1>
                      : P.W <= 64 ? (const void *)gdi_grid_sorted_kernel<2>
                      : P.W <= 128 ? (const void *)gdi_grid_sorted_kernel<4>
@@ -1950,8 +1633,7 @@ int gdi_launch_grid_anneal(const GdiDevProblem &P, const GdiDevRun &R, const Gdi
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, GB, smem);
     if (e != cudaSuccess) return (int)e;
     if (per_sm < 1) return (int)cudaErrorCooperativeLaunchTooLarge;
-    // the sorted path's chain buffers (exact G, flags, byte tables) live in the table area
-    if (sorted && chain_bytes(sms) > (size_t)sms * 8 * TW * sizeof(int16_t)) return (int)cudaErrorInvalidValue;
+    if (chain_bytes(sms) > GDI_GRID_CHAIN_BYTES(sms)) return (int)cudaErrorInvalidValue;
     const int pg = (int)((P.N + 255) / 256) < 4096 ? (int)((P.N + 255) / 256) : 4096;
     for (int g0 = 0; g0 < P.replicas; g0 += 8) {
         const int nrep = P.replicas - g0 < 8 ? P.replicas - g0 : 8;
@@ -1959,7 +1641,7 @@ int gdi_launch_grid_anneal(const GdiDevProblem &P, const GdiDevRun &R, const Gdi
         cudaMemsetAsync(X.Gcls, 0, 8 * sizeof(int32_t), st);
         cudaMemsetAsync(X.bar, 0, 4 * sizeof(unsigned int), st);
         if (X.bar_start) set_word_kernel<<<1, 1, 0, st>>>(X.bar + 2, 1u);
-        if (sorted) cudaMemsetAsync(X.tables, 0, chain_bytes(sms), st);
+        if (!racy) cudaMemsetAsync(X.chain, 0, chain_bytes(sms), st);
         GridArgs A;
         A.P = P;
         A.R = R;
@@ -1968,14 +1650,14 @@ int gdi_launch_grid_anneal(const GdiDevProblem &P, const GdiDevRun &R, const Gdi
         A.nrep = nrep;
         A.spc = spc;
         A.wpc = wpc;
-        A.wbnd = (sorted || racy) ? wbnd : nullptr;
-        A.hf = sorted ? X.hfield : nullptr;
+        A.wbnd = wbnd;
+        A.hf = racy ? nullptr : X.hfield;
         // the level the plan's size stands for
         int level = 3;
         while (level > 0 && smem < planned_layout(spc, wpc, R.max_row, sms, level).total) --level;
-        A.es_pre = sorted && level >= 1 && R.max_row < 32000;
-        A.tables = sorted && level >= 2;
-        A.binned = sorted && level >= 3;
+        A.es_pre = level >= 1 && R.max_row < 32000;
+        A.tables = level >= 2;
+        A.binned = level >= 3;
         void *args[] = {&A};
         const bool timed = timer && timer->ev && timer->n < timer->cap;
         if (timed) cudaEventRecord(timer->ev[2 * timer->n], st);

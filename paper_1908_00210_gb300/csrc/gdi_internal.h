@@ -34,10 +34,8 @@ struct GdiDevProblem {
 // Global scratch of the grid-scale path (single large instance).
 struct GdiGridScratch {
     uint8_t *packed;                 // [N] spins of one replica group: bit r set = replica r is -1
-    int16_t *tables;                 // [P][8][TW] composed window tables of every block (W > 256);
-                                     // for W <= 256 the same bytes hold the sorted path's exact-G
-                                     // words and [P][8][64] byte block and run tables
-    int32_t *gin;                    // [P][8] exact G entering every block's windows
+    unsigned char *chain;            // [GDI_GRID_CHAIN_BYTES(P)] exact-G words, [P][8][64] byte block tables and run
+                                     // tables
     int32_t *Gcls;                   // [8] G at class start / after the class
     unsigned int *bar;               // [4] grid barrier: 64-bit arrival count, gate, unused
     int32_t *err;                    // [1] device error word
@@ -46,8 +44,8 @@ struct GdiGridScratch {
     uint8_t *rflags;                 // [N] repair flips (bit per replica)
     int32_t *rties;                  // [8][blocks] repair ties per block
     int32_t *rparams;                // [8][4] repair k, majority, kappa, ties to take
-    unsigned long long *hfield;      // [N][2] maintained local fields of the replica group (the
-                                     // sorted-window path), or null: fields gathered every class
+    unsigned long long *hfield;      // [N][2] maintained local fields of the replica group, or null: fields
+                                     // gathered every class
     long long spin_limit;            // polls before a device wait gives up (error word set)
     unsigned int bar_start;          // nonzero: the barrier's gate starts closed (test hook)
 };
@@ -104,11 +102,10 @@ struct GdiCtaPlan {
 int32_t gdi_cta_piece(int32_t W, int32_t cluster);
 int gdi_cta_plan(const GdiDevProblem &P, const GdiDevRun &R, int block, int grid_limit, GdiCtaPlan *plan);
 // Grid plan for `sms` blocks: spans of ranks (spc) and windows (wpc) per block and per class, and
-// the dynamic shared memory; counted: the counted-window kernel runs it (else the tabulated one); -1 if
-// the instance does not fit smem_limit.
+// the dynamic shared memory; -1 if the instance does not fit smem_limit.
 int gdi_grid_plan(const GdiDevProblem &P, int max_row, int sms, size_t smem_limit, int *spc, int *wpc,
-                  size_t *smem, bool *counted);
-// Host: first window of every block, per class, for the sorted-window grid path.  cost[k] is the
+                  size_t *smem);
+// Host: first window of every block, per class, for the grid path.  cost[k] is the
 // cost of window k of the class (windows of one class consecutive, class c starting at
 // cost_off[c]); every block gets at most wpc windows.  bnd has num_classes * (blocks + 1) entries.
 void gdi_grid_window_bounds(const int64_t *cost, const int64_t *cost_off, int num_classes, int blocks,
@@ -120,8 +117,8 @@ struct GdiKernelTimer {
     int n;                           // pairs recorded
 };
 int gdi_launch_grid_anneal(const GdiDevProblem &P, const GdiDevRun &R, const GdiGridScratch &X,
-                           int8_t *spins, int sms, int spc, int wpc, size_t smem, bool counted,
-                           const int32_t *wbnd, GdiKernelTimer *timer, void *stream);
+                           int8_t *spins, int sms, int spc, int wpc, size_t smem, const int32_t *wbnd,
+                           GdiKernelTimer *timer, void *stream);
 int gdi_launch_grid_finish(const GdiDevProblem &P, const GdiDevRun &R, const GdiGridScratch &X,
                            int8_t *spins, int do_repair, void *stream);
 int gdi_launch_gather_spins(const GdiDevProblem &P, const int8_t *spins_rank, int8_t *out_orig,
@@ -138,4 +135,5 @@ int gdi_launch_gather_spins(const GdiDevProblem &P, const int8_t *spins_rank, in
 #define GDI_DEVERR_TIMEOUT 2
 #define GDI_DEVERR_INPUT 3     // an input check of the launch failed (sizes the caller passed)
 
-#define GDI_GRID_TW 129   // entries of a window table (2 * 64 + 1)
+// chain buffers of P blocks: 64 + 512 bytes a block, 512 for every 16, alignment
+#define GDI_GRID_CHAIN_BYTES(P) ((size_t)(P) * 608 + 1024)

@@ -4,8 +4,8 @@
 // allocator (a framework's caching pool or a fixed arena), or a process that must not grow its
 // device footprint after start-up.  gdi_anneal allocates its table, staging and grid scratch on
 // first use, so those callers cannot use it.  This entry point runs the same grid-scale sweep
-// kernel, but its scratch (packed spins of one 8-replica group, the per-block window tables, the
-// chain inputs, the class-start magnetisations, the barrier counters and the error word) lives in
+// kernel, but its scratch (packed spins of one 8-replica group, the blocks' chain tables,
+// the class-start magnetisations, the barrier counters and the error word) lives in
 // one file-scope __device__ array of fixed size, which every GPU that loads the library holds
 // until the process exits.  The caller passes every input and output as device pointers.
 #include <cuda_runtime.h>
@@ -24,9 +24,8 @@ constexpr size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 constexpr size_t ST_MAX_N = (size_t)GDI_STATIC_MAX_VERTICES;
 constexpr size_t ST_MAX_BLOCKS = (size_t)GDI_STATIC_MAX_BLOCKS;
 constexpr size_t OFF_PACKED = 0;
-constexpr size_t OFF_TABLES = OFF_PACKED + align256(ST_MAX_N);
-constexpr size_t OFF_GIN = OFF_TABLES + align256(ST_MAX_BLOCKS * 8 * GDI_GRID_TW * sizeof(int16_t));
-constexpr size_t OFF_GCLS = OFF_GIN + align256(ST_MAX_BLOCKS * 8 * sizeof(int32_t));
+constexpr size_t OFF_CHAIN = OFF_PACKED + align256(ST_MAX_N);
+constexpr size_t OFF_GCLS = OFF_CHAIN + align256(GDI_GRID_CHAIN_BYTES(ST_MAX_BLOCKS));
 constexpr size_t OFF_BAR = OFF_GCLS + 256;
 constexpr size_t OFF_ERR = OFF_BAR + 256;
 constexpr size_t OFF_STATUS = OFF_ERR + 256;
@@ -190,15 +189,13 @@ extern "C" int gdi_anneal_static(int32_t n, const int64_t *row_ptr, const uint32
     P.max_item_nnz = 0;
     int spc = 0, wpc = 0;
     size_t smem = 0;
-    bool counted = false;
-    if (gdi_grid_plan(P, max_row, nblk, (size_t)optin, &spc, &wpc, &smem, &counted) != 0)
+    if (gdi_grid_plan(P, max_row, nblk, (size_t)optin, &spc, &wpc, &smem) != 0)
         return gdi_set_error(GDI_ERR_TOO_LARGE, "gdi_anneal_static: the plan needs " + std::to_string(smem) +
                                                     " bytes of shared memory per block; use a smaller W");
 
     GdiGridScratch X;
     X.packed = base + OFF_PACKED;
-    X.tables = reinterpret_cast<int16_t *>(base + OFF_TABLES);
-    X.gin = reinterpret_cast<int32_t *>(base + OFF_GIN);
+    X.chain = base + OFF_CHAIN;
     X.Gcls = reinterpret_cast<int32_t *>(base + OFF_GCLS);
     X.bar = reinterpret_cast<unsigned int *>(base + OFF_BAR);
     X.err = reinterpret_cast<int32_t *>(base + OFF_ERR);
@@ -248,7 +245,7 @@ extern "C" int gdi_anneal_static(int32_t n, const int64_t *row_ptr, const uint32
         static_rows_check_kernel<<<cb, 256, 0, st>>>(n, row_ptr, max_degree, X.err);
         static_cols_check_kernel<<<cb, 256, 0, st>>>(n, row_ptr, col, class_ptr, num_classes, X.err);
     }
-    const int ke = gdi_launch_grid_anneal(P, R, X, spins, nblk, spc, wpc, smem, counted, nullptr, nullptr, st);
+    const int ke = gdi_launch_grid_anneal(P, R, X, spins, nblk, spc, wpc, smem, nullptr, nullptr, st);
     if (ke) return gdi_set_error(GDI_ERR_CUDA, std::string("gdi_anneal_static launch: ") +
                                                    cudaGetErrorString((cudaError_t)ke));
     return GDI_OK;

@@ -17,8 +17,6 @@
 namespace gdi {
 namespace win {
 
-constexpr int KC = 31;                  // flips per group the exact counting histogram covers at once
-constexpr int HA = 2 * KC + 1;          // histogram bins of the exact counting replay
 constexpr int NT = 64;                  // lattice points of a stage map
 constexpr int WBINS = 256;              // words a window's distances are counted in
 constexpr int BIN_L = 190;              // distance -BIN_L is bin 0 (everything below too) in 256 bins
@@ -29,174 +27,6 @@ struct StageMap {
     int32_t ylo;                        // output index of lattice point 0
     int32_t pad;
 };
-
-// In-place cumulative counts of bins[0, nb) by one warp: forward (bins[x] = base + sum_{b <= x})
-// or backward (bins[x] = base + sum_{b >= x}); each lane scans a contiguous chunk.
-__device__ inline void warp_cumulate(int32_t *bins, int nb, int32_t base, bool forward)
-{
-    const int lane = threadIdx.x & 31;
-    const int ch = (nb + 31) / 32;
-    const int l = forward ? lane : 31 - lane;          // chunk order along the scan direction
-    const int b0 = l * ch, b1 = min(b0 + ch, nb);
-    int32_t loc = 0;
-    for (int b = b0; b < b1; ++b) loc += bins[b];
-    // lanes in increasing order hold the chunks in scan order (backward: lane 0 owns the top
-    // chunk), so an inclusive scan over lane order gives the sum up to and including my chunk
-    int32_t x = loc;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int32_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
-        if (lane >= o) x += y;
-    }
-    int32_t run = base + x - loc;                       // everything before my chunk
-    if (forward) {
-        for (int b = b0; b < b1; ++b) { run += bins[b]; bins[b] = run; }
-    } else {
-        for (int b = b1 - 1; b >= b0; --b) { run += bins[b]; bins[b] = run; }
-    }
-    __syncwarp();
-}
-
-// ---------------------------------------------------------------------------------------------
-// Exact decision of one group of one window for one replica, by one warp.
-// Members are window positions i in [ws, we) whose start sign (bit r of s0[i]) is the group's;
-// gam[i * gs + r] are their thresholds.  +1 group: the k-th member in (gamma asc, position asc)
-// order flips iff g - 2k >= gamma_(k).  -1 group: (gamma desc, position asc), flips iff
-// g + 2k <= gamma_(k).  Returns the number of flips K; marks them in fm (if fm != null).
-__device__ inline int32_t warp_count(const int32_t *gam, int gs, int gc, const uint8_t *s0, int r, int ws,
-                              int we, bool plus, int64_t v)
-{
-    const int lane = threadIdx.x & 31;
-    int32_t c = 0;
-    for (int i = ws + lane; i < we; i += 32) {
-        const bool neg = (s0[i] >> r) & 1;
-        if (plus != !neg) continue;
-        const int64_t gm = gam[(size_t)i * gs + gc];
-        c += plus ? (gm <= v) : (gm >= v);
-    }
-    return warp_sum(c);
-}
-
-__device__ inline int32_t warp_group(const int32_t *gam, int gs, int gc, const uint8_t *s0, int r, int ws,
-                              int we, int32_t g, bool plus, int32_t *bins, uint32_t *fm)
-{
-    const int lane = threadIdx.x & 31;
-    // histogram of thresholds over [g - 2KC, g] (+) or [g, g + 2KC] (-); beyond: "deep" members
-    const int64_t base = plus ? (int64_t)g - 2 * KC : (int64_t)g;
-    for (int b = lane; b < HA; b += 32) bins[b] = 0;
-    __syncwarp();
-    int32_t deep = 0;
-    for (int i = ws + lane; i < we; i += 32) {
-        const bool neg = (s0[i] >> r) & 1;
-        if (plus == neg) continue;
-        const int64_t gm = gam[(size_t)i * gs + gc];
-        const int64_t b = gm - base;
-        if (plus) {
-            if (b < 0) ++deep;
-            else if (b < HA) atomicAdd(&bins[b], 1);
-        } else {
-            if (b >= HA) ++deep;
-            else if (b >= 0) atomicAdd(&bins[b], 1);
-        }
-    }
-    deep = warp_sum(deep);
-    __syncwarp();
-    // cumulative counts toward the deep side: plus: C(base + x) = deep + sum_{b <= x};
-    // minus: D(base + x) = deep + sum_{b >= x}
-    warp_cumulate(bins, HA, deep, plus);
-    // K = #{k : count(g -/+ 2k) >= k + 1}, k in [0, KC] (one lane per k)
-    int32_t K;
-    int64_t vstar = 0;
-    int32_t t = 0;
-    bool slow;
-    {
-        const int k = lane;   // KC + 1 == 32 lanes
-        const int x = plus ? (HA - 1) - 2 * k : 2 * k;
-        const bool pred = bins[x] >= k + 1;
-        const unsigned m = __ballot_sync(0xFFFFFFFFu, pred);
-        K = __popc(m);
-        slow = (m >> 31) & 1;   // K may exceed KC
-    }
-    if (!slow) {
-        if (K == 0) return 0;
-        if (K <= deep) {
-            // all K flips are deep members (K == deep here: K >= min(deep, KC + 1))
-            vstar = plus ? base : base + HA - 1;   // flips: exactly the deep members
-            t = 0;
-        } else {
-            // v* = the K-th value in group order; t = ties at v* that flip
-            int first = -1;
-            for (int x0 = 0; x0 < HA; x0 += 32) {
-                const int x = x0 + lane;
-                bool pred = false;
-                if (x < HA) pred = plus ? (bins[x] >= K) : (bins[HA - 1 - x] >= K);
-                const unsigned m = __ballot_sync(0xFFFFFFFFu, pred);
-                if (m) { first = x0 + __ffs(m) - 1; break; }
-            }
-            if (plus) {
-                vstar = base + first;
-                const int32_t before = first > 0 ? bins[first - 1] : deep;
-                t = K - before;
-            } else {
-                const int xb = HA - 1 - first;
-                vstar = base + xb;
-                const int32_t before = xb < HA - 1 ? bins[xb + 1] : deep;
-                t = K - before;
-            }
-        }
-    } else {
-        // exact counting path: K = max{k + 1 : count(g -/+ 2k) >= k + 1}
-        const int32_t n0 = warp_count(gam, gs, gc, s0, r, ws, we, plus, g);
-        int32_t lo = 0, hi = n0;   // K in [0, n0]
-        while (lo < hi) {
-            const int32_t mid = (lo + hi + 1) >> 1;   // test k = mid - 1
-            const int64_t v = plus ? (int64_t)g - 2 * (int64_t)(mid - 1) : (int64_t)g + 2 * (int64_t)(mid - 1);
-            if (warp_count(gam, gs, gc, s0, r, ws, we, plus, v) >= mid) lo = mid; else hi = mid - 1;
-        }
-        K = lo;
-        if (K == 0) return 0;
-        // v*: plus: smallest v with C(v) >= K; minus: largest v with D(v) >= K
-        int64_t a = -((int64_t)1 << 31), b = (int64_t)1 << 31;
-        if (plus) {
-            b = (int64_t)g - 2 * (int64_t)(K - 1);
-            while (a < b) {
-                const int64_t mid = a + ((b - a) >> 1);
-                if (warp_count(gam, gs, gc, s0, r, ws, we, true, mid) >= K) b = mid; else a = mid + 1;
-            }
-            vstar = a;
-            t = K - warp_count(gam, gs, gc, s0, r, ws, we, true, vstar - 1);
-        } else {
-            a = (int64_t)g + 2 * (int64_t)(K - 1);
-            while (a < b) {
-                const int64_t mid = a + ((b - a + 1) >> 1);
-                if (warp_count(gam, gs, gc, s0, r, ws, we, false, mid) >= K) a = mid; else b = mid - 1;
-            }
-            vstar = a;
-            t = K - warp_count(gam, gs, gc, s0, r, ws, we, false, vstar + 1);
-        }
-    }
-    if (fm) {
-        int32_t run = 0;
-        for (int i0 = ws; i0 < we; i0 += 32) {
-            const int i = i0 + lane;
-            bool mem = false, strict = false, tie = false;
-            if (i < we) {
-                const bool neg = (s0[i] >> r) & 1;
-                mem = (plus != neg);
-                if (mem) {
-                    const int64_t gm = gam[(size_t)i * gs + gc];
-                    strict = plus ? (gm < vstar) : (gm > vstar);
-                    tie = (gm == vstar);
-                }
-            }
-            const unsigned tm = __ballot_sync(0xFFFFFFFFu, tie);
-            const int32_t idx = run + __popc(tm & ((1u << lane) - 1u));
-            run += __popc(tm);
-            if (strict || (tie && idx < t)) atomicOr(&fm[i >> 2], 1u << (8 * (i & 3) + r));
-        }
-    }
-    return K;
-}
 
 // counts of all bins before this lane's PER, by one warp
 template <int PER>
