@@ -456,7 +456,7 @@ __device__ __forceinline__ void team_thresholds(const GdiDevProblem &P, const in
 // reads both groups' flips off the bins -- members flip in e order, the k-th iff e >= 2k, so the first
 // k with N(2k) <= k is the number of flips K, and the last one has e >= 2K, = 2K - 1 or = 2K - 2; the
 // second group sees the same margins shifted by the first group's 2K -- and then every thread decides its
-// ranks, equal margins by position.  Four block barriers per window (two less where no tie is cut); a
+// ranks, equal margins by position.  Three block barriers per window, four where a tie is cut; a
 // counting pass and a scan per group with its own barriers took about 26.  Draws and rows of the next
 // window are prepared by the other warps while one reads the bins, as in the counting kernel.  Measured:
 // ER 2000, 8 replicas, whole-class windows, 200 sweeps 23.7 -> 7.3 ms; Algorithm 2 on a 71 x 71 torus, 100 sweeps
@@ -856,7 +856,7 @@ __global__ void __launch_bounds__(BS, 1024 / BS) gdi_cta_block_kernel(GdiDevProb
 }
 
 // ---------------------------------------------------------------------------------------------
-// CTA-resident counting kernel (1 <= W <= 256): the same results as gdi_cta_anneal_kernel with far
+// CTA-resident counting kernel (1 <= W <= 256): the same results as gdi_cta_block_kernel with far
 // fewer block barriers per window.  Per colour class:
 //   1. thresholds of the class's ranks: a team of T lanes sums a rank's row over the shared spins;
 //   2. a class of three or more windows: the counts of each window's threshold distances give its stage
@@ -876,7 +876,7 @@ __global__ void __launch_bounds__(BS, 1024 / BS) gdi_cta_block_kernel(GdiDevProb
 // is a few shared loads.  Measured, whole call, with sorted windows, draws and rows on the chain -> now:
 // ER-800, one replica, 1000 sweeps 63.7 -> 42.6 ms; 640 ER instances, 500 sweeps 98.7 -> 43.9 ms; 1024 anneals
 // of 25 sweeps 8.0 -> 4.8 ms; torus 100 x 100, 64 replicas, 5000 sweeps (two blocks each) 148 -> 98.8 ms; BA
-// 20,000, one replica, 300 sweeps (eight blocks) 20.7 (grid path) -> 14.8 ms.
+// 20,000, one replica, 300 sweeps (eight blocks) 20.7 (grid path) -> 15.3 ms.
 struct SortedCta {
     int32_t *gam;       // [own ranks] flip thresholds of my share of the class
     int32_t *es;        // [own ranks] E* of the next class's, drawn ahead
@@ -1393,7 +1393,7 @@ __global__ void gdi_gather_kernel(GdiDevProblem P, const int8_t *spins, int8_t *
 
 // the sorted-window kernel serves every window size 1 .. 256 (one instantiation per members per
 // lane) of the running-G method when its whole-class buffers fit in a block's shared memory;
-// Algorithm 2 (GDI_DEV_STANDARD), larger windows and larger classes take gdi_cta_anneal_kernel
+// Algorithm 2 (GDI_DEV_STANDARD), larger windows and larger classes take gdi_cta_block_kernel
 constexpr size_t CTA_STATIC_SMEM = 3072;     // the kernel's class bounds and single words, rounded up
 
 // the problem as the counting kernel with clusters of cl blocks sees it: no class larger than a piece
